@@ -508,7 +508,7 @@ int chfsi_filter(const chfsi_matrix* H, const double* X, int64_t ldx, double* Y,
     coefficients(m, a, b, a0, al, be, R.c);
     CHFSI_CUDA_TRY(cudaMemsetAsync(R.st, 0, sizeof(unsigned), R.s));
     make_devs(H, H->csr.val, H->bsr.val, Buf::F64, &R.csr64, &R.bsr64);
-    if (oz_tail && (rc = ozaki_bsr_prepare(R.bsr64, slab, R.fl.oz, R.fl.oz_bytes, R.st, R.s))) return rc;
+    if (oz_tail && (rc = ozaki_bsr_prepare(R.bsr64, slab, R.c, R.fl.oz, R.fl.oz_bytes, R.st, R.s))) return rc;
     if (H->kind == CHFSI_SPLIT) {
         // the off-diagonal part through the CSR kernel; the dense blocks sliced once
         const chfsi_csr& o = H->split.off;
@@ -963,7 +963,7 @@ int rr_run_ozaki(const chfsi_matrix* H, const double* Y, int64_t ldy, int64_t N,
         CsrDev csr{};
         BsrDev bsr{};
         make_devs(H, H->csr.val, H->bsr.val, Buf::F64, &csr, &bsr);
-        if ((rc = ozaki_bsr_prepare(bsr, n, rl.oz, rl.oz_bytes, st, s))) return rc;
+        if ((rc = ozaki_bsr_prepare(bsr, n, 0.0, rl.oz, rl.oz_bytes, st, s))) return rc;
         if ((rc = ozaki_bsr_step(bsr, n, XF, ldw, nullptr, 0, HXF, ldw, 1.0, 0.0, 0.0, rl.oz, rl.oz_bytes, st, s)))
             return rc;
     } else if (has_csr(H)) {

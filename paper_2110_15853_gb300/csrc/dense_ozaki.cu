@@ -10,50 +10,56 @@
 // |A_hat[r][k]| 2^{-e_r} < 1/2 for all k, and the scaled value a is rounded to a
 // 56-bit fixed-point number and written as seven balanced base-256 digits
 //     a = sum_{t=1..7} d_t 2^{-8t},   d_t integer, |d_t| <= 128,
-// (integer arithmetic on the FP64 bit pattern; no FP64 instructions).  Slice t
-// stores d_t 2^{-8t} in BF16, which is exact (8 significant bits).  Then
-//     C_ij = 2^{e_i + f_j} sum_{t + u <= 8} sum_k a_t[i][k] b_u[j][k]
+// (integer arithmetic on the FP64 bit pattern; no FP64 instructions).  Slice t stores the
+// integers d_t in BF16, which is exact (8 significant bits).  Then
+//     C_ij = 2^{e_i + f_j} sum_{t + u <= 8} 2^{-8(t+u)} sum_k a_t[i][k] b_u[j][k]
 // keeps every digit product of weight 2^{-64} and above (28 slice pairs; the
 // dropped pairs and the 56-bit rounding are below about 2^{-55} of the row scales
 // per term, i.e. about 2^{-48} of a typical term).
 //
-// Exact accumulation.  A product of two slices is d_t g_u 2^{-8(t+u)}, an integer
-// multiple of 2^{-8l} at level l = t + u with |d_t g_u| <= 2^14.  Every level l = 2 .. 8
-// has its own FP32 accumulator E_l in TMEM, and each is drained before its sums can
-// pass 2^24 units (levels 2-5 every 256 K, levels 6-8 every 128 K; at most 4 and 7
-// pairs per level), so the tensor-core accumulation -- which truncates rather than
-// rounds -- never rounds at all: the sums are exact integers.  The drains add them to
-// two 64-bit integers per output element, levels 2-5 in units of 2^{-40} and levels
-// 6-8 in units of 2^{-64}.  A work item spans at most 8192 K (longer sums are split
-// over items and the FP64 partial tiles added), which bounds the integers by 2^51 and
-// 2^46.  C = 2^{e_i + f_j} (2^{-40} hi + 2^{-64} lo), converted once at the end, so the
-// only errors are the 56-bit rounding of the inputs and the dropped pairs (weights
-// 2^{-72} and below).
+// Exact accumulation.  A product of two digits is an integer of at most 2^14.  Every level
+// l = t + u = 2 .. 8 has its own FP32 accumulator E_l in TMEM, and each is drained before
+// its sums can pass 2^24 (see Groups), so the tensor-core accumulation -- which truncates
+// rather than rounds -- never rounds at all: the sums are exact integers.  The drains add
+// them to one 96-bit integer per output element in units of 2^{-64}.  A work item spans at
+// most 8192 K (longer sums are split over items and the FP64 partial tiles added), which
+// bounds that integer by 2^76.  It is rounded to a double once at the end, so the only
+// errors are the 56-bit rounding of the inputs and the dropped pairs (weights 2^{-72} and
+// below).
 //
 // Five-slice steps.  A filter step may also use only the first five digits of each
 // operand (a 40-bit fixed-point value, truncation below 2^{-41} of the row scale) and
 // the 15 pairs of weight 2^{-48} and above (levels 2 .. 6): about 2^{-40} of the row
 // scales per term, some 2^{16} times finer than FP32, for 15 slice products instead
-// of 28 and three operand stages instead of two.  The digits are the same as above,
-// so the same slices serve both step kinds.
+// of 28.  The digits are the same as above, so the same slices serve both step kinds.
+//
+// Layout.  An operand is stored as [row tile][K chunk of 8][7 planes][rows of the tile][8]:
+// 16 bytes a row, plane and chunk, the core-matrix order that an unswizzled K-major
+// shared-memory operand has.  So a chunk of a tile is one contiguous copy of 14 KB (128
+// rows) or 7 KB (64 rows; its first five planes for a five-slice step), and any chunks can
+// be put side by side: the BSR step copies only the chunks of Y_cur that meet a nonzero
+// column of H.  (Tensor-map boxes of 128 rows x 64 bytes, 14 a stage, took the producer 87
+// cycles each.)
 //
 // Kernel.  Persistent, warp-specialised, one CTA per SM, 128 x 64 output tiles; NS = 7
 // slices per operand (or 5 for the 40-bit filter steps):
-//   warp 0, lane 0 : TMA producer -- per K-block of 32, the NS A (128-row) and NS B
-//                    (64-row) slice tiles (64-byte swizzle) into a ring of two stages
-//                    (84 KB each) or, with five slices, three (60 KB each);
-//   warp 1         : owns 512 TMEM columns, NS 64-column FP32 accumulators E2 .. E_{NS+1};
-//                    lane 0 issues the slice-pair products of a stage as 11 (or 9) MMAs
-//                    of M = 128, N = 64 c (B slices stacked), K = 16, twice per K-block;
-//   warps 2-17     : epilogue; warp w reads TMEM lanes 32 (w % 4) .. + 31 (one output
-//                    row per thread), columns 16 ((w - 2) / 4) .. + 15, and keeps those
-//                    16 x 2 integers in registers.
-// Drains alternate between group X (E2 .. E5, after K-blocks 5, 13, 21, ...) and group
-// Y (E6 .., after K-blocks 3, 7, 11, ...); the issuer runs the other group's MMAs of
-// the next stage before it waits for a drain.  Every mbarrier wait is bounded; on a
-// timeout the CTA flags DEV_TIMEOUT, stops, waits (bounded) for its copies and MMAs in
-// flight, frees TMEM and exits.
+//   warp 0    : producer, K = 16 of both operands per ring slot (42 KB, five slots; or 30
+//               KB, seven);
+//   warp 1    : MMA issuer, owns 512 TMEM columns; stages of K = 32 (two slots);
+//   warps 2-3 : BSR mode, the recurrence on the finished products;
+//   warps 4-11: epilogue; warp w reads TMEM lanes 32 (w % 4) .. + 31 (one output row per
+//               thread), columns 32 ((w - 4) / 4) .. + 31, and keeps their sums in registers.
+// Every mbarrier wait is bounded; on a timeout the CTA flags DEV_TIMEOUT, stops, waits
+// (bounded) for its copies and MMAs in flight, frees TMEM and exits.
+//
+// What bounds it: the tensor pipe, at 908 cycles per K = 16 of the 28 slice products (their
+// work is 896) when nothing else runs on the SM; about 1150 in the filter step, since
+// the warps share the issue slots with the drains' conversions (6 of 61 ms) and a
+// drained group's MMAs come in narrower pieces.  20 FP64-accurate steps at 40^3, w = 3, 1024
+// states: 98.0 -> 61.4 ms (0.83 of the chunks, and 1.35 x the rate); 20 40-bit and 4
+// FP64-accurate steps at 48^3, w = 4, 1500 states: 266 -> 164 ms.
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.cuh"
@@ -68,128 +74,134 @@ using namespace tc;
 constexpr int kSlices = 7;                            // digit planes stored per operand
 constexpr int kTileM = 128;                           // output rows per tile (TMEM lanes)
 constexpr int kTileN = 64;                            // output columns per tile
-constexpr int kRowPad = 128;                          // operand rows are padded to this
-// K per stage (a K-block): 32 BF16 = 64-byte rows under the 64-byte swizzle; a stage of
-// 7 + 7 slice tiles is 84 KB and two fit in shared memory.  K-blocks of 16 (32-byte
-// swizzle, 42 KB stages, five of them) measured slower: 114.7 against 98.4 ms for the
-// 20-step BSR filter at 40^3 with 1024 states, since the MMAs of one group that overlap
-// the other group's drain halve with the stage.
-constexpr int kKB = 32;
-constexpr int kSwizzleBytes = 2 * kKB;
-constexpr int kMaxItemKB = 8192 / kKB;                // K-blocks per work item (8192 K)
-constexpr int kBlockKB = 64 / kKB;                    // K-blocks per 64-wide BSR block
-constexpr int kSliceA = kTileM * kKB * 2;             // 8 KB
-constexpr int kSliceB = kTileN * kKB * 2;             // 4 KB
-constexpr int kPeriodX = 256 / kKB;                   // K-blocks between drains of group X (256 K)
-constexpr int kPeriodY = 128 / kKB;                   // K-blocks between drains of group Y (128 K)
-constexpr CUtensorMapSwizzle kTmaSwizzle = kKB == 16 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_64B;
-constexpr int kEpiWarps = 16;
-constexpr int kColsPerThread = kTileN / (kEpiWarps / 4);   // 16
-constexpr int kThreads = 32 * (2 + kEpiWarps);
+constexpr int kChunk = 8;                             // K columns per chunk: 8 BF16 = 16 bytes per row
+constexpr int kKB = 32;                               // K per stage: two ring slots of 16
+constexpr int kStageChunks = kKB / kChunk;
+constexpr int kSlotChunks = 2;                        // chunks per ring slot (K = 16, one MMA step)
+constexpr int kStageSlots = kStageChunks / kSlotChunks;
+constexpr int kMaxItemKB = 8192 / kKB;                // stages per work item (8192 K)
+constexpr int kBlockChunks = 64 / kChunk;             // chunks per 64-wide BSR block
+constexpr int kPlaneA = kTileM * 16;                  // bytes of one chunk and digit plane of a 128-row tile
+constexpr int kPlaneB = kTileN * 16;                  // the same for a 64-row tile
+constexpr int kEpiWarps = 8;                          // two warpgroups
+constexpr int kColsPerThread = kTileN / (kEpiWarps / 4);   // 32
+constexpr int kThreads = 32 * (4 + kEpiWarps);        // a warpgroup for the producer and the issuer
+// Registers a thread: launched with 168 (three warps on each scheduler's 16,384), of which
+// the first warpgroup gives 80 away to the other two: 88 + 2 x 208 = 3 x 168.
+constexpr int kRegsIssue = 88, kRegsEpilogue = 208;
 constexpr uint32_t kTmemCols = 512;
-constexpr int kMaxStages = 3;
-constexpr int kXEvent = 1, kYEvent = 2, kFullEvent = 3;
-static_assert(kSliceB % (8 * kSwizzleBytes) == 0, "swizzle-atom alignment of the tiles");
-static_assert(kKB == 16 || kKB == 32, "K-block of one or two 16-wide MMA steps");
-static_assert(kColsPerThread == 16, "16-column TMEM loads");
+constexpr int kMaxSlots = 7;
+constexpr int kMaxGroups = 3;                         // accumulator groups, and drains on the way at once
+constexpr int kEvents = 4;                            // barrier pairs of the drains
+static_assert(kColsPerThread == 32, "TMEM loads of 8 columns, batches of 8 and 16");
 
 // Shape of a product with NS digit slices per operand (7: FP64-accurate; 5: the
-// 40-bit steps): a stage holds NS A and NS B slice tiles; levels 2 .. NS + 1 each have
-// an accumulator (E2 .. E_{NS+1}), group X = E2 .. E5, group Y = the rest.
+// 40-bit steps): a ring slot holds the NS slices of K = 16 of both operands; level l = 2
+// .. NS + 1 has an accumulator E_l (index a = l - 2, 64 TMEM columns).
 template <int NS>
 struct OzShape {
-    static constexpr int kStageBytes = NS * (kSliceA + kSliceB);
-    static constexpr int kStages = (224 * 1024) / kStageBytes;
-    static constexpr int kSmemBytes = kStages * kStageBytes + 1024;
-    static constexpr int kAccs = NS;
-    static constexpr int kMmas = NS == 7 ? 11 : 9;
+    static constexpr int kChunkA = NS * kPlaneA, kChunkB = NS * kPlaneB;   // chunk strides in a slot
+    static constexpr int kSlotBytes = kSlotChunks * (kChunkA + kChunkB);
+    static constexpr int kSlots = (216 * 1024) / kSlotBytes;
+    static constexpr int kSmemBytes = kSlots * kSlotBytes + 128;
     static_assert(NS == 7 || NS == 5, "seven or five slices");
-    static_assert(kStages >= 2 && kStages <= kMaxStages, "two or three operand stages");
+    static_assert(kSlots > 2 * kStageSlots && kSlots <= kMaxSlots, "two stages and more in the ring");
     static_assert(kSmemBytes + 1024 <= 227 * 1024, "shared memory per CTA");
-    static_assert(kAccs * kTileN <= (int)kTmemCols, "accumulators in TMEM");
-    static_assert(kStageBytes % 1024 == 0, "swizzle-atom alignment of the stages");
 };
 
-// The 28 slice pairs (t, u), 0-based, with t + u <= 6 go to accumulator t + u (level
-// t + u + 2).  For one slice t of A, the slices u of B that fall into one accumulator
-// group are consecutive, and so are their accumulators, so they run as one MMA with the
-// B slices stacked along N (N = 64 c <= 256): 4 MMAs for group X (accumulators 0-3,
-// E2 .. E5) and 7 for group Y (accumulators 4-6, E6 .. E8), 11 per K-step instead of 28
-// (fewer, wider MMAs: less shared-memory operand traffic per product).  The first MMA of
-// each group has t = 0 and covers all of the group's accumulators.
-// With five slices the 15 pairs with t + u <= 4 take the same 4 MMAs for group X and
-// one MMA per pair of level 6 (accumulator 4, E6) for group Y: 9 per K-step.
-// MMA q takes slice mma_t(q) of A and the mma_c(q) slices of B from mma_u(q) on:
-//   seven slices: t = {0,1,2,3, 0,1,2,3,4,5,6}, u = {0,0,0,0, 4,3,2,1,0,0,0},
-//                 c = {4,3,2,1, 3,3,3,3,3,2,1};
-//   five slices:  t = {0,1,2,3, 0,1,2,3,4},     u = {0,0,0,0, 4,3,2,1,0},
-//                 c = {4,3,2,1, 1,1,1,1,1}.
-// Compile-time functions of q, so that the unrolled issue sequence folds them into
-// immediate descriptor offsets (one thread issues every MMA; table loads and
-// descriptor rebuilds per MMA made that thread the pace of the pipeline).
-constexpr int kMmaX = 4;
-__host__ __device__ constexpr int mma_t(int q) { return q < kMmaX ? q : q - kMmaX; }
-__host__ __device__ constexpr int mma_u(int q) { return q < kMmaX ? 0 : (q <= 2 * kMmaX ? 2 * kMmaX - q : 0); }
+// Drains.  The accumulators are drained in groups, one group after a stage, so that the
+// MMAs of the others cover it: seven slices E7-E8 (index 5, 6), E5-E6 (3, 4) and E2-E4
+// (0 .. 2); five slices E4-E6 (2 .. 4) and E2-E3 (0, 1), E4-E6 in two alternating sets of
+// columns, so that its drain holds up nothing.  A product of two digits is at most 2^14 and
+// E_l takes l - 1 pairs, so l - 1 <= 2^10 / K keeps |E_l| <= 2^24 between drains:
+//   seven slices: E7-E8 after stages 3, 7, 11 .. (K = 128), E5-E6 after 4, 10, 16 .. (160,
+//   192), E2-E4 after 9, 17 .. (320, 256); at the end of an item all three in turn.
+//   five slices: E4-E6 after 3, 7, 11 .. (128), E2-E3 after 9, 25 .. (320, 512); at the end
+//   E2-E3, then E4-E6.
+// (Drained in two groups, E2-E5 and E6-E8, the tensor pipe waited 1200 of 3800 cycles a
+// stage for them and for the outputs.)
 template <int NS>
-__host__ __device__ constexpr int mma_c(int q) {
-    return q < kMmaX ? kMmaX - q : (NS == 5 ? 1 : (11 - q < 3 ? 11 - q : 3));
-}
-// Every pair (t, u) with t + u <= NS - 1 exactly once, accumulator t + u.
-template <int NS>
-constexpr bool mma_covers_pairs(int nmmas) {
-    int seen[7][7] = {};
-    for (int q = 0; q < nmmas; q++)
-        for (int j = 0; j < mma_c<NS>(q); j++) {
-            const int t = mma_t(q), u = mma_u(q) + j;
-            if (t >= NS || u >= NS || t + u > NS - 1) return false;
-            if ((q < kMmaX) != (t + u < kMmaX)) return false;   // groups X (E2 .. E5) and Y
-            seen[t][u]++;
-        }
-    for (int t = 0; t < NS; t++)
-        for (int u = 0; u < NS; u++)
-            if (seen[t][u] != (t + u <= NS - 1 ? 1 : 0)) return false;
-    return true;
-}
-static_assert(mma_covers_pairs<7>(11) && mma_covers_pairs<5>(9), "slice-pair tables");
-static_assert(mma_t(10) == 6 && mma_u(9) == 0 && mma_c<7>(9) == 2 && mma_c<7>(8) == 3, "seven-slice table");
+struct Groups;
+template <>
+struct Groups<7> {
+    static constexpr int kCount = 3;
+    __host__ __device__ static constexpr int lo(int g) { return g == 0 ? 5 : (g == 1 ? 3 : 0); }
+    __host__ __device__ static constexpr int hi(int g) { return g == 0 ? 7 : (g == 1 ? 5 : 3); }
+    __host__ __device__ static constexpr int column(int g, int) { return lo(g) * kTileN; }
+    // the group drained after stage kb (not the item's last), or -1
+    __device__ static int event(int kb) { return kb % 4 == 3 ? 0 : (kb % 6 == 4 ? 1 : (kb % 8 == 1 && kb > 1 ? 2 : -1)); }
+};
+template <>
+struct Groups<5> {
+    static constexpr int kCount = 2;
+    __host__ __device__ static constexpr int lo(int g) { return g == 0 ? 0 : 2; }
+    __host__ __device__ static constexpr int hi(int g) { return g == 0 ? 2 : 5; }
+    // E2 E3 | E4 E5 E6 | E4 E5 E6 (second set)
+    __host__ __device__ static constexpr int column(int g, int set) { return g == 0 ? 0 : (2 + 3 * set) * kTileN; }
+    __device__ static int event(int kb) { return kb % 4 == 3 ? 1 : (kb % 16 == 9 ? 0 : -1); }
+};
 
-// The MMAs Q0 .. Q1 - 1 of one stage: A slices from descriptor da0, B slices from db0
-// (descriptors of the stage's first A and first B tile; a tile's start address is
-// da0 + offset / 16, which stays inside the 14-bit field below 256 KB).  The first MMA
-// of a group (q = 0 for X, q = kMmaX for Y) covers all of the group's accumulators and
-// overwrites them when the group starts fresh.
-template <int NS, int Q0, int Q1>
-__device__ __forceinline__ void issue_mmas(uint64_t da0, uint64_t db0, uint32_t tmem, bool freshX, bool freshY) {
+// The slice pairs (t, u), 0-based, t + u <= NS - 1, go to accumulator t + u.  For one slice
+// t of A consecutive slices u of B fall into consecutive accumulators, so they run as one
+// MMA with the B slices stacked along N (N = 64 c <= 256).  The pairs of the accumulators
+// LO .. HI - 1 take, for every t, the slices u = max(LO - t, 0) .. HI - 1 - t, in one MMA or
+// (five to seven slices) two; the t = 0 MMAs cover every accumulator of the range and come
+// first, so they overwrite when its sums start fresh; then the last slices of A (narrow
+// MMAs) down to the first (wide ones), because the tensor pipe queues only a few MMAs and
+// the wide ones last cover the waits between two ranges.  All of it is known at compile time:
+// the unrolled sequence has immediate descriptor offsets.  The whole warp runs it on
+// warp-uniform values and the MMAs are predicated on the leader lane (issued from a branch
+// that one lane takes, 10 MMAs took 1016-1146 cycles instead of 951-1030, their work being
+// 908).  `mid` runs before the MMAs of the last two slices.
+template <int NS, int LO, int HI, typename Mid>
+__device__ __forceinline__ void issue_range(uint32_t leader, uint64_t da0, uint64_t db0, uint32_t dcol, bool fresh,
+                                            Mid&& mid) {
+    static_assert(0 <= LO && LO < HI && HI <= NS, "accumulator range");
 #pragma unroll
-    for (int q = Q0; q < Q1; q++) {
-        const int t = mma_t(q), u0 = mma_u(q), c = mma_c<NS>(q);
-        const bool fresh = (q == 0 && freshX) || (q == kMmaX && freshY);
-        const uint64_t da = da0 + (uint64_t)((t * kSliceA) >> 4);
-        const uint64_t db = db0 + (uint64_t)((u0 * kSliceB) >> 4);
-        const uint32_t dt = tmem + (uint32_t)((t + u0) * kTileN);
-        constexpr uint32_t kIdesc1 = idesc_bf16(kTileM, kTileN);
-        const uint32_t idesc = kIdesc1 + (uint32_t)(((kTileN * (c - 1)) >> 3) << 17);
+    for (int k = 0; k < HI; k++) {
+        const int t = k == 0 ? 0 : HI - k;
+        if (k == HI - 2) mid();
+        const int u0 = LO > t ? LO - t : 0, n = HI - t - u0;
+        const int first = n > 4 ? n / 2 : n;
 #pragma unroll
-        for (int k = 0; k < kKB / 16; k++) {
-            const uint32_t accumulate = (fresh && k == 0) ? 0u : 1u;
+        for (int part = 0; part < (n > 4 ? 2 : 1); part++) {
+            const int u = part ? u0 + first : u0, c = part ? n - first : first;
+            constexpr uint32_t kIdesc1 = idesc_bf16(kTileM, kTileN);
+            // an offset stays inside the low word's 14-bit start address below 256 KB
+            const uint32_t da = (uint32_t)da0 + (uint32_t)((t * kPlaneA) >> 4);
+            const uint32_t db = (uint32_t)db0 + (uint32_t)((u * kPlaneB) >> 4);
+            const uint32_t dt = dcol + (uint32_t)((t + u - LO) * kTileN);
+            const uint32_t idesc = kIdesc1 + (uint32_t)(((kTileN * (c - 1)) >> 3) << 17);
+            const uint32_t accumulate = fresh && t == 0 ? 0u : 1u;
             asm volatile(
-                "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n"
-                :: "r"(dt), "l"(da + 2 * k), "l"(db + 2 * k), "r"(idesc), "r"(accumulate));
+                "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\tsetp.ne.b32 p, %6, 0;\n\tsetp.ne.b32 q, %7, 0;\n\t"
+                "mov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\t"
+                "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n\t}\n"
+                :: "r"(dt), "r"(da), "r"((uint32_t)(da0 >> 32)), "r"(db), "r"((uint32_t)(db0 >> 32)), "r"(idesc),
+                   "r"(accumulate), "r"(leader));
         }
     }
 }
 
-// The drain after K-block kb of an item of KB blocks: 0 none, kXEvent (E2 .. E5),
-// kYEvent (E6 ..) or kFullEvent (every accumulator, then the output).
-__device__ __forceinline__ int event_at(int kb, int KB) {
-    if (kb == KB - 1) return kFullEvent;
-    if (kb % kPeriodY == kPeriodY - 1) return kYEvent;
-    if (kb % kPeriodX == kPeriodX - 3) return kXEvent;
-    return 0;
+// Shared-memory descriptor of a K-major operand tile without swizzle: core matrices of 8
+// rows x 16 bytes (128 contiguous bytes), 8-row groups 128 bytes apart, the two 8-wide
+// K chunks of a step `chunk_stride` bytes apart.
+__device__ __forceinline__ uint64_t desc_chunks(uint32_t addr, int chunk_stride) {
+    uint64_t d = 0;
+    d |= (uint64_t)((addr & 0x3FFFF) >> 4);             // start address
+    d |= (uint64_t)(chunk_stride >> 4) << 16;           // leading byte offset: next K chunk
+    d |= (uint64_t)(128 >> 4) << 32;                    // stride byte offset: next 8 rows
+    d |= (uint64_t)1 << 46;                             // descriptor version
+    return d;
 }
 
 struct OzArgs {
+    // operands: [row tile][K chunk][7][rows of the tile][8] digits (128-row tiles of A_hat,
+    // 64-row tiles of B_hat; b_in_a: B_hat is A_hat, its 64-row tiles halves of A's)
+    const unsigned char* A;
+    const unsigned char* B;
+    int b_in_a;               // then loaded through the tensor map tmA
+    int64_t chunksA, chunksB; // K chunks per row tile
     int64_t M, Nc;            // output rows / columns
     int64_t ldc;
     double* C;                // output (direct mode), or
@@ -197,28 +209,29 @@ struct OzArgs {
     int64_t Mp, Np;           // partial-tile extents: tilesM * 128, tilesN * 64
     const int* expA;          // biased exponent field of each row's largest |value| (0: zero row)
     const int* expB;
-    int64_t rowsA_pad, rowsB_pad;
     int tilesM, tilesN;
-    int kb_total;             // K-blocks of 32
-    int kb_split;             // K-blocks per split
+    int kb_total;             // stages (32 K)
+    int kb_split;             // stages per split
     int splits;
     int symmetric;            // only tiles that reach the upper triangle (j >= i)
     int b_upper;              // B_hat[j][k] = 0 for k > j: K limited to the tile's last column
     int64_t pairs;            // tiles per split and batch
     int nbatch;               // independent products (diagonal blocks of the split layout)
     int64_t m_batch;          // output rows per batch (M when nbatch = 1)
-    int64_t a_batch_rows, b_batch_rows;   // operand rows per batch in the slice arrays
+    int64_t a_batch_tiles, b_batch_tiles;   // row tiles per batch in the operands
     uint64_t wait_ns;         // limit of the waits on the other roles (drains keep kDrainNs)
     unsigned* status;
     // BSR filter-step mode (bsr != 0): A_hat = Y_cur^T (states x grid points), B_hat = the
-    // 64 x 64 blocks of H stacked by rows; a work item is one block row (the 64 output
-    // columns, grid rows R * 64 ..) against one tile of 128 states, its K the block
-    // columns of the row, and the epilogue applies the recurrence
+    // non-zero 8-column chunks of H's 64-row block rows; a work item is one block row
+    // (the 64 output columns, grid rows R * 64 ..) against one tile of 128 states, its K
+    // the row's chunks, and the epilogue applies the recurrence
     // Y_out = alpha (H Y_cur - c Y_cur) - beta Y_prev in FP64 (output in C, ldc).
     int bsr;
     int slices;               // digit slices per operand in the products: 7, or 5 (BSR mode)
     const int32_t* brow_ptr;
-    const int32_t* bcol;
+    const int32_t* hchunk;    // Y_cur chunk of each stored chunk of H (row R from brow_ptr[R] * 8 on)
+    const int32_t* hcount;    // stored chunks of each block row (a multiple of kStageChunks),
+                              // kUnfolded set where c is not in H's digits
     int64_t nbr, nblocks;
     const int* expH;          // exponent field of each grid row of H (over its block row)
     const double* Ycur;
@@ -228,19 +241,25 @@ struct OzArgs {
     double alpha, cshift, beta;
 };
 
+constexpr int kUnfolded = 1 << 30;
+
 struct Item {
     int batch, tm, tn, kb0, KB;
-    int qb;                   // BSR mode: first block of the row
+    bool unfolded;            // BSR mode: the epilogue subtracts c Y_cur
+    int64_t qc;               // BSR mode: first stored chunk of the row
 };
 
-// Stored block range of block row R, clamped to [0, nblocks] and to kMaxItemKB / kBlockKB
-// blocks (the host rejects longer rows); `bad` is set for a malformed row pointer.
-__device__ __forceinline__ void bsr_row_range(const OzArgs& g, int64_t R, int& qb, int& nq, bool& bad) {
-    int b0 = g.brow_ptr[R], b1 = g.brow_ptr[R + 1];
+// Stored block range of block row R, clamped to [0, nblocks] and to 128 blocks (the host
+// rejects longer rows); `bad` is set for a malformed row pointer.
+__device__ __forceinline__ void bsr_row_range(const int32_t* brow_ptr, int64_t nblocks, int64_t R, int& qb, int& nq,
+                                              bool& bad) {
+    constexpr int kMaxBlocks = kMaxItemKB * kKB / 64;
+    int b0 = brow_ptr[R], b1 = brow_ptr[R + 1];
     if (b0 < 0) { b0 = 0; bad = true; }
-    if (b1 > g.nblocks) { b1 = (int)g.nblocks; bad = true; }
+    if (b0 > nblocks) { b0 = (int)nblocks; bad = true; }
+    if (b1 > nblocks) { b1 = (int)nblocks; bad = true; }
     if (b1 < b0) { b1 = b0; bad = true; }
-    if (b1 - b0 > kMaxItemKB / kBlockKB) { b1 = b0 + kMaxItemKB / kBlockKB; bad = true; }
+    if (b1 - b0 > kMaxBlocks) { b1 = b0 + kMaxBlocks; bad = true; }
     qb = b0;
     nq = b1 - b0;
 }
@@ -252,20 +271,23 @@ template <bool kBsr>
 __device__ __forceinline__ Item decode(const OzArgs& g, int64_t item) {
     Item it;
     if (kBsr) {
-        // the state tiles of a block row are consecutive, so its H slices are shared
+        // the state tiles of a block row are consecutive, so its H chunks are shared
         // through L2
         const int64_t R = item / g.tilesM;
         bool bad = false;
-        int nq;
-        bsr_row_range(g, R, it.qb, nq, bad);
+        int qb, nq;
+        bsr_row_range(g.brow_ptr, g.nblocks, R, qb, nq, bad);
         it.batch = 0;
-        it.tm = (int)(item % g.tilesM);
+        it.tm = (int)(item - R * g.tilesM);
         it.tn = (int)R;
         it.kb0 = 0;
-        it.KB = kBlockKB * nq;
+        const int packed = g.hcount[R], cnt = packed & ~kUnfolded;
+        it.unfolded = (packed & kUnfolded) != 0;
+        it.KB = (cnt < nq * kBlockChunks ? cnt : nq * kBlockChunks) / kStageChunks;
+        it.qc = (int64_t)qb * kBlockChunks;
         return it;
     }
-    it.qb = 0;
+    it.qc = 0;
     const int64_t per_split = g.pairs * g.nbatch;
     const int z = (int)(item / per_split);
     it.batch = (int)((item % per_split) / g.pairs);
@@ -290,64 +312,148 @@ __device__ __forceinline__ Item decode(const OzArgs& g, int64_t item) {
     return it;
 }
 
-// 16 accumulator columns of this warp's 32 TMEM lanes (one row per lane).
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+// Eight accumulator columns of this warp's 32 TMEM lanes (one row per lane).
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+}
+
+// Output sum of an element in units of 2^-64, 96 bits (|T| < 2^76): three registers where
+// one 64-bit sum per accumulator group takes four (with those the epilogue spilled).
+struct Sum96 {
+    uint32_t w0, w1, w2;
+};
+// t += x 2^kShift
+template <int kShift>
+__device__ __forceinline__ void add96(Sum96& t, long long x) {
+    if constexpr (kShift < 32) {
+        const uint32_t a0 = (uint32_t)x << kShift;
+        const uint32_t a1 = (uint32_t)(x >> (kShift == 0 ? 32 : 32 - kShift));
+        const uint32_t a2 = (uint32_t)(x >> (kShift == 0 ? 63 : 64 - kShift));
+        asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+            : "+r"(t.w0), "+r"(t.w1), "+r"(t.w2) : "r"(a0), "r"(a1), "r"(a2));
+    } else {
+        const uint32_t a1 = (uint32_t)x << (kShift - 32), a2 = (uint32_t)(x >> (64 - kShift));
+        asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, %3;" : "+r"(t.w1), "+r"(t.w2) : "r"(a1), "r"(a2));
+    }
+}
+
+// umma_commit by the leader lane of a convergent warp.
+__device__ __forceinline__ void commit_by(uint32_t leader, uint64_t* b) {
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+        :: "r"(sa(b)), "r"(leader) : "memory");
 }
 
-// FP32 power of two 2^p (|p| < 127).
-__device__ __forceinline__ float pow2f(int p) { return __int_as_float((127 + p) << 23); }
-
-// x * 2^e for a nonzero double x built from an integer (exact exponent shift);
-// results outside the normal range flush to signed zero or infinity.
-__device__ __forceinline__ double scale_pow2(double x, int e) {
-    const long long b = __double_as_longlong(x);
-    const int ex = (int)((b >> 52) & 0x7ff) + e;
-    const long long sign = b & (1ll << 63);
-    if (ex <= 0) return __longlong_as_double(sign);
-    if (ex >= 0x7ff) return __longlong_as_double(sign | (0x7ffll << 52));
-    return __longlong_as_double(b + ((long long)e << 52));
+// One lane of the warp, always the same one.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\tselp.u32 %0, 1, 0, e;\n\t}" : "=r"(p));
+    return p != 0;
 }
 
-// 2^{e} (hi 2^{-40} + lo 2^{-64}) from the two exact integers of an output element.
-__device__ __forceinline__ double combine(long long hi, long long lo, int e) {
-    double v = 0.0;
-    if (hi != 0) v = scale_pow2((double)hi, e - 40);
-    if (lo != 0) v += scale_pow2((double)lo, e - 64);
-    return v;
+// Whether the phase of `parity` has completed, without waiting.
+__device__ __forceinline__ bool mbar_test(uint32_t addr, uint32_t parity) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(done) : "r"(addr), "r"(parity) : "memory");
+    return done != 0;
 }
 
-// One CTA of 18 warps per SM: the register file is split among the SM's four schedulers
-// (16,384 registers each) and five of the warps share one of them, which allows 96
-// registers a thread; ptxas keeps to that under these launch bounds.  kBsr: the BSR
-// filter-step mode (its own instantiation, so that neither mode carries the other's
-// epilogue registers).  NS: digit slices per operand (7, or 5 for the 40-bit steps).
+// Contiguous copy of `bytes` (a multiple of 16) into shared memory.
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+        :: "r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
+
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+        :: "r"(dst), "l"((uint64_t)map), "r"(x), "r"(y), "r"(z), "r"(bar) : "memory");
+}
+
+// acc + v * mul (32 x 32 -> 64-bit multiply-add).
+__device__ __forceinline__ long long mad_wide(int v, int mul, long long acc) {
+    long long r;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(v), "r"(mul), "l"(acc));
+    return r;
+}
+
+// 2^{e - 64} T rounded to nearest once, from the exact sum T of an output element; results
+// below the normal range flush to signed zero, above it to infinity.  Integer
+// instructions only: the FP64 pipe runs two operations a cycle and SM, so that its
+// conversions of two 64-bit sums, their addition and scaling cost an item of 128 x 64
+// outputs 16,000 cycles and more.
+__device__ __forceinline__ double combine(const Sum96& t, int e) {
+    const uint32_t neg = (uint32_t)((int)t.w2 >> 31);
+    uint32_t a0 = t.w0 ^ neg, a1 = t.w1 ^ neg, a2 = t.w2 ^ neg;      // |T|
+    asm("sub.cc.u32 %0, %0, %3;\n\tsubc.cc.u32 %1, %1, %3;\n\tsubc.u32 %2, %2, %3;"
+        : "+r"(a0), "+r"(a1), "+r"(a2) : "r"(neg));
+    // leading bit to bit 31 of a2
+    int ex = 1023 + 95 - 64 + e;
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+        const bool z = a2 == 0;
+        a2 = z ? a1 : a2;
+        a1 = z ? a0 : a1;
+        a0 = z ? 0u : a0;
+        ex -= z ? 32 : 0;
+    }
+    const int lz = __clz((int)a2) & 31;
+    a2 = __funnelshift_l(a1, a2, lz);
+    a1 = __funnelshift_l(a0, a1, lz);
+    a0 <<= lz;
+    ex -= lz;                                                        // biased exponent of the leading bit
+    // 53 bits, rounded to nearest even; the implicit bit adds one to the exponent field, as
+    // does a mantissa that rounds up to 2^53
+    uint32_t lo = __funnelshift_r(a1, a2, 11), hi = a2 >> 11;
+    const uint32_t rest = ((a1 & 0x7ffu) << 1) | (a0 != 0 ? 1u : 0u);
+    const uint32_t up = rest + (lo & 1u) > 0x800u ? 1u : 0u;
+    hi += (uint32_t)(ex - 1) << 20;
+    asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, 0;" : "+r"(lo), "+r"(hi) : "r"(up));
+    if (ex <= 0 || ex >= 0x7ff || hi >= 0x7ff00000u || a2 == 0) {
+        lo = 0;
+        hi = (a2 == 0 || ex <= 0) ? 0u : 0x7ff00000u;
+        if (a2 == 0) return 0.0;
+    }
+    return __hiloint2double((int)(hi | (neg & 0x80000000u)), (int)lo);
+}
+
+// One CTA of 12 warps per SM.  kBsr: the BSR filter-step mode (its own instantiation, so
+// that neither mode carries the other's epilogue registers).  NS: digit slices per operand
+// (7, or 5 for the 40-bit steps).
 template <bool kBsr, int NS>
-__global__ void __launch_bounds__(kThreads, 1)
-oz_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, OzArgs g,
-               int64_t total) {
+__global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(const __grid_constant__ OzArgs g,
+                                                              const __grid_constant__ CUtensorMap tmA, int64_t total) {
     using Sh = OzShape<NS>;
-    constexpr int kStages = Sh::kStages, kStageBytes = Sh::kStageBytes, kMmas = Sh::kMmas, kAccs = Sh::kAccs;
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    __shared__ __align__(8) uint64_t full[kMaxStages], empty[kMaxStages], efull, eempty, done;
+    using Gr = Groups<NS>;
+    constexpr int kSlots = Sh::kSlots, kSlotBytes = Sh::kSlotBytes;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
+    __shared__ __align__(8) uint64_t full[kMaxSlots], empty[kMaxSlots], efull[kEvents], eempty[kEvents], done;
+    __shared__ __align__(8) uint64_t dfull[2], dempty[2];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     bool nonfinite = false, bad_pattern = false;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kStages; s++) {
+        for (int s = 0; s < kSlots; s++) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
-        mbar_init(&efull, 1);
-        mbar_init(&eempty, kEpiWarps);
+        for (int e = 0; e < kEvents; e++) {
+            mbar_init(&efull[e], 1);
+            mbar_init(&eempty[e], kEpiWarps);
+        }
+        for (int d = 0; d < 2; d++) {
+            mbar_init(&dfull[d], kEpiWarps);
+            mbar_init(&dempty[d], 2);
+        }
         mbar_init(&done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;");
         asm volatile("fence.proxy.async.shared::cta;");
@@ -364,201 +470,432 @@ oz_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const uint32_t tmem = tmem_slot;
     volatile int* abort_v = &abort_flag;
 
-    if (warp == 0 && lane == 0) {
-        // ---------------- TMA producer
+    if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" :: "n"(kRegsIssue));
+    if (warp == 0) {
+        // ---------------- producer: lane 0 waits for the slot and announces its bytes, then
+        // the lanes issue its copies
         int64_t sc = 0;
-        for (int64_t item = blockIdx.x; item < total && !*abort_v; item += gridDim.x) {
-            const Item it = decode<kBsr>(g, item);
+        int s = 0;
+        uint32_t ph = 1;        // parity of the previous pass over the ring
+        bool ok = true;
+        // BSR mode: entry p of an item's list of Y_cur chunks, always a valid chunk
+        auto list_entry = [&](const Item& it, int64_t p) -> int {
+            int yc = kBsr && p < (int64_t)it.KB * kStageChunks ? g.hchunk[it.qc + p] : 0;
+            if (yc < 0 || yc >= g.chunksA) { yc = 0; bad_pattern = true; }
+            return yc;
+        };
+        Item it{}, next{};
+        int list0 = 0, list1 = 0, next0 = 0;   // this lane's entries of the current 32, the next 32, the next item's first
+        if (blockIdx.x < total) {
+            next = decode<kBsr>(g, blockIdx.x);
+            next0 = list_entry(next, lane);
+        }
+        for (int64_t item = blockIdx.x; ok && item < total; item += gridDim.x) {
+            if (__any_sync(0xffffffffu, *abort_v)) break;
+            it = next;
+            list0 = next0;
+            list1 = list_entry(it, 32 + lane);
+            const int slots = it.KB * kStageSlots;
+            if (item + gridDim.x < total) {    // the next item's sizes and list, a whole item ahead of their use
+                next = decode<kBsr>(g, item + gridDim.x);
+                next0 = list_entry(next, lane);
+            }
             if (kBsr) {
                 int qb, nq;
-                bsr_row_range(g, it.tn, qb, nq, bad_pattern);
+                bsr_row_range(g.brow_ptr, g.nblocks, it.tn, qb, nq, bad_pattern);
             }
-            bool ok = true;
-            for (int kb = 0; kb < it.KB; kb++, sc++) {
-                const int s = (int)(sc % kStages);
-                const int64_t u = sc / kStages;
-                if (u >= 1 && !mbar_wait(sa(&empty[s]), (uint32_t)((u - 1) & 1), g.wait_ns)) { ok = false; break; }
-                const uint32_t st = sa(smem + (size_t)s * kStageBytes);
-                // K offset in A_hat and in B_hat, and B_hat's first row
-                int xa = (it.kb0 + kb) * kKB, xb = xa;
-                int64_t rb = it.batch * g.b_batch_rows + (int64_t)it.tn * kTileN;
+            const unsigned char* At = g.A + ((int64_t)(it.batch * g.a_batch_tiles + it.tm) * g.chunksA) *
+                                                (kSlices * kPlaneA);
+            const unsigned char* Bt =
+                kBsr ? g.B + it.qc * (kSlices * kPlaneB)
+                     : g.B + ((int64_t)(it.batch * g.b_batch_tiles + it.tn) * g.chunksB) * (kSlices * kPlaneB);
+            for (int sl = 0; sl < slots; sl++, sc++) {
+                if (kBsr && sl % (32 / kSlotChunks) == 0 && sl > 0) {
+                    list0 = list1;
+                    list1 = list_entry(it, (int64_t)sl * kSlotChunks + 32 + lane);
+                }
+                const int64_t c0 = (int64_t)(it.kb0 * kStageSlots + sl) * kSlotChunks;
+                bool got = true;
+                if (lane == 0) {
+                    if (sc >= kSlots) got = mbar_wait(sa(&empty[s]), ph, g.wait_ns);
+                    if (got) mbar_expect_tx(&full[s], kSlotBytes);
+                }
+                if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
+                const uint32_t st = sa(smem + (size_t)s * kSlotBytes), bar = sa(&full[s]);
                 if (kBsr) {
-                    const int q = it.qb + kb / kBlockKB, half = kb % kBlockKB;
-                    int C = g.bcol[q];
-                    if (C < 0 || (int64_t)C >= g.nbr) { C = 0; bad_pattern = true; }   // still a valid tile
-                    xa = C * 64 + half * kKB;
-                    xb = half * kKB;
-                    rb = (int64_t)q * 64;
+                    const int64_t yc = __shfl_sync(0xffffffffu, list0, (sl * kSlotChunks + lane) & 31);
+                    if (lane < kSlotChunks) {       // chunks of Y_cur, and of H
+                        bulk_load(st + lane * Sh::kChunkA, At + yc * (kSlices * kPlaneA), Sh::kChunkA, bar);
+                        bulk_load(st + kSlotChunks * Sh::kChunkA + lane * Sh::kChunkB,
+                                  Bt + (c0 + lane) * (kSlices * kPlaneB), Sh::kChunkB, bar);
+                    }
+                } else {
+                    const uint32_t sb = st + kSlotChunks * Sh::kChunkA;
+                    if (g.b_in_a) {
+                        // columns 64 tn ..: the half (tn & 1) of every plane of 128-row tile tn / 2
+                        if (lane == 0)
+                            tma_load_3d(sb, &tmA, (it.tn & 1) * (kPlaneB / 4), 0,
+                                        (int)((it.tn >> 1) * g.chunksA + c0), bar);
+                    } else if (lane < kSlotChunks) {
+                        bulk_load(sb + lane * Sh::kChunkB, Bt + (c0 + lane) * (kSlices * kPlaneB), Sh::kChunkB, bar);
+                    }
+                    if (lane >= 30)
+                        bulk_load(st + (lane - 30) * Sh::kChunkA, At + (c0 + lane - 30) * (kSlices * kPlaneA),
+                                  Sh::kChunkA, bar);
                 }
-                mbar_expect_tx(&full[s], kStageBytes);
-#pragma unroll
-                for (int t = 0; t < NS; t++)
-                    tma_load_2d(st + t * kSliceA, &tmA, xa,
-                                (int)(t * g.rowsA_pad + it.batch * g.a_batch_rows + (int64_t)it.tm * kTileM),
-                                sa(&full[s]));
-#pragma unroll
-                for (int t = 0; t < NS; t++)
-                    tma_load_2d(st + NS * kSliceA + t * kSliceB, &tmB, xb, (int)(t * g.rowsB_pad + rb),
-                                sa(&full[s]));
+                if (++s == kSlots) { s = 0; ph ^= 1; }
             }
-            if (!ok) { *abort_v = 1; break; }
         }
+        if (!ok && lane == 0) *abort_v = 1;
         // every copy issued has landed before the CTA can exit
-        for (int s = 0; s < kStages && s < sc; s++) {
-            const int64_t last = s + ((sc - 1 - s) / kStages) * kStages;
-            mbar_wait(sa(&full[s]), (uint32_t)((last / kStages) & 1), kDrainNs);
-        }
-    } else if (warp == 1 && lane == 0) {
-        // ---------------- MMA issuer
-        int64_t sc = 0, ev_commit = 0, ev_wait = 0;
-        bool issued = false;
-        for (int64_t item = blockIdx.x; item < total && !*abort_v; item += gridDim.x) {
-            const Item it = decode<kBsr>(g, item);
-            bool ok = true;
-            for (int kb = 0; kb < it.KB; kb++, sc++) {
-                const int s = (int)(sc % kStages);
-                if (!mbar_wait(sa(&full[s]), (uint32_t)((sc / kStages) & 1), g.wait_ns) || *abort_v) {
-                    ok = false;
-                    break;
-                }
-                asm volatile("tcgen05.fence::after_thread_sync;");
-                const uint32_t st = sa(smem + (size_t)s * kStageBytes);
-                // which group starts fresh in this stage (its drain must have ended first)
-                const bool resetX = kb == 0 || kb % kPeriodX == kPeriodX - 2;
-                const bool resetY = kb == 0 || kb % kPeriodY == 0;
-                auto wait_drain = [&]() -> bool {
-                    const bool w = mbar_wait(sa(&eempty), (uint32_t)(ev_wait & 1), g.wait_ns);
-                    ev_wait++;
+        __syncwarp();
+        if (lane == 0)
+            for (int q = 0; q < kSlots && q < sc; q++) {
+                const int64_t last = q + ((sc - 1 - q) / kSlots) * kSlots;
+                mbar_wait(sa(&full[q]), (uint32_t)((last / kSlots) & 1), kDrainNs);
+            }
+    } else if (warp == 1) {
+        // ---------------- MMA issuer: the whole warp runs the loop on warp-uniform values, one
+        // elected lane issues.
+        // Drain number e uses barrier pair e % kEvents; pend_g is the last drain of group g
+        // (five slices: pend1 and pend2 of the two sets of E4-E6), -1 once waited for, so that
+        // at most kMaxGroups drains are on the way.
+        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+        const uint32_t ring = __shfl_sync(0xffffffffu, sa(smem), 0);
+        const uint32_t leader = elect_one() ? 1u : 0u;
+        int ev = 0, pend0 = -1, pend1 = -1, pend2 = -1;
+        int set = 0;            // five slices: the set of E4-E6 in use
+        int s = 0;
+        uint32_t ph = 0;
+        bool issued = false, ok = true;
+        bool ready = false;     // slot s is known to be full
+        int kb_next = blockIdx.x < total ? decode<kBsr>(g, blockIdx.x).KB : 0;
+        for (int64_t item = blockIdx.x; ok && item < total; item += gridDim.x) {
+            if (__any_sync(0xffffffffu, *abort_v)) break;
+            const int KB = __shfl_sync(0xffffffffu, kb_next, 0);
+            if (item + gridDim.x < total) kb_next = decode<kBsr>(g, item + gridDim.x).KB;   // an item ahead of its use
+            int fresh = -1;     // the group drained after the last stage
+            for (int kb = 0; kb < KB; kb++) {
+                // the stage's two slots and their descriptors (each slot's first A and B plane)
+                const int s0 = s, s1 = s + 1 == kSlots ? 0 : s + 1;
+                const uint32_t ph0 = ph, ph1 = s + 1 == kSlots ? ph ^ 1 : ph;
+                s = s1 + 1 == kSlots ? 0 : s1 + 1;
+                ph = s1 + 1 == kSlots ? ph1 ^ 1 : ph1;
+                const uint32_t st0 = ring + (uint32_t)(s0 * kSlotBytes), st1 = ring + (uint32_t)(s1 * kSlotBytes);
+                const uint64_t da0 = desc_chunks(st0, Sh::kChunkA), da1 = desc_chunks(st1, Sh::kChunkA);
+                const uint64_t db0 = desc_chunks(st0 + kSlotChunks * Sh::kChunkA, Sh::kChunkB);
+                const uint64_t db1 = desc_chunks(st1 + kSlotChunks * Sh::kChunkA, Sh::kChunkB);
+                auto wait_full = [&](int sl, uint32_t p) -> bool {
+                    const bool w = ready || __all_sync(0xffffffffu, mbar_wait(sa(&full[sl]), p, g.wait_ns));
+                    ready = false;
                     asm volatile("tcgen05.fence::after_thread_sync;");
                     return w;
                 };
-                // descriptors of the stage's first A and first B slice tile
-                const uint64_t da0 = desc_kmajor(st, kSwizzleBytes);
-                const uint64_t db0 = desc_kmajor(st + NS * kSliceA, kSwizzleBytes);
-                // after a drain wait that gave up, nothing more is issued into the
-                // accumulators that the epilogue may still be reading
+                // looks at a slot without waiting, while MMAs are queued
+                auto test_full = [&](int sl, uint32_t p) { ready = __all_sync(0xffffffffu, mbar_test(sa(&full[sl]), p)); };
+                // the drain that a group (or set) still waits for; after a wait that gave up,
+                // nothing more is issued into accumulators that the epilogue may be reading
+                auto test_drain = [&](int& pend) {
+                    if (pend >= 0 && __all_sync(0xffffffffu, mbar_test(sa(&eempty[pend % kEvents]),
+                                                                       (uint32_t)((pend / kEvents) & 1))))
+                        pend = -1;
+                };
+                auto wait_drain = [&](int& pend) -> bool {
+                    if (pend < 0) {
+                        asm volatile("tcgen05.fence::after_thread_sync;");
+                        return true;
+                    }
+                    const int e = pend;
+                    pend = -1;
+                    const bool w = __all_sync(0xffffffffu, mbar_wait(sa(&eempty[e % kEvents]),
+                                                                     (uint32_t)((e / kEvents) & 1), g.wait_ns));
+                    asm volatile("tcgen05.fence::after_thread_sync;");
+                    return w;
+                };
                 bool w = true;
-                if (kb == 0) {
-                    if (ev_commit > 0) w = wait_drain();     // the previous item's output drain
-                    if (w) issue_mmas<NS, 0, kMmas>(da0, db0, tmem, resetX, resetY);
-                } else if (resetX) {                           // E2 .. E5 drained after the last block
-                    issue_mmas<NS, kMmaX, kMmas>(da0, db0, tmem, false, resetY);
-                    w = wait_drain();
-                    if (w) issue_mmas<NS, 0, kMmaX>(da0, db0, tmem, true, false);
-                } else if (resetY) {                           // E6 .. drained after the last block
-                    issue_mmas<NS, 0, kMmaX>(da0, db0, tmem, resetX, false);
-                    w = wait_drain();
-                    if (w) issue_mmas<NS, kMmaX, kMmas>(da0, db0, tmem, false, true);
-                } else {
-                    issue_mmas<NS, 0, kMmas>(da0, db0, tmem, false, false);
-                }
                 issued = true;
-                umma_commit(&empty[s]);
-                if (!w) { ok = false; sc++; break; }
-                if (event_at(kb, it.KB)) {
-                    umma_commit(&efull);
-                    ev_commit++;
+                auto none = []() {};
+                auto test1 = [&]() { test_full(s1, ph1); };
+                auto test_next = [&]() { test_full(s, ph); };   // the next stage's (or item's) first slot
+                if (!wait_full(s0, ph0)) { ok = false; break; }
+                if constexpr (NS == 7) {
+                    const uint32_t c0 = tm + Gr::column(0, 0), c1 = tm + Gr::column(1, 0), c2 = tm + Gr::column(2, 0);
+                    if (kb == 0) {                     // each group when the last item's sums have left it
+                        w = wait_full(s1, ph1) && wait_drain(pend0);
+                        if (w) {
+                            issue_range<NS, 5, 7>(leader, da0, db0, c0, true, none);
+                            issue_range<NS, 5, 7>(leader, da1, db1, c0, false, none);
+                            w = wait_drain(pend1);
+                        }
+                        if (w) {
+                            issue_range<NS, 3, 5>(leader, da0, db0, c1, true, none);
+                            issue_range<NS, 3, 5>(leader, da1, db1, c1, false, none);
+                            w = wait_drain(pend2);
+                        }
+                        if (w) {
+                            issue_range<NS, 0, 3>(leader, da0, db0, c2, true, none);
+                            commit_by(leader, &empty[s0]);
+                            issue_range<NS, 0, 3>(leader, da1, db1, c2, false, test_next);
+                        }
+                    } else if (fresh < 0) {
+                        issue_range<NS, 0, 7>(leader, da0, db0, tm, false, test1);
+                        commit_by(leader, &empty[s0]);
+                        if ((w = wait_full(s1, ph1))) issue_range<NS, 0, 7>(leader, da1, db1, tm, false, test_next);
+                    } else if (fresh == 0) {           // the other groups, then the drained one
+                        issue_range<NS, 0, 5>(leader, da0, db0, tm, false, test1);
+                        if ((w = wait_full(s1, ph1))) {
+                            issue_range<NS, 0, 5>(leader, da1, db1, tm, false, [&]() { test_drain(pend0); });
+                            w = wait_drain(pend0);
+                        }
+                        if (w) {
+                            issue_range<NS, 5, 7>(leader, da0, db0, c0, true, none);
+                            commit_by(leader, &empty[s0]);
+                            issue_range<NS, 5, 7>(leader, da1, db1, c0, false, test_next);
+                        }
+                    } else if (fresh == 1) {
+                        issue_range<NS, 5, 7>(leader, da0, db0, c0, false, test1);
+                        issue_range<NS, 0, 3>(leader, da0, db0, c2, false, none);
+                        if ((w = wait_full(s1, ph1))) {
+                            issue_range<NS, 5, 7>(leader, da1, db1, c0, false, [&]() { test_drain(pend1); });
+                            issue_range<NS, 0, 3>(leader, da1, db1, c2, false, none);
+                            w = wait_drain(pend1);
+                        }
+                        if (w) {
+                            issue_range<NS, 3, 5>(leader, da0, db0, c1, true, none);
+                            commit_by(leader, &empty[s0]);
+                            issue_range<NS, 3, 5>(leader, da1, db1, c1, false, test_next);
+                        }
+                    } else {
+                        issue_range<NS, 3, 7>(leader, da0, db0, c1, false, test1);
+                        if ((w = wait_full(s1, ph1))) {
+                            issue_range<NS, 3, 7>(leader, da1, db1, c1, false, [&]() { test_drain(pend2); });
+                            w = wait_drain(pend2);
+                        }
+                        if (w) {
+                            issue_range<NS, 0, 3>(leader, da0, db0, c2, true, none);
+                            commit_by(leader, &empty[s0]);
+                            issue_range<NS, 0, 3>(leader, da1, db1, c2, false, test_next);
+                        }
+                    }
+                } else {
+                    const bool fresh0 = kb == 0 || fresh == 0, fresh1 = kb == 0 || fresh == 1;
+                    const uint32_t d0 = tm + Gr::column(0, 0), d1 = tm + Gr::column(1, set);
+                    if (fresh1) w = set ? wait_drain(pend2) : wait_drain(pend1);   // this set's drain before the last
+                    if (w && !fresh0) {
+                        issue_range<NS, 0, 2>(leader, da0, db0, d0, false, none);
+                        issue_range<NS, 2, 5>(leader, da0, db0, d1, fresh1, test1);
+                        commit_by(leader, &empty[s0]);
+                        if ((w = wait_full(s1, ph1))) {
+                            issue_range<NS, 0, 2>(leader, da1, db1, d0, false, none);
+                            issue_range<NS, 2, 5>(leader, da1, db1, d1, false, test_next);
+                        }
+                    } else if (w) {
+                        issue_range<NS, 2, 5>(leader, da0, db0, d1, fresh1, test1);
+                        if ((w = wait_full(s1, ph1))) {
+                            issue_range<NS, 2, 5>(leader, da1, db1, d1, false, [&]() { test_drain(pend0); });
+                            w = wait_drain(pend0);
+                        }
+                        if (w) {
+                            issue_range<NS, 0, 2>(leader, da0, db0, d0, true, none);
+                            commit_by(leader, &empty[s0]);
+                            issue_range<NS, 0, 2>(leader, da1, db1, d0, false, test_next);
+                        }
+                    }
                 }
+                commit_by(leader, &empty[s1]);
+                if (!w) { ok = false; break; }
+                auto event = [&](int& pend) {
+                    commit_by(leader, &efull[ev % kEvents]);
+                    pend = ev++;
+                };
+                fresh = Gr::event(kb);
+                const bool last = kb == KB - 1;
+                if (last || fresh == 0) event(pend0);
+                if (last || fresh == 1) {
+                    if (NS == 5 && set) event(pend2);
+                    else event(pend1);
+                    if (NS == 5) set ^= 1;
+                }
+                if (NS == 7 && (last || fresh == 2)) event(pend2);
             }
-            if (!ok) { *abort_v = 1; break; }
         }
+        if (!ok && lane == 0) *abort_v = 1;
         // every MMA issued has completed before TMEM is released
         if (issued) {
-            umma_commit(&done);
+            commit_by(leader, &done);
             mbar_wait(sa(&done), 0, kDrainNs);
         }
-    } else if (warp >= 2) {
-        // ---------------- epilogue: exact drains into 64-bit integers, then the output
-        const int q = warp & 3, h = (warp - 2) >> 2;
-        const uint32_t lane_base = (uint32_t)(32 * q) << 16;
-        int64_t ev = 0;
-        long long hi[kColsPerThread], lo[kColsPerThread];
-        // BSR mode: Y_out at grid rows col0 + c of state `row` from the product D of
-        // the tile (zero for an empty block row)
-        auto bsr_out = [&](const Item& it, bool have) {
-            const int64_t j = (int64_t)it.tm * kTileM + 32 * q + lane;      // state
-            if (j >= g.M) return;
-            const int64_t i0 = (int64_t)it.tn * kTileN + h * kColsPerThread;   // first grid row
-            const int ea = have ? g.expA[j] : 0;
+    } else if (kBsr) {
+        // ---------------- output of the BSR mode (two warps, 64 states each): Y_out = alpha D -
+        // beta Y_prev from the products D that the epilogue has left in Y_out, with D already
+        // of H - c unless the row is unfolded.  Warps of their own: the two FP64 operations an
+        // element take 8200 cycles an item at least and wait for Y_prev; done by the epilogue
+        // warps (at once, or in pieces between the drains) they kept the drains and so
+        // the MMAs waiting for a fifth of the time, and no registers or shared memory are left
+        // to hold an item's products for later, but L2 is.
+        int n = 0;
+        bool ok = true;
+        for (int64_t item = blockIdx.x; ok && item < total; item += gridDim.x, n++) {
+            if (__any_sync(0xffffffffu, *abort_v)) break;
+            const Item it = decode<kBsr>(g, item);
+            ok = __all_sync(0xffffffffu, mbar_wait(sa(&dfull[n & 1]), (uint32_t)((n >> 1) & 1), g.wait_ns));
+            if (!ok) break;
+            constexpr int kStep = 4;
+            const int64_t i0 = (int64_t)it.tn * kTileN;
+#pragma unroll 1
+            for (int half = 0; half < 2; half++) {
+                const int64_t j = (int64_t)it.tm * kTileM + 64 * (warp - 2) + 32 * half + lane;
+                if (j >= g.M) continue;
+                double* out = g.C + i0 * g.ldc + j;
+                const double* prev = g.Yprev ? g.Yprev + i0 * g.ldprev + j : nullptr;
+                double d[2][kStep], p[2][kStep];
+                auto load = [&](int b, int r) {
 #pragma unroll
-            for (int c = 0; c < kColsPerThread; c++) {
-                const int64_t i = i0 + c;
-                const int eb = have ? g.expH[i] : 0;
-                const double D = (ea != 0 && eb != 0) ? combine(hi[c], lo[c], (ea - 1021) + (eb - 1021)) : 0.0;
-                double y = g.alpha * fma(-g.cshift, g.Ycur[i * g.ldcur + j], D);
-                if (g.Yprev) y = fma(-g.beta, g.Yprev[i * g.ldprev + j], y);
-                nonfinite |= !isfinite(y);
-                g.C[i * g.ldc + j] = y;
+                    for (int c = 0; c < kStep; c++) {
+                        d[b][c] = out[(r + c) * g.ldc];
+                        p[b][c] = prev ? prev[(r + c) * g.ldprev] : 0.0;
+                    }
+                };
+                load(0, 0);
+#pragma unroll 2
+                for (int r = 0; r < kTileN; r += kStep) {
+                    const int b = (r / kStep) & 1;
+                    if (r + kStep < kTileN) load(b ^ 1, r + kStep);   // on the way before this step's stores
+#pragma unroll
+                    for (int c = 0; c < kStep; c++) {
+                        double D = d[b][c];
+                        if (it.unfolded) D = fma(-g.cshift, g.Ycur[(i0 + r + c) * g.ldcur + j], D);
+                        double y = g.alpha * D;
+                        if (prev) y = fma(-g.beta, p[b][c], y);
+                        nonfinite |= (__double2hiint(y) & 0x7ff00000) == 0x7ff00000;
+                        out[(r + c) * g.ldc] = y;
+                    }
+                }
             }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&dempty[n & 1]);
+        }
+        if (!ok && lane == 0) *abort_v = 1;
+    }
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" :: "n"(kRegsEpilogue));
+        // ---------------- epilogue: exact drains into 96-bit integers, then the output
+        const int q = warp & 3, h = (warp - 4) >> 2;
+        const uint32_t lane_base = (uint32_t)(32 * q) << 16;
+        int ev = 0, set = 0;
+        Sum96 sum[kColsPerThread];
+        // drain number ev, of group GI: its accumulators are given back as soon as they are in
+        // registers, the last conversions (16 lanes a cycle and SM) overlap the next MMAs
+        auto drain = [&](auto gc) -> bool {
+            constexpr int GI = decltype(gc)::value, LO = Gr::lo(GI), HI = Gr::hi(GI), kAccs = HI - LO;
+            constexpr int kBatch = kAccs > 2 ? 16 : 32;       // columns read before they are converted
+            constexpr int kShift = 64 - 8 * (HI + 1);         // unit of E_{HI + 1}
+            const int slot = ev % kEvents;
+            if (!__all_sync(0xffffffffu,
+                            !*abort_v && mbar_wait(sa(&efull[slot]), (uint32_t)((ev / kEvents) & 1), g.wait_ns)))
+                return false;
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            const uint32_t at = tmem + lane_base + (uint32_t)(Gr::column(GI, set) + h * kColsPerThread);
+#pragma unroll
+            for (int c0 = 0; c0 < kColsPerThread; c0 += kBatch) {
+                uint32_t v[kAccs][kBatch / 8][8];
+#pragma unroll
+                for (int a = 0; a < kAccs; a++)
+#pragma unroll
+                    for (int k = 0; k < kBatch / 8; k++) tmem_ld8(at + (uint32_t)(a * kTileN + c0 + 8 * k), v[a][k]);
+                asm volatile("tcgen05.wait::ld.sync.aligned;");
+                if (c0 + kBatch == kColsPerThread) {
+                    asm volatile("tcgen05.fence::before_thread_sync;");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&eempty[slot]);
+                }
+#pragma unroll
+                for (int c = 0; c < kBatch; c++) {
+                    // E_l holds an integer of at most 2^24, in units of 2^-8l
+                    long long x = __float2int_rn(__uint_as_float(v[kAccs - 1][c / 8][c % 8]));
+#pragma unroll
+                    for (int a = kAccs - 2; a >= 0; a--)
+                        x = mad_wide(__float2int_rn(__uint_as_float(v[a][c / 8][c % 8])), 1 << (8 * (kAccs - 1 - a)), x);
+                    add96<kShift>(sum[c0 + c], x);
+                }
+            }
+            if (NS == 5 && GI == 1) set ^= 1;
+            ev++;
+            return true;
         };
-        for (int64_t item = blockIdx.x; item < total; item += gridDim.x) {
+        auto drain_group = [&](int gi) -> bool {
+            if (gi == 0) return drain(std::integral_constant<int, 0>{});
+            if (NS == 5 || gi == 1) return drain(std::integral_constant<int, 1>{});
+            return drain(std::integral_constant<int, Gr::kCount - 1>{});
+        };
+        int n = 0;
+        for (int64_t item = blockIdx.x; item < total; item += gridDim.x, n++) {
             const Item it = decode<kBsr>(g, item);
 #pragma unroll
-            for (int c = 0; c < kColsPerThread; c++) hi[c] = lo[c] = 0;
-            if (kBsr && it.KB == 0) {   // empty block row: no MMA, no drain
-                if (*abort_v) break;
-                bsr_out(it, false);
-                continue;
+            for (int c = 0; c < kColsPerThread; c++) sum[c] = Sum96{0, 0, 0};
+            if (kBsr && *abort_v) break;
+            // exponents of the item's state and (one a lane) of its grid rows
+            int ea = 0, eh = 0;
+            if (kBsr && it.KB > 0) {
+                const int j = it.tm * kTileM + 32 * q + lane;
+                if (j < g.M) ea = g.expA[j];
+                eh = g.expH[it.tn * kTileN + h * kColsPerThread + lane];
             }
             bool ok = true;
-            for (int kb = 0; kb < it.KB; kb++) {
-                const int kind = event_at(kb, it.KB);
-                if (!kind) continue;
-                if (!__all_sync(0xffffffffu, !*abort_v && mbar_wait(sa(&efull), (uint32_t)(ev & 1), g.wait_ns))) {
-                    ok = false;
+            for (int kb = 0; ok && kb < it.KB; kb++) {
+                const bool end = kb == it.KB - 1;
+                const int gi0 = end ? 0 : Gr::event(kb);
+                if (gi0 < 0) continue;
+                for (int gi = gi0; ok && (gi == gi0 || (end && gi < Gr::kCount)); gi++) ok = drain_group(gi);
+            }
+            if (!ok) { *abort_v = 1; break; }
+            if constexpr (kBsr) {
+                // the products (zero for an empty block row) for the output warps
+                const int64_t j = (int64_t)it.tm * kTileM + 32 * q + lane;
+                double* out = g.C + ((int64_t)it.tn * kTileN + h * kColsPerThread) * g.ldc + j;
+#pragma unroll
+                for (int c = 0; c < kColsPerThread; c++) {
+                    const int eb = __shfl_sync(0xffffffffu, eh, c);
+                    const double D = (ea != 0 && eb != 0) ? combine(sum[c], (ea - 1021) + (eb - 1021)) : 0.0;
+                    if (j < g.M) out[c * g.ldc] = D;
+                }
+                if (n >= 2 && !__all_sync(0xffffffffu, mbar_wait(sa(&dempty[n & 1]), (uint32_t)(((n - 2) >> 1) & 1),
+                                                                 g.wait_ns))) {
+                    *abort_v = 1;
                     break;
                 }
-                asm volatile("tcgen05.fence::after_thread_sync;");
-#pragma unroll
-                for (int a = 0; a < kAccs; a++) {
-                    const bool take = (a < 4) ? (kind & kXEvent) : (kind & kYEvent);
-                    if (!take) continue;
-                    // E_l (l = a + 2) holds an exact multiple of 2^-8l below 2^24 units
-                    const float up = pow2f(8 * (a + 2));
-                    const long long mul = 1ll << (a < 4 ? 40 - 8 * (a + 2) : 64 - 8 * (a + 2));
-                    uint32_t v[16];
-                    tmem_ld16(tmem + lane_base + (uint32_t)(a * kTileN + h * kColsPerThread), v);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;");
-#pragma unroll
-                    for (int c = 0; c < 16; c++) {
-                        const long long iv = (long long)__float2int_rn(__uint_as_float(v[c]) * up) * mul;
-                        if (a < 4) hi[c] += iv;
-                        else lo[c] += iv;
-                    }
-                }
-                asm volatile("tcgen05.fence::before_thread_sync;");
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&eempty);
-                ev++;
-                if (kind == kFullEvent && kBsr) {
-                    bsr_out(it, true);
-                } else if (kind == kFullEvent) {
-                    const int64_t row = (int64_t)it.tm * kTileM + 32 * q + lane;        // within the batch
-                    const int64_t orow = it.batch * g.m_batch + row;                     // output row
-                    const int64_t col0 = (int64_t)it.tn * kTileN + h * kColsPerThread;
-                    const bool valid = row < g.m_batch && orow < g.M;
-                    const int ea = valid ? g.expA[it.batch * g.a_batch_rows + row] : 0;
-                    const int* expB = g.expB + it.batch * g.b_batch_rows;
-                    if (g.part) {
-                        const int z = it.kb0 / g.kb_split;
-                        double* dst = g.part + ((int64_t)z * g.Mp + row) * g.Np + col0;
+                if (lane == 0) mbar_arrive(&dfull[n & 1]);
+            } else if (it.KB > 0) {
+                const int64_t row = (int64_t)it.tm * kTileM + 32 * q + lane;        // within the batch
+                const int64_t orow = it.batch * g.m_batch + row;                     // output row
+                const int64_t col0 = (int64_t)it.tn * kTileN + h * kColsPerThread;
+                const bool valid = row < g.m_batch && orow < g.M;
+                const int ea = valid ? g.expA[it.batch * g.a_batch_tiles * kTileM + row] : 0;
+                const int* expB = g.expB + it.batch * g.b_batch_tiles * kTileN;
+                double* dst = g.part ? g.part + ((int64_t)(it.kb0 / g.kb_split) * g.Mp + row) * g.Np + col0
+                                     : g.C + orow * g.ldc + col0;
+                const bool whole = g.part || (valid && col0 + kColsPerThread <= g.Nc &&
+                                              (reinterpret_cast<uintptr_t>(dst) & 31u) == 0);
 #pragma unroll
-                        for (int c = 0; c < kColsPerThread; c++) {
-                            const int eb = (col0 + c < g.Nc) ? expB[col0 + c] : 0;
-                            dst[c] = (ea != 0 && eb != 0) ? combine(hi[c], lo[c], (ea - 1021) + (eb - 1021)) : 0.0;
-                        }
+                for (int c0 = 0; c0 < kColsPerThread; c0 += 4) {
+                    double v[4];
+#pragma unroll
+                    for (int c = 0; c < 4; c++) {
+                        const int eb = (col0 + c0 + c < g.Nc) ? expB[col0 + c0 + c] : 0;
+                        v[c] = (ea != 0 && eb != 0) ? combine(sum[c0 + c], (ea - 1021) + (eb - 1021)) : 0.0;
+                    }
+                    if (whole) {     // a thread's columns as whole 32-byte sectors
+                        asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};"
+                                     :: "l"(dst + c0), "d"(v[0]), "d"(v[1]), "d"(v[2]), "d"(v[3]) : "memory");
                     } else if (valid) {
-                        double* dst = g.C + orow * g.ldc + col0;
 #pragma unroll
-                        for (int c = 0; c < kColsPerThread; c++) {
-                            if (col0 + c >= g.Nc) break;
-                            const int eb = expB[col0 + c];
-                            dst[c] = (ea != 0 && eb != 0) ? combine(hi[c], lo[c], (ea - 1021) + (eb - 1021)) : 0.0;
-                        }
+                        for (int c = 0; c < 4; c++)
+                            if (col0 + c0 + c < g.Nc) dst[c0 + c] = v[c];
                     }
                 }
             }
-            if (!ok) { *abort_v = 1; break; }
         }
     }
 
@@ -616,80 +953,112 @@ __global__ void oz_exponents_kernel(const double* __restrict__ src, int64_t ld, 
     if (bad) raise_status(status, DEV_NONFINITE);
 }
 
-// The seven BF16 slices of one value x of a row whose largest exponent field is efm.
-__device__ __forceinline__ void digits_of(double x, int efm, __nv_bfloat16 (&out)[kSlices]) {
+// Fixed-point form of x in a row whose largest exponent field is efm: sign(x) |x| 2^{-e}
+// 2^{56} rounded to nearest, e = efm - 1021, below 2^55 in magnitude.
+__device__ __forceinline__ long long fixed_point(double x, int efm) {
     const long long b = __double_as_longlong(x);
     const int ef = (int)((b >> 52) & 0x7ff);
-    long long F = 0;
-    if (ef != 0 && efm != 0 && ef != 0x7ff) {
-        // F = |x| 2^{-e} 2^{56} < 2^55 with e = efm - 1021: mant 2^{ef - efm + 2}, the
-        // right shifts rounded to nearest
-        const long long mant = (b & ((1ll << 52) - 1)) | (1ll << 52);
-        const int sh = efm - ef - 2;
-        if (sh <= 0) F = mant << (-sh);
-        else F = sh < 60 ? (mant + (1ll << (sh - 1))) >> sh : 0;
-    }
-    // balanced base-256 digits, least significant first; the top digit keeps its carry
-    int d[kSlices];
-    int carry = 0;
-#pragma unroll
-    for (int t = kSlices - 1; t >= 1; t--) {
-        int byte = (int)((F >> (8 * (kSlices - 1 - t))) & 255) + carry;
-        carry = byte >= 128;
-        d[t] = carry ? byte - 256 : byte;
-    }
-    d[0] = (int)(F >> (8 * (kSlices - 1))) + carry;
-    const bool neg = b < 0;
-#pragma unroll
-    for (int t = 0; t < kSlices; t++) {
-        const float v = (float)(neg ? -d[t] : d[t]) * pow2f(-8 * (t + 1));
-        out[t] = __float2bfloat16_rn(v);
-    }
+    if (ef == 0 || efm == 0 || ef == 0x7ff) return 0;
+    const long long mant = (b & ((1ll << 52) - 1)) | (1ll << 52);
+    const int sh = efm - ef - 2;
+    long long F;
+    if (sh <= 0) F = mant << (-sh);
+    else F = sh < 60 ? (mant + (1ll << (sh - 1))) >> sh : 0;
+    return b < 0 ? -F : F;
 }
 
-// Slices of A_hat into [kSlices][nbatch * rows_pad][K_pad] (K contiguous), zero in
-// the padding; batch z = blockIdx.z as in oz_exponents_kernel, at rows z * rows_pad.
-// Only the first nplanes planes are written (the five-slice steps read no others).
-// 32 x 32 tiles through shared memory so that reads and writes are both coalesced
-// when A_hat is the transpose of src.
-template <bool kTrans>
-__global__ void oz_slice_kernel(const double* __restrict__ src, int64_t ld, int64_t rows, int64_t Kb, int64_t Ktot,
-                                int64_t src_bstride, const int* __restrict__ exps, int64_t rows_pad, int64_t K_pad,
-                                size_t plane, int nplanes, __nv_bfloat16* __restrict__ slices) {
-    __shared__ double tile[32][33];
-    const int64_t z = blockIdx.z;
-    src += z * src_bstride;
-    exps += z * rows_pad;
-    slices += (size_t)z * rows_pad * K_pad;
-    const int64_t K = Ktot - z * Kb < Kb ? Ktot - z * Kb : Kb;
-    const int64_t k0 = (int64_t)blockIdx.x * 32;
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    // row tiles in a grid-stride loop: gridDim.y is at most 65535
-    for (int64_t rt = blockIdx.y; rt * 32 < rows_pad; rt += gridDim.y) {
-        const int64_t r0 = rt * 32;
-        __syncthreads();   // the previous tile has been read
-        for (int i = ty; i < 32; i += blockDim.y) {
-            double v = 0.0;
-            if (kTrans) {   // src row k0 + i, column r0 + tx  ->  tile[k][r]
-                const int64_t k = k0 + i, r = r0 + tx;
-                if (k < K && r < rows) v = src[k * ld + r];
-                tile[i][tx] = v;
-            } else {        // src row r0 + i, column k0 + tx  ->  tile[k][r]
-                const int64_t r = r0 + i, k = k0 + tx;
-                if (k < K && r < rows) v = src[r * ld + k];
-                tile[tx][i] = v;
+// The seven digit planes of eight consecutive K entries of a row, 16 bytes per plane.
+// Balanced base-256 digits in [-128, 127] (the top one keeps the carry): adding 128 to
+// each of the six low digits at once turns them into the bytes of G, so digit = byte -
+// 128 without a carry chain; bytes become floats by placing them under 2^23, and an exact
+// BF16 is the upper half of its float.
+__device__ __forceinline__ void digits8(const long long (&F)[kChunk], uint4 (&out)[kSlices]) {
+    uint32_t w[kSlices][4];
+#pragma unroll
+    for (int pr = 0; pr < kChunk / 2; pr++) {
+        float f[2][kSlices];
+#pragma unroll
+        for (int k = 0; k < 2; k++) {
+            const long long G = F[2 * pr + k] + 0x0000808080808080ll;
+            const uint32_t glo = (uint32_t)G, ghi = (uint32_t)((unsigned long long)G >> 32);
+            f[k][0] = __int_as_float(0x4B400000 + ((int)ghi >> 16)) - 12582912.0f;
+#pragma unroll
+            for (int t = 1; t < kSlices; t++) {
+                const int byte = kSlices - 1 - t;
+                const uint32_t u = __byte_perm(byte < 4 ? glo : ghi, 0x4B000000u, 0x7440u + (uint32_t)(byte & 3));
+                f[k][t] = __uint_as_float(u) - 8388736.0f;
             }
         }
-        __syncthreads();
-        for (int i = ty; i < 32; i += blockDim.y) {
-            const int64_t r = r0 + i, k = k0 + tx;
-            if (r >= rows_pad || k >= K_pad) continue;
-            const int efm = r < rows ? exps[r] : 0;
-            __nv_bfloat16 dg[kSlices];
-            digits_of(tile[tx][i], efm, dg);
 #pragma unroll
-            for (int t = 0; t < kSlices; t++)
-                if (t < nplanes) slices[t * plane + (size_t)r * K_pad + k] = dg[t];
+        for (int t = 0; t < kSlices; t++)
+            w[t][pr] = __byte_perm(__float_as_uint(f[0][t]), __float_as_uint(f[1][t]), 0x7632);
+    }
+#pragma unroll
+    for (int t = 0; t < kSlices; t++) out[t] = make_uint4(w[t][0], w[t][1], w[t][2], w[t][3]);
+}
+
+// Digit planes of A_hat in tiles of kRows rows: [batch z][row tile][K chunk][7][kRows][8],
+// zero in the padding; batch z = blockIdx.z as in oz_exponents_kernel.  Only the first
+// nplanes planes are written (the five-slice steps read no others).  A thread makes the
+// eight digits of one row and chunk, so that each plane is written 16 bytes a thread and
+// 512 contiguous bytes a warp: bounded by the reads of src and those writes.
+// kTrans (A_hat[r][k] = src[k * ld + r]): a warp reads 32 consecutive columns of each of
+// the chunk's src rows, straight into the threads that need them.  Otherwise 32 rows x 64
+// columns pass through shared memory.
+template <bool kTrans, int kRows>
+__global__ void __launch_bounds__(256) oz_slice_kernel(const double* __restrict__ src, int64_t ld, int64_t rows,
+                                                       int64_t Kb, int64_t Ktot, int64_t src_bstride,
+                                                       const int* __restrict__ exps, int64_t tiles, int64_t chunks,
+                                                       int nplanes, unsigned char* __restrict__ slices) {
+    const int64_t z = blockIdx.z;
+    src += z * src_bstride;
+    exps += z * tiles * kRows;
+    slices += (size_t)(z * tiles * chunks) * (kSlices * kRows * 16);
+    const int64_t K = Ktot - z * Kb < Kb ? Ktot - z * Kb : Kb;
+    auto store = [&](const double (&x)[kChunk], int64_t r, int64_t ch, int efm) {
+        long long F[kChunk];
+#pragma unroll
+        for (int k = 0; k < kChunk; k++) F[k] = fixed_point(x[k], efm);
+        uint4 dg[kSlices];
+        digits8(F, dg);
+        uint4* dst = reinterpret_cast<uint4*>(slices) + ((r / kRows) * chunks + ch) * (kSlices * kRows) + r % kRows;
+#pragma unroll
+        for (int t = 0; t < kSlices; t++)
+            if (t < nplanes) dst[t * kRows] = dg[t];
+    };
+    if (kTrans) {
+        // blocks of 256 / kRows chunks x one row tile
+        const int64_t ch = (int64_t)blockIdx.x * (256 / kRows) + threadIdx.x / kRows;
+        if (ch >= chunks) return;
+        const int64_t k0 = ch * kChunk;
+        for (int64_t rt = blockIdx.y; rt < tiles; rt += gridDim.y) {
+            const int64_t r = rt * kRows + threadIdx.x % kRows;
+            double x[kChunk];
+#pragma unroll
+            for (int k = 0; k < kChunk; k++) x[k] = (r < rows && k0 + k < K) ? src[(k0 + k) * ld + r] : 0.0;
+            store(x, r, ch, r < rows ? exps[r] : 0);
+        }
+    } else {
+        __shared__ double tile[32][65];
+        const int64_t k0 = (int64_t)blockIdx.x * 64;
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        for (int64_t rt = blockIdx.y; rt < tiles * (kRows / 32); rt += gridDim.y) {
+            const int64_t r0 = rt * 32;
+            __syncthreads();   // the previous tile has been read
+            for (int i = warp; i < 32; i += 8)
+#pragma unroll
+                for (int e = 0; e < 2; e++) {
+                    const int64_t k = k0 + 32 * e + lane;
+                    tile[i][32 * e + lane] = (r0 + i < rows && k < K) ? src[(r0 + i) * ld + k] : 0.0;
+                }
+            __syncthreads();
+            const int64_t ch = (int64_t)blockIdx.x * 8 + warp, r = r0 + lane;
+            if (ch < chunks) {
+                double x[kChunk];
+#pragma unroll
+                for (int k = 0; k < kChunk; k++) x[k] = tile[lane][warp * kChunk + k];
+                store(x, r, ch, r < rows ? exps[r] : 0);
+            }
         }
     }
 }
@@ -719,54 +1088,62 @@ struct CountAr {
     }
 };
 
-// Workspace pieces of one operand: exponents (int32 per padded row) and slices
-// [kSlices][nbatch * rows_pad][K_pad]; batch b holds rows b * rows_pad ...
+// Workspace pieces of one operand: exponents (int32 per padded row) and digit planes
+// [nbatch][row tile][K chunk][7][tile_rows][8]; tile_rows 128 for A_hat, 64 for B_hat.
 struct OzOperand {
     int* exps = nullptr;
-    __nv_bfloat16* slices = nullptr;
-    int64_t rows = 0, K = 0, rows_pad = 0, K_pad = 0;
+    unsigned char* slices = nullptr;
+    int64_t rows = 0, K = 0, tiles = 0, chunks = 0;
+    int tile_rows = kTileM;
     int nbatch = 1;
-    int64_t plane_rows() const { return (int64_t)nbatch * rows_pad; }
+    int64_t padded_rows() const { return (int64_t)nbatch * tiles * tile_rows; }
 };
 
 template <typename Ar>
-void oz_operand_layout(Ar& ar, int64_t rows, int64_t K, int nbatch, int64_t row_pad, OzOperand* op) {
+void oz_operand_layout(Ar& ar, int64_t rows, int64_t K, int nbatch, int tile_rows, OzOperand* op) {
     OzOperand o;
     o.rows = rows;
     o.K = K;
     o.nbatch = nbatch;
-    o.rows_pad = round_up(rows, row_pad);
-    o.K_pad = round_up(K, 32);   // the slicing kernel's tiles are 32 wide in K
-    o.exps = ar.template take<int>((size_t)o.plane_rows());
-    o.slices = ar.template take<__nv_bfloat16>((size_t)kSlices * o.plane_rows() * o.K_pad);
+    o.tile_rows = tile_rows;
+    o.tiles = (rows + tile_rows - 1) / tile_rows;
+    o.chunks = round_up(K, kKB) / kChunk;
+    o.exps = ar.template take<int>((size_t)o.padded_rows());
+    o.slices = ar.template take<unsigned char>((size_t)o.padded_rows() * o.chunks * (kSlices * 16));
     if (op) *op = o;
 }
 
-// Exponents and slices of an operand; batch b reads src + b * src_bstride over
-// min(o.K, Ktot - b o.K) of the K dimension.  nplanes: slice planes written.
-int oz_prepare(const double* src, int64_t ld, bool trans, const OzOperand& o, int64_t Ktot, int64_t src_bstride,
-               unsigned* status, cudaStream_t s, int nplanes = kSlices) {
-    CHFSI_CUDA_TRY(cudaMemsetAsync(o.exps, 0, sizeof(int) * (size_t)o.plane_rows(), s));
-    if (trans) {
-        dim3 grid((unsigned)((o.rows + 255) / 256), (unsigned)((o.K + 255) / 256), (unsigned)o.nbatch);
-        oz_exponents_kernel<true><<<grid, 256, 0, s>>>(src, ld, o.rows, o.K, Ktot, src_bstride, o.rows_pad, o.exps,
-                                                      status);
-    } else {
-        dim3 grid((unsigned)((o.rows * 32 + 255) / 256), 1, (unsigned)o.nbatch);
-        oz_exponents_kernel<false><<<grid, 256, 0, s>>>(src, ld, o.rows, o.K, Ktot, src_bstride, o.rows_pad, o.exps,
-                                                       status);
-    }
-    CHFSI_LAUNCH_CHECK();
-    dim3 grid((unsigned)(o.K_pad / 32), (unsigned)std::min<int64_t>(o.rows_pad / 32, 65535), (unsigned)o.nbatch);
-    const size_t plane = (size_t)o.plane_rows() * o.K_pad;
-    if (trans)
-        oz_slice_kernel<true><<<grid, dim3(32, 8), 0, s>>>(src, ld, o.rows, o.K, Ktot, src_bstride, o.exps, o.rows_pad,
-                                                          o.K_pad, plane, nplanes, o.slices);
-    else
-        oz_slice_kernel<false><<<grid, dim3(32, 8), 0, s>>>(src, ld, o.rows, o.K, Ktot, src_bstride, o.exps,
-                                                           o.rows_pad, o.K_pad, plane, nplanes, o.slices);
+template <bool kTrans, int kRows>
+int launch_slices(const double* src, int64_t ld, const OzOperand& o, int64_t Ktot, int64_t src_bstride, int nplanes,
+                  cudaStream_t s) {
+    const int64_t per = kTrans ? 256 / kRows : 8, ytiles = kTrans ? o.tiles : o.tiles * (kRows / 32);
+    const dim3 grid((unsigned)((o.chunks + per - 1) / per), (unsigned)std::min<int64_t>(ytiles, 65535),
+                    (unsigned)o.nbatch);
+    oz_slice_kernel<kTrans, kRows><<<grid, 256, 0, s>>>(src, ld, o.rows, o.K, Ktot, src_bstride, o.exps, o.tiles,
+                                                        o.chunks, nplanes, o.slices);
     CHFSI_LAUNCH_CHECK();
     return CHFSI_OK;
+}
+
+// Exponents and digit planes of an operand; batch b reads src + b * src_bstride over
+// min(o.K, Ktot - b o.K) of the K dimension.  nplanes: digit planes written.
+int oz_prepare(const double* src, int64_t ld, bool trans, const OzOperand& o, int64_t Ktot, int64_t src_bstride,
+               unsigned* status, cudaStream_t s, int nplanes = kSlices) {
+    CHFSI_CUDA_TRY(cudaMemsetAsync(o.exps, 0, sizeof(int) * (size_t)o.padded_rows(), s));
+    const int64_t brows = o.tiles * o.tile_rows;
+    if (trans) {
+        dim3 grid((unsigned)((o.rows + 255) / 256), (unsigned)((o.K + 255) / 256), (unsigned)o.nbatch);
+        oz_exponents_kernel<true><<<grid, 256, 0, s>>>(src, ld, o.rows, o.K, Ktot, src_bstride, brows, o.exps, status);
+    } else {
+        dim3 grid((unsigned)((o.rows * 32 + 255) / 256), 1, (unsigned)o.nbatch);
+        oz_exponents_kernel<false><<<grid, 256, 0, s>>>(src, ld, o.rows, o.K, Ktot, src_bstride, brows, o.exps, status);
+    }
+    CHFSI_LAUNCH_CHECK();
+    if (o.tile_rows == kTileM)
+        return trans ? launch_slices<true, kTileM>(src, ld, o, Ktot, src_bstride, nplanes, s)
+                     : launch_slices<false, kTileM>(src, ld, o, Ktot, src_bstride, nplanes, s);
+    return trans ? launch_slices<true, kTileN>(src, ld, o, Ktot, src_bstride, nplanes, s)
+                 : launch_slices<false, kTileN>(src, ld, o, Ktot, src_bstride, nplanes, s);
 }
 
 // Split-K count for a product whose output has `tiles` tiles: at most kMaxItemKB
@@ -794,19 +1171,19 @@ template <typename Ar>
 void oz_layout(Ar& ar, bool tn_form, int64_t M, int64_t Nc, int64_t K, bool same, int sms, OzPlan* plan) {
     OzPlan p;
     p.same = same;
-    oz_operand_layout(ar, M, K, 1, kRowPad, &p.A);
+    oz_operand_layout(ar, M, K, 1, kTileM, &p.A);
     if (same) p.B = p.A;
-    else oz_operand_layout(ar, Nc, K, 1, kRowPad, &p.B);
+    else oz_operand_layout(ar, Nc, K, 1, kTileN, &p.B);
     if (tn_form) {
         const int64_t tm = (M + kTileM - 1) / kTileM, tn = (Nc + kTileN - 1) / kTileN;
-        p.splits = oz_splits(tm * tn, (int)(p.A.K_pad / kKB), sms > 0 ? sms : 148);
+        p.splits = oz_splits(tm * tn, (int)(p.A.chunks / kStageChunks), sms > 0 ? sms : 148);
         p.part = ar.template take<double>((size_t)p.splits * (tm * kTileM) * (tn * kTileN));
     }
     if (plan) *plan = p;
 }
 
 // One persistent CTA per SM (or per work item, if fewer).
-int launch_oz(const CUtensorMap& tmA, const CUtensorMap& tmB, const OzArgs& g, int64_t total, cudaStream_t s) {
+int launch_oz(const OzArgs& g, const CUtensorMap& tmA, int64_t total, cudaStream_t s) {
     if (total <= 0) return CHFSI_OK;
     const int dev = current_device();
     if (dev < 0) return CHFSI_ERR_CUDA;
@@ -825,13 +1202,27 @@ int launch_oz(const CUtensorMap& tmA, const CUtensorMap& tmB, const OzArgs& g, i
     if (sms <= 0) return CHFSI_ERR_CUDA;
     const unsigned grid = (unsigned)(total < sms ? total : sms);
     if (g.bsr && g.slices == 5)
-        oz_gemm_kernel<true, 5><<<grid, kThreads, OzShape<5>::kSmemBytes, s>>>(tmA, tmB, g, total);
+        oz_gemm_kernel<true, 5><<<grid, kThreads, OzShape<5>::kSmemBytes, s>>>(g, tmA, total);
     else if (g.bsr)
-        oz_gemm_kernel<true, 7><<<grid, kThreads, OzShape<7>::kSmemBytes, s>>>(tmA, tmB, g, total);
+        oz_gemm_kernel<true, 7><<<grid, kThreads, OzShape<7>::kSmemBytes, s>>>(g, tmA, total);
     else
-        oz_gemm_kernel<false, 7><<<grid, kThreads, OzShape<7>::kSmemBytes, s>>>(tmA, tmB, g, total);
+        oz_gemm_kernel<false, 7><<<grid, kThreads, OzShape<7>::kSmemBytes, s>>>(g, tmA, total);
     CHFSI_LAUNCH_CHECK();
     return CHFSI_OK;
+}
+
+// Tensor map over the planes of an operand with 128-row tiles, [tile and chunk][7][512
+// words]: a box is 64 rows of the seven planes of a slot's two chunks.
+int make_map_planes(CUtensorMap* map, const OzOperand& o) {
+    EncodeTiledFn enc = encode_fn();
+    if (!enc) return CHFSI_ERR_CUDA;
+    const cuuint64_t dims[3] = {kPlaneA / 4, kSlices, (cuuint64_t)(o.nbatch * o.tiles * o.chunks)};
+    const cuuint64_t strides[2] = {kPlaneA, kSlices * kPlaneA};
+    const cuuint32_t box[3] = {kPlaneB / 4, kSlices, kSlotChunks}, es[3] = {1, 1, 1};
+    const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, o.slices, dims, strides, box, es,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? CHFSI_OK : CHFSI_ERR_CUDA;
 }
 
 // The product of prepared operands.  nbatch > 1: independent products, batch b of the
@@ -839,21 +1230,16 @@ int launch_oz(const CUtensorMap& tmA, const CUtensorMap& tmB, const OzArgs& g, i
 int oz_run(const OzPlan& p, bool tn_form, double* C, int64_t ldc, int64_t M, int64_t Nc, bool symmetric,
            bool b_upper, unsigned* status, cudaStream_t s, int nbatch = 1, int64_t m_batch = 0) {
     if (M <= 0 || Nc <= 0) return CHFSI_OK;
-    const int64_t K_pad = p.A.K_pad;
-    if (K_pad > (int64_t)1 << 21 || p.A.plane_rows() * kSlices > INT32_MAX || p.B.plane_rows() * kSlices > INT32_MAX)
+    const int64_t K_pad = p.A.chunks * kChunk;
+    if (K_pad > (int64_t)1 << 21 || p.A.padded_rows() * kSlices > INT32_MAX || p.B.padded_rows() * kSlices > INT32_MAX)
         return CHFSI_ERR_UNSUPPORTED;
     if (!tn_form && K_pad > (int64_t)kMaxItemKB * kKB) return CHFSI_ERR_UNSUPPORTED;   // no split-K in the nn form
     if (nbatch > 1 && (tn_form || symmetric || p.A.nbatch != nbatch || p.B.nbatch != nbatch || m_batch <= 0 ||
-                       m_batch > p.A.rows_pad))
+                       m_batch > p.A.tiles * kTileM))
         return CHFSI_ERR_ARG;
-    CUtensorMap tmA, tmB;
     int rc;
-    if ((rc = make_map_bf16(&tmA, p.A.slices, K_pad, kSlices * p.A.plane_rows(), kKB, kTileM,
-                            kTmaSwizzle)))
-        return rc;
-    if ((rc = make_map_bf16(&tmB, p.B.slices, K_pad, kSlices * p.B.plane_rows(), kKB, kTileN,
-                            kTmaSwizzle)))
-        return rc;
+    CUtensorMap tmA{};
+    if (p.same && (rc = make_map_planes(&tmA, p.A))) return rc;
     OzArgs g{};
     const int64_t mb = nbatch > 1 ? m_batch : M;
     g.M = M;
@@ -861,16 +1247,19 @@ int oz_run(const OzPlan& p, bool tn_form, double* C, int64_t ldc, int64_t M, int
     g.ldc = ldc;
     g.nbatch = nbatch;
     g.m_batch = mb;
-    g.a_batch_rows = p.A.rows_pad;
-    g.b_batch_rows = p.B.rows_pad;
+    g.A = p.A.slices;
+    g.B = p.B.slices;
+    g.b_in_a = p.same ? 1 : 0;
+    g.chunksA = p.A.chunks;
+    g.chunksB = p.B.chunks;
+    g.a_batch_tiles = p.A.tiles;
+    g.b_batch_tiles = p.B.tiles;
     g.tilesM = (int)((mb + kTileM - 1) / kTileM);
     g.tilesN = (int)((Nc + kTileN - 1) / kTileN);
     g.Mp = (int64_t)g.tilesM * kTileM;
     g.Np = (int64_t)g.tilesN * kTileN;
     g.expA = p.A.exps;
     g.expB = p.B.exps;
-    g.rowsA_pad = p.A.plane_rows();
-    g.rowsB_pad = p.B.plane_rows();
     g.kb_total = (int)(K_pad / kKB);
     g.splits = tn_form ? p.splits : 1;
     g.kb_split = (g.kb_total + g.splits - 1) / g.splits;
@@ -893,7 +1282,7 @@ int oz_run(const OzPlan& p, bool tn_form, double* C, int64_t ldc, int64_t M, int
     }
     g.pairs = pairs;
     const int64_t total = pairs * g.splits * nbatch;
-    if ((rc = launch_oz(tmA, tmB, g, total, s))) return rc;
+    if ((rc = launch_oz(g, tmA, total, s))) return rc;
     if (tn_form) {
         const int64_t cnt = M * Nc;
         oz_reduce_kernel<<<(unsigned)((cnt + 255) / 256), 256, 0, s>>>(p.part, g.splits, g.Mp, g.Np, M, Nc, C, ldc,
@@ -913,54 +1302,152 @@ template <typename Ar>
 void oz_blockdiag_layout(Ar& ar, int64_t N, int B, int64_t n, OzBlockDiag* out) {
     OzBlockDiag b;
     const int nblk = (int)((N + B - 1) / B);
-    oz_operand_layout(ar, (int64_t)nblk * B, B, 1, kRowPad, &b.D);   // rows of all blocks, K = B
-    oz_operand_layout(ar, n, B, nblk, 32, &b.Y);                      // per block: n rows (Y columns), K = B
+    oz_operand_layout(ar, (int64_t)nblk * B, B, 1, kTileM, &b.D);   // rows of all blocks, K = B
+    oz_operand_layout(ar, n, B, nblk, kTileN, &b.Y);                 // per block: n rows (Y columns), K = B
     if (out) *out = b;
 }
 
-// BSR filter step: slices of H's blocks (made once per filter call; rows = the 64
-// rows of every stored block, K = the block's 64 columns, each row scaled by the
-// largest exponent of its grid row over the whole block row, so that the products of
-// all block columns share one scale) and of Y_cur^T (made per step; rows = states,
-// K = grid points).
+// BSR filter step: digit planes of the chunks of H (made once per filter call) and of
+// Y_cur^T (made per step; rows = states, K = grid points).  H is stored by block rows:
+// of a row's blocks only the chunks of eight columns with a nonzero entry are kept, in
+// order, [chunk][7][64 rows][8], from chunk brow_ptr[R] * 8 on; chunk[] names the chunk of
+// Y_cur that each multiplies, count[] how many a row has (rounded up to a whole stage by
+// zero chunks).  Every grid row has one scale over its whole block row, so that the
+// products of all its chunks share it.
 struct OzBsr {
-    OzOperand H, Y;
+    OzOperand Y;
+    unsigned char* H = nullptr;
+    int32_t *chunk = nullptr, *count = nullptr;
     int* expH = nullptr;      // per grid row
 };
 
 template <typename Ar>
 void oz_bsr_layout(Ar& ar, int64_t nbr, int64_t nblocks, int64_t n, OzBsr* out) {
     OzBsr b;
-    // at least one tile of rows, so that the tensor map is valid without stored blocks
-    oz_operand_layout(ar, (nblocks > 2 ? nblocks : 2) * 64, 64, 1, kRowPad, &b.H);
-    oz_operand_layout(ar, n, nbr * 64, 1, kRowPad, &b.Y);
+    const size_t stored = (size_t)(nblocks > 0 ? nblocks : 1) * kBlockChunks;
+    b.H = ar.template take<unsigned char>(stored * (kSlices * kPlaneB));
+    b.chunk = ar.template take<int32_t>(stored);
+    b.count = ar.template take<int32_t>((size_t)nbr);
+    oz_operand_layout(ar, n, nbr * 64, 1, kTileM, &b.Y);
     b.expH = ar.template take<int>((size_t)(nbr * 64));
     if (out) *out = b;
 }
 
-// Largest exponent field of each grid row of H over its block row: thread r of block R
-// scans row r of every block of the row; the result goes to expH[R * 64 + r] and to
-// the slice exponent of that row in each of the row's blocks.
-__global__ void bsr_row_exponents_kernel(const double* __restrict__ val, const int32_t* __restrict__ brow_ptr,
-                                         int64_t nblocks, int* expH, int* exps, unsigned* status) {
+// Exponents, chunk list and digit planes of one block row per CTA.  The first pass reads
+// the row's blocks with a warp per grid row (512 contiguous bytes a load) for the row's
+// largest exponent and the chunks' nonzero flags, the second makes the kept chunks'
+// digits, a thread per grid row: bounded by reading H twice and writing 14 bytes an entry.
+// A chunk whose entries are all zero (as on the faces of a block that the stencil does
+// not reach) adds nothing to the product and is left out of it.
+// The shift c goes into the digits of the diagonal (of H_ii - c as a two-float sum), so that
+// the step's output need not read Y_cur again nor spend a third FP64 operation an element
+// (8192 outputs an item at two operations a cycle) on it -- where that leaves no grid row
+// of the block row with a larger scale, so that no digit loses weight; other block rows,
+// and those without a stored diagonal block, are marked kUnfolded.
+__global__ void __launch_bounds__(256) oz_bsr_prepare_kernel(const double* __restrict__ val,
+                                                             const int32_t* __restrict__ brow_ptr,
+                                                             const int32_t* __restrict__ bcol, int64_t nblocks,
+                                                             double c, int* expH, int32_t* chunk, int32_t* count,
+                                                             unsigned char* __restrict__ H, unsigned* status) {
+    constexpr int kMaxChunks = kMaxItemKB * kStageChunks;
+    __shared__ int rowmax[64];
+    __shared__ unsigned char flag[kMaxChunks];
+    __shared__ int16_t list[kMaxChunks + kStageChunks];
+    __shared__ int kept, padded, grown;
     const int64_t R = blockIdx.x;
-    const int r = threadIdx.x;
-    int b0 = brow_ptr[R], b1 = brow_ptr[R + 1];
-    b0 = b0 < 0 ? 0 : (b0 > nblocks ? (int)nblocks : b0);
-    b1 = b1 < b0 ? b0 : (b1 > nblocks ? (int)nblocks : b1);
-    int m = 0;
-    bool bad = false;
-    for (int q = b0; q < b1; q++) {
-        const double* row = val + ((int64_t)q * 64 + r) * 64;
-        for (int k = 0; k < 64; k++) {
-            const int ef = (int)((__double_as_longlong(row[k]) >> 52) & 0x7ff);
-            bad |= ef == 0x7ff;
-            m = ef > m ? ef : m;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int qb, nq;
+    bool bad_ptr = false, bad = false;
+    bsr_row_range(brow_ptr, nblocks, R, qb, nq, bad_ptr);
+    for (int p = threadIdx.x; p < nq * kBlockChunks; p += 256) flag[p] = 0;
+    if (threadIdx.x == 0) grown = 0;
+    __syncthreads();
+    int qd = -1;        // the first diagonal block of the row
+    int m[8] = {};      // largest exponent fields, without that block's diagonal
+    for (int q = 0; q < nq; q++) {
+        const bool diag = qd < 0 && bcol[qb + q] == (int)R;
+        if (diag) qd = q;
+        const double* blk = val + (int64_t)(qb + q) * 4096;
+        bool any0 = false, any1 = false;
+#pragma unroll
+        for (int i = 0; i < 8; i++) {       // grid rows warp, warp + 8, ...
+            const double* row = blk + (warp + 8 * i) * 64;
+            const int e0 = (__double2hiint(row[lane]) >> 20) & 0x7ff;
+            const int e1 = (__double2hiint(row[32 + lane]) >> 20) & 0x7ff;
+            bad |= e0 == 0x7ff || e1 == 0x7ff;
+            any0 |= e0 != 0;
+            any1 |= e1 != 0;
+            const int d = diag ? warp + 8 * i : -1;      // column of the diagonal entry
+            if (lane != d && e0 > m[i]) m[i] = e0;
+            if (32 + lane != d && e1 > m[i]) m[i] = e1;
+        }
+        const unsigned b0 = __ballot_sync(0xffffffffu, any0), b1 = __ballot_sync(0xffffffffu, any1);
+        if (lane < kBlockChunks && (((lane < 4 ? b0 : b1) >> (8 * (lane & 3))) & 255u)) flag[q * kBlockChunks + lane] = 1;
+    }
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+        const int e = __reduce_max_sync(0xffffffffu, m[i]);
+        if (lane == 0) rowmax[warp + 8 * i] = e;
+    }
+    __syncthreads();
+    // H_ii of this thread's grid row, and its scale without and with the shift
+    const int r = threadIdx.x & 63;
+    const double hii = qd >= 0 ? val[(int64_t)(qb + qd) * 4096 + r * 65] : 0.0;
+    const double sd = hii - c, back = sd + c, err = (hii - back) + ((back - sd) - c);   // hii - c = sd + err
+    const int ed = (__double2hiint(hii) >> 20) & 0x7ff, es = (__double2hiint(sd) >> 20) & 0x7ff;
+    const int em = rowmax[r], plain = em > ed ? em : ed, shifted = em > es ? em : es;
+    if (threadIdx.x < 64 && shifted > plain) grown = 1;
+    __syncthreads();
+    const bool fold = qd >= 0 && c != 0.0 && !grown;
+    const int efm = fold ? shifted : plain;
+    if (fold && threadIdx.x < kBlockChunks) flag[qd * kBlockChunks + threadIdx.x] = 1;
+    __syncthreads();
+    if (warp == 0) {
+        int k = 0;
+        for (int c0 = 0; c0 < nq * kBlockChunks; c0 += 32) {
+            const int p = c0 + lane;
+            const bool f = p < nq * kBlockChunks && flag[p];
+            const unsigned b = __ballot_sync(0xffffffffu, f);
+            if (f) list[k + __popc(b & ((1u << lane) - 1))] = (int16_t)p;
+            k += __popc(b);
+        }
+        const int up = (k + kStageChunks - 1) / kStageChunks * kStageChunks;   // at most nq * 8
+        if (lane < up - k) list[k + lane] = -1;
+        if (lane == 0) {
+            kept = k;
+            padded = up;
+            count[R] = up | (fold || c == 0.0 ? 0 : kUnfolded);
         }
     }
-    expH[R * 64 + r] = m;
-    for (int q = b0; q < b1; q++) exps[(int64_t)q * 64 + r] = m;
+    __syncthreads();
+    const int64_t base = (int64_t)qb * kBlockChunks;
+    if (threadIdx.x < 64) expH[R * 64 + r] = efm;
+    for (int p = threadIdx.x >> 6; p < padded; p += 4) {
+        const int l = p < kept ? list[p] : 0, blk = l / kBlockChunks, k0 = (l % kBlockChunks) * kChunk;
+        double x[kChunk];
+        const double* src = val + (int64_t)(qb + blk) * 4096 + r * 64 + k0;
+#pragma unroll
+        for (int k = 0; k < kChunk; k++) x[k] = p < kept ? src[k] : 0.0;
+        long long F[kChunk];
+#pragma unroll
+        for (int k = 0; k < kChunk; k++) {
+            F[k] = fixed_point(x[k], efm);
+            if (fold && p < kept && blk == qd && k0 + k == r) F[k] = fixed_point(sd, efm) + fixed_point(err, efm);
+        }
+        uint4 dg[kSlices];
+        digits8(F, dg);
+        uint4* dst = reinterpret_cast<uint4*>(H) + (base + p) * (kSlices * 64) + r;
+#pragma unroll
+        for (int t = 0; t < kSlices; t++) dst[t * 64] = dg[t];
+        if (r == 0) {
+            const int C = p < kept ? bcol[qb + blk] : 0;
+            const bool in = C >= 0 && C < (int64_t)gridDim.x;
+            bad_ptr |= !in;
+            chunk[base + p] = p < kept && in ? C * kBlockChunks + l % kBlockChunks : 0;   // always a valid chunk
+        }
+    }
     if (bad) raise_status(status, DEV_NONFINITE);
+    if (bad_ptr) raise_status(status, DEV_PATTERN);
 }
 
 }  // namespace
@@ -971,21 +1458,16 @@ size_t ozaki_bsr_bytes(int64_t nbr, int64_t nblocks, int64_t n) {
     return ar.s.used;
 }
 
-int ozaki_bsr_prepare(const BsrDev& h, int64_t n, void* ws, size_t ws_bytes, unsigned* status, cudaStream_t s) {
+int ozaki_bsr_prepare(const BsrDev& h, int64_t n, double c, void* ws, size_t ws_bytes, unsigned* status, cudaStream_t s) {
     if (h.bdim != 64 || h.nbr <= 0) return CHFSI_ERR_UNSUPPORTED;
     if (ws_bytes < ozaki_bsr_bytes(h.nbr, h.nblocks, n)) return CHFSI_ERR_NOMEM;
     Arena ar(ws, ws_bytes);
     OzBsr b;
     oz_bsr_layout(ar, h.nbr, h.nblocks, n, &b);
-    if (b.H.plane_rows() * kSlices > INT32_MAX || b.Y.plane_rows() * kSlices > INT32_MAX) return CHFSI_ERR_UNSUPPORTED;
-    const double* val = static_cast<const double*>(h.val);
-    CHFSI_CUDA_TRY(cudaMemsetAsync(b.H.exps, 0, sizeof(int) * (size_t)b.H.plane_rows(), s));
-    bsr_row_exponents_kernel<<<(unsigned)h.nbr, 64, 0, s>>>(val, h.brow_ptr, h.nblocks, b.expH, b.H.exps, status);
-    CHFSI_LAUNCH_CHECK();
-    dim3 grid((unsigned)(b.H.K_pad / 32), (unsigned)std::min<int64_t>(b.H.rows_pad / 32, 65535), 1);
-    oz_slice_kernel<false><<<grid, dim3(32, 8), 0, s>>>(val, 64, h.nblocks * 64, 64, 64, 0, b.H.exps, b.H.rows_pad,
-                                                       b.H.K_pad, (size_t)b.H.plane_rows() * b.H.K_pad, kSlices,
-                                                       b.H.slices);
+    if (std::max<int64_t>(h.nblocks, 2) * 64 * kSlices > INT32_MAX || b.Y.padded_rows() * kSlices > INT32_MAX)
+        return CHFSI_ERR_UNSUPPORTED;
+    oz_bsr_prepare_kernel<<<(unsigned)h.nbr, 256, 0, s>>>(static_cast<const double*>(h.val), h.brow_ptr, h.bcol,
+                                                          h.nblocks, c, b.expH, b.chunk, b.count, b.H, status);
     CHFSI_LAUNCH_CHECK();
     return CHFSI_OK;
 }
@@ -1002,27 +1484,19 @@ int ozaki_bsr_step(const BsrDev& h, int64_t n, const double* Yc, int64_t ldc, co
     const int64_t N = h.nbr * 64;
     int rc;
     if ((rc = oz_prepare(Yc, ldc, true, b.Y, N, 0, status, s, slices))) return rc;
-    CUtensorMap tmA, tmB;
-    if ((rc = make_map_bf16(&tmA, b.Y.slices, b.Y.K_pad, kSlices * b.Y.plane_rows(), kKB, kTileM,
-                            kTmaSwizzle)))
-        return rc;
-    if ((rc = make_map_bf16(&tmB, b.H.slices, b.H.K_pad, kSlices * b.H.plane_rows(), kKB, kTileN,
-                            kTmaSwizzle)))
-        return rc;
     OzArgs g{};
+    g.A = b.Y.slices;
+    g.B = b.H;
+    g.chunksA = b.Y.chunks;
     g.M = n;
     g.Nc = N;
     g.ldc = ldo;
     g.C = Yo;
     g.nbatch = 1;
     g.m_batch = n;
-    g.a_batch_rows = b.Y.rows_pad;
     g.tilesM = (int)((n + kTileM - 1) / kTileM);
     g.tilesN = (int)h.nbr;
     g.expA = b.Y.exps;
-    g.expB = b.H.exps;
-    g.rowsA_pad = b.Y.plane_rows();
-    g.rowsB_pad = b.H.plane_rows();
     g.kb_total = kMaxItemKB;
     g.kb_split = kMaxItemKB;
     g.splits = 1;
@@ -1032,7 +1506,8 @@ int ozaki_bsr_step(const BsrDev& h, int64_t n, const double* Yc, int64_t ldc, co
     g.bsr = 1;
     g.slices = slices;
     g.brow_ptr = h.brow_ptr;
-    g.bcol = h.bcol;
+    g.hchunk = b.chunk;
+    g.hcount = b.count;
     g.nbr = h.nbr;
     g.nblocks = h.nblocks;
     g.expH = b.expH;
@@ -1043,7 +1518,7 @@ int ozaki_bsr_step(const BsrDev& h, int64_t n, const double* Yc, int64_t ldc, co
     g.alpha = alpha;
     g.cshift = c;
     g.beta = beta;
-    return launch_oz(tmA, tmB, g, g.pairs, s);
+    return launch_oz(g, CUtensorMap{}, g.pairs, s);
 }
 
 size_t ozaki_workspace_bytes(bool tn_form, int64_t M, int64_t Nc, int64_t K, bool same) {
@@ -1116,7 +1591,7 @@ int ozaki_blockdiag_apply(const double* Y, int64_t ldy, int64_t N, int B, int64_
     OzPlan p;
     p.A = bd.D;
     p.A.nbatch = bd.Y.nbatch;
-    p.A.rows_pad = B;      // rows per batch in the stacked D operand
+    p.A.tiles = B / kTileM;      // row tiles per batch in the stacked D operand
     p.B = bd.Y;
     return oz_run(p, false, T, ldt, N, n, false, false, status, s, bd.Y.nbatch, B);
 }
