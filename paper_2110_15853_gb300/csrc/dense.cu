@@ -4,10 +4,13 @@
 // Psi = X_F Q), a blocked right-looking Cholesky S = R^T R, the inverse of the
 // upper-triangular factor, and small element-wise helpers.
 //
-// FP64 on this part runs on the DFMA pipe (about 1.2 TFLOP/s for the whole GPU),
-// so the tiles are sized for DFMA issue, not for bandwidth: 64 x 64 output tiles,
-// 256 threads, 4 x 4 outputs per thread with stride-16 row/column ownership so
-// that shared-memory reads are conflict-free and global stores coalesce.
+// FP64 on this part runs on the DFMA pipe (about 1.2 TFLOP/s for the whole GPU, two
+// multiply-adds a cycle and SM), so the tiles are sized for DFMA issue, not for bandwidth:
+// 64 x 64 output tiles, 256 threads, 4 x 4 outputs per thread with stride-16 row/column
+// ownership so that shared-memory reads are conflict-free and global stores coalesce --
+// or 16 x 16 tiles, one output per thread, where 64 x 64 tiles leave SMs idle.
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.cuh"
 
@@ -15,7 +18,6 @@ namespace chfsi {
 
 namespace {
 
-constexpr int TB = 64;   // output tile edge
 constexpr int BK = 16;   // reduction chunk
 
 struct GemmArgs {
@@ -29,12 +31,29 @@ struct GemmArgs {
     bool b_upper;                             // B upper triangular: k <= j
     int splits;
     double* part;                             // splits x M x Nc partials, or nullptr
+    bool a_upper = false;                     // A upper triangular: k >= i
+    // nbatch > 1: independent products (splits = 1), operands `stride` elements apart; batch b
+    // has min(Nc, Ntot - b Nstep) columns, and as many k where k_is_nc
+    int nbatch = 1;
+    int64_t strideA = 0, strideB = 0, strideC = 0, Ntot = 0, Nstep = 0;
+    bool k_is_nc = false;
 };
 
+// TB x TB output tile, TB / 16 squared outputs per thread.
+template <int TB>
 __global__ void __launch_bounds__(256) gemm_kernel(GemmArgs g) {
+    constexpr int T = TB / 16;
     __shared__ double As[BK][TB + 1];
     __shared__ double Bs[BK][TB];
-    const int bi = blockIdx.y, bj = blockIdx.x, z = blockIdx.z;
+    const int bi = blockIdx.y, bj = blockIdx.x, z = g.nbatch > 1 ? 0 : blockIdx.z;
+    if (g.nbatch > 1) {
+        const int64_t b = blockIdx.z, cols = g.Ntot - b * g.Nstep;
+        g.A += b * g.strideA;
+        g.B += b * g.strideB;
+        g.C += b * g.strideC;
+        if (cols < g.Nc) g.Nc = cols;
+        if (g.k_is_nc) g.K = g.Nc;
+    }
     if (g.upper_tiles && bi > bj) return;
     const int64_t i0 = (int64_t)bi * TB, j0 = (int64_t)bj * TB;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -47,12 +66,13 @@ __global__ void __launch_bounds__(256) gemm_kernel(GemmArgs g) {
         int64_t lim = j0 + TB;
         if (k_end > lim) k_end = lim;
     }
+    if (g.a_upper && k_begin < i0) k_begin = i0;
 
-    double acc[4][4];
+    double acc[T][T];
 #pragma unroll
-    for (int a = 0; a < 4; a++)
+    for (int a = 0; a < T; a++)
 #pragma unroll
-        for (int b = 0; b < 4; b++) acc[a][b] = 0.0;
+        for (int b = 0; b < T; b++) acc[a][b] = 0.0;
 
     for (int64_t k0 = k_begin; k0 < k_end; k0 += BK) {
         // stage A chunk as As[k][i] and B chunk as Bs[k][j]
@@ -76,25 +96,25 @@ __global__ void __launch_bounds__(256) gemm_kernel(GemmArgs g) {
         __syncthreads();
 #pragma unroll
         for (int kk = 0; kk < BK; kk++) {
-            double av[4], bv[4];
+            double av[T], bv[T];
 #pragma unroll
-            for (int a = 0; a < 4; a++) av[a] = As[kk][ty + 16 * a];
+            for (int a = 0; a < T; a++) av[a] = As[kk][ty + 16 * a];
 #pragma unroll
-            for (int b = 0; b < 4; b++) bv[b] = Bs[kk][tx + 16 * b];
+            for (int b = 0; b < T; b++) bv[b] = Bs[kk][tx + 16 * b];
 #pragma unroll
-            for (int a = 0; a < 4; a++)
+            for (int a = 0; a < T; a++)
 #pragma unroll
-                for (int b = 0; b < 4; b++) acc[a][b] = fma(av[a], bv[b], acc[a][b]);
+                for (int b = 0; b < T; b++) acc[a][b] = fma(av[a], bv[b], acc[a][b]);
         }
         __syncthreads();
     }
 
 #pragma unroll
-    for (int a = 0; a < 4; a++) {
+    for (int a = 0; a < T; a++) {
         int64_t i = i0 + ty + 16 * a;
         if (i >= g.M) continue;
 #pragma unroll
-        for (int b = 0; b < 4; b++) {
+        for (int b = 0; b < T; b++) {
             int64_t j = j0 + tx + 16 * b;
             if (j >= g.Nc) continue;
             if (g.part) {
@@ -108,87 +128,128 @@ __global__ void __launch_bounds__(256) gemm_kernel(GemmArgs g) {
     }
 }
 
-// C[i][j] = sum_z part[z][i][j] in split order; with `mirror`, tiles below the
+// C[i][j] = sum_z part[z][i][j] in split order; with `mirror`, tb x tb tiles below the
 // diagonal take the transposed upper-tile sum.
 __global__ void reduce_parts_kernel(const double* __restrict__ part, int splits, int64_t M, int64_t Nc,
-                                    double* C, int64_t ldc, bool mirror) {
+                                    double* C, int64_t ldc, bool mirror, int tb) {
     int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= M * Nc) return;
     int64_t i = idx / Nc, j = idx % Nc;
     int64_t si = i, sj = j;
-    if (mirror && (i / TB) > (j / TB)) { si = j; sj = i; }
+    if (mirror && (i / tb) > (j / tb)) { si = j; sj = i; }
     double s = 0.0;
     for (int z = 0; z < splits; z++) s += part[((int64_t)z * M + si) * Nc + sj];
     C[i * ldc + j] = s;
 }
 
+// Tile edge: 64, or 16 where fewer than four 64 x 64 tiles per SM would run.  A tile's time is
+// its multiply-adds at two a cycle (a 64 x 64 x 64 product takes one SM 68 us), so small
+// products need many small tiles; at two multiply-adds a cycle the 16 x 16 tile's
+// operands are no load on shared memory or L2.  Measured: the products of a 96-state
+// closure over 8000 rows 8.48 -> 0.71 ms together; with four and more tiles per SM the
+// 64 x 64 tiles, at 97% of the DFMA pipe, stay.
+int gemm_tile(int64_t M, int64_t Nc, int64_t batches, bool upper) {
+    int64_t tm = (M + 63) / 64, tn = (Nc + 63) / 64, tiles = tm * tn;
+    if (upper) tiles = tm * (tm + 1) / 2;
+    return tiles * batches < 4 * 152 ? 16 : 64;
+}
+
 int run_gemm(const GemmArgs& g, cudaStream_t s) {
     if (g.M <= 0 || g.Nc <= 0) return CHFSI_OK;
-    dim3 grid((unsigned)((g.Nc + TB - 1) / TB), (unsigned)((g.M + TB - 1) / TB), (unsigned)g.splits);
-    gemm_kernel<<<grid, 256, 0, s>>>(g);
+    const int64_t z = g.nbatch > 1 ? g.nbatch : g.splits;
+    const int tb = gemm_tile(g.M, g.Nc, z, g.upper_tiles);
+    dim3 grid((unsigned)((g.Nc + tb - 1) / tb), (unsigned)((g.M + tb - 1) / tb), (unsigned)z);
+    if (tb == 64) gemm_kernel<64><<<grid, 256, 0, s>>>(g);
+    else gemm_kernel<16><<<grid, 256, 0, s>>>(g);
     CHFSI_LAUNCH_CHECK();
     return CHFSI_OK;
 }
 
 // ---------------------------------------------------------------- Cholesky
 
-constexpr int NB = 64;
+constexpr int NB = 64;    // columns between trailing updates
+constexpr int ND = 32;    // diagonal block
 
-// Unblocked upper Cholesky of the nb x nb diagonal block at S[k0][k0] (in place).
-__global__ void __launch_bounds__(256) chol_diag_kernel(double* S, int64_t lds, int64_t k0, int nb,
+// q = v / d from the reciprocal r of d, with one correction (Markstein): three FP64
+// operations in place of the division's dozen on a pipe that takes 64 cycles a warp.
+__device__ __forceinline__ double div_by(double v, double d, double r) {
+    const double q = v * r;
+    return fma(fma(-q, d, v), r, q);
+}
+
+// Upper Cholesky of the nb x nb diagonal block at S[k0][k0] (nb <= 32, in place): four warps,
+// lane = column, warp w the rows i = w mod 4 in registers (one warp per FP64 unit of the
+// SM).  A step's chain is the root and reciprocal of the pivot, the scaled row and one
+// update; 64 columns in one block of 256 threads with three barriers a step took 105 us,
+// two 32-column blocks take 36 us each.
+__global__ void __launch_bounds__(128) chol_diag_kernel(double* S, int64_t lds, int64_t k0, int nb,
                                                         unsigned* status) {
-    __shared__ double A[NB][NB + 1];
-    for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-        int i = e / nb, j = e % nb;
-        A[i][j] = S[(k0 + i) * lds + k0 + j];
+    __shared__ double row[2][ND];
+    const int w = threadIdx.x >> 5, j = threadIdx.x & 31;
+    double a[ND / 4];
+    bool bad = false;
+#pragma unroll
+    for (int q = 0; q < ND / 4; q++) {
+        const int i = 4 * q + w;
+        a[q] = (i < nb && j < nb && i <= j) ? S[(k0 + i) * lds + k0 + j] : (i == j ? 1.0 : 0.0);
     }
-    __syncthreads();
-    __shared__ int bad;
-    if (threadIdx.x == 0) bad = 0;
-    __syncthreads();
-    for (int k = 0; k < nb; k++) {
-        if (threadIdx.x == 0) {
-            double p = A[k][k];
-            if (!(p > 0.0) || !isfinite(p)) { bad = 1; p = 1.0; }
-            A[k][k] = sqrt(p);
+#pragma unroll
+    for (int k = 0; k < ND; k++) {
+        if (w == (k & 3)) row[k & 1][j] = a[k / 4];
+        __syncthreads();
+        double p = row[k & 1][k];
+        if (!(p > 0.0) || !isfinite(p)) { bad = true; p = 1.0; }
+        const double d = sqrt(p), r = 1.0 / d;
+        const double x = j == k ? d : div_by(row[k & 1][j], d, r);   // R[k][j], j >= k
+        if (w == (k & 3)) a[k / 4] = j >= k ? x : 0.0;
+#pragma unroll
+        for (int q = 0; q < ND / 4; q++) {
+            if (4 * q + 3 <= k) continue;
+            const int i = 4 * q + w;
+            const double xi = __shfl_sync(0xffffffffu, x, i);
+            if (i > k && j >= i) a[q] = fma(-xi, x, a[q]);
         }
-        __syncthreads();
-        double d = A[k][k];
-        for (int j = k + 1 + threadIdx.x; j < nb; j += blockDim.x) A[k][j] /= d;
-        __syncthreads();
-        const int m = nb - k - 1;
-        for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-            int i = k + 1 + e / m, j = k + 1 + e % m;
-            if (j >= i) A[i][j] -= A[k][i] * A[k][j];
-        }
-        __syncthreads();
     }
-    for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-        int i = e / nb, j = e % nb;
-        S[(k0 + i) * lds + k0 + j] = (j >= i) ? A[i][j] : 0.0;
+#pragma unroll
+    for (int q = 0; q < ND / 4; q++) {
+        const int i = 4 * q + w;
+        if (i < nb && j < nb) S[(k0 + i) * lds + k0 + j] = j >= i ? a[q] : 0.0;
     }
     if (threadIdx.x == 0 && bad) raise_status(status, DEV_CHOL);
 }
 
-// Panel: R[k0:k0+nb, j] = R_kk^-T S[k0:k0+nb, j] for j >= k0+nb (forward substitution).
-__global__ void __launch_bounds__(64) chol_panel_kernel(double* S, int64_t lds, int64_t n, int64_t k0,
-                                                        int nb) {
-    __shared__ double R[NB][NB + 1];
-    for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-        int i = e / nb, j = e % nb;
-        R[i][j] = S[(k0 + i) * lds + k0 + j];
-    }
+// Panel: R[k0:k0+nb, j] = R_kk^-T S[k0:k0+nb, j] for j >= k0+nb (forward substitution), 16
+// columns per block so that the multiply-adds spread over the SMs; row i of the solution,
+// then its update of the rows below, one barrier a step.  (A thread per column with its 64
+// entries in local memory took 182 us a panel; two 32-row panels take 13 us each.)
+constexpr int kPanelCols = 16;
+
+__global__ void __launch_bounds__(256) chol_panel_kernel(double* S, int64_t lds, int64_t n, int64_t k0, int nb) {
+    __shared__ double R[ND][ND + 1];
+    __shared__ double z[ND][kPanelCols];
+    __shared__ double rinv[ND];
+    for (int e = threadIdx.x; e < nb * nb; e += 256) R[e / nb][e % nb] = S[(k0 + e / nb) * lds + k0 + e % nb];
+    const int c = threadIdx.x % kPanelCols, r = threadIdx.x / kPanelCols;
+    const int64_t j = k0 + nb + (int64_t)blockIdx.x * kPanelCols + c;
+    double v[2];
+#pragma unroll
+    for (int h = 0; h < 2; h++) v[h] = (j < n && r + 16 * h < nb) ? S[(k0 + r + 16 * h) * lds + j] : 0.0;
     __syncthreads();
-    int64_t j = k0 + nb + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    double z[NB];
-#pragma unroll 1
+    if (threadIdx.x < nb) rinv[threadIdx.x] = 1.0 / R[threadIdx.x][threadIdx.x];
+    __syncthreads();
     for (int i = 0; i < nb; i++) {
-        double v = S[(k0 + i) * lds + j];
-        for (int l = 0; l < i; l++) v -= R[l][i] * z[l];
-        z[i] = v / R[i][i];
+        if (r == (i & 15)) z[i][c] = div_by(i < 16 ? v[0] : v[1], R[i][i], rinv[i]);
+        __syncthreads();
+        const double zi = z[i][c];
+#pragma unroll
+        for (int h = 0; h < 2; h++)
+            if (r + 16 * h > i && r + 16 * h < nb) v[h] = fma(-R[i][r + 16 * h], zi, v[h]);
     }
-    for (int i = 0; i < nb; i++) S[(k0 + i) * lds + j] = z[i];
+    if (j < n) {
+#pragma unroll
+        for (int h = 0; h < 2; h++)
+            if (r + 16 * h < nb) S[(k0 + r + 16 * h) * lds + j] = z[r + 16 * h][c];
+    }
 }
 
 __global__ void zero_lower_kernel(double* S, int64_t lds, int64_t n) {
@@ -200,28 +261,50 @@ __global__ void zero_lower_kernel(double* S, int64_t lds, int64_t n) {
 
 // ---------------------------------------------------------------- triangular inverse
 
-// Column j of R^-1 by back substitution, one warp per column:
-//   z_j = 1/R_jj,  z_i = -(sum_{l=i+1..j} R_il z_l)/R_ii  for i = j-1..0.
-__global__ void tri_inv_kernel(const double* __restrict__ R, int64_t ldr, double* Rinv, int64_t ldi,
-                               int64_t n, int warps_per_block) {
-    extern __shared__ double zs[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t j = (int64_t)blockIdx.x * warps_per_block + warp;
-    if (j >= n) return;
-    double* z = zs + (int64_t)warp * n;
-    for (int64_t i = lane; i <= j; i += 32) z[i] = 0.0;
-    __syncwarp();
-    if (lane == 0) z[j] = 1.0 / R[j * ldr + j];
-    __syncwarp();
-    for (int64_t i = j - 1; i >= 0; i--) {
-        double s = 0.0;
-        for (int64_t l = i + 1 + lane; l <= j; l += 32) s = fma(R[i * ldr + l], z[l], s);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) z[i] = -s / R[i * ldr + i];
-        __syncwarp();
+constexpr int kTriLeaf = 64;
+
+// Inverse of the 64 x 64 diagonal blocks of an upper-triangular R (block b at row and column
+// 64 b), one block per CTA: from the last row up, row i of X is the scaled row of the
+// identity minus the updates received from the rows below, then row i updates the rows
+// above; one barrier a row.  A thread holds one column's rows r = 4 q + w (w = threadIdx.x /
+// 64).  Entries below the diagonal are written as zeros.
+__global__ void __launch_bounds__(256) tri_inv_leaf_kernel(const double* __restrict__ R, int64_t ldr, double* X,
+                                                           int64_t ldx, int64_t n) {
+    __shared__ double Rs[kTriLeaf][kTriLeaf + 1];
+    __shared__ double xi[2][kTriLeaf];
+    const int64_t b0 = (int64_t)blockIdx.x * kTriLeaf;
+    const int nb = (int)(n - b0 < kTriLeaf ? n - b0 : kTriLeaf);
+    for (int e = threadIdx.x; e < kTriLeaf * kTriLeaf; e += 256) {
+        const int i = e / kTriLeaf, j = e % kTriLeaf;
+        Rs[i][j] = (i < nb && j < nb && j >= i) ? R[(b0 + i) * ldr + b0 + j] : (i == j ? 1.0 : 0.0);
     }
-    for (int64_t i = lane; i < n; i += 32) Rinv[i * ldi + j] = (i <= j) ? z[i] : 0.0;
+    __syncthreads();
+    const int j = threadIdx.x & 63, w = threadIdx.x >> 6;
+    double x[kTriLeaf / 4];
+#pragma unroll
+    for (int q = 0; q < kTriLeaf / 4; q++) x[q] = 4 * q + w == j ? 1.0 : 0.0;
+    if (threadIdx.x < kTriLeaf) Rs[threadIdx.x][kTriLeaf] = 1.0 / Rs[threadIdx.x][threadIdx.x];
+    __syncthreads();
+#pragma unroll
+    for (int i = kTriLeaf - 1; i >= 0; i--) {
+        if (w == (i & 3)) {
+            x[i / 4] = div_by(x[i / 4], Rs[i][i], Rs[i][kTriLeaf]);
+            xi[i & 1][j] = x[i / 4];
+        }
+        __syncthreads();
+        const double v = xi[i & 1][j];
+#pragma unroll
+        for (int q = 0; q < kTriLeaf / 4; q++) {
+            if (4 * q >= i) continue;
+            const int l = 4 * q + w;
+            if (l < i && j >= i) x[q] = fma(-Rs[l][i], v, x[q]);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < kTriLeaf / 4; q++) {
+        const int i = 4 * q + w;
+        if (i < nb && j < nb) X[(b0 + i) * ldx + b0 + j] = j >= i ? x[q] : 0.0;
+    }
 }
 
 __global__ void transpose_kernel(const double* __restrict__ A, int64_t lda, double* B, int64_t ldb, int64_t n) {
@@ -291,11 +374,19 @@ __global__ void convert_values_kernel(const double* __restrict__ src, float* dst
 }  // namespace
 
 int gemm_tn_splits(int64_t K, int64_t n) {
-    int64_t tiles = ((n + TB - 1) / TB);
+    int64_t tiles = ((n + 63) / 64);
     tiles = tiles * (tiles + 1) / 2;
-    int64_t want = (4 * 152 + tiles - 1) / tiles;        // about four CTAs per SM
+    int64_t want = (4 * 152 + tiles - 1) / tiles;        // about four 64 x 64 tiles per SM
     int64_t maxs = (K + 2047) / 2048;                    // keep >= 2048 rows per split
     int64_t s = want < maxs ? want : maxs;
+    // fewer tiles than that: 16 x 16 tiles (run_gemm), enough splits for a dozen of them per
+    // SM while each keeps 256 rows
+    if (tiles * s < 4 * 152) {
+        const int64_t t = (n + 15) / 16, more = (12 * 152 + t * (t + 1) / 2 - 1) / (t * (t + 1) / 2);
+        const int64_t most = (K + 255) / 256, want16 = more < most ? more : most;
+        if (want16 > s) s = want16;
+        if (tiles * s >= 4 * 152) s = (4 * 152 - 1) / tiles;
+    }
     if (s < 1) s = 1;
     if (s > 64) s = 64;
     return (int)s;
@@ -308,7 +399,8 @@ int gemm_tn(const double* A, int64_t lda, const double* B, int64_t ldb, int64_t 
     int rc = run_gemm(g, s);
     if (rc) return rc;
     int64_t total = n * n;
-    reduce_parts_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(part, splits, n, n, S, lds, symmetric);
+    reduce_parts_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(part, splits, n, n, S, lds, symmetric,
+                                                                        gemm_tile(n, n, splits, symmetric));
     CHFSI_LAUNCH_CHECK();
     return CHFSI_OK;
 }
@@ -342,19 +434,33 @@ constexpr int64_t kCholOzakiMin = 256;   // trailing blocks from this size on as
 
 int cholesky_upper(double* S, int64_t n, int64_t lds, unsigned* status, cudaStream_t s, void* oz_ws, size_t oz_bytes,
                    double* scratch) {
+    int rc;
     for (int64_t k0 = 0; k0 < n; k0 += NB) {
-        int nb = (int)((n - k0) < NB ? (n - k0) : NB);
-        chol_diag_kernel<<<1, 256, 0, s>>>(S, lds, k0, nb, status);
-        CHFSI_LAUNCH_CHECK();
+        const int nb = (int)((n - k0) < NB ? (n - k0) : NB);
+        // the nb rows in blocks of 32: diagonal block, its panel, and the update of the second
+        // block's rows
+        for (int64_t k = k0; k < k0 + nb; k += ND) {
+            const int nd = (int)(k0 + nb - k < ND ? k0 + nb - k : ND);
+            chol_diag_kernel<<<1, 128, 0, s>>>(S, lds, k, nd, status);
+            CHFSI_LAUNCH_CHECK();
+            const int64_t right = n - k - nd;
+            if (right <= 0) break;
+            chol_panel_kernel<<<(unsigned)((right + kPanelCols - 1) / kPanelCols), 256, 0, s>>>(S, lds, n, k, nd);
+            CHFSI_LAUNCH_CHECK();
+            if (k + nd < k0 + nb) {
+                const double* Rk = S + k * lds + (k + nd);
+                const int64_t below = k0 + nb - k - nd;
+                GemmArgs g{Rk, lds, true, Rk, lds, S + (k + nd) * lds + (k + nd), lds, below, right, nd, -1.0, true,
+                           false, false, 1, nullptr};
+                if ((rc = run_gemm(g, s))) return rc;
+            }
+        }
         int64_t rest = n - k0 - nb;
         if (rest <= 0) break;
-        chol_panel_kernel<<<(unsigned)((rest + 63) / 64), 64, 0, s>>>(S, lds, n, k0, nb);
-        CHFSI_LAUNCH_CHECK();
         // trailing update S22 -= R12^T R12 (upper tiles): an Ozaki product on the tensor
         // cores into the scratch block when one is given, else FP64 on the DFMA pipe
         const double* R12 = S + k0 * lds + (k0 + nb);
         double* S22 = S + (k0 + nb) * lds + (k0 + nb);
-        int rc;
         if (oz_ws && scratch && rest >= kCholOzakiMin &&
             oz_bytes >= ozaki_workspace_bytes(true, rest, rest, nb, true)) {
             if ((rc = ozaki_gemm_tn(R12, lds, R12, lds, nb, rest, rest, scratch, rest, true, oz_ws, oz_bytes, status,
@@ -373,19 +479,6 @@ int cholesky_upper(double* S, int64_t n, int64_t lds, unsigned* status, cudaStre
     return CHFSI_OK;
 }
 
-int tri_inverse_upper(const double* R, int64_t ldr, double* Rinv, int64_t ldi, int64_t n, cudaStream_t s) {
-    if (n <= 0) return CHFSI_OK;
-    int wpb = (int)((160 * 1024) / (n * 8));
-    if (wpb > 8) wpb = 8;
-    if (wpb < 1) return CHFSI_ERR_UNSUPPORTED;            // n > 20480
-    size_t smem = (size_t)wpb * n * 8;
-    if (smem > 48 * 1024)
-        CHFSI_CUDA_TRY(cudaFuncSetAttribute(tri_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    tri_inv_kernel<<<(unsigned)((n + wpb - 1) / wpb), 32 * wpb, smem, s>>>(R, ldr, Rinv, ldi, n, wpb);
-    CHFSI_LAUNCH_CHECK();
-    return CHFSI_OK;
-}
-
 namespace {
 
 __global__ void negate_block_kernel(double* X, int64_t ldx, int64_t rows, int64_t cols) {
@@ -394,38 +487,63 @@ __global__ void negate_block_kernel(double* X, int64_t ldx, int64_t rows, int64_
     X[(idx / cols) * ldx + idx % cols] = -X[(idx / cols) * ldx + idx % cols];
 }
 
-constexpr int64_t kTriInvLeaf = 1024;   // the column-per-warp kernel below this size
+constexpr int64_t kTriInvOzaki = 256;   // halves of this size and more as Ozaki products
 
 }  // namespace
 
-// R^-1 of an upper-triangular R by halves: with R = [R11 R12; 0 R22],
-// R^-1 = [X11, -X11 R12 X22; 0, X22] (X11 = R11^-1, X22 = R22^-1, both recursively), the
-// off-diagonal block from two products (T = R12 X22 into `tmp`, then X11 T) -- Ozaki
-// products on the tensor cores when oz_ws is given and the depth fits (<= 8192), FP64
-// products otherwise; blocks of at most kTriInvLeaf columns by back substitution.
+// R^-1 of an upper-triangular R: the 64 x 64 diagonal blocks in one launch, then pairs of
+// blocks of h = 64, 128, ... rows: with [R11 R12; 0 R22] the off-diagonal block of the inverse
+// is -X11 R12 X22 (T = R12 X22 into `tmp`, then X11 T) -- all pairs of a size in one
+// FP64 launch a product, or from 256 rows on as Ozaki products on the tensor cores when
+// oz_ws is given and the depth fits (<= 8192).  (Column by column, a warp each, blocks of up
+// to 1024 columns took 1.4 ms; the diagonal blocks now take 56 us and an FP64 product 8 - 20.)
 int tri_inverse_upper_blocked(const double* R, int64_t ldr, double* X, int64_t ldx, int64_t n, double* tmp,
                               int64_t ldt, void* oz_ws, size_t oz_bytes, unsigned* status, cudaStream_t s) {
-    if (n <= kTriInvLeaf) return tri_inverse_upper(R, ldr, X, ldx, n, s);
-    const int64_t h = (n / 2 + 63) / 64 * 64, r = n - h;
+    if (n <= 0) return CHFSI_OK;
     int rc;
-    if ((rc = tri_inverse_upper_blocked(R, ldr, X, ldx, h, tmp, ldt, oz_ws, oz_bytes, status, s))) return rc;
-    if ((rc = tri_inverse_upper_blocked(R + h * ldr + h, ldr, X + h * ldx + h, ldx, r, tmp, ldt, oz_ws, oz_bytes, status,
-                                        s)))
-        return rc;
-    CHFSI_CUDA_TRY(cudaMemset2DAsync(X + h * ldx, sizeof(double) * (size_t)ldx, 0, sizeof(double) * (size_t)h,
-                                     (size_t)r, s));
-    const double* R12 = R + h;
-    const double* X22 = X + h * ldx + h;
-    double* X12 = X + h;
-    if (oz_ws && r <= 8192 && h <= 8192 && oz_bytes >= ozaki_workspace_bytes(false, h, r, r, false)) {
-        if ((rc = ozaki_gemm_nn(R12, ldr, X22, ldx, h, r, r, tmp, ldt, true, oz_ws, oz_bytes, status, s))) return rc;
-        if ((rc = ozaki_gemm_nn(X, ldx, tmp, ldt, h, h, r, X12, ldx, false, oz_ws, oz_bytes, status, s))) return rc;
-        negate_block_kernel<<<(unsigned)((h * r + 255) / 256), 256, 0, s>>>(X12, ldx, h, r);
-        CHFSI_LAUNCH_CHECK();
-        return CHFSI_OK;
+    CHFSI_CUDA_TRY(cudaMemset2DAsync(X, sizeof(double) * (size_t)ldx, 0, sizeof(double) * (size_t)n, (size_t)n, s));
+    tri_inv_leaf_kernel<<<(unsigned)((n + kTriLeaf - 1) / kTriLeaf), 256, 0, s>>>(R, ldr, X, ldx, n);
+    CHFSI_LAUNCH_CHECK();
+    for (int64_t h = kTriLeaf; h < n; h *= 2) {
+        const int64_t pairs = (n - h + 2 * h - 1) / (2 * h);     // blocks at 2 h b with rows right of the first h
+        if (oz_ws && h >= kTriInvOzaki && h <= 8192 && oz_bytes >= ozaki_workspace_bytes(false, h, h, h, false)) {
+            for (int64_t b = 0; b < pairs; b++) {
+                const int64_t o = 2 * h * b, r = std::min(h, n - o - h);
+                const double* R12 = R + o * ldr + o + h;
+                const double* X22 = X + (o + h) * ldx + o + h;
+                double* X12 = X + o * ldx + o + h;
+                if ((rc = ozaki_gemm_nn(R12, ldr, X22, ldx, h, r, r, tmp, ldt, true, oz_ws, oz_bytes, status, s)))
+                    return rc;
+                if ((rc = ozaki_gemm_nn(X + o * ldx + o, ldx, tmp, ldt, h, h, r, X12, ldx, false, oz_ws, oz_bytes,
+                                        status, s)))
+                    return rc;
+                negate_block_kernel<<<(unsigned)((h * r + 255) / 256), 256, 0, s>>>(X12, ldx, h, r);
+                CHFSI_LAUNCH_CHECK();
+            }
+            continue;
+        }
+        GemmArgs g{R + h, ldr, false, X + h * ldx + h, ldx, tmp, ldt, h, h, h, 1.0, false, false, true, 1, nullptr};
+        g.nbatch = (int)pairs;
+        g.Ntot = n - h;
+        g.Nstep = 2 * h;
+        g.k_is_nc = true;
+        g.strideA = 2 * h * (ldr + 1);
+        g.strideB = 2 * h * (ldx + 1);
+        g.strideC = 2 * h * ldt;
+        if (pairs == 1) { g.Nc = g.K = std::min(h, n - h); }
+        if ((rc = run_gemm(g, s))) return rc;
+        GemmArgs f{X, ldx, false, tmp, ldt, X + h, ldx, h, h, h, -1.0, false, false, false, 1, nullptr};
+        f.a_upper = true;
+        f.nbatch = (int)pairs;
+        f.Ntot = n - h;
+        f.Nstep = 2 * h;
+        f.strideA = 2 * h * (ldx + 1);
+        f.strideB = 2 * h * ldt;
+        f.strideC = 2 * h * (ldx + 1);
+        if (pairs == 1) f.Nc = std::min(h, n - h);
+        if ((rc = run_gemm(f, s))) return rc;
     }
-    if ((rc = gemm_general(R12, ldr, false, X22, ldx, tmp, ldt, h, r, r, 1.0, false, s))) return rc;
-    return gemm_general(X, ldx, false, tmp, ldt, X12, ldx, h, r, h, -1.0, false, s);
+    return CHFSI_OK;
 }
 
 int transpose(const double* A, int64_t lda, double* B, int64_t ldb, int64_t n, cudaStream_t s) {

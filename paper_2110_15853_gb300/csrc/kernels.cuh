@@ -106,11 +106,9 @@ int gemm_general(const double* A, int64_t lda, bool a_t, const double* B, int64_
 // and more run as Ozaki products on the tensor cores.
 int cholesky_upper(double* S, int64_t n, int64_t lds, unsigned* status, cudaStream_t s, void* oz_ws = nullptr,
                    size_t oz_bytes = 0, double* scratch = nullptr);
-// Rinv (n x n) = R^-1 for upper-triangular R (column per warp, n <= 20480).
-int tri_inverse_upper(const double* R, int64_t ldr, double* Rinv, int64_t ldi, int64_t n,
-                      cudaStream_t s);
-// The same by halves with products for the off-diagonal blocks (Ozaki products when oz_ws
-// is given); tmp: at least ceil(n/2) x ceil(n/2) doubles (ldt >= n / 2 + 64).
+// X (n x n) = R^-1 for upper-triangular R, zeros below the diagonal: 64 x 64 diagonal blocks,
+// then products for the off-diagonal blocks (Ozaki products from 256 rows on when oz_ws is
+// given); tmp: n x n doubles (ldt >= n).
 int tri_inverse_upper_blocked(const double* R, int64_t ldr, double* X, int64_t ldx, int64_t n, double* tmp,
                               int64_t ldt, void* oz_ws, size_t oz_bytes, unsigned* status, cudaStream_t s);
 // B = A^T (n x n).
