@@ -968,31 +968,62 @@ __global__ void panel_v_kernel(const double* A, int64_t lda, int64_t n, int64_t 
     Vp[t * mr + i] = v;
 }
 
-// Gv[s][t] = Vp[s] . Vp[t] (s <= t), one block per pair.
-__global__ void panel_gram_kernel(const double* Vp, int64_t mr, int nb, double* Gv) {
+// Gv[p][s][t] = v_s . v_t (s <= t) for every panel p = blockIdx.z of kPanel reflectors, one
+// block per pair, straight from A's rows (v of reflector j: zeros, 1 at j + 1, A[j][j+2:]).
+__global__ void panel_gram_kernel(const double* __restrict__ A, int64_t lda, int64_t n, int64_t nref, double* Gv) {
     const int s = blockIdx.x, t = blockIdx.y;
-    if (s > t) return;
+    const int64_t j0 = (int64_t)blockIdx.z * kPanel;
+    const int nb = (int)(nref - j0 < kPanel ? nref - j0 : kPanel);
+    if (s > t || t >= nb) return;
+    const double* vs = A + (j0 + s) * lda;
+    const int64_t jt = j0 + t;
+    const double* vt = A + jt * lda;
     double acc = 0.0;
-    for (int64_t i = threadIdx.x; i < mr; i += blockDim.x) acc = fma(Vp[s * mr + i], Vp[t * mr + i], acc);
+    for (int64_t i = jt + 2 + threadIdx.x; i < n; i += blockDim.x) acc = fma(vs[i], vt[i], acc);
+    if (threadIdx.x == 0) acc += s == t ? 1.0 : vs[jt + 1];
     acc = block_sum(acc);
-    if (threadIdx.x == 0) Gv[s * nb + t] = acc;
+    if (threadIdx.x == 0) Gv[(int64_t)blockIdx.z * kPanel * kPanel + s * nb + t] = acc;
 }
 
 // T of H_j0 ... H_{j0+nb-1} = I - V T V^T (upper triangular, forward accumulation):
-// T[t][t] = tau_t, T[0:t, t] = -tau_t T[0:t, 0:t] Gv[0:t, t].  One block.
-__global__ void panel_t_kernel(const double* Gv, const double* tau, int64_t j0, int nb, double* T) {
-    for (int idx = threadIdx.x; idx < nb * nb; idx += blockDim.x) T[idx] = 0.0;
+// T[t][t] = tau_t, T[s][t] = -tau_t sum_{s <= u < t} T[s][u] Gv[u][t]; one block per panel.
+// The rows of T are independent: four lanes share a row, each keeps the sums of sixteen
+// columns in registers, and T[s][u], final at step u, goes round by shuffle, so there is no
+// barrier in the chain.  (One panel a launch, the sums over u in one thread from global
+// memory, took 145 us a panel; all panels together now take 50 us.)
+__global__ void __launch_bounds__(256) panel_t_kernel(const double* __restrict__ Gv, const double* __restrict__ tau,
+                                                      int64_t nref, double* T) {
+    __shared__ double G[kPanel][kPanel + 1];
+    __shared__ double ts[kPanel];
+    const int64_t j0 = (int64_t)blockIdx.x * kPanel;
+    const int nb = (int)(nref - j0 < kPanel ? nref - j0 : kPanel);
+    Gv += (int64_t)blockIdx.x * kPanel * kPanel;
+    T += (int64_t)blockIdx.x * kPanel * kPanel;
+    for (int e = threadIdx.x; e < kPanel * kPanel; e += 256) {
+        const int s = e / kPanel, t = e % kPanel;
+        G[s][t] = (s <= t && t < nb) ? Gv[s * nb + t] : 0.0;
+    }
+    if (threadIdx.x < kPanel) ts[threadIdx.x] = (int)threadIdx.x < nb ? tau[j0 + threadIdx.x] : 0.0;
     __syncthreads();
-    for (int t = 0; t < nb; t++) {
-        const double tt = tau[j0 + t];
-        if (threadIdx.x < t) {
-            const int s = threadIdx.x;
-            double acc = 0.0;
-            for (int u = s; u < t; u++) acc = fma(T[s * nb + u], Gv[u * nb + t], acc);
-            T[s * nb + t] = -tt * acc;
+    const int s = threadIdx.x >> 2, g = threadIdx.x & 3;
+    double w[kPanel / 4];
+#pragma unroll
+    for (int q = 0; q < kPanel / 4; q++) w[q] = 0.0;
+#pragma unroll
+    for (int u = 0; u < kPanel; u++) {
+        double v = s < u ? -ts[u] * w[u / 4] : (s == u ? ts[u] : 0.0);
+        v = __shfl_sync(0xffffffffu, v, u & 3, 4);
+        if (g == (u & 3)) w[u / 4] = v;              // T[s][u]
+#pragma unroll
+        for (int q = 0; q < kPanel / 4; q++) {
+            if (4 * q + 3 <= u) continue;
+            if (4 * q + g > u) w[q] = fma(v, G[u][4 * q + g], w[q]);
         }
-        if (threadIdx.x == 0) T[t * nb + t] = tt;
-        __syncthreads();
+    }
+#pragma unroll
+    for (int q = 0; q < kPanel / 4; q++) {
+        const int t = 4 * q + g;
+        if (s < nb && t < nb) T[s * nb + t] = w[q];
     }
 }
 
@@ -1061,8 +1092,9 @@ void eigh_layout(Ar& ar, int64_t n, EighBufs* out) {
     b.U = ar.template take<double>((size_t)n * n);
     b.Gn = ar.template take<double>((size_t)n * n);
     u.Vp = ar.template take<double>((size_t)kPanel * n);
-    u.Gv = ar.template take<double>((size_t)kPanel * kPanel);
-    u.T = ar.template take<double>((size_t)kPanel * kPanel);
+    const size_t panels = (size_t)((n + kPanel - 1) / kPanel);
+    u.Gv = ar.template take<double>(panels * kPanel * kPanel);
+    u.T = ar.template take<double>(panels * kPanel * kPanel);
     u.W1 = ar.template take<double>((size_t)kPanel * n);
     u.W2 = ar.template take<double>((size_t)kPanel * n);
     u.oz_bytes = eigh_ozaki_bytes(n);
@@ -1232,27 +1264,31 @@ int eigh(double* A, int64_t lda, int64_t n, double* w, double* Q, int64_t ldq, v
 
     // 3. back-transformation Q = H_0 H_1 ... H_{n-3} Q, panels from the last
     const int64_t nref = n - 2;   // reflectors j = 0 .. n - 3
+    if (nref > 0) {
+        const unsigned panels = (unsigned)((nref + kPanel - 1) / kPanel);
+        panel_gram_kernel<<<dim3(kPanel, kPanel, panels), 256, 0, s>>>(A, lda, n, nref, Gv);
+        CHFSI_LAUNCH_CHECK();
+        panel_t_kernel<<<panels, 256, 0, s>>>(Gv, tau, nref, T);
+        CHFSI_LAUNCH_CHECK();
+    }
     for (int64_t j0 = ((nref - 1) / kPanel) * kPanel; nref > 0 && j0 >= 0; j0 -= kPanel) {
         const int nb = (int)std::min<int64_t>(kPanel, nref - j0);
         const int64_t mr = n - j0 - 1;
         panel_v_kernel<<<dim3((unsigned)((mr + 255) / 256), (unsigned)nb), 256, 0, s>>>(A, lda, n, j0, nb, Vp);
         CHFSI_LAUNCH_CHECK();
-        panel_gram_kernel<<<dim3((unsigned)nb, (unsigned)nb), 256, 0, s>>>(Vp, mr, nb, Gv);
-        CHFSI_LAUNCH_CHECK();
-        panel_t_kernel<<<1, 128, 0, s>>>(Gv, tau, j0, nb, T);
-        CHFSI_LAUNCH_CHECK();
+        const double* Tp = T + (j0 / kPanel) * (kPanel * kPanel);
         double* ZR = Q + (j0 + 1) * ldq;
         int rc;
         if (oz) {
             // W1 = V^T Z, W2 = T W1 (small, DFMA), Z -= V W2 through a product block
             if ((rc = ozaki_gemm_nn(Vp, mr, ZR, ldq, nb, mr, n, W1, n, false, u.oz, u.oz_bytes, status, s))) return rc;
-            if ((rc = gemm_general(T, nb, false, W1, n, W2, n, nb, n, nb, 1.0, false, s))) return rc;
+            if ((rc = gemm_general(Tp, nb, false, W1, n, W2, n, nb, n, nb, 1.0, false, s))) return rc;
             if ((rc = ozaki_gemm_tn(Vp, mr, W2, n, nb, mr, n, mb.G, n, false, u.oz, u.oz_bytes, status, s))) return rc;
             sub_block_kernel<<<(unsigned)((mr * n + 255) / 256), 256, 0, s>>>(ZR, ldq, mb.G, mr, n);
             CHFSI_LAUNCH_CHECK();
         } else {
             if ((rc = gemm_general(Vp, mr, false, ZR, ldq, W1, n, nb, n, mr, 1.0, false, s))) return rc;
-            if ((rc = gemm_general(T, nb, false, W1, n, W2, n, nb, n, nb, 1.0, false, s))) return rc;
+            if ((rc = gemm_general(Tp, nb, false, W1, n, W2, n, nb, n, nb, 1.0, false, s))) return rc;
             if ((rc = gemm_general(Vp, mr, true, W2, n, ZR, ldq, mr, n, nb, -1.0, true, s))) return rc;
         }
     }
