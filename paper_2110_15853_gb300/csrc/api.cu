@@ -863,6 +863,7 @@ int rr_finish(const RRLayout& rl, unsigned* st, cudaStream_t s) {
     CHFSI_CUDA_TRY(cudaMemcpy(&word, st, sizeof(unsigned), cudaMemcpyDeviceToHost));
     if (word & DEV_PATTERN) return CHFSI_ERR_PATTERN;
     if (word & DEV_CHOL) return CHFSI_ERR_CHOL;
+    if (word & DEV_TIMEOUT) return CHFSI_ERR_TIMEOUT;
     if (word & DEV_NONFINITE) return CHFSI_ERR_NONFINITE;
     return CHFSI_OK;
 }

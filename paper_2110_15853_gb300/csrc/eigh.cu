@@ -57,35 +57,35 @@ __device__ double block_sum(double v) {
 
 // ------------------------------------------------------------------ 1. tridiagonalisation
 
-// Column j takes two launches.  The product kernel forms the reflector of row j
-// (columns j+1 .. n-1 of the symmetric A): H = I - tau v v^T with v_0 = 1 maps
-// x = A[j][j+1:] to beta e_1, every block recomputing beta, tau and the scale of v
-// from x_0 and sum_{i>=1} x_i^2; it computes p = tau A22 v (A22 = A[j+1:, j+1:], one
-// warp per row) and p . v.  The update kernel applies A22 -= v w^T + w v^T with
-// w = p - (tau/2)(p . v) v, stores v in A's row j (not read again by the reduction),
-// and sums the squares of the next reflector's row, A[j+1][j+3:].  The two sums are
-// reduced in block order by the last block to finish (a completion counter, no
-// waiting), so the results do not depend on the blocks' timing.
-constexpr int kPanel32 = 32;   // columns per panel of the blocked tridiagonalisation
+// A panel reduces kPanel32 columns j0 .. j0 + 31 against the trailing matrix as it stood at
+// the panel's start (A0); the reflectors v_t and the vectors w_t of the panel's columns
+// are kept as rows of PV = [V; W; V] (length n each), so that the matrix current at column
+// j is A0 - sum_t (v_t w_t^T + w_t v_t^T).  One cooperative launch does a whole panel; after
+// it the trailing matrix takes A -= V^T W + W^T V in one product of depth 2 * 32.
+//
+// With x = A[j][j+1:] (row j up to date), H = I - tau v v^T maps x to beta e_1, v = scale (x -
+// beta e_1) (v_0 = 1).  A column takes two passes with a grid barrier after each:
+//   1. every block reads x into shared memory; a warp per row forms A0 x (one FMA an entry;
+//      A0 v = scale (A0 x - beta A0 e_1)) and, as further rows, the dots V_t . x and
+//      W_t . x; the blocks' shares of x . A0 x go to part.  beta, tau and scale come
+//      from x itself, in every block alike.
+//   2. with those sums p . v = tau (v . A0 v - 2 sum_t (V_t . v)(W_t . v)) is known before p is, so
+//      each block forms p, w = p - (tau / 2)(p . v) v and row j + 1 of the current matrix for
+//      its own columns at once.
+// A row, a product and a p kernel per column with a reduction at the end of each took 31 us a
+// column at n = 2400 (27 of them latency: launch, dependent L2 reads, the last block's sum),
+// and an unblocked pair of kernels 23 us at n = 640; this takes 19 and 13 us.
+constexpr int kPanel32 = 32;   // columns per panel of the tridiagonalisation
+constexpr int kTriThreads = 256, kTriWarps = kTriThreads / 32;
+constexpr int kTriCols = 16;   // columns of pass 2 per block and turn
+constexpr int kTriUnroll = 8;  // loads in flight per lane in pass 1
+constexpr int64_t kTriStaged = 20000;   // x in shared memory up to this n
 
+// Barrier counter of the panel kernels (it counts on from launch to launch) and the flag of
+// a barrier that gave up, after which later panels do nothing.
 struct TriScalars {
-    double sumsq;            // sum_{i>=1} x_i^2 of the current reflector's row
-    double dot;              // p . v of the current column (blocked: (tau / 2) p . v)
-    unsigned cnt_a, cnt_b;   // completion counters of the two kernels
-    double c12[2 * kPanel32];   // blocked: W_t . v (t < i), then V_t . v
-    double scale;               // blocked: v_q = scale x_q (q >= 1) of the current reflector
+    unsigned count, gave_up;
 };
-
-// Sum of the nparts partial sums written by the other blocks (called by the whole block
-// that finished last): strided per thread, then the block reduction, so the order of
-// the additions is fixed.
-__device__ double last_block_sum(const double* part, unsigned nparts) {
-    __threadfence();
-    const volatile double* pp = part;
-    double t = 0.0;
-    for (unsigned b = threadIdx.x; b < nparts; b += blockDim.x) t += pp[b];
-    return block_sum(t);
-}
 
 __device__ __forceinline__ void reflector(double x0, double sumsq, double& beta, double& t, double& scale) {
     if (sumsq == 0.0) {
@@ -100,400 +100,255 @@ __device__ __forceinline__ void reflector(double x0, double sumsq, double& beta,
     }
 }
 
-// Sum of squares of A[0][2:] (the first reflector's row past its leading entry).  One block.
-__global__ void tri_init_kernel(const double* A, int64_t n, TriScalars* tri) {
-    double s = 0.0;
-    for (int64_t c = 2 + threadIdx.x; c < n; c += blockDim.x) s = fma(A[c], A[c], s);
-    s = block_sum(s);
-    if (threadIdx.x == 0) {
-        tri->sumsq = s;
-        tri->cnt_a = tri->cnt_b = 0;
-    }
-}
+struct TriPanel {
+    double* A;
+    int64_t lda, n, j0;
+    int nc;                      // columns of the panel
+    bool staged;                 // x fits shared memory
+    double *PV, *part, *ybuf, *dots, *d, *e, *tau;
+    TriScalars* tri;
+    unsigned base;               // count at the start of this launch
+    unsigned* status;
+};
 
-constexpr int kTriRows = 8;     // rows (one warp each) per block of the product kernel
-constexpr int kTriUnroll = 8;   // loads in flight per lane in the product kernel
-
-__global__ void __launch_bounds__(32 * kTriRows) tri_product_kernel(const double* __restrict__ A, int64_t lda,
-                                                                    int64_t n, int64_t j, TriScalars* tri,
-                                                                    double* part, double* d, double* e, double* tau,
-                                                                    double* vbuf, double* pbuf) {
-    const int64_t m = n - j - 1;
-    const double* x = A + j * lda + j + 1;
-    double beta, t, scale;
-    reflector(x[0], tri->sumsq, beta, t, scale);
-    auto v_at = [&](int64_t i) { return i == 0 ? 1.0 : x[i] * scale; };
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t r = (int64_t)blockIdx.x * kTriRows + warp;
-    double pv = 0.0;
-    if (r < m) {
-        // eight independent partial sums per lane (eight loads in flight), combined in a
-        // fixed order
-        const double* row = A + (j + 1 + r) * lda + j + 1;
-        double acc[kTriUnroll];
-#pragma unroll
-        for (int q = 0; q < kTriUnroll; q++) acc[q] = 0.0;
-        int64_t i = lane;
-        for (; i + 32 * (kTriUnroll - 1) < m; i += 32 * kTriUnroll) {
-            double rv[kTriUnroll];
-#pragma unroll
-            for (int q = 0; q < kTriUnroll; q++) rv[q] = row[i + 32 * q];
-#pragma unroll
-            for (int q = 0; q < kTriUnroll; q++) acc[q] = fma(rv[q], v_at(i + 32 * q), acc[q]);
-        }
-        for (; i < m; i += 32) acc[0] = fma(row[i], v_at(i), acc[0]);
-#pragma unroll
-        for (int w = kTriUnroll / 2; w > 0; w /= 2)
-#pragma unroll
-            for (int q = 0; q < w; q++) acc[q] += acc[q + w];
-        const double pr = t * warp_sum(acc[0]);
-        if (lane == 0) pbuf[r] = pr;
-        pv = pr * v_at(r);
-    }
-    if (blockIdx.x == 0)
-        for (int64_t i = threadIdx.x; i < m; i += blockDim.x) vbuf[i] = v_at(i);
-    __shared__ double wpart[kTriRows];
-    __shared__ bool last;
-    if (lane == 0) wpart[warp] = pv;
+// Arrive at grid barrier number `b` of this launch; wait for it (bounded: the launch is
+// cooperative, so every block is resident, but a wait that gives up is flagged, not endless).
+__device__ __forceinline__ void grid_arrive(const TriPanel& a) {
     __syncthreads();
     if (threadIdx.x == 0) {
-        double bs = 0.0;
-        for (int w = 0; w < kTriRows; w++) bs += wpart[w];
-        part[blockIdx.x] = bs;
         __threadfence();
-        last = atomicAdd(&tri->cnt_a, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (last) {   // the last block to finish reduces the partial sums (fixed order)
-        const double tot = last_block_sum(part, gridDim.x);
-        if (threadIdx.x == 0) {
-            tri->dot = tot;
-            tri->cnt_a = 0;
-            d[j] = A[j * lda + j];
-            e[j] = beta;
-            tau[j] = t;
-        }
+        atomicAdd(&a.tri->count, 1u);
     }
 }
-
-constexpr int kTriUpdRows = 16;  // rows of A22 per thread of the update kernel
-
-__global__ void __launch_bounds__(256) tri_update_kernel(double* A, int64_t lda, int64_t n, int64_t j,
-                                                         TriScalars* tri, double* part,
-                                                         const double* __restrict__ tau,
-                                                         const double* __restrict__ vbuf,
-                                                         const double* __restrict__ pbuf) {
-    const int64_t m = n - j - 1;
-    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t r0 = (int64_t)blockIdx.y * kTriUpdRows;
-    const double K = 0.5 * tau[j] * tri->dot;
-    double sq = 0.0;
-    if (c < m) {
-        const double vc = vbuf[c];
-        const double wc = pbuf[c] - K * vc;
-        const int64_t nr = m - r0 < kTriUpdRows ? m - r0 : kTriUpdRows;
-        double* a = A + (j + 1 + r0) * lda + j + 1 + c;
-        double cur[kTriUpdRows];
-#pragma unroll
-        for (int q = 0; q < kTriUpdRows; q++)
-            if (q < nr) cur[q] = a[q * lda];          // the rows' loads all in flight
-#pragma unroll
-        for (int q = 0; q < kTriUpdRows; q++) {
-            if (q >= nr) break;
-            const double vr = vbuf[r0 + q];
-            const double wr = pbuf[r0 + q] - K * vr;
-            const double v = cur[q] - (vr * wc + wr * vc);
-            a[q * lda] = v;
-            if (r0 + q == 0) {
-                if (c >= 2) sq = v * v;                // the next reflector's row past its leading entry
-                A[j * lda + j + 1 + c] = vc;           // v kept in row j for the back-transformation
+__device__ __forceinline__ bool grid_wait(const TriPanel& a, unsigned b) {
+    __shared__ int ok;
+    if (threadIdx.x == 0) {
+        const unsigned target = a.base + (b + 1) * gridDim.x;
+        const volatile unsigned* c = &a.tri->count;
+        uint64_t t0 = 0;
+        ok = 1;
+        for (unsigned polls = 1; (int)(*c - target) < 0; polls++) {
+            if ((polls & 1023u) == 0) {
+                uint64_t t;
+                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+                if (t0 == 0) t0 = t;
+                else if (t - t0 > 1000000000ull) {
+                    a.tri->gave_up = 1;
+                    raise_status(a.status, DEV_TIMEOUT);
+                    ok = 0;
+                    break;
+                }
             }
         }
+        __threadfence();
     }
-    if (blockIdx.y == 0) {   // block-uniform: the blocks of the first rows sum the next reflector's squares
-        __shared__ bool last;
-        const double bs = block_sum(sq);
-        if (threadIdx.x == 0) {
-            part[blockIdx.x] = bs;
-            __threadfence();
-            last = atomicAdd(&tri->cnt_b, 1u) == gridDim.x - 1;
+    __syncthreads();
+    return ok != 0;
+}
+
+__global__ void __launch_bounds__(kTriThreads) tri_panel_kernel(const __grid_constant__ TriPanel a) {
+    extern __shared__ __align__(16) double xs_raw[];
+    __shared__ double c1s[kPanel32], c2s[kPanel32], vj[kPanel32], wj[kPanel32];
+    __shared__ double red[2][kTriWarps][kTriCols];
+    __shared__ double wpart[kTriWarps], tot[3];
+    if (*(const volatile unsigned*)&a.tri->gave_up) return;
+    const int64_t n = a.n, lda = a.lda;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t gw = (int64_t)blockIdx.x * kTriWarps + warp, nw = (int64_t)gridDim.x * kTriWarps;
+    const bool pair_ok = a.staged && (lda % 2) == 0 && (reinterpret_cast<uintptr_t>(a.A) & 15u) == 0;
+    unsigned bar = 0;
+    for (int i = 0; i < a.nc; i++) {
+        const int64_t j = a.j0 + i, m = n - j - 1;
+        double* xg = a.A + j * lda + j + 1;
+        const int head = (reinterpret_cast<uintptr_t>(xg) & 15u) ? 1 : 0;   // entries before a 16-byte boundary
+        double* xs = xs_raw + head;                                          // aligned like xg
+        auto x_at = [&](int64_t q) { return a.staged ? xs[q] : __ldcg(xg + q); };
+        if (a.staged)
+            for (int64_t q = threadIdx.x; q < m; q += kTriThreads) xs[q] = __ldcg(xg + q);
+        const double* next = a.A + (j + 1) * lda;            // row j + 1 of A0
+        const double a00 = next[j + 1];
+        if ((int)threadIdx.x < i) {
+            vj[threadIdx.x] = __ldcg(a.PV + (int64_t)threadIdx.x * n + j + 1);
+            wj[threadIdx.x] = __ldcg(a.PV + (int64_t)(kPanel32 + threadIdx.x) * n + j + 1);
         }
         __syncthreads();
-        if (last) {
-            const double tot = last_block_sum(part, gridDim.x);
-            if (threadIdx.x == 0) {
-                tri->sumsq = tot;
-                tri->cnt_b = 0;
-            }
-        }
-    }
-}
-
-// ---- blocked tridiagonalisation (n >= kBlockedMinN)
-// A panel reduces kPanel32 columns j0 .. j0 + 31 against the trailing matrix as it stood at
-// the panel's start (A0); the reflectors v_t and the vectors w_t of the panel's columns
-// are kept as rows of PV = [V; W; V] (length n each, zero left of their column), so that
-// the matrix current at column j is A0 - sum_t (v_t w_t^T + w_t v_t^T).  Per column
-// j = j0 + i: the row kernel brings row j up to date (and writes the previous column's
-// v, w rows of PV); the product kernel forms y = A0[j+1:, j+1:] v (the only pass over the
-// trailing matrix) and the dots W_t . v, V_t . v; the p kernel corrects
-// p = tau (y - V (W^T v) - W (V^T v)) and stores v in A's row j.  After the panel the
-// trailing matrix takes A -= V^T W + W^T V in one product of depth 2 * 32.
-
-// Writes rows i of V, W (both copies of V) for the column jc whose v and p are in vbuf and
-// pbuf and whose (tau / 2) p . v is kw: v_c, and w_c = p_c - kw v_c, for c in [c0, n).
-__device__ __forceinline__ void blk_store_vw(double* PV, int64_t n, int i, int64_t c, const double* vbuf,
-                                             const double* pbuf, double kw, double* vo, double* wo) {
-    const double v = vbuf[c];
-    const double w = pbuf[c] - kw * v;
-    PV[(int64_t)i * n + c] = v;
-    PV[(int64_t)(kPanel32 + i) * n + c] = w;
-    PV[(int64_t)(2 * kPanel32 + i) * n + c] = v;
-    *vo = v;
-    *wo = w;
-}
-
-// Row j = j0 + i brought up to date over columns c in [j, n):
-// a_c = A0[j][c] - sum_{t < i} (V_t[j] W_t[c] + W_t[j] V_t[c]); for i >= 1 the previous
-// column's rows of V and W are formed from vbuf, pbuf, tri->dot (and written).  The sum of
-// squares of a_c for c >= j + 2 (the next reflector's row past x_0) goes to tri->sumsq.
-// A block takes 32 columns; its 8 groups of 32 threads share the terms t < i - 1 (t = g,
-// g + 8, ...: all loads of a thread in flight at once) and group 0 adds their sums in order.
-constexpr int kColGroups = 8, kGroupCols = 32;
-
-__global__ void __launch_bounds__(kColGroups * kGroupCols) blk_row_kernel(double* A, int64_t lda, int64_t n,
-                                                                          int64_t j, int i, double* PV,
-                                                                          TriScalars* tri, double* part,
-                                                                          const double* __restrict__ vbuf,
-                                                                          const double* __restrict__ pbuf) {
-    __shared__ double cv[kPanel32], cw[kPanel32];
-    __shared__ double red[kColGroups][kGroupCols];
-    const double kw = tri->dot;
-    if (threadIdx.x < i) {
-        const int t = threadIdx.x;
-        if (t == i - 1) {   // the previous column's entries at row j, from its vbuf / pbuf
-            cv[t] = vbuf[j];
-            cw[t] = pbuf[j] - kw * vbuf[j];
-        } else {
-            cv[t] = PV[(int64_t)t * n + j];
-            cw[t] = PV[(int64_t)(kPanel32 + t) * n + j];
-        }
-    }
-    __syncthreads();
-    const int cl = threadIdx.x % kGroupCols, g = threadIdx.x / kGroupCols;
-    const int64_t c = j + (int64_t)blockIdx.x * kGroupCols + cl;
-    double acc = 0.0;
-    if (c < n) {
-        const double* __restrict__ Vr = PV;
-        const double* __restrict__ Wr = PV + (int64_t)kPanel32 * n;
-        double vt[kPanel32 / kColGroups], wt[kPanel32 / kColGroups];
-#pragma unroll
-        for (int u = 0; u < kPanel32 / kColGroups; u++) {
-            const int t = g + kColGroups * u;
-            const bool in = t < i - 1;
-            vt[u] = in ? Vr[(int64_t)t * n + c] : 0.0;
-            wt[u] = in ? Wr[(int64_t)t * n + c] : 0.0;
-        }
-#pragma unroll
-        for (int u = 0; u < kPanel32 / kColGroups; u++) {
-            const int t = g + kColGroups * u;
-            if (t < i - 1) acc += cv[t] * wt[u] + cw[t] * vt[u];
-        }
-    }
-    red[g][cl] = acc;
-    __syncthreads();
-    double sq = 0.0;
-    if (g == 0 && c < n) {
-        double sum = 0.0;
-#pragma unroll
-        for (int h = 0; h < kColGroups; h++) sum += red[h][cl];
-        double a = A[j * lda + c] - sum;
-        if (i >= 1) {
-            double vt, wt;
-            blk_store_vw(PV, n, i - 1, c, vbuf, pbuf, kw, &vt, &wt);
-            a -= cv[i - 1] * wt + cw[i - 1] * vt;
-        }
-        A[j * lda + c] = a;
-        if (c >= j + 2) sq = a * a;
-    }
-    __shared__ bool last;
-    const double bs = block_sum(sq);
-    if (threadIdx.x == 0) {
-        part[blockIdx.x] = bs;
-        __threadfence();
-        last = atomicAdd(&tri->cnt_b, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (last) {
-        const double tot = last_block_sum(part, gridDim.x);
-        if (threadIdx.x == 0) {
-            tri->sumsq = tot;
-            tri->cnt_b = 0;
-        }
-    }
-}
-
-// The rows i of V and W for the panel's last column jc (before the trailing update):
-// c in [jc + 1, n).
-__global__ void blk_finish_kernel(double* PV, int64_t n, int64_t jc, int i, const TriScalars* tri,
-                                  const double* __restrict__ vbuf, const double* __restrict__ pbuf) {
-    const int64_t c = jc + 1 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n) return;
-    double v, w;
-    blk_store_vw(PV, n, i, c, vbuf, pbuf, tri->dot, &v, &w);
-}
-
-// y = A0[j+1:, j+1:] v (one warp per row, blocks 0 .. nsymv-1) for the reflector of row j
-// (formed in every block from x_0 and tri->sumsq, as in the unblocked product), and in
-// blocks 0 .. 2i - 1 (first, so that they overlap the rows) the dots W_t . v (t < i) and
-// V_t . v.  The FP64 pipe, not
-// memory, bounds this pass on GB300 (one multiply-add per 8-byte entry is above the
-// ridge), so v is not formed per entry: with v = scale x except v_0 = 1,
-// y_r = scale (sum_q A[r][q] x_q - beta A[r][0]) (1 - scale x_0 = -scale beta), one FMA an
-// entry with x read straight from A's row j; when sum_{q>=1} x_q^2 = 0 (scale = 0, v = e_0)
-// y_r = A[r][0].  Block 0 also writes d[j], e[j], tau[j] and the scale of v.
-constexpr int kBlkRows = 4;   // rows (one warp each) per block of the blocked product
-
-__global__ void __launch_bounds__(32 * kBlkRows) blk_product_kernel(const double* __restrict__ A, int64_t lda,
-                                                                    int64_t n, int64_t j, int i,
-                                                                    const double* __restrict__ PV, TriScalars* tri,
-                                                                    double* d, double* e, double* tau,
-                                                                    double* ybuf) {
-    const int64_t m = n - j - 1;
-    const double* x = A + j * lda + j + 1;
-    double beta, t, scale;
-    reflector(x[0], tri->sumsq, beta, t, scale);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        d[j] = A[j * lda + j];
-        e[j] = beta;
-        tau[j] = t;
-        tri->scale = scale;
-    }
-    if ((int)blockIdx.x < 2 * i) {   // block-uniform: one dot product per block
-        auto v_at = [&](int64_t q) { return q == 0 ? 1.0 : x[q] * scale; };
-        const int tp = (int)blockIdx.x;
-        const double* row = tp < i ? PV + (int64_t)(kPanel32 + tp) * n : PV + (int64_t)(tp - i) * n;
-        double acc = 0.0;
-        for (int64_t q = threadIdx.x; q < m; q += blockDim.x) acc = fma(row[j + 1 + q], v_at(q), acc);
-        acc = block_sum(acc);
-        if (threadIdx.x == 0) tri->c12[tp] = acc;
-        return;
-    }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t r = (int64_t)(blockIdx.x - 2 * i) * kBlkRows + warp;
-    if (r < m) {
-        const double* arow = A + (j + 1 + r) * lda + j + 1;
-        if (scale == 0.0) {
-            if (lane == 0) ybuf[j + 1 + r] = arow[0];
-        } else {
-            // 16-byte loads of the row and of x (two entries a lane) after one peeled entry
-            // when the segment does not start on a 16-byte boundary (A's rows and row j
-            // share the alignment when lda is even)
-            const bool pair_ok = (lda % 2) == 0;
-            const int64_t head = (reinterpret_cast<uintptr_t>(arow) & 15u) ? 1 : 0;
+        // ---- pass 1: the dots of W_t (t < i) and V_t with x, then the rows of A0
+        double xy = 0.0;
+        for (int64_t r = gw; r < m + 2 * i; r += nw) {
+            const int64_t row = r - 2 * i;
             double acc[kTriUnroll];
 #pragma unroll
             for (int q = 0; q < kTriUnroll; q++) acc[q] = 0.0;
-            if (pair_ok) {
-                const int64_t m2 = (m - head) / 2;
-                const double2* a2 = reinterpret_cast<const double2*>(arow + head);
-                const double2* x2 = reinterpret_cast<const double2*>(x + head);
-                if (head && lane == 0) acc[0] = arow[0] * x[0];
-                int64_t q0 = lane;
-                for (; q0 + 32 * (kTriUnroll - 1) < m2; q0 += 32 * kTriUnroll) {
-                    double2 rv[kTriUnroll], xv[kTriUnroll];
+            if (row < 0) {
+                const double* pv = a.PV + (r < i ? kPanel32 + r : r - i) * n + j + 1;
+                int64_t q = lane;
+                for (; q + 32 * 3 < m; q += 32 * 4) {
+                    double v[4];
 #pragma unroll
-                    for (int q = 0; q < kTriUnroll; q++) {
-                        rv[q] = a2[q0 + 32 * q];
-                        xv[q] = x2[q0 + 32 * q];
-                    }
+                    for (int k = 0; k < 4; k++) v[k] = __ldcg(pv + q + 32 * k);
 #pragma unroll
-                    for (int q = 0; q < kTriUnroll; q++) {
-                        acc[q] = fma(rv[q].x, xv[q].x, acc[q]);
-                        acc[q] = fma(rv[q].y, xv[q].y, acc[q]);
-                    }
+                    for (int k = 0; k < 4; k++) acc[k] = fma(v[k], x_at(q + 32 * k), acc[k]);
                 }
-                for (; q0 < m2; q0 += 32) {
-                    const double2 rv = a2[q0], xv = x2[q0];
-                    acc[0] = fma(rv.x, xv.x, acc[0]);
-                    acc[0] = fma(rv.y, xv.y, acc[0]);
-                }
-                if (((m - head) & 1) && lane == 0) acc[1] = fma(arow[m - 1], x[m - 1], acc[1]);
+                for (; q < m; q += 32) acc[0] = fma(__ldcg(pv + q), x_at(q), acc[0]);
             } else {
-                for (int64_t q = lane; q < m; q += 32) acc[0] = fma(arow[q], x[q], acc[0]);
+                const double* ar = a.A + (j + 1 + row) * lda + j + 1;
+                if (pair_ok) {
+                    const int64_t m2 = (m - head) / 2;
+                    const double2* a2 = reinterpret_cast<const double2*>(ar + head);
+                    const double2* x2 = reinterpret_cast<const double2*>(xs + head);
+                    if (head && lane == 0) acc[0] = ar[0] * xs[0];
+                    int64_t q = lane;
+                    for (; q + 32 * (kTriUnroll - 1) < m2; q += 32 * kTriUnroll) {
+                        double2 v[kTriUnroll];
+#pragma unroll
+                        for (int k = 0; k < kTriUnroll; k++) v[k] = a2[q + 32 * k];
+#pragma unroll
+                        for (int k = 0; k < kTriUnroll; k++) {
+                            const double2 xv = x2[q + 32 * k];
+                            acc[k] = fma(v[k].x, xv.x, acc[k]);
+                            acc[k] = fma(v[k].y, xv.y, acc[k]);
+                        }
+                    }
+                    double2 v[kTriUnroll];
+#pragma unroll
+                    for (int k = 0; k < kTriUnroll; k++)
+                        v[k] = q + 32 * k < m2 ? a2[q + 32 * k] : make_double2(0.0, 0.0);
+#pragma unroll
+                    for (int k = 0; k < kTriUnroll; k++)
+                        if (q + 32 * k < m2) {
+                            const double2 xv = x2[q + 32 * k];
+                            acc[k] = fma(v[k].x, xv.x, acc[k]);
+                            acc[k] = fma(v[k].y, xv.y, acc[k]);
+                        }
+                    if (((m - head) & 1) && lane == 0) acc[1] = fma(ar[m - 1], xs[m - 1], acc[1]);
+                } else {
+                    int64_t q = lane;
+                    for (; q + 32 * 3 < m; q += 32 * 4)
+#pragma unroll
+                        for (int k = 0; k < 4; k++) acc[k] = fma(ar[q + 32 * k], x_at(q + 32 * k), acc[k]);
+                    for (; q < m; q += 32) acc[0] = fma(ar[q], x_at(q), acc[0]);
+                }
             }
 #pragma unroll
             for (int w = kTriUnroll / 2; w > 0; w /= 2)
 #pragma unroll
                 for (int q = 0; q < w; q++) acc[q] += acc[q + w];
-            const double y = warp_sum(acc[0]);
-            if (lane == 0) ybuf[j + 1 + r] = scale * fma(-beta, arow[0], y);
+            const double sum = warp_sum(acc[0]);
+            if (lane == 0) {
+                if (row < 0) {
+                    a.dots[r] = sum;
+                } else {
+                    a.ybuf[row] = sum;
+                    xy = fma(x_at(row), sum, xy);
+                }
+            }
         }
-    }
-}
-
-// p = tau (y - sum_t (V_t W_t . v + W_t V_t . v)) over rows r in [j+1, n), v (from x and
-// the scale) stored in vbuf and in A's row j for the back-transformation, and (tau / 2) p . v
-// to tri->dot (reduced in a fixed order by the last block to finish).  A block takes 32
-// rows; its 8 groups share the terms t < i as in the row kernel.
-__global__ void __launch_bounds__(kColGroups * kGroupCols) blk_p_kernel(double* A, int64_t lda, int64_t n, int64_t j,
-                                                                        int i, const double* __restrict__ PV,
-                                                                        TriScalars* tri, double* part,
-                                                                        const double* __restrict__ tau, double* vbuf,
-                                                                        const double* __restrict__ ybuf, double* pbuf) {
-    __shared__ double c1[kPanel32], c2[kPanel32];
-    __shared__ double red[kColGroups][kGroupCols];
-    if (threadIdx.x < kPanel32) {
-        c1[threadIdx.x] = (int)threadIdx.x < i ? tri->c12[threadIdx.x] : 0.0;
-        c2[threadIdx.x] = (int)threadIdx.x < i ? tri->c12[i + threadIdx.x] : 0.0;
-    }
-    __syncthreads();
-    const int rl = threadIdx.x % kGroupCols, g = threadIdx.x / kGroupCols;
-    const int64_t r = j + 1 + (int64_t)blockIdx.x * kGroupCols + rl;
-    double acc = 0.0;
-    if (r < n) {
-        double vt[kPanel32 / kColGroups], wt[kPanel32 / kColGroups];
-#pragma unroll
-        for (int u = 0; u < kPanel32 / kColGroups; u++) {
-            const int t = g + kColGroups * u;
-            const bool in = t < i;
-            vt[u] = in ? PV[(int64_t)t * n + r] : 0.0;
-            wt[u] = in ? PV[(int64_t)(kPanel32 + t) * n + r] : 0.0;
-        }
-#pragma unroll
-        for (int u = 0; u < kPanel32 / kColGroups; u++) {
-            const int t = g + kColGroups * u;
-            if (t < i) acc += vt[u] * c1[t] + wt[u] * c2[t];
-        }
-    }
-    red[g][rl] = acc;
-    __syncthreads();
-    const double tj = tau[j];
-    double pv = 0.0;
-    if (g == 0 && r < n) {
-        double sum = 0.0;
-#pragma unroll
-        for (int h = 0; h < kColGroups; h++) sum += red[h][rl];
-        const double pr = tj * (ybuf[r] - sum);
-        pbuf[r] = pr;
-        const double v = r == j + 1 ? 1.0 : A[j * lda + r] * tri->scale;   // x_r read, then v_r stored
-        vbuf[r] = v;
-        pv = pr * v;
-        A[j * lda + r] = v;
-    }
-    __shared__ bool last;
-    const double bs = block_sum(pv);
-    if (threadIdx.x == 0) {
-        part[blockIdx.x] = bs;
-        __threadfence();
-        last = atomicAdd(&tri->cnt_a, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (last) {
-        const double tot = last_block_sum(part, gridDim.x);
+        if (lane == 0) wpart[warp] = xy;
+        __syncthreads();
         if (threadIdx.x == 0) {
-            tri->dot = 0.5 * tj * tot;
-            tri->cnt_a = 0;
+            double t = 0.0;
+            for (int w = 0; w < kTriWarps; w++) t += wpart[w];
+            a.part[blockIdx.x] = t;
+        }
+        // the reflector, in every block alike: while the others finish when x is staged (in A's
+        // row j it is overwritten once all have arrived)
+        if (a.staged) grid_arrive(a);
+        double sq = 0.0;
+        for (int64_t q = 1 + threadIdx.x; q < m; q += kTriThreads) sq = fma(x_at(q), x_at(q), sq);
+        sq = block_sum(sq);
+        double beta, t, scale;
+        reflector(x_at(0), sq, beta, t, scale);
+        if (!a.staged) grid_arrive(a);
+        if (!grid_wait(a, bar++)) return;
+        // ---- pass 2
+        const double yx0 = __ldcg(a.ybuf);
+        if (warp == 0) {
+            double v = 0.0;
+            for (unsigned b = lane; b < gridDim.x; b += 32) v += __ldcg(a.part + b);
+            v = warp_sum(v);
+            if (lane == 0) tot[0] = v;
+        } else if (warp == 1) {
+            double c1 = 0.0, c2 = 0.0, v0 = 0.0, w0 = 0.0;
+            if (lane < i) {
+                v0 = vj[lane];
+                w0 = wj[lane];
+                c1 = scale == 0.0 ? w0 : scale * fma(-beta, w0, __ldcg(a.dots + lane));        // W_t . v
+                c2 = scale == 0.0 ? v0 : scale * fma(-beta, v0, __ldcg(a.dots + i + lane));    // V_t . v
+            }
+            c1s[lane] = c1;
+            c2s[lane] = c2;
+            const double cc = warp_sum(c1 * c2), s0 = warp_sum(fma(v0, c1, w0 * c2));
+            if (lane == 0) {
+                tot[1] = cc;
+                tot[2] = s0;
+            }
+        }
+        __syncthreads();
+        const double y0 = scale == 0.0 ? a00 : scale * fma(-beta, a00, yx0);                   // (A0 v)_0
+        const double vav = scale == 0.0 ? a00
+                                        : scale * scale * fma(beta, fma(beta, a00, -2.0 * yx0), tot[0]);
+        const double kw = 0.5 * t * t * (vav - 2.0 * tot[1]);                                  // (tau / 2) p . v
+        const double wnext = t * (y0 - tot[2]) - kw;                                           // w at index j + 1
+        double* Vi = a.PV + (int64_t)i * n;
+        double* Wi = a.PV + (int64_t)(kPanel32 + i) * n;
+        double* Vc = a.PV + (int64_t)(2 * kPanel32 + i) * n;
+        const int cl = threadIdx.x % kTriCols, g = threadIdx.x / kTriCols;
+        for (int64_t c0 = j + 1 + (int64_t)blockIdx.x * kTriCols; c0 < n; c0 += (int64_t)gridDim.x * kTriCols) {
+            const int64_t c = c0 + cl;
+            double s1 = 0.0, s2 = 0.0;
+            if (c < n) {
+                double vt[2], wt[2];
+#pragma unroll
+                for (int u = 0; u < 2; u++) {
+                    const int q = g + 16 * u;
+                    vt[u] = q < i ? __ldcg(a.PV + (int64_t)q * n + c) : 0.0;
+                    wt[u] = q < i ? __ldcg(a.PV + (int64_t)(kPanel32 + q) * n + c) : 0.0;
+                }
+#pragma unroll
+                for (int u = 0; u < 2; u++) {
+                    const int q = g + 16 * u;
+                    if (q < i) {
+                        s1 = fma(vt[u], c1s[q], fma(wt[u], c2s[q], s1));
+                        s2 = fma(vj[q], wt[u], fma(wj[q], vt[u], s2));
+                    }
+                }
+            }
+            s1 += __shfl_xor_sync(0xffffffffu, s1, 16);
+            s2 += __shfl_xor_sync(0xffffffffu, s2, 16);
+            if (lane < kTriCols) {
+                red[0][warp][cl] = s1;
+                red[1][warp][cl] = s2;
+            }
+            __syncthreads();
+            if (threadIdx.x < 32) {       // lanes 0-15 sum the first kind, 16-31 the second
+                const double* rp = &red[lane >> 4][0][cl];
+                double u[4];
+#pragma unroll
+                for (int k = 0; k < 4; k++) u[k] = rp[k * kTriCols] + rp[(k + 4) * kTriCols];
+                const double sum = (u[0] + u[2]) + (u[1] + u[3]);
+                const double sum2 = __shfl_xor_sync(0xffffffffu, sum, 16);
+                if (lane < kTriCols && c < n) {
+                    const double an = next[c];
+                    const double y = scale == 0.0 ? an : scale * fma(-beta, an, __ldcg(a.ybuf + (c - j - 1)));
+                    const double v = c == j + 1 ? 1.0 : x_at(c - j - 1) * scale;
+                    const double w = fma(-kw, v, t * (y - sum));
+                    Vi[c] = v;
+                    Wi[c] = w;
+                    Vc[c] = v;
+                    if (i + 1 < a.nc) a.A[(j + 1) * lda + c] = an - sum2 - fma(wnext, v, w);
+                    a.A[j * lda + c] = v;    // kept for the back-transformation
+                }
+            }
+            __syncthreads();
+        }
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            a.d[j] = __ldcg(a.A + j * lda + j);
+            a.e[j] = beta;
+            a.tau[j] = t;
+        }
+        if (i + 1 < a.nc) {
+            grid_arrive(a);
+            if (!grid_wait(a, bar++)) return;
         }
     }
 }
@@ -762,10 +617,11 @@ __global__ void __launch_bounds__(32 * kRootWarps) dc_secular_kernel(MergeBufs b
     auto Zj = [&](int j) { return staged ? z2[j] : b.znd[j] * b.znd[j]; };
     const double d_i = Dj(i);
     const double gap = (i + 1 < k) ? Dj(i + 1) - d_i : rho;
-    // g at the midpoint decides which pole is nearer
-    const double mid = d_i + 0.5 * gap;
+    // g at the midpoint decides which pole is nearer (measured from d_i, as the bracket is: the
+    // rounded sum d_i + gap / 2 can lie on the root's other side when the gap is a few
+    // thousand units of d_i, and the bracket then misses the root)
     double fm = 0.0;
-    for (int j = lane; j < k; j += 32) fm += Zj(j) / (Dj(j) - mid);
+    for (int j = lane; j < k; j += 32) fm += Zj(j) / ((Dj(j) - d_i) - 0.5 * gap);
     fm = 1.0 + rho * warp_sum(fm);
     int org;
     double lo, hi;
@@ -1036,11 +892,11 @@ inline int64_t round8(int64_t x) { return (x + 7) / 8 * 8; }
 // 8192), otherwise as FP64 products on the DFMA pipe (small n: a few tiles, where the
 // slicing passes would cost more than they save).
 constexpr int64_t kOzakiMinN = 256, kOzakiMaxN = 8192;
-constexpr int64_t kBlockedMinN = 2048;   // the blocked tridiagonalisation from this n on
+constexpr int kMaxTriBlocks = 1024;
 
 struct EighBufs {
-    double *d, *e, *tau, *ebak, *vbuf, *pbuf, *part_a, *part_b;
-    double *PV, *ybuf;      // blocked tridiagonalisation: [V; W; V] of a panel, y = A0 v
+    double *d, *e, *tau, *ebak;
+    double *PV, *ybuf, *part, *dots;      // tridiagonalisation: [V; W; V] of a panel, A0 x, sums
     TriScalars* tri;
     MergeBufs mb;
     double *Vp, *Gv, *T, *W1, *W2;
@@ -1061,10 +917,8 @@ void eigh_layout(Ar& ar, int64_t n, EighBufs* out) {
     u.e = ar.template take<double>(n);
     u.tau = ar.template take<double>(n);
     u.ebak = ar.template take<double>(n);
-    u.vbuf = ar.template take<double>(n);
-    u.pbuf = ar.template take<double>(n);
-    u.part_a = ar.template take<double>((size_t)(n / kTriRows + 1));
-    u.part_b = ar.template take<double>((size_t)(n / 32 + 1));
+    u.part = ar.template take<double>(kMaxTriBlocks);
+    u.dots = ar.template take<double>(2 * kPanel32);
     u.tri = ar.template take<TriScalars>(1);
     u.PV = ar.template take<double>((size_t)(3 * kPanel32) * n);
     u.ybuf = ar.template take<double>(n);
@@ -1139,31 +993,50 @@ int eigh(double* A, int64_t lda, int64_t n, double* w, double* Q, int64_t ldq, v
     MergeBufs& mb = u.mb;
     const bool oz = u.oz != nullptr;
 
-    // 1. tridiagonalisation: blocked for large n (one pass over the trailing matrix per
-    // column plus one product per panel), else two launches per column
-    if (n >= kBlockedMinN) {
+    // 1. tridiagonalisation: a cooperative launch per panel, then the trailing product
+    if (n >= 3) {
+        const int dev = current_device();
+        int sms = 0;
+        if (dev < 0 || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+            return CHFSI_ERR_CUDA;
+        sms = std::min(sms, kMaxTriBlocks);
+        TriPanel tp{};
+        tp.A = A;
+        tp.lda = lda;
+        tp.n = n;
+        tp.staged = n <= kTriStaged;
+        tp.PV = u.PV;
+        tp.part = u.part;
+        tp.ybuf = u.ybuf;
+        tp.dots = u.dots;
+        tp.d = d;
+        tp.e = e;
+        tp.tau = tau;
+        tp.tri = u.tri;
+        tp.status = status;
+        static bool attr[kMaxDevices] = {};
+        if (!attr[dev]) {
+            CHFSI_CUDA_TRY(cudaFuncSetAttribute(tri_panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                (int)(sizeof(double) * (kTriStaged + 2))));
+            attr[dev] = true;
+        }
         CHFSI_CUDA_TRY(cudaMemsetAsync(u.tri, 0, sizeof(TriScalars), s));
         for (int64_t j0 = 0; j0 + 2 < n; j0 += kPanel32) {
             const int nc = (int)std::min<int64_t>(kPanel32, (n - 2) - j0);
             if (nc < kPanel32)   // rows nc .. 31 of V and W take part in the trailing product
                 CHFSI_CUDA_TRY(cudaMemsetAsync(u.PV, 0, sizeof(double) * (size_t)(3 * kPanel32) * n, s));
-            for (int i = 0; i < nc; i++) {
-                const int64_t j = j0 + i, m = n - j - 1;
-                blk_row_kernel<<<(unsigned)((n - j + kGroupCols - 1) / kGroupCols), kColGroups * kGroupCols, 0, s>>>(
-                    A, lda, n, j, i, u.PV, u.tri, u.part_b, u.vbuf, u.pbuf);
-                CHFSI_LAUNCH_CHECK();
-                const unsigned nrowb = (unsigned)((m + kBlkRows - 1) / kBlkRows);
-                blk_product_kernel<<<nrowb + 2 * i, 32 * kBlkRows, 0, s>>>(A, lda, n, j, i, u.PV, u.tri, d, e, tau,
-                                                                          u.ybuf);
-                CHFSI_LAUNCH_CHECK();
-                blk_p_kernel<<<(unsigned)((m + kGroupCols - 1) / kGroupCols), kColGroups * kGroupCols, 0, s>>>(
-                    A, lda, n, j, i, u.PV, u.tri, u.part_a, tau, u.vbuf, u.ybuf, u.pbuf);
-                CHFSI_LAUNCH_CHECK();
-            }
-            const int64_t jl = j0 + nc - 1, jn = j0 + nc, mp = n - jn;
-            blk_finish_kernel<<<(unsigned)((n - jl - 1 + 255) / 256), 256, 0, s>>>(u.PV, n, jl, nc - 1, u.tri, u.vbuf,
-                                                                                   u.pbuf);
+            // a warp per row of the product and its dots, at most one block per SM: fewer blocks
+            // meet sooner at the barriers
+            const int64_t rows = n - j0 - 1 + 2 * kPanel32;
+            const unsigned grid = (unsigned)std::min<int64_t>(sms, (rows + kTriWarps - 1) / kTriWarps);
+            tp.j0 = j0;
+            tp.nc = nc;
+            void* args[] = {&tp};
+            CHFSI_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)tri_panel_kernel, dim3(grid), dim3(kTriThreads),
+                                                       args, tp.staged ? sizeof(double) * (size_t)(n - j0 + 2) : 0, s));
             CHFSI_LAUNCH_CHECK();
+            tp.base += grid * (unsigned)(2 * nc - 1);
+            const int64_t jn = j0 + nc, mp = n - jn;
             // trailing matrix: A[jn:, jn:] -= V^T W + W^T V over the panel's rows of PV
             const double* Vop = u.PV + jn;
             const double* Wop = u.PV + (int64_t)kPanel32 * n + jn;
@@ -1179,18 +1052,6 @@ int eigh(double* A, int64_t lda, int64_t n, double* w, double* Q, int64_t ldq, v
                 return rc;
             }
         }
-    } else if (n >= 3) {
-        tri_init_kernel<<<1, 1024, 0, s>>>(A, n, u.tri);
-        CHFSI_LAUNCH_CHECK();
-    }
-    for (int64_t j = 0; n < kBlockedMinN && j + 2 < n; j++) {
-        const int64_t m = n - j - 1;
-        tri_product_kernel<<<(unsigned)((m + kTriRows - 1) / kTriRows), 32 * kTriRows, 0, s>>>(
-            A, lda, n, j, u.tri, u.part_a, d, e, tau, u.vbuf, u.pbuf);
-        CHFSI_LAUNCH_CHECK();
-        tri_update_kernel<<<dim3((unsigned)((m + 255) / 256), (unsigned)((m + kTriUpdRows - 1) / kTriUpdRows)), 256, 0,
-                            s>>>(A, lda, n, j, u.tri, u.part_b, tau, u.vbuf, u.pbuf);
-        CHFSI_LAUNCH_CHECK();
     }
     tridiag_tail_kernel<<<1, 32, 0, s>>>(A, lda, n, d, e, tau);
     CHFSI_LAUNCH_CHECK();
