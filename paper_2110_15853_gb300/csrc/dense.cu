@@ -37,6 +37,10 @@ struct GemmArgs {
     int nbatch = 1;
     int64_t strideA = 0, strideB = 0, strideC = 0, Ntot = 0, Nstep = 0;
     bool k_is_nc = false;
+    // merge products of the eigensolver: K = Nc = lda = ldb = ldc = the count at kn[b kn_stride],
+    // min(M, Ntot - b M) rows
+    const double* kn = nullptr;
+    int kn_stride = 0;
 };
 
 // TB x TB output tile, TB / 16 squared outputs per thread.
@@ -46,13 +50,19 @@ __global__ void __launch_bounds__(256) gemm_kernel(GemmArgs g) {
     __shared__ double As[BK][TB + 1];
     __shared__ double Bs[BK][TB];
     const int bi = blockIdx.y, bj = blockIdx.x, z = g.nbatch > 1 ? 0 : blockIdx.z;
-    if (g.nbatch > 1) {
+    if (g.nbatch > 1 || g.kn) {
         const int64_t b = blockIdx.z, cols = g.Ntot - b * g.Nstep;
         g.A += b * g.strideA;
         g.B += b * g.strideB;
         g.C += b * g.strideC;
-        if (cols < g.Nc) g.Nc = cols;
-        if (g.k_is_nc) g.K = g.Nc;
+        if (g.kn) {
+            if (g.Ntot - b * g.M < g.M) g.M = g.Ntot - b * g.M;
+            g.K = g.Nc = g.lda = g.ldb = g.ldc = (int64_t)g.kn[b * g.kn_stride];
+            if ((int64_t)bj * TB >= g.Nc || (int64_t)bi * TB >= g.M) return;
+        } else {
+            if (cols < g.Nc) g.Nc = cols;
+            if (g.k_is_nc) g.K = g.Nc;
+        }
     }
     if (g.upper_tiles && bi > bj) return;
     const int64_t i0 = (int64_t)bi * TB, j0 = (int64_t)bj * TB;
@@ -409,6 +419,23 @@ int gemm_nn(const double* A, int64_t lda, const double* B, int64_t ldb, double* 
             int64_t n, bool b_upper, cudaStream_t s) {
     GemmArgs g{A, lda, false, B, ldb, C, ldc, M, n, n, 1.0, false, false, b_upper, 1, nullptr};
     return run_gemm(g, s);
+}
+
+int gemm_merges(const double* G, const double* U, double* Gn, int64_t k, int64_t n, int nm, const double* kn,
+                int kn_stride, cudaStream_t s) {
+    GemmArgs g{G, k, false, U, k, Gn, k, k < n ? k : n, k < n ? k : n, k, 1.0, false, false, false, 1, nullptr};
+    g.M = k;
+    g.nbatch = nm;
+    g.Ntot = n;
+    g.strideA = g.strideB = g.strideC = k * k;
+    g.kn = kn;
+    g.kn_stride = kn_stride;
+    const int tb = gemm_tile(g.Nc, g.Nc, nm, false);
+    const dim3 grid((unsigned)((g.Nc + tb - 1) / tb), (unsigned)((g.Nc + tb - 1) / tb), (unsigned)nm);
+    if (tb == 64) gemm_kernel<64><<<grid, 256, 0, s>>>(g);
+    else gemm_kernel<16><<<grid, 256, 0, s>>>(g);
+    CHFSI_LAUNCH_CHECK();
+    return CHFSI_OK;
 }
 
 int gemm_general(const double* A, int64_t lda, bool a_t, const double* B, int64_t ldb, double* C, int64_t ldc,

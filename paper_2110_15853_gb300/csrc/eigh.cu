@@ -3,8 +3,8 @@
 //   1. Householder tridiagonalisation  A = Q_H T Q_H^T, one reflector per column
 //      (reflector of row j, symmetric matrix-vector product with the trailing block,
 //      symmetric rank-2 update);
-//   2. divide and conquer on T (Cuppen's splitting T = diag(T1, T2) + rho u u^T):
-//      leaves of 32 rows by parallel-ordered Jacobi in shared memory; each merge
+//   2. divide and conquer on T (Cuppen's splitting T = diag(T1, T2) + rho u u^T), the merges
+//      of a level together: leaves of 16 rows by parallel-ordered Jacobi in shared memory; each merge
 //      deflates (small components of z, nearly equal poles rotated together), finds
 //      the roots of the secular equation 1 + rho sum z_j^2 / (d_j - lambda) (one warp
 //      per root, bracketed steps of a two-pole rational model from the nearer pole), recomputes z
@@ -27,7 +27,8 @@ namespace chfsi {
 namespace {
 
 constexpr double kEps = 2.220446049250313e-16;
-constexpr int kLeaf = 32;
+// Jacobi on a leaf takes 800 us for 32 rows and 236 us for 16; one more level of merges about 150.
+constexpr int kLeaf = 16;
 constexpr int kPanel = 64;
 constexpr int kSecularSmem = 6144;   // poles and weights staged in shared memory up to this size
 
@@ -483,77 +484,153 @@ struct MergeBufs {
     double *G, *U, *Gn;
 };
 
+// The merges of a level run together: merge b = blockIdx.z joins the blocks [l, m) and [m, r) of
+// half = kLeaf 2^level rows (the last block may be shorter), l = 2 half b.  Every launch of a
+// level takes all of them; one merge at a time, the launches of 74 merges at n = 2400
+// mostly waited for one block or one warp per root.
+struct Merge {
+    int64_t l, m, r, k;
+};
+__device__ __forceinline__ Merge merge_at(int64_t half, int64_t n, MergeBufs& b) {
+    const int64_t i = blockIdx.z;
+    Merge g;
+    g.l = 2 * half * i;
+    g.m = g.l + half;
+    g.r = g.l + 2 * half < n ? g.l + 2 * half : n;
+    g.k = g.r - g.l;
+    b.D += g.l; b.z += g.l; b.Dnd += g.l; b.znd += g.l; b.tau_r += g.l; b.zhat += g.l; b.norm += g.l; b.val += g.l;
+    b.rot_c += g.l; b.rot_s += g.l;
+    b.perm += g.l; b.defl += g.l; b.ndidx += g.l; b.pos += g.l; b.org += g.l; b.rot_a += g.l; b.rot_b += g.l;
+    b.rank += g.l;
+    b.par += 8 * i;
+    const int64_t mat = i * (2 * half) * (2 * half);   // at most n^2 - k^2: 2 half <= l for i > 0
+    b.G += mat; b.U += mat; b.Gn += mat;
+    return g;
+}
+
 // par[] = {rho_hat, sign, k_nd, nrot}.
 // Merge preparation: z from the boundary rows, signs, the sorted poles, deflation with
-// the Givens rotations of nearly equal poles.  One block (the scans on thread 0).
-__global__ void __launch_bounds__(1024) dc_merge_prep_kernel(int64_t l, int64_t m, int64_t r, const double* w,
+// the Givens rotations of nearly equal poles.  One block per merge.  Each pole finds its
+// place in the merged order by a binary search in the other half; the poles that stay are
+// numbered by a block-wide count.  Only when two neighbouring ones are close enough for a
+// rotation does one thread walk through them (the walk alone took 115 us a merge).
+__global__ void __launch_bounds__(1024) dc_merge_prep_kernel(int64_t half, int64_t n, const double* w,
                                                              const double* Q, int64_t ldq, const double* ebak,
                                                              MergeBufs b) {
-    const int64_t n1 = m - l, k = r - l;
+    __shared__ int wcount[32], total;
+    __shared__ double wmax[32];
+    const Merge g = merge_at(half, n, b);
+    const int64_t l = g.l, m = g.m;
+    const int n1 = (int)(m - l), k = (int)g.k, n2 = k - n1;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const double rho0 = ebak[m - 1];
     const double sg = rho0 >= 0.0 ? 1.0 : -1.0;
-    double zz = 0.0;
-    for (int64_t p = threadIdx.x; p < k; p += blockDim.x) {
+    double zz = 0.0, dmax = 0.0;
+    for (int p = threadIdx.x; p < k; p += blockDim.x) {
         const double zp = p < n1 ? Q[(m - 1) * ldq + l + p] : Q[m * ldq + m + (p - n1)];
+        const double d = sg * w[l + p];
         b.z[p] = zp;
-        b.D[p] = sg * w[l + p];
+        b.D[p] = d;
+        dmax = fmax(dmax, fabs(d));
         zz += zp * zp;
     }
     zz = block_sum(zz);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
+    if (lane == 0) wmax[warp] = dmax;
     __syncthreads();
+    dmax = wmax[lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
+    const double rho_hat = fabs(rho0) * zz;
+    const double zs = 1.0 / sqrt(zz > 0.0 ? zz : 1.0);
+    // merged order of the two sorted halves (ascending when sg > 0, descending otherwise):
+    // entry t of a half goes behind the entries of the other half that come before it (those
+    // of the first half also when equal)
+    auto at1 = [&](int t) { return sg > 0.0 ? t : n1 - 1 - t; };
+    auto at2 = [&](int t) { return sg > 0.0 ? n1 + t : k - 1 - t; };
+    for (int p = threadIdx.x; p < k; p += blockDim.x) {
+        const bool first = p < n1;
+        const int t = first ? p : p - n1, q = first ? at1(t) : at2(t);
+        const double d = b.D[q];
+        int lo = 0, hi = first ? n2 : n1;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            const double o = first ? b.D[at2(mid)] : b.D[at1(mid)];
+            if (first ? o < d : o <= d) lo = mid + 1;
+            else hi = mid;
+        }
+        b.perm[t + lo] = q;
+        b.val[t + lo] = d;                 // sorted poles (modified by the rotations below)
+        b.tau_r[t + lo] = b.z[q] * zs;     // sorted, normalised z (temporarily)
+    }
+    __syncthreads();
+    const double tol = 8.0 * kEps * fmax(dmax, rho_hat);
+    // small components of z, and the numbers of the others
+    auto number = [&](bool small) {
+        int kn = 0;
+        for (int p0 = 0; p0 < k; p0 += blockDim.x) {
+            const int p = p0 + threadIdx.x;
+            bool stay = false;
+            if (p < k) {
+                if (small) b.defl[p] = fabs(rho_hat * b.tau_r[p]) <= tol;
+                stay = !b.defl[p];
+            }
+            const unsigned bits = __ballot_sync(0xffffffffu, stay);
+            if (lane == 0) wcount[warp] = __popc(bits);
+            __syncthreads();
+            int before = 0, sum = 0;
+            for (int q = 0; q < (int)(blockDim.x >> 5); q++) {
+                before += q < warp ? wcount[q] : 0;
+                sum += wcount[q];
+            }
+            const int c = kn + before + __popc(bits & ((1u << lane) - 1));
+            if (p < k) b.pos[p] = stay ? c : -1;
+            if (stay) b.ndidx[c] = p;
+            kn += sum;
+            __syncthreads();
+        }
+        return kn;
+    };
+    int kn = number(true);
+    if (threadIdx.x == 0) total = 0;
+    __syncthreads();
+    for (int c = threadIdx.x; c + 1 < kn; c += blockDim.x)
+        if (fabs(b.val[b.ndidx[c + 1]] - b.val[b.ndidx[c]]) <= tol) total = 1;
+    __syncthreads();
+    int nrot = 0;
+    if (total) {
+        if (threadIdx.x == 0) {
+            int last = -1;
+            for (int p = 0; p < k; p++) {
+                if (b.defl[p]) continue;
+                if (last >= 0 && fabs(b.val[p] - b.val[last]) <= tol) {
+                    const double zl = b.tau_r[last], zp = b.tau_r[p];
+                    const double rr = hypot(zl, zp), c = zp / rr, s = -zl / rr;
+                    const double dl = b.val[last], dp = b.val[p];
+                    b.val[last] = c * c * dl + s * s * dp;
+                    b.val[p] = s * s * dl + c * c * dp;
+                    b.tau_r[p] = rr;
+                    b.tau_r[last] = 0.0;
+                    b.defl[last] = 1;
+                    b.rot_a[nrot] = last;
+                    b.rot_b[nrot] = p;
+                    b.rot_c[nrot] = c;
+                    b.rot_s[nrot] = s;
+                    nrot++;
+                }
+                last = p;
+            }
+        }
+        __syncthreads();
+        kn = number(false);
+    }
+    for (int c = threadIdx.x; c < kn; c += blockDim.x) {
+        const int p = b.ndidx[c];
+        b.Dnd[c] = b.val[p];
+        b.znd[c] = b.tau_r[p];
+    }
     if (threadIdx.x == 0) {
-        const double rho_hat = fabs(rho0) * zz;
-        const double zs = 1.0 / sqrt(zz > 0.0 ? zz : 1.0);
-        // merge the two sorted halves (ascending when sg > 0, descending otherwise)
-        int64_t i = 0, j = 0, o = 0;
-        auto at1 = [&](int64_t t) { return sg > 0.0 ? t : n1 - 1 - t; };
-        auto at2 = [&](int64_t t) { return sg > 0.0 ? n1 + t : k - 1 - t; };
-        while (i < n1 || j < k - n1) {
-            if (j >= k - n1 || (i < n1 && b.D[at1(i)] <= b.D[at2(j)])) b.perm[o++] = (int)at1(i++);
-            else b.perm[o++] = (int)at2(j++);
-        }
-        double dmax = 0.0;
-        for (int64_t p = 0; p < k; p++) {
-            const int q = b.perm[p];
-            b.val[p] = b.D[q];                 // sorted poles (modified by the rotations below)
-            b.tau_r[p] = b.z[q] * zs;          // sorted, normalised z (temporarily)
-            dmax = fmax(dmax, fabs(b.val[p]));
-        }
-        const double tol = 8.0 * kEps * fmax(dmax, rho_hat);
-        int nrot = 0;
-        int64_t last = -1;
-        for (int64_t p = 0; p < k; p++) {
-            b.defl[p] = fabs(rho_hat * b.tau_r[p]) <= tol;
-            if (b.defl[p]) continue;
-            if (last >= 0 && fabs(b.val[p] - b.val[last]) <= tol) {
-                const double zl = b.tau_r[last], zp = b.tau_r[p];
-                const double rr = hypot(zl, zp), c = zp / rr, s = -zl / rr;
-                const double dl = b.val[last], dp = b.val[p];
-                b.val[last] = c * c * dl + s * s * dp;
-                b.val[p] = s * s * dl + c * c * dp;
-                b.tau_r[p] = rr;
-                b.tau_r[last] = 0.0;
-                b.defl[last] = 1;
-                b.rot_a[nrot] = (int)last;
-                b.rot_b[nrot] = (int)p;
-                b.rot_c[nrot] = c;
-                b.rot_s[nrot] = s;
-                nrot++;
-            }
-            last = p;
-        }
-        int64_t kn = 0;
-        for (int64_t p = 0; p < k; p++) {
-            if (!b.defl[p]) {
-                b.ndidx[kn] = (int)p;
-                b.pos[p] = (int)kn;
-                b.Dnd[kn] = b.val[p];
-                b.znd[kn] = b.tau_r[p];
-                kn++;
-            } else {
-                b.pos[p] = -1;
-            }
-        }
         b.par[0] = rho_hat;
         b.par[1] = sg;
         b.par[2] = (double)kn;
@@ -563,7 +640,9 @@ __global__ void __launch_bounds__(1024) dc_merge_prep_kernel(int64_t l, int64_t 
 
 // The deflation rotations on the block's columns (column p of the sorted problem is
 // block column perm[p]); one thread per row applies them in order.
-__global__ void dc_rotate_kernel(int64_t l, int64_t k, double* Q, int64_t ldq, MergeBufs b) {
+__global__ void dc_rotate_kernel(int64_t half, int64_t n, double* Q, int64_t ldq, MergeBufs b) {
+    const Merge g = merge_at(half, n, b);
+    const int64_t l = g.l, k = g.k;
     const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (row >= k) return;
     const int nrot = (int)b.par[3];
@@ -596,8 +675,9 @@ __device__ __forceinline__ double warp_prod(double v) {
 // behind the classical secular-equation solvers of Bunch, Nielsen and Sorensen and of
 // R.-C. Li), kept inside a bracket [lo, hi] with g(lo) < 0 < g(hi) by a bisection step
 // whenever the model's step would leave it.
-__global__ void __launch_bounds__(32 * kRootWarps) dc_secular_kernel(MergeBufs b, int cap) {
+__global__ void __launch_bounds__(32 * kRootWarps) dc_secular_kernel(int64_t half, int64_t n, MergeBufs b, int cap) {
     extern __shared__ double sh[];
+    merge_at(half, n, b);
     const int k = (int)b.par[2];
     const double rho = b.par[0];
     const bool staged = k <= cap;   // cap: poles the dynamic shared memory was sized for
@@ -710,7 +790,8 @@ __global__ void __launch_bounds__(32 * kRootWarps) dc_secular_kernel(MergeBufs b
 // (sign of the original z_i); one warp per i, each lane a strided part of the product.
 // By interlacing, every partial product of the ratios stays between the bounds of the
 // telescoping products, far from overflow.
-__global__ void __launch_bounds__(32 * kRootWarps) dc_lowner_kernel(MergeBufs b) {
+__global__ void __launch_bounds__(32 * kRootWarps) dc_lowner_kernel(int64_t half, int64_t n, MergeBufs b) {
+    merge_at(half, n, b);
     const int k = (int)b.par[2];
     const double rho = b.par[0];
     const int lane = threadIdx.x & 31;
@@ -730,7 +811,8 @@ __global__ void __launch_bounds__(32 * kRootWarps) dc_lowner_kernel(MergeBufs b)
 }
 
 // Norms of the eigenvectors u_i = (zhat_j / (d_j - lambda_i))_j; one warp per i.
-__global__ void __launch_bounds__(32 * kRootWarps) dc_norm_kernel(MergeBufs b) {
+__global__ void __launch_bounds__(32 * kRootWarps) dc_norm_kernel(int64_t half, int64_t n, MergeBufs b) {
+    merge_at(half, n, b);
     const int k = (int)b.par[2];
     const int lane = threadIdx.x & 31;
     const int i = blockIdx.x * kRootWarps + (threadIdx.x >> 5);
@@ -746,7 +828,8 @@ __global__ void __launch_bounds__(32 * kRootWarps) dc_norm_kernel(MergeBufs b) {
 }
 
 // U[j][i] = zhat_j / (d_j - lambda_i) / |u_i|  (k_nd x k_nd, row-major).
-__global__ void dc_build_u_kernel(MergeBufs b) {
+__global__ void dc_build_u_kernel(int64_t half, int64_t n, MergeBufs b) {
+    merge_at(half, n, b);
     const int k = (int)b.par[2];
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y;
@@ -755,7 +838,9 @@ __global__ void dc_build_u_kernel(MergeBufs b) {
 }
 
 // G[row][c] = block column perm[ndidx[c]] of Q.
-__global__ void dc_gather_kernel(int64_t l, int64_t k, const double* Q, int64_t ldq, MergeBufs b) {
+__global__ void dc_gather_kernel(int64_t half, int64_t n, const double* Q, int64_t ldq, MergeBufs b) {
+    const Merge g = merge_at(half, n, b);
+    const int64_t l = g.l, k = g.k;
     const int kn = (int)b.par[2];
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t row = blockIdx.y;
@@ -764,7 +849,8 @@ __global__ void dc_gather_kernel(int64_t l, int64_t k, const double* Q, int64_t 
 }
 
 // Final eigenvalues of the merged problem (sign restored) and their ascending ranks.
-__global__ void dc_rank_kernel(int64_t k, MergeBufs b) {
+__global__ void dc_rank_kernel(int64_t half, int64_t n, MergeBufs b) {
+    const int64_t k = merge_at(half, n, b).k;
     const double sg = b.par[1];
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < k; p += (int64_t)gridDim.x * blockDim.x) {
         const int q = b.pos[p];
@@ -773,7 +859,8 @@ __global__ void dc_rank_kernel(int64_t k, MergeBufs b) {
 }
 
 // Ascending rank of each merged eigenvalue (ties by index); one warp per value.
-__global__ void __launch_bounds__(32 * kRootWarps) dc_rank2_kernel(int64_t k, MergeBufs b) {
+__global__ void __launch_bounds__(32 * kRootWarps) dc_rank2_kernel(int64_t half, int64_t n, MergeBufs b) {
+    const int64_t k = merge_at(half, n, b).k;
     const int lane = threadIdx.x & 31;
     const int64_t p = (int64_t)blockIdx.x * kRootWarps + (threadIdx.x >> 5);
     if (p >= k) return;
@@ -790,8 +877,10 @@ __global__ void __launch_bounds__(32 * kRootWarps) dc_rank2_kernel(int64_t k, Me
 
 // Writes the merged eigenvalues w[l + rank] and the block's new columns into F
 // (k x k): deflated columns from Q, the others from Gn = G U.
-__global__ void dc_scatter_kernel(int64_t l, int64_t k, const double* Q, int64_t ldq, double* w, double* F,
-                                  MergeBufs b) {
+__global__ void dc_scatter_kernel(int64_t half, int64_t n, const double* Q, int64_t ldq, double* w, MergeBufs b) {
+    const Merge g = merge_at(half, n, b);
+    const int64_t l = g.l, k = g.k;
+    double* F = b.U;
     const int kn = (int)b.par[2];
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t row = blockIdx.y;
@@ -802,7 +891,10 @@ __global__ void dc_scatter_kernel(int64_t l, int64_t k, const double* Q, int64_t
     if (row == 0) w[l + dst] = b.D[p];
 }
 
-__global__ void copy_block_kernel(const double* F, int64_t k, double* Q, int64_t ldq, int64_t l) {
+__global__ void copy_block_kernel(int64_t half, int64_t n, double* Q, int64_t ldq, MergeBufs b) {
+    const Merge g = merge_at(half, n, b);
+    const int64_t l = g.l, k = g.k;
+    const double* F = b.U;
     const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t row = blockIdx.y;
     if (c >= k || row >= k) return;
@@ -893,6 +985,9 @@ inline int64_t round8(int64_t x) { return (x + 7) / 8 * 8; }
 // slicing passes would cost more than they save).
 constexpr int64_t kOzakiMinN = 256, kOzakiMaxN = 8192;
 constexpr int kMaxTriBlocks = 1024;
+// Merges of up to 256 rows multiply in FP64 (n k^2 multiply-adds a level, 0.27 ms at n = 2400
+// and k = 256, against about 40 us of launches a merge for an Ozaki product).
+constexpr int64_t kMergeFp64 = 256;
 
 struct EighBufs {
     double *d, *e, *tau, *ebak;
@@ -933,7 +1028,7 @@ void eigh_layout(Ar& ar, int64_t n, EighBufs* out) {
     b.val = ar.template take<double>(n);
     b.rot_c = ar.template take<double>(n);
     b.rot_s = ar.template take<double>(n);
-    b.par = ar.template take<double>(8);
+    b.par = ar.template take<double>((size_t)(n / kLeaf + 8) * 4);   // 8 per merge
     b.perm = ar.template take<int>(n);
     b.defl = ar.template take<int>(n);
     b.ndidx = ar.template take<int>(n);
@@ -1063,64 +1158,66 @@ int eigh(double* A, int64_t lda, int64_t n, double* w, double* Q, int64_t ldq, v
     const int64_t nleaf = (n + kLeaf - 1) / kLeaf;
     dc_leaf_kernel<<<(unsigned)nleaf, 256, 0, s>>>(n, d, e, w, Q, ldq);
     CHFSI_LAUNCH_CHECK();
-    std::vector<int64_t> bounds;
-    for (int64_t i = 0; i <= nleaf; i++) bounds.push_back(std::min(i * kLeaf, n));
-    while (bounds.size() > 2) {
-        std::vector<int64_t> next;
-        next.push_back(bounds[0]);
-        for (size_t i = 0; i + 2 < bounds.size(); i += 2) {
-            const int64_t l = bounds[i], m = bounds[i + 1], r = bounds[i + 2];
-            const int64_t k = r - l;
-            dc_merge_prep_kernel<<<1, 1024, 0, s>>>(l, m, r, w, Q, ldq, ebak, mb);
-            CHFSI_LAUNCH_CHECK();
-            dc_rotate_kernel<<<(unsigned)((k + 255) / 256), 256, 0, s>>>(l, k, Q, ldq, mb);
-            CHFSI_LAUNCH_CHECK();
-            const size_t sh = k <= kSecularSmem ? 2 * sizeof(double) * (size_t)k : 0;
-            if (sh > 48 * 1024) {
-                static bool attr[kMaxDevices] = {};
-                const int dev = current_device();
-                if (dev < 0) return CHFSI_ERR_CUDA;
-                if (!attr[dev]) {
-                    CHFSI_CUDA_TRY(cudaFuncSetAttribute(dc_secular_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                        (int)(2 * sizeof(double) * kSecularSmem)));
-                    attr[dev] = true;
-                }
+    std::vector<double> kns;
+    for (int64_t half = kLeaf; half < n; half *= 2) {
+        // all merges of the level: blocks at 2 half b with rows beyond the first half
+        const unsigned nm = (unsigned)((n - half + 2 * half - 1) / (2 * half));
+        const int64_t k = std::min(2 * half, n);      // the largest of them
+        const unsigned kb = (unsigned)((k + 255) / 256);
+        dc_merge_prep_kernel<<<dim3(1, 1, nm), 1024, 0, s>>>(half, n, w, Q, ldq, ebak, mb);
+        CHFSI_LAUNCH_CHECK();
+        dc_rotate_kernel<<<dim3(kb, 1, nm), 256, 0, s>>>(half, n, Q, ldq, mb);
+        CHFSI_LAUNCH_CHECK();
+        const size_t sh = k <= kSecularSmem ? 2 * sizeof(double) * (size_t)k : 0;
+        if (sh > 48 * 1024) {
+            static bool attr[kMaxDevices] = {};
+            const int dev = current_device();
+            if (dev < 0) return CHFSI_ERR_CUDA;
+            if (!attr[dev]) {
+                CHFSI_CUDA_TRY(cudaFuncSetAttribute(dc_secular_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                    (int)(2 * sizeof(double) * kSecularSmem)));
+                attr[dev] = true;
             }
-            // the non-deflated count is only known on the device: size the grids for k
-            const unsigned root_blocks = (unsigned)((k + kRootWarps - 1) / kRootWarps);
-            dc_secular_kernel<<<root_blocks, 32 * kRootWarps, sh, s>>>(mb, sh ? (int)k : 0);
-            CHFSI_LAUNCH_CHECK();
-            dc_lowner_kernel<<<root_blocks, 32 * kRootWarps, 0, s>>>(mb);
-            CHFSI_LAUNCH_CHECK();
-            dc_norm_kernel<<<root_blocks, 32 * kRootWarps, 0, s>>>(mb);
-            CHFSI_LAUNCH_CHECK();
-            dc_build_u_kernel<<<dim3((unsigned)((k + 255) / 256), (unsigned)k), 256, 0, s>>>(mb);
-            CHFSI_LAUNCH_CHECK();
-            dc_gather_kernel<<<dim3((unsigned)((k + 255) / 256), (unsigned)k), 256, 0, s>>>(l, k, Q, ldq, mb);
-            CHFSI_LAUNCH_CHECK();
-            // Gn (k x kn) = G (k x kn) U (kn x kn); kn <= k is read on the device, so the
-            // product runs at the full size k with G, U and Gn laid out for kn: a host copy
-            // of kn keeps the shapes exact
-            double kn_d = 0.0;
-            CHFSI_CUDA_TRY(cudaMemcpyAsync(&kn_d, mb.par + 2, sizeof(double), cudaMemcpyDeviceToHost, s));
-            CHFSI_CUDA_TRY(cudaStreamSynchronize(s));
-            const int64_t kn = (int64_t)kn_d;
-            int rc = oz ? ozaki_gemm_nn(mb.G, kn, mb.U, kn, k, kn, kn, mb.Gn, kn, false, u.oz, u.oz_bytes, status, s)
-                        : gemm_general(mb.G, kn, false, mb.U, kn, mb.Gn, kn, k, kn, kn, 1.0, false, s);
-            if (rc) return rc;
-            dc_rank_kernel<<<(unsigned)((k + 255) / 256), 256, 0, s>>>(k, mb);
-            CHFSI_LAUNCH_CHECK();
-            dc_rank2_kernel<<<root_blocks, 32 * kRootWarps, 0, s>>>(k, mb);
-            CHFSI_LAUNCH_CHECK();
-            dc_scatter_kernel<<<dim3((unsigned)((k + 255) / 256), (unsigned)k), 256, 0, s>>>(l, k, Q, ldq, w, mb.U,
-                                                                                          mb);
-            CHFSI_LAUNCH_CHECK();
-            copy_block_kernel<<<dim3((unsigned)((k + 255) / 256), (unsigned)k), 256, 0, s>>>(mb.U, k, Q, ldq, l);
-            CHFSI_LAUNCH_CHECK();
-            next.push_back(r);
         }
-        if (bounds.size() % 2 == 0) next.push_back(bounds.back());   // an unpaired last block carries over
-        bounds.swap(next);
+        // the non-deflated counts are only known on the device: size the grids for k
+        const dim3 roots((unsigned)((k + kRootWarps - 1) / kRootWarps), 1, nm), cells(kb, (unsigned)k, nm);
+        dc_secular_kernel<<<roots, 32 * kRootWarps, sh, s>>>(half, n, mb, sh ? (int)k : 0);
+        CHFSI_LAUNCH_CHECK();
+        dc_lowner_kernel<<<roots, 32 * kRootWarps, 0, s>>>(half, n, mb);
+        CHFSI_LAUNCH_CHECK();
+        dc_norm_kernel<<<roots, 32 * kRootWarps, 0, s>>>(half, n, mb);
+        CHFSI_LAUNCH_CHECK();
+        dc_build_u_kernel<<<cells, 256, 0, s>>>(half, n, mb);
+        CHFSI_LAUNCH_CHECK();
+        dc_gather_kernel<<<cells, 256, 0, s>>>(half, n, Q, ldq, mb);
+        CHFSI_LAUNCH_CHECK();
+        // Gn (k x kn) = G (k x kn) U (kn x kn), kn <= k the merge's count of non-deflated poles:
+        // FP64 products of all merges in one launch that reads kn on the device, or from
+        // 512 rows on Ozaki products one by one (kn copied to the host, once a level)
+        int rc;
+        if (oz && k > kMergeFp64) {
+            kns.resize(nm);
+            CHFSI_CUDA_TRY(cudaMemcpy2DAsync(kns.data(), sizeof(double), mb.par + 2, 8 * sizeof(double), sizeof(double),
+                                             nm, cudaMemcpyDeviceToHost, s));
+            CHFSI_CUDA_TRY(cudaStreamSynchronize(s));
+            for (unsigned b = 0; b < nm; b++) {
+                const int64_t kn = (int64_t)kns[b], mat = (int64_t)b * (2 * half) * (2 * half);
+                const int64_t kk = std::min(2 * half, n - 2 * half * b);
+                if ((rc = ozaki_gemm_nn(mb.G + mat, kn, mb.U + mat, kn, kk, kn, kn, mb.Gn + mat, kn, false, u.oz,
+                                        u.oz_bytes, status, s)))
+                    return rc;
+            }
+        } else if ((rc = gemm_merges(mb.G, mb.U, mb.Gn, 2 * half, n, (int)nm, mb.par + 2, 8, s))) {
+            return rc;
+        }
+        dc_rank_kernel<<<dim3(kb, 1, nm), 256, 0, s>>>(half, n, mb);
+        CHFSI_LAUNCH_CHECK();
+        dc_rank2_kernel<<<roots, 32 * kRootWarps, 0, s>>>(half, n, mb);
+        CHFSI_LAUNCH_CHECK();
+        dc_scatter_kernel<<<cells, 256, 0, s>>>(half, n, Q, ldq, w, mb);
+        CHFSI_LAUNCH_CHECK();
+        copy_block_kernel<<<cells, 256, 0, s>>>(half, n, Q, ldq, mb);
+        CHFSI_LAUNCH_CHECK();
     }
 
     // 3. back-transformation Q = H_0 H_1 ... H_{n-3} Q, panels from the last

@@ -101,6 +101,11 @@ int gemm_nn(const double* A, int64_t lda, const double* B, int64_t ldb, double* 
 // a_t, the transpose of A stored K x M; B: K x Nc (ldb).  FP64 on the DFMA pipe.
 int gemm_general(const double* A, int64_t lda, bool a_t, const double* B, int64_t ldb, double* C, int64_t ldc,
                  int64_t M, int64_t Nc, int64_t K, double alpha, bool accumulate, cudaStream_t s);
+// Gn_b = G_b U_b for the merges b < nm of a level of the eigensolver, matrices k * k apart,
+// dense with kn_b columns (kn_b = kn[b kn_stride], read on the device): G_b min(k, n - b k) x
+// kn_b, U_b kn_b x kn_b.  FP64.
+int gemm_merges(const double* G, const double* U, double* Gn, int64_t k, int64_t n, int nm, const double* kn,
+                int kn_stride, cudaStream_t s);
 // In place: upper Cholesky S = R^T R (R in the upper triangle, lower zeroed).
 // With oz_ws and scratch (at least (n - 64)^2 doubles) the trailing updates of 256 rows
 // and more run as Ozaki products on the tensor cores.
