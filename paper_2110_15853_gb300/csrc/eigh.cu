@@ -4,7 +4,7 @@
 //      (reflector of row j, symmetric matrix-vector product with the trailing block,
 //      symmetric rank-2 update);
 //   2. divide and conquer on T (Cuppen's splitting T = diag(T1, T2) + rho u u^T), the merges
-//      of a level together: leaves of 16 rows by parallel-ordered Jacobi in shared memory; each merge
+//      of a level together: leaves of 32 rows by parallel-ordered Jacobi in shared memory; each merge
 //      deflates (small components of z, nearly equal poles rotated together), finds
 //      the roots of the secular equation 1 + rho sum z_j^2 / (d_j - lambda) (one warp
 //      per root, bracketed steps of a two-pole rational model from the nearer pole), recomputes z
@@ -27,8 +27,7 @@ namespace chfsi {
 namespace {
 
 constexpr double kEps = 2.220446049250313e-16;
-// Jacobi on a leaf takes 800 us for 32 rows and 236 us for 16; one more level of merges about 150.
-constexpr int kLeaf = 16;
+constexpr int kLeaf = 32;
 constexpr int kPanel = 64;
 constexpr int kSecularSmem = 6144;   // poles and weights staged in shared memory up to this size
 
@@ -75,7 +74,7 @@ __device__ double block_sum(double v) {
 //      its own columns at once.
 // A row, a product and a p kernel per column with a reduction at the end of each took 31 us a
 // column at n = 2400 (27 of them latency: launch, dependent L2 reads, the last block's sum),
-// and an unblocked pair of kernels 23 us at n = 640; this takes 19 and 13 us.
+// and an unblocked pair of kernels 23 us at n = 640; this takes 18 and 12 us.
 constexpr int kPanel32 = 32;   // columns per panel of the tridiagonalisation
 constexpr int kTriThreads = 256, kTriWarps = kTriThreads / 32;
 constexpr int kTriCols = 16;   // columns of pass 2 per block and turn
@@ -246,10 +245,11 @@ __global__ void __launch_bounds__(kTriThreads) tri_panel_kernel(const __grid_con
         }
         if (lane == 0) wpart[warp] = xy;
         __syncthreads();
-        if (threadIdx.x == 0) {
-            double t = 0.0;
-            for (int w = 0; w < kTriWarps; w++) t += wpart[w];
-            a.part[blockIdx.x] = t;
+        if (warp == 0) {
+            double v = lane < kTriWarps ? wpart[lane] : 0.0;
+#pragma unroll
+            for (int o = kTriWarps / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (lane == 0) a.part[blockIdx.x] = v;
         }
         // the reflector, in every block alike: while the others finish when x is staged (in A's
         // row j it is overwritten once all have arrived)
@@ -260,15 +260,30 @@ __global__ void __launch_bounds__(kTriThreads) tri_panel_kernel(const __grid_con
         double beta, t, scale;
         reflector(x_at(0), sq, beta, t, scale);
         if (!a.staged) grid_arrive(a);
+        // this thread's entries of V, W and row j + 1 for pass 2, ready since the last column
+        const int cl = threadIdx.x % kTriCols, g = threadIdx.x / kTriCols;
+        const int64_t cfirst = j + 1 + (int64_t)blockIdx.x * kTriCols + cl;
+        double vt[2], wt[2], an = 0.0;
+        auto load_vw = [&](int64_t c) {
+#pragma unroll
+            for (int u = 0; u < 2; u++) {
+                const int q = g + 16 * u;
+                vt[u] = c < n && q < i ? __ldcg(a.PV + (int64_t)q * n + c) : 0.0;
+                wt[u] = c < n && q < i ? __ldcg(a.PV + (int64_t)(kPanel32 + q) * n + c) : 0.0;
+            }
+            if (threadIdx.x < kTriCols && c < n) an = next[c];
+        };
+        load_vw(cfirst);
         if (!grid_wait(a, bar++)) return;
         // ---- pass 2
         const double yx0 = __ldcg(a.ybuf);
+        double yc = threadIdx.x < kTriCols && cfirst < n ? __ldcg(a.ybuf + (cfirst - j - 1)) : 0.0;
         if (warp == 0) {
             double v = 0.0;
             for (unsigned b = lane; b < gridDim.x; b += 32) v += __ldcg(a.part + b);
             v = warp_sum(v);
             if (lane == 0) tot[0] = v;
-        } else if (warp == 1) {
+        } else if (warp <= 2) {
             double c1 = 0.0, c2 = 0.0, v0 = 0.0, w0 = 0.0;
             if (lane < i) {
                 v0 = vj[lane];
@@ -276,13 +291,12 @@ __global__ void __launch_bounds__(kTriThreads) tri_panel_kernel(const __grid_con
                 c1 = scale == 0.0 ? w0 : scale * fma(-beta, w0, __ldcg(a.dots + lane));        // W_t . v
                 c2 = scale == 0.0 ? v0 : scale * fma(-beta, v0, __ldcg(a.dots + i + lane));    // V_t . v
             }
-            c1s[lane] = c1;
-            c2s[lane] = c2;
-            const double cc = warp_sum(c1 * c2), s0 = warp_sum(fma(v0, c1, w0 * c2));
-            if (lane == 0) {
-                tot[1] = cc;
-                tot[2] = s0;
+            if (warp == 1) {
+                c1s[lane] = c1;
+                c2s[lane] = c2;
             }
+            const double sum = warp_sum(warp == 1 ? c1 * c2 : fma(v0, c1, w0 * c2));
+            if (lane == 0) tot[warp] = sum;
         }
         __syncthreads();
         const double y0 = scale == 0.0 ? a00 : scale * fma(-beta, a00, yx0);                   // (A0 v)_0
@@ -293,25 +307,15 @@ __global__ void __launch_bounds__(kTriThreads) tri_panel_kernel(const __grid_con
         double* Vi = a.PV + (int64_t)i * n;
         double* Wi = a.PV + (int64_t)(kPanel32 + i) * n;
         double* Vc = a.PV + (int64_t)(2 * kPanel32 + i) * n;
-        const int cl = threadIdx.x % kTriCols, g = threadIdx.x / kTriCols;
         for (int64_t c0 = j + 1 + (int64_t)blockIdx.x * kTriCols; c0 < n; c0 += (int64_t)gridDim.x * kTriCols) {
             const int64_t c = c0 + cl;
             double s1 = 0.0, s2 = 0.0;
-            if (c < n) {
-                double vt[2], wt[2];
 #pragma unroll
-                for (int u = 0; u < 2; u++) {
-                    const int q = g + 16 * u;
-                    vt[u] = q < i ? __ldcg(a.PV + (int64_t)q * n + c) : 0.0;
-                    wt[u] = q < i ? __ldcg(a.PV + (int64_t)(kPanel32 + q) * n + c) : 0.0;
-                }
-#pragma unroll
-                for (int u = 0; u < 2; u++) {
-                    const int q = g + 16 * u;
-                    if (q < i) {
-                        s1 = fma(vt[u], c1s[q], fma(wt[u], c2s[q], s1));
-                        s2 = fma(vj[q], wt[u], fma(wj[q], vt[u], s2));
-                    }
+            for (int u = 0; u < 2; u++) {
+                const int q = g + 16 * u;
+                if (q < i) {
+                    s1 = fma(vt[u], c1s[q], fma(wt[u], c2s[q], s1));
+                    s2 = fma(vj[q], wt[u], fma(wj[q], vt[u], s2));
                 }
             }
             s1 += __shfl_xor_sync(0xffffffffu, s1, 16);
@@ -329,8 +333,7 @@ __global__ void __launch_bounds__(kTriThreads) tri_panel_kernel(const __grid_con
                 const double sum = (u[0] + u[2]) + (u[1] + u[3]);
                 const double sum2 = __shfl_xor_sync(0xffffffffu, sum, 16);
                 if (lane < kTriCols && c < n) {
-                    const double an = next[c];
-                    const double y = scale == 0.0 ? an : scale * fma(-beta, an, __ldcg(a.ybuf + (c - j - 1)));
+                    const double y = scale == 0.0 ? an : scale * fma(-beta, an, yc);
                     const double v = c == j + 1 ? 1.0 : x_at(c - j - 1) * scale;
                     const double w = fma(-kw, v, t * (y - sum));
                     Vi[c] = v;
@@ -341,6 +344,11 @@ __global__ void __launch_bounds__(kTriThreads) tri_panel_kernel(const __grid_con
                 }
             }
             __syncthreads();
+            const int64_t cn = c + (int64_t)gridDim.x * kTriCols;      // a further turn
+            if (cn - cl < n) {
+                load_vw(cn);
+                if (threadIdx.x < kTriCols && cn < n) yc = __ldcg(a.ybuf + (cn - j - 1));
+            }
         }
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             a.d[j] = __ldcg(a.A + j * lda + j);
@@ -424,10 +432,11 @@ __global__ void __launch_bounds__(256) dc_leaf_kernel(int64_t n, const double* d
                 if (p > q) { const int t = p; p = q; q = t; }
                 const double apq = A[p][q];
                 double c = 1.0, sn = 0.0;
-                if (apq != 0.0 && fabs(apq) > 1e-300) {
+                // an entry below 1e-19 |A| is left (the sweeps end at 1e-15 |A| over all of them)
+                if (apq != 0.0 && fabs(apq) > 1e-300 && apq * apq > 1e-38 * t2) {
                     const double theta = (A[q][q] - A[p][p]) / (2.0 * apq);
                     const double t = (theta >= 0.0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-                    c = 1.0 / sqrt(t * t + 1.0);
+                    c = rsqrt(t * t + 1.0);
                     sn = t * c;
                 }
                 rp[k] = p; rq[k] = q; rc[k] = c; rs[k] = sn;
@@ -438,6 +447,7 @@ __global__ void __launch_bounds__(256) dc_leaf_kernel(int64_t n, const double* d
                 const int k = idx / kLeaf, col = idx % kLeaf;
                 const int p = rp[k], q = rq[k];
                 const double c = rc[k], sn = rs[k];
+                if (sn == 0.0) continue;                 // uniform in the warp
                 const double ap = A[p][col], aq = A[q][col];
                 A[p][col] = c * ap - sn * aq;
                 A[q][col] = sn * ap + c * aq;
@@ -448,6 +458,7 @@ __global__ void __launch_bounds__(256) dc_leaf_kernel(int64_t n, const double* d
                 const int k = idx / kLeaf, row = idx % kLeaf;
                 const int p = rp[k], q = rq[k];
                 const double c = rc[k], sn = rs[k];
+                if (sn == 0.0) continue;
                 const double ap = A[row][p], aq = A[row][q];
                 A[row][p] = c * ap - sn * aq;
                 A[row][q] = sn * ap + c * aq;

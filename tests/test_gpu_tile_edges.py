@@ -27,7 +27,7 @@ def _dev(a):
 
 @pytest.mark.parametrize("n", [4, 15, 16, 17, 34, 35, 48, 66, 255, 256, 258, 511, 513, 546])
 def test_eigh_leaves_panels_and_merge_products(P, n):
-    """Leaves of 16 rows, panels of 32 (and the last two rows), merges on either side of
+    """Leaves and panels of 32 rows (and the last two rows), merges on either side of
     the FP64 / Ozaki product line, odd leading dimensions, on a random matrix and on one
     with threefold clusters (rotations in the merges)."""
     rng = np.random.default_rng(n)
