@@ -191,7 +191,7 @@ __device__ __forceinline__ double div_by(double v, double d, double r) {
 // lane = column, warp w the rows i = w mod 4 in registers (one warp per FP64 unit of the
 // SM).  A step's chain is the root and reciprocal of the pivot, the scaled row and one
 // update; 64 columns in one block of 256 threads with three barriers a step took 105 us,
-// two 32-column blocks take 36 us each.
+// two 32-column blocks take 28 us each.
 __global__ void __launch_bounds__(128) chol_diag_kernel(double* S, int64_t lds, int64_t k0, int nb,
                                                         unsigned* status) {
     __shared__ double row[2][ND];
@@ -209,7 +209,9 @@ __global__ void __launch_bounds__(128) chol_diag_kernel(double* S, int64_t lds, 
         __syncthreads();
         double p = row[k & 1][k];
         if (!(p > 0.0) || !isfinite(p)) { bad = true; p = 1.0; }
-        const double d = sqrt(p), r = 1.0 / d;
+        // root and reciprocal from one reciprocal square root and a correction each: a shorter
+        // chain than sqrt and a division (a block 37 -> 28 us)
+        const double r = rsqrt(p), d0 = p * r, d = fma(fma(-d0, d0, p), 0.5 * r, d0);
         const double x = j == k ? d : div_by(row[k & 1][j], d, r);   // R[k][j], j >= k
         if (w == (k & 3)) a[k / 4] = j >= k ? x : 0.0;
 #pragma unroll
@@ -447,20 +449,12 @@ int gemm_general(const double* A, int64_t lda, bool a_t, const double* B, int64_
 
 namespace {
 
-// Z -= D on the upper triangle of a rows x rows block (D dense, leading dimension rows).
-__global__ void sub_upper_kernel(double* Z, int64_t ldz, const double* __restrict__ D, int64_t rows) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= rows * rows) return;
-    const int64_t i = idx / rows, c = idx % rows;
-    if (c >= i) Z[i * ldz + c] -= D[idx];
-}
-
 constexpr int64_t kCholOzakiMin = 256;   // trailing blocks from this size on as Ozaki products
 
 }  // namespace
 
-int cholesky_upper(double* S, int64_t n, int64_t lds, unsigned* status, cudaStream_t s, void* oz_ws, size_t oz_bytes,
-                   double* scratch) {
+int cholesky_upper(double* S, int64_t n, int64_t lds, unsigned* status, cudaStream_t s, void* oz_ws,
+                   size_t oz_bytes) {
     int rc;
     for (int64_t k0 = 0; k0 < n; k0 += NB) {
         const int nb = (int)((n - k0) < NB ? (n - k0) : NB);
@@ -484,17 +478,15 @@ int cholesky_upper(double* S, int64_t n, int64_t lds, unsigned* status, cudaStre
         }
         int64_t rest = n - k0 - nb;
         if (rest <= 0) break;
-        // trailing update S22 -= R12^T R12 (upper tiles): an Ozaki product on the tensor
-        // cores into the scratch block when one is given, else FP64 on the DFMA pipe
+        // trailing update S22 -= R12^T R12: an Ozaki product on the tensor cores when its
+        // workspace is given, else FP64 on the DFMA pipe (upper tiles)
         const double* R12 = S + k0 * lds + (k0 + nb);
         double* S22 = S + (k0 + nb) * lds + (k0 + nb);
-        if (oz_ws && scratch && rest >= kCholOzakiMin &&
+        if (oz_ws && rest >= kCholOzakiMin &&
             oz_bytes >= ozaki_workspace_bytes(true, rest, rest, nb, true)) {
-            if ((rc = ozaki_gemm_tn(R12, lds, R12, lds, nb, rest, rest, scratch, rest, true, oz_ws, oz_bytes, status,
-                                    s)))
+            if ((rc = ozaki_gemm_tn(R12, lds, R12, lds, nb, rest, rest, S22, lds, true, oz_ws, oz_bytes, status, s,
+                                    true)))
                 return rc;
-            sub_upper_kernel<<<(unsigned)((rest * rest + 255) / 256), 256, 0, s>>>(S22, lds, scratch, rest);
-            CHFSI_LAUNCH_CHECK();
             continue;
         }
         GemmArgs g{R12, lds, true, R12, lds, S22, lds, rest, rest, nb, -1.0, true, true, false, 1, nullptr};

@@ -914,9 +914,14 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(const __grid_const
 // when trans, else src[r * ld + k]); 0 for a row of zeros (subnormals count as zero).
 // Batch z = blockIdx.z reads src + z * src_bstride over K_z = min(Kb, Ktot - z Kb) and
 // writes exps + z * rows_pad.  exps must be zeroed first.
+// kTrans: a thread per column of src, span of its rows per block row, eight loads in
+// flight.  Short spans where K is small: the loads of a span follow one another (64 rows
+// in one span, four at a time, took 13 us).
+inline int exponent_span(int64_t K) { return K <= 4096 ? 32 : 256; }
+
 template <bool kTrans>
 __global__ void oz_exponents_kernel(const double* __restrict__ src, int64_t ld, int64_t rows, int64_t Kb,
-                                    int64_t Ktot, int64_t src_bstride, int64_t rows_pad, int* exps,
+                                    int64_t Ktot, int64_t src_bstride, int64_t rows_pad, int span, int* exps,
                                     unsigned* status) {
     const int64_t z = blockIdx.z;
     src += z * src_bstride;
@@ -925,16 +930,21 @@ __global__ void oz_exponents_kernel(const double* __restrict__ src, int64_t ld, 
     int m = 0;
     bool bad = false;
     if (kTrans) {
-        // thread per column of src (row of A_hat), a range of src rows per block row
         const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-        const int64_t k0 = (int64_t)blockIdx.y * 256;
+        const int64_t k0 = (int64_t)blockIdx.y * span;
         if (r >= rows) return;
-        const int64_t k1 = k0 + 256 < K ? k0 + 256 : K;
-        for (int64_t k = k0; k < k1; k++) {
-            const int ef = (int)((__double_as_longlong(src[k * ld + r]) >> 52) & 0x7ff);
-            bad |= ef == 0x7ff;
-            m = ef > m ? ef : m;
+        const int64_t k1 = k0 + span < K ? k0 + span : K;
+        for (int64_t k = k0; k < k1; k += 8) {
+            double x[8];
+#pragma unroll
+            for (int u = 0; u < 8; u++) x[u] = k + u < k1 ? src[(k + u) * ld + r] : 0.0;
+#pragma unroll
+            for (int u = 0; u < 8; u++) {
+                const int ef = (__double2hiint(x[u]) >> 20) & 0x7ff;
+                m = ef > m ? ef : m;
+            }
         }
+        bad = m == 0x7ff;
         if (m) atomicMax(exps + r, m);
     } else {
         // warp per row
@@ -1063,17 +1073,23 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(const double* __restrict_
     }
 }
 
-// C = sum over splits of the partial tiles; for a symmetric product an element
-// below the diagonal takes its mirror above it (always in a computed tile).
-__global__ void oz_reduce_kernel(const double* __restrict__ part, int splits, int64_t Mp, int64_t Np, int64_t M,
-                                 int64_t Nc, double* C, int64_t ldc, int symmetric) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= M * Nc) return;
-    int64_t i = idx / Nc, j = idx % Nc;
-    if (symmetric && i > j) { const int64_t t = i; i = j; j = t; }
-    double s = 0.0;
-    for (int z = 0; z < splits; z++) s += part[((int64_t)z * Mp + i) * Np + j];
-    C[(idx / Nc) * ldc + idx % Nc] = s;
+// C (= C - when subtract) the sum over splits of the partial tiles; for a symmetric product
+// an element below the diagonal takes its mirror above it (always in a computed tile).  A
+// block per 256 columns of a row: with the row and column from a 64-bit division per element
+// the pass took twice as long.
+__global__ void __launch_bounds__(256) oz_reduce_kernel(const double* __restrict__ part, int splits, int64_t Mp,
+                                                        int64_t Np, int64_t M, int64_t Nc, double* C, int64_t ldc,
+                                                        int symmetric, int subtract) {
+    const int64_t c = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (c >= Nc) return;
+    for (int64_t r = blockIdx.y; r < M; r += gridDim.y) {
+        const bool below = symmetric && r > c;
+        const double* p = part + (below ? c * Np + r : r * Np + c);
+        double s = 0.0;
+        for (int z = 0; z < splits; z++) s += p[(int64_t)z * Mp * Np];
+        double* d = C + r * ldc + c;
+        *d = subtract ? *d - s : s;
+    }
 }
 
 inline int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
@@ -1132,11 +1148,14 @@ int oz_prepare(const double* src, int64_t ld, bool trans, const OzOperand& o, in
     CHFSI_CUDA_TRY(cudaMemsetAsync(o.exps, 0, sizeof(int) * (size_t)o.padded_rows(), s));
     const int64_t brows = o.tiles * o.tile_rows;
     if (trans) {
-        dim3 grid((unsigned)((o.rows + 255) / 256), (unsigned)((o.K + 255) / 256), (unsigned)o.nbatch);
-        oz_exponents_kernel<true><<<grid, 256, 0, s>>>(src, ld, o.rows, o.K, Ktot, src_bstride, brows, o.exps, status);
+        const int span = exponent_span(o.K);
+        dim3 grid((unsigned)((o.rows + 255) / 256), (unsigned)((o.K + span - 1) / span), (unsigned)o.nbatch);
+        oz_exponents_kernel<true><<<grid, 256, 0, s>>>(src, ld, o.rows, o.K, Ktot, src_bstride, brows, span, o.exps,
+                                                      status);
     } else {
         dim3 grid((unsigned)((o.rows * 32 + 255) / 256), 1, (unsigned)o.nbatch);
-        oz_exponents_kernel<false><<<grid, 256, 0, s>>>(src, ld, o.rows, o.K, Ktot, src_bstride, brows, o.exps, status);
+        oz_exponents_kernel<false><<<grid, 256, 0, s>>>(src, ld, o.rows, o.K, Ktot, src_bstride, brows, 0, o.exps,
+                                                       status);
     }
     CHFSI_LAUNCH_CHECK();
     if (o.tile_rows == kTileM)
@@ -1228,7 +1247,7 @@ int make_map_planes(CUtensorMap* map, const OzOperand& o) {
 // The product of prepared operands.  nbatch > 1: independent products, batch b of the
 // output at rows b * m_batch (m_batch rows each, the last one clipped at M).
 int oz_run(const OzPlan& p, bool tn_form, double* C, int64_t ldc, int64_t M, int64_t Nc, bool symmetric,
-           bool b_upper, unsigned* status, cudaStream_t s, int nbatch = 1, int64_t m_batch = 0) {
+           bool b_upper, unsigned* status, cudaStream_t s, int nbatch = 1, int64_t m_batch = 0, bool subtract = false) {
     if (M <= 0 || Nc <= 0) return CHFSI_OK;
     const int64_t K_pad = p.A.chunks * kChunk;
     if (K_pad > (int64_t)1 << 21 || p.A.padded_rows() * kSlices > INT32_MAX || p.B.padded_rows() * kSlices > INT32_MAX)
@@ -1284,9 +1303,9 @@ int oz_run(const OzPlan& p, bool tn_form, double* C, int64_t ldc, int64_t M, int
     const int64_t total = pairs * g.splits * nbatch;
     if ((rc = launch_oz(g, tmA, total, s))) return rc;
     if (tn_form) {
-        const int64_t cnt = M * Nc;
-        oz_reduce_kernel<<<(unsigned)((cnt + 255) / 256), 256, 0, s>>>(p.part, g.splits, g.Mp, g.Np, M, Nc, C, ldc,
-                                                                       g.symmetric);
+        const dim3 grid((unsigned)((Nc + 255) / 256), (unsigned)std::min<int64_t>(M, 65535));
+        oz_reduce_kernel<<<grid, 256, 0, s>>>(p.part, g.splits, g.Mp, g.Np, M, Nc, C, ldc, g.symmetric,
+                                              subtract ? 1 : 0);
         CHFSI_LAUNCH_CHECK();
     }
     return CHFSI_OK;
@@ -1529,7 +1548,7 @@ size_t ozaki_workspace_bytes(bool tn_form, int64_t M, int64_t Nc, int64_t K, boo
 
 int ozaki_gemm_tn(const double* A, int64_t lda, const double* B, int64_t ldb, int64_t K, int64_t M, int64_t Nc,
                   double* C, int64_t ldc, bool symmetric, void* ws, size_t ws_bytes, unsigned* status,
-                  cudaStream_t s) {
+                  cudaStream_t s, bool subtract) {
     if (M <= 0 || Nc <= 0) return CHFSI_OK;
     // the same operand twice (a Gram matrix) is sliced once; `symmetric` says that the
     // product is known to be symmetric (a Gram matrix, or X^T (H X) for symmetric H):
@@ -1543,7 +1562,7 @@ int ozaki_gemm_tn(const double* A, int64_t lda, const double* B, int64_t ldb, in
     int rc;
     if ((rc = oz_prepare(A, lda, true, p.A, K, 0, status, s))) return rc;
     if (!same && (rc = oz_prepare(B, ldb, true, p.B, K, 0, status, s))) return rc;
-    return oz_run(p, true, C, ldc, M, Nc, symmetric, false, status, s);
+    return oz_run(p, true, C, ldc, M, Nc, symmetric, false, status, s, 1, 0, subtract);
 }
 
 int ozaki_gemm_nn(const double* A, int64_t lda, const double* B, int64_t ldb, int64_t M, int64_t K, int64_t Nc,

@@ -1062,14 +1062,6 @@ void eigh_layout(Ar& ar, int64_t n, EighBufs* out) {
     if (out) *out = u;
 }
 
-// Z[i][c] -= D[i][c] (rows x cols; Z with leading dimension ldz, D dense).
-__global__ void sub_block_kernel(double* Z, int64_t ldz, const double* __restrict__ D, int64_t rows, int64_t cols) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= rows * cols) return;
-    const int64_t i = idx / cols, c = idx % cols;
-    Z[i * ldz + c] -= D[idx];
-}
-
 struct CountOnly {
     Sizer s;
     template <typename T>
@@ -1149,11 +1141,9 @@ int eigh(double* A, int64_t lda, int64_t n, double* w, double* Q, int64_t ldq, v
             double* C22 = A + jn * lda + jn;
             int rc;
             if (oz && mp >= kOzakiMinN) {
-                if ((rc = ozaki_gemm_tn(Vop, n, Wop, n, 2 * kPanel32, mp, mp, mb.G, mp, true, u.oz, u.oz_bytes, status,
-                                        s)))
+                if ((rc = ozaki_gemm_tn(Vop, n, Wop, n, 2 * kPanel32, mp, mp, C22, lda, true, u.oz, u.oz_bytes, status,
+                                        s, true)))
                     return rc;
-                sub_block_kernel<<<(unsigned)((mp * mp + 255) / 256), 256, 0, s>>>(C22, lda, mb.G, mp, mp);
-                CHFSI_LAUNCH_CHECK();
             } else if ((rc = gemm_general(Vop, n, true, Wop, n, C22, lda, mp, mp, 2 * kPanel32, -1.0, true, s))) {
                 return rc;
             }
@@ -1249,12 +1239,11 @@ int eigh(double* A, int64_t lda, int64_t n, double* w, double* Q, int64_t ldq, v
         double* ZR = Q + (j0 + 1) * ldq;
         int rc;
         if (oz) {
-            // W1 = V^T Z, W2 = T W1 (small, DFMA), Z -= V W2 through a product block
+            // W1 = V^T Z, W2 = T W1 (small, DFMA), Z -= V W2
             if ((rc = ozaki_gemm_nn(Vp, mr, ZR, ldq, nb, mr, n, W1, n, false, u.oz, u.oz_bytes, status, s))) return rc;
             if ((rc = gemm_general(Tp, nb, false, W1, n, W2, n, nb, n, nb, 1.0, false, s))) return rc;
-            if ((rc = ozaki_gemm_tn(Vp, mr, W2, n, nb, mr, n, mb.G, n, false, u.oz, u.oz_bytes, status, s))) return rc;
-            sub_block_kernel<<<(unsigned)((mr * n + 255) / 256), 256, 0, s>>>(ZR, ldq, mb.G, mr, n);
-            CHFSI_LAUNCH_CHECK();
+            if ((rc = ozaki_gemm_tn(Vp, mr, W2, n, nb, mr, n, ZR, ldq, false, u.oz, u.oz_bytes, status, s, true)))
+                return rc;
         } else {
             if ((rc = gemm_general(Vp, mr, false, ZR, ldq, W1, n, nb, n, mr, 1.0, false, s))) return rc;
             if ((rc = gemm_general(Tp, nb, false, W1, n, W2, n, nb, n, nb, 1.0, false, s))) return rc;

@@ -107,10 +107,10 @@ int gemm_general(const double* A, int64_t lda, bool a_t, const double* B, int64_
 int gemm_merges(const double* G, const double* U, double* Gn, int64_t k, int64_t n, int nm, const double* kn,
                 int kn_stride, cudaStream_t s);
 // In place: upper Cholesky S = R^T R (R in the upper triangle, lower zeroed).
-// With oz_ws and scratch (at least (n - 64)^2 doubles) the trailing updates of 256 rows
-// and more run as Ozaki products on the tensor cores.
+// With oz_ws the trailing updates of 256 rows and more run as Ozaki products on the tensor
+// cores.
 int cholesky_upper(double* S, int64_t n, int64_t lds, unsigned* status, cudaStream_t s, void* oz_ws = nullptr,
-                   size_t oz_bytes = 0, double* scratch = nullptr);
+                   size_t oz_bytes = 0);
 // X (n x n) = R^-1 for upper-triangular R, zeros below the diagonal: 64 x 64 diagonal blocks,
 // then products for the off-diagonal blocks (Ozaki products from 256 rows on when oz_ws is
 // given); tmp: n x n doubles (ldt >= n).
@@ -147,13 +147,14 @@ int eigh(double* A, int64_t lda, int64_t n, double* w, double* Q, int64_t ldq, v
 
 // FP64-accurate products on the BF16 tensor cores (Ozaki-scheme slices, dense_ozaki.cu).
 // tn form: C (M x Nc) = A^T B with A: K x M (lda), B: K x Nc (ldb); symmetric: the
-// product is known to be symmetric (M == Nc), only the upper tiles are computed.
+// product is known to be symmetric (M == Nc), only the upper tiles are computed;
+// subtract: C -= A^T B.
 // nn form: C (M x Nc) = A B with A: M x K (lda), B: K x Nc (ldb); b_upper: B is upper
 // triangular.  Scratch from ws (ozaki_workspace_bytes; same = the tn form's A is B).
 size_t ozaki_workspace_bytes(bool tn_form, int64_t M, int64_t Nc, int64_t K, bool same);
 int ozaki_gemm_tn(const double* A, int64_t lda, const double* B, int64_t ldb, int64_t K, int64_t M, int64_t Nc,
                   double* C, int64_t ldc, bool symmetric, void* ws, size_t ws_bytes, unsigned* status,
-                  cudaStream_t s);
+                  cudaStream_t s, bool subtract = false);
 int ozaki_gemm_nn(const double* A, int64_t lda, const double* B, int64_t ldb, int64_t M, int64_t K, int64_t Nc,
                   double* C, int64_t ldc, bool b_upper, void* ws, size_t ws_bytes, unsigned* status,
                   cudaStream_t s);
