@@ -28,7 +28,7 @@ namespace chfsi {
 
 namespace {
 
-constexpr int kWarps = 8;            // rows (warps) per CTA
+constexpr int kWarps = 8;            // rows (warps) per CTA, at most
 constexpr int kThreads = kWarps * 32;
 
 template <typename A, typename T> __device__ __forceinline__ A cvt(T x);
@@ -193,8 +193,9 @@ csr_step_body(int64_t N, const int64_t* __restrict__ row_ptr, const int32_t* __r
     int32_t* s_col = reinterpret_cast<int32_t*>(smem_raw + sizeof(TH) * (size_t)cap);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t r0 = (int64_t)blockIdx.x * kWarps;
-    const int64_t r_end = (r0 + kWarps < N) ? r0 + kWarps : N;
+    const int warps = blockDim.x >> 5, threads = blockDim.x;
+    const int64_t r0 = (int64_t)blockIdx.x * warps;
+    const int64_t r_end = (r0 + warps < N) ? r0 + warps : N;
 
     auto clampp = [&](int64_t p) { return p < 0 ? (int64_t)0 : (p > nnz ? nnz : p); };
     const int64_t p_lo = clampp(row_ptr[r0]);
@@ -204,10 +205,10 @@ csr_step_body(int64_t N, const int64_t* __restrict__ row_ptr, const int32_t* __r
     bool bad = false;
 
     if (staged) {
-        for (int64_t q = threadIdx.x; q < cnt; q += kThreads) stage_entry(s_val + q, s_col + q, val, col, p_lo + q);
+        for (int64_t q = threadIdx.x; q < cnt; q += threads) stage_entry(s_val + q, s_col + q, val, col, p_lo + q);
         cp_async_wait_all();
         __syncthreads();
-        for (int64_t q = threadIdx.x; q < cnt; q += kThreads) {
+        for (int64_t q = threadIdx.x; q < cnt; q += threads) {
             if ((uint64_t)(uint32_t)s_col[q] >= (uint64_t)N || s_col[q] < 0) {
                 s_col[q] = 0;
                 s_val[q] = (TH)0;
@@ -227,6 +228,90 @@ csr_step_body(int64_t N, const int64_t* __restrict__ row_ptr, const int32_t* __r
         const int len = (int)(re - rb);
         bool nonfinite = false;
 
+        // The output of VV columns from j on, from their sums.
+        auto finish = [&](int64_t j, auto& acc) {
+            constexpr int VV = sizeof(acc) / sizeof(acc[0]);
+            ACC yc[VV], out[VV];
+            ldv<ACC, TC, VV>(Yc + r * ldc + j, yc);
+            if (Yp) {
+                ACC yp[VV];
+                ldv<ACC, TP, VV>(Yp + r * ldp + j, yp);
+#pragma unroll
+                for (int v = 0; v < VV; v++) out[v] = fma(-beta, yp[v], alpha * fma(-c, yc[v], acc[v]));
+            } else {
+#pragma unroll
+                for (int v = 0; v < VV; v++) out[v] = alpha * fma(-c, yc[v], acc[v]);
+            }
+#pragma unroll
+            for (int v = 0; v < VV; v++) nonfinite |= !isfinite(out[v]);
+            stv<ACC, TO, VV>(Yo + r * ldo + j, out);
+            if constexpr (kShadow) stv<ACC, __nv_bfloat16, VV>(Ys + r * lds + j, out);
+        };
+        if constexpr (std::is_same<ACC, double>::value) {
+            // FP64: bound by the pipe, on which an instruction takes the same time whatever its
+            // active lanes, so that the last columns are matched to the warp: W lanes a row
+            // entry, 32 / W entries at once (their sums added at the end), VV columns a lane.
+            // Entries are accumulated in their stored order when W = 32.  Two alternating
+            // buffers: the gathers of the next entry are in flight while one is accumulated; a
+            // bad column index (unstaged rows only) becomes a zero entry on row 0.
+            auto pass = [&](auto vv, auto ww, int64_t jbase) {
+                constexpr int VV = decltype(vv)::value, W = decltype(ww)::value, kGroups = 32 / W;
+                using G = Gathered<ACC, TG, VV>;
+                const int g = lane / W;
+                const int64_t j = jbase + (int64_t)(lane % W) * VV;
+                const bool on = j < n;
+                ACC acc[VV];
+#pragma unroll
+                for (int v = 0; v < VV; v++) acc[v] = (ACC)0;
+                if (Ya && on && g == 0) ldv<double, double, VV>(Ya + r * lda + j, acc);
+                auto fetch = [&](int t, G& y, ACC& h) {
+                    const int q = t * kGroups + g;
+                    h = (ACC)0;
+                    y.zero();
+                    if (kGroups > 1 && q >= len) return;
+                    int32_t cj = hc[q];
+                    h = cvt<ACC>(hv[q]);
+                    if (!staged && (cj < 0 || (int64_t)cj >= N)) { bad = true; cj = 0; h = (ACC)0; }
+                    if (on) y.load(Yg + (int64_t)cj * ldg + j);
+                };
+                const int steps = (len + kGroups - 1) / kGroups;
+                G ya, yb;
+                ACC ha = (ACC)0, hb = (ACC)0;
+                if (steps > 0) fetch(0, ya, ha);
+                int t = 0;
+                for (; t + 1 < steps; t += 2) {
+                    fetch(t + 1, yb, hb);
+                    ya.madd(ha, acc);
+                    if (t + 2 < steps) fetch(t + 2, ya, ha);
+                    yb.madd(hb, acc);
+                }
+                if (t < steps) ya.madd(ha, acc);
+#pragma unroll
+                for (int o = W; o < 32; o <<= 1)
+#pragma unroll
+                    for (int v = 0; v < VV; v++) acc[v] += __shfl_xor_sync(0xffffffffu, acc[v], o);
+                if (on && g == 0) finish(j, acc);
+            };
+            using std::integral_constant;
+            // FP64 instructions an entry: 2 for 64 columns, 1 for 32, 1/2 for 16, 1/4 for 8
+            int64_t j = 0;
+            while (j < n) {
+                const int64_t rest = n - j;
+                if (V == 2 && rest > 48) {
+                    pass(integral_constant<int, V>{}, integral_constant<int, 32>{}, j);
+                    j += 32 * V;
+                } else if (rest > 16) {
+                    pass(integral_constant<int, 1>{}, integral_constant<int, 32>{}, j);
+                    j += 32;
+                } else if (rest > 8) {
+                    pass(integral_constant<int, 1>{}, integral_constant<int, 16>{}, j);
+                    j += 16;
+                } else {
+                    pass(integral_constant<int, 1>{}, integral_constant<int, 8>{}, j);
+                    j += 8;
+                }
+            }
+        } else {
         for (int64_t jbase = 0; jbase < n; jbase += 32 * V * U) {
             ACC acc[U][V];
             bool on[U];
@@ -236,16 +321,12 @@ csr_step_body(int64_t N, const int64_t* __restrict__ row_ptr, const int32_t* __r
                 on[u] = jbase + (int64_t)(u * 32 + lane) * V < n;
 #pragma unroll
                 for (int v = 0; v < V; v++) acc[u][v] = (ACC)0;
-                if constexpr (std::is_same<ACC, double>::value) {
-                    if (Ya && on[u]) ldv<double, double, V>(Ya + r * lda + j0 + u * 32 * V, acc[u]);
-                }
             }
             // Register pipeline with two alternating buffers: the gathers of entry q+1
             // are in flight while entry q is accumulated.  Full chunks take a
             // predicate-free path; a bad column index (unstaged rows only) becomes a
-            // zero entry on row 0.  In the low-precision steps the common case (a
-            // staged slice and a full chunk) is compiled as its own loop with no
-            // per-entry checks; the FP64 step, bound by its pipe, keeps one loop.
+            // zero entry on row 0.  The common case (a staged slice and a full chunk) is
+            // compiled as its own loop with no per-entry checks.
             const bool full = jbase + 32 * V * U <= n;
             using G = Gathered<ACC, TG, V>;
             auto pass = [&](auto fast_tag) {
@@ -277,32 +358,14 @@ csr_step_body(int64_t N, const int64_t* __restrict__ row_ptr, const int32_t* __r
                 }
                 if (q < len) accumulate(ya, ha);
             };
-            if constexpr (std::is_same<ACC, double>::value) {
-                pass(std::false_type{});
-            } else {
-                if (staged && full) pass(std::true_type{});
-                else pass(std::false_type{});
-            }
+            if (staged && full) pass(std::true_type{});
+            else pass(std::false_type{});
 #pragma unroll
             for (int u = 0; u < U; u++) {
                 if (!on[u]) continue;
-                const int64_t j = j0 + u * 32 * V;
-                ACC yc[V], out[V];
-                ldv<ACC, TC, V>(Yc + r * ldc + j, yc);
-                if (Yp) {
-                    ACC yp[V];
-                    ldv<ACC, TP, V>(Yp + r * ldp + j, yp);
-#pragma unroll
-                    for (int v = 0; v < V; v++) out[v] = fma(-beta, yp[v], alpha * fma(-c, yc[v], acc[u][v]));
-                } else {
-#pragma unroll
-                    for (int v = 0; v < V; v++) out[v] = alpha * fma(-c, yc[v], acc[u][v]);
-                }
-#pragma unroll
-                for (int v = 0; v < V; v++) nonfinite |= !isfinite(out[v]);
-                stv<ACC, TO, V>(Yo + r * ldo + j, out);
-                if constexpr (kShadow) stv<ACC, __nv_bfloat16, V>(Ys + r * lds + j, out);
+                finish(j0 + u * 32 * V, acc[u]);
             }
+        }
         }
         if (__any_sync(0xffffffffu, nonfinite) && lane == 0) raise_status(status, DEV_NONFINITE);
     }
@@ -349,6 +412,13 @@ int launch(const CsrDev& h, const void* hval, int64_t n, const StepIO& io, doubl
         int64_t want = (kWarps * mean * 5 / 4 + 127) / 128 * 128;
         cap = (int)(want < 256 ? 256 : (want > kCapMax ? kCapMax : want));
     }
+    // FP64 on few rows: 4 rows a CTA, for an even share of them on every SM (1728 rows: 432
+    // CTAs, at most 3 an SM, where 216 of 8 rows gave some SMs twice the rows of others)
+    int warps = kWarps;
+    if (std::is_same<ACC, double>::value && h.N < 152 * 8 * kWarps) {
+        warps = kWarps / 2;
+        cap = kCapMax / 2;
+    }
     const size_t smem = (sizeof(TH) + sizeof(int32_t)) * (size_t)cap;
     const size_t smem_max = (sizeof(TH) + sizeof(int32_t)) * (size_t)kCapMax;
     auto kern = [] {
@@ -362,8 +432,8 @@ int launch(const CsrDev& h, const void* hval, int64_t n, const StepIO& io, doubl
         CHFSI_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
         attr_set[dev] = true;
     }
-    const int64_t blocks = (h.N + kWarps - 1) / kWarps;
-    kern<<<(unsigned)blocks, kThreads, smem, s>>>(
+    const int64_t blocks = (h.N + warps - 1) / warps;
+    kern<<<(unsigned)blocks, 32 * warps, smem, s>>>(
         h.N, h.row_ptr, h.col, static_cast<const TH*>(hval), h.nnz, n,
         static_cast<const TG*>(io.gather), io.ldg, static_cast<const TC*>(io.cur), io.ldc,
         static_cast<const TP*>(io.prev), io.ldp, static_cast<TO*>(io.out), io.ldo,

@@ -47,7 +47,7 @@ __device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
 // Y blocks row-major in the pair-split layout with leading dimension ld (in elements,
 // even).  Each lane owns 2 consecutive states (one float4); U chunks per pass.
 template <int U>
-__global__ void __launch_bounds__(kThreads, (U >= 4 ? 2 : 3))
+__global__ void __launch_bounds__(kThreads, (U >= 3 ? 2 : 3))
 csr_step_f32x2_kernel(int64_t N, const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                       const float2* __restrict__ val, int64_t nnz, int64_t n, const float2* __restrict__ Yc,
                       int64_t ldc, const float2* __restrict__ Yp, int64_t ldp, float2* __restrict__ Yo, int64_t ldo,
@@ -254,26 +254,27 @@ int csr_step_f32x2(const CsrDev& h, int64_t n, const void* Yc, int64_t ldc, cons
     if (cap < 256) cap = 256;
     if (cap > kCapMax) cap = kCapMax;
     const size_t smem = (sizeof(float2) + sizeof(int32_t)) * (size_t)cap;
-    static bool attr[kMaxDevices] = {};
+    // Chunks of 64 states per pass: at most 4, and so that the passes are of nearly the same
+    // number -- a pass does its U chunks' work whether there are states for them or not (301
+    // states: 3 + 3 chunks, where passes of 4 took twice as long as one; 64: one chunk).
+    const int64_t chunks = (n + 63) / 64, passes = (chunks + 3) / 4;
+    auto kern = csr_step_f32x2_kernel<4>;
+    const int per = (int)((chunks + passes - 1) / passes);
+    if (per == 3) kern = csr_step_f32x2_kernel<3>;
+    else if (per == 2) kern = csr_step_f32x2_kernel<2>;
+    else if (per == 1) kern = csr_step_f32x2_kernel<1>;
+    static bool attr[kMaxDevices][5] = {};
     const int dev = current_device();
     if (dev < 0) return CHFSI_ERR_CUDA;
-    if (!attr[dev]) {
-        CHFSI_CUDA_TRY(cudaFuncSetAttribute(csr_step_f32x2_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (!attr[dev][per]) {
+        CHFSI_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             (int)((sizeof(float2) + sizeof(int32_t)) * kCapMax)));
-        CHFSI_CUDA_TRY(cudaFuncSetAttribute(csr_step_f32x2_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)((sizeof(float2) + sizeof(int32_t)) * kCapMax)));
-        attr[dev] = true;
+        attr[dev][per] = true;
     }
     const int64_t blocks = (h.N + kWarps - 1) / kWarps;
-    // 4 chunks of 64 states per pass when n fills them, else 2
-    if (n >= 256)
-        csr_step_f32x2_kernel<4><<<(unsigned)blocks, kThreads, smem, s>>>(
-            h.N, h.row_ptr, h.col, static_cast<const float2*>(h.val), h.nnz, n, static_cast<const float2*>(Yc), ldc,
-            static_cast<const float2*>(Yp), ldp, static_cast<float2*>(Yo), ldo, alpha, c, beta, (int)cap, status);
-    else
-        csr_step_f32x2_kernel<2><<<(unsigned)blocks, kThreads, smem, s>>>(
-            h.N, h.row_ptr, h.col, static_cast<const float2*>(h.val), h.nnz, n, static_cast<const float2*>(Yc), ldc,
-            static_cast<const float2*>(Yp), ldp, static_cast<float2*>(Yo), ldo, alpha, c, beta, (int)cap, status);
+    kern<<<(unsigned)blocks, kThreads, smem, s>>>(
+        h.N, h.row_ptr, h.col, static_cast<const float2*>(h.val), h.nnz, n, static_cast<const float2*>(Yc), ldc,
+        static_cast<const float2*>(Yp), ldp, static_cast<float2*>(Yo), ldo, alpha, c, beta, (int)cap, status);
     CHFSI_LAUNCH_CHECK();
     return CHFSI_OK;
 }
