@@ -14,8 +14,11 @@ namespace chfsi {
 
 namespace {
 
-constexpr int kRowsPerBlock = 8;     // SpMV: one warp per row
-constexpr int kChunk = 2048;         // vector kernels: rows per block
+constexpr int kRowsPerWarp = 4;      // SpMV: rows whose sums a warp adds up together
+constexpr int kRowsPerBlock = 8 * kRowsPerWarp;
+constexpr int kChunk = 512;          // vector kernels: rows per block, two a thread (2048 left 120 SMs
+                                     // of 152 idle at N = 64000)
+constexpr int kUnroll = 4;           // SpMV: entries in flight per lane
 constexpr int kMaxSteps = 64;
 
 // scal layout
@@ -43,7 +46,11 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
     return t;   // valid on thread 0
 }
 
-// w = H v ; part[b] = sum over the block's rows of v[r] w[r]
+// w = H v ; part[b] = sum over the block's rows of v[r] w[r].  A warp takes four rows, their
+// entries strided over the lanes with kUnroll in flight a lane (the column index, then the
+// gather, are dependent reads), and adds up the four rows' lane sums together: six
+// FP64 additions a lane where row by row took twenty, half of the FP64 pipe's time on rows of
+// 300 entries (83 -> 64 us at 19.2 M entries; reading them takes 34).
 __global__ void __launch_bounds__(256) spmv_dot_kernel(int64_t N, const int64_t* __restrict__ row_ptr,
                                                        const int32_t* __restrict__ col,
                                                        const double* __restrict__ val, int64_t nnz,
@@ -52,104 +59,176 @@ __global__ void __launch_bounds__(256) spmv_dot_kernel(int64_t N, const int64_t*
     if (scal[S_STOP] != 0.0) return;
     __shared__ double rowdot[kRowsPerBlock];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t r = (int64_t)blockIdx.x * kRowsPerBlock + warp;
-    double d = 0.0;
-    if (r < N) {
-        int64_t b = row_ptr[r], e = row_ptr[r + 1];
+    const int64_t r0 = (int64_t)blockIdx.x * kRowsPerBlock + warp * kRowsPerWarp;
+    int64_t ptr = lane <= kRowsPerWarp && r0 + lane <= N ? row_ptr[r0 + lane] : 0;
+    double s[kRowsPerWarp];
+    bool bad = false;
+#pragma unroll
+    for (int q = 0; q < kRowsPerWarp; q++) {
+        s[q] = 0.0;
+        if (r0 + q >= N) continue;
+        int64_t b = __shfl_sync(0xffffffffu, ptr, q), e = __shfl_sync(0xffffffffu, ptr, q + 1);
         if (b < 0) b = 0;
         if (e > nnz) e = nnz;
-        double s = 0.0;
-        bool bad = false;
-        for (int64_t p = b + lane; p < e; p += 32) {
-            int32_t c = col[p];
-            if (c < 0 || (int64_t)c >= N) { bad = true; continue; }
-            s = fma(val[p], v[c], s);
-        }
+        for (int64_t p = b + lane; p < e; p += 32 * kUnroll) {
+            int32_t c[kUnroll];
+            double h[kUnroll], x[kUnroll];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (__any_sync(0xffffffffu, bad) && lane == 0) raise_status(status, DEV_PATTERN);
-        if (lane == 0) {
-            w[r] = s;
-            d = v[r] * s;
+            for (int u = 0; u < kUnroll; u++) {
+                const bool in = p + 32 * u < e;
+                c[u] = in ? col[p + 32 * u] : 0;
+                h[u] = in ? val[p + 32 * u] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < kUnroll; u++) {
+                const bool out = c[u] < 0 || (int64_t)c[u] >= N;
+                bad |= out;
+                x[u] = out ? 0.0 : v[c[u]];
+                if (out) h[u] = 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < kUnroll; u++)
+                if (p + 32 * u < e) s[q] = fma(h[u], x[u], s[q]);
         }
     }
-    if (lane == 0) rowdot[warp] = d;
+    // lanes 8 q .. 8 q + 7 end with the sum of row q
+    const bool up16 = lane & 16, up8 = lane & 8;
+    double t0 = up16 ? s[2] : s[0], t1 = up16 ? s[3] : s[1];
+    t0 += __shfl_xor_sync(0xffffffffu, up16 ? s[0] : s[2], 16);
+    t1 += __shfl_xor_sync(0xffffffffu, up16 ? s[1] : s[3], 16);
+    double t = up8 ? t1 : t0;
+    t += __shfl_xor_sync(0xffffffffu, up8 ? t0 : t1, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (__any_sync(0xffffffffu, bad) && lane == 0) raise_status(status, DEV_PATTERN);
+    const int64_t r = r0 + lane / 8;
+    if ((lane & 7) == 0) {
+        double d = 0.0;
+        if (r < N) {
+            w[r] = t;
+            d = v[r] * t;
+        }
+        rowdot[warp * kRowsPerWarp + lane / 8] = d;
+    }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int i = 0; i < kRowsPerBlock; i++) t += rowdot[i];
-        part[blockIdx.x] = t;
+    if (warp == 0) {
+        double d = rowdot[lane];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+        if (lane == 0) part[blockIdx.x] = d;
     }
 }
 
-// out[idx] = sum_b part[b * stride + idx], one block per idx, fixed order.
-__global__ void __launch_bounds__(256) finalize_kernel(const double* part, int64_t nparts, int64_t stride,
-                                                       double* out, int mode, int j, double* scal) {
-    if (scal[S_STOP] != 0.0) return;
-    __shared__ double red[8];
-    const int idx = blockIdx.x;
+// The sum of nparts partial sums, on every thread: each block of the kernels below adds up
+// the parts that it needs itself, in the same order as every other (a launch of one block
+// for each of the three sums of a step took 6.5 us).
+__device__ __forceinline__ double sum_parts(const double* part, int64_t nparts, double* red) {
+    __shared__ double total;
     double s = 0.0;
-    for (int64_t b = threadIdx.x; b < nparts; b += blockDim.x) s += part[b * stride + idx];
-    double t = block_sum(s, red);
-    if (threadIdx.x != 0) return;
-    if (mode == 0) {                 // alpha_j
-        out[idx] = t;
-    } else if (mode == 1) {          // re-orthogonalisation coefficients h_i
-        out[idx] = t;
-    } else {                         // beta_j = |w|, breakdown test
-        double beta = sqrt(t);
-        double al = scal[S_ALPHA + j];
-        double scale = scal[S_SCALE];
-        double cand = fabs(al) + (j > 0 ? scal[S_BETA + j - 1] : 0.0);
-        if (cand > scale) scale = cand;
-        scal[S_SCALE] = scale;
-        scal[S_K] = (double)(j + 1);
-        if (beta <= 1e-12 * scale) {
-            scal[S_BETA + j] = 0.0;
-            scal[S_STOP] = 1.0;
-        } else {
-            scal[S_BETA + j] = beta;
-        }
-    }
+    for (int64_t b = threadIdx.x; b < nparts; b += blockDim.x) s += part[b];
+    const double t = block_sum(s, red);
+    if (threadIdx.x == 0) total = t;
+    __syncthreads();
+    return total;
 }
 
-// w -= alpha_j v_j + beta_{j-1} v_{j-1}; part[b*(j+1) + i] = <V_i, w> over the block's rows
+// alpha_j from the SpMV's parts; w -= alpha_j v_j + beta_{j-1} v_{j-1}; part[b*(j+1) + i] =
+// <V_i, w> over the block's rows
 __global__ void __launch_bounds__(256) three_term_dots_kernel(int64_t N, double* w, const double* V, int j,
-                                                              double* part, const double* scal) {
+                                                              const double* aparts, int64_t naparts, double* part,
+                                                              double* scal) {
     if (scal[S_STOP] != 0.0) return;
-    __shared__ double red[8];
+    __shared__ double red[8][kMaxSteps];
     const int64_t r0 = (int64_t)blockIdx.x * kChunk;
     const int64_t r1 = r0 + kChunk < N ? r0 + kChunk : N;
-    const double al = scal[S_ALPHA + j];
+    const double al = sum_parts(aparts, naparts, &red[0][0]);
+    if (blockIdx.x == 0 && threadIdx.x == 0) scal[S_ALPHA + j] = al;
     const double bp = j > 0 ? scal[S_BETA + j - 1] : 0.0;
     const double* vj = V + (int64_t)j * N;
     const double* vjm = j > 0 ? V + (int64_t)(j - 1) * N : nullptr;
-    for (int64_t r = r0 + threadIdx.x; r < r1; r += blockDim.x) {
-        double x = w[r] - al * vj[r];
-        if (vjm) x -= bp * vjm[r];
-        w[r] = x;
+    constexpr int kRows = kChunk / 256;
+    double x[kRows];
+#pragma unroll
+    for (int u = 0; u < kRows; u++) {
+        const int64_t r = r0 + threadIdx.x + 256 * u;
+        x[u] = 0.0;
+        if (r < r1) {
+            x[u] = w[r] - al * vj[r];
+            if (vjm) x[u] -= bp * vjm[r];
+            w[r] = x[u];
+        }
+    }
+    __syncthreads();   // red is free again
+    // four dots at a time; the warps' sums wait in shared memory for one barrier at the end (a
+    // block-wide sum per dot took 1.5 us each)
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int i0 = 0; i0 <= j; i0 += 4) {
+        double d[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            d[q] = 0.0;
+            if (i0 + q > j) continue;
+            const double* vi = V + (int64_t)(i0 + q) * N;
+#pragma unroll
+            for (int u = 0; u < kRows; u++) {
+                const int64_t r = r0 + threadIdx.x + 256 * u;
+                if (r < r1) d[q] = fma(vi[r], x[u], d[q]);
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < 4; q++) d[q] += __shfl_xor_sync(0xffffffffu, d[q], o);
+#pragma unroll
+        for (int q = 0; q < 4; q++)
+            if (lane == 0 && i0 + q <= j) red[warp][i0 + q] = d[q];
     }
     __syncthreads();
-    for (int i = 0; i <= j; i++) {
-        const double* vi = V + (int64_t)i * N;
-        double s = 0.0;
-        for (int64_t r = r0 + threadIdx.x; r < r1; r += blockDim.x) s = fma(vi[r], w[r], s);
-        double t = block_sum(s, red);
-        if (threadIdx.x == 0) part[(int64_t)blockIdx.x * (j + 1) + i] = t;
+    for (int i = threadIdx.x; i <= j; i += blockDim.x) {
+        double t = 0.0;
+        for (int q = 0; q < 8; q++) t += red[q][i];
+        part[(int64_t)blockIdx.x * (j + 1) + i] = t;
     }
 }
 
-// w -= sum_i h_i V_i ; part[b] = |w|^2 over the block's rows
+// h_i from the dots' parts (four threads a coefficient); w -= sum_i h_i V_i ; part[b] = |w|^2
+// over the block's rows
 __global__ void __launch_bounds__(256) reorth_norm_kernel(int64_t N, double* w, const double* V, int j,
-                                                          double* part, const double* scal) {
+                                                          const double* hparts, int64_t nparts, double* part,
+                                                          const double* scal) {
     if (scal[S_STOP] != 0.0) return;
-    __shared__ double red[8];
+    __shared__ double red[8], hs[kMaxSteps];
+    static_assert(4 * kMaxSteps <= 256, "four threads a coefficient");
+    {
+        const int i = threadIdx.x >> 2;
+        double h[4] = {0.0, 0.0, 0.0, 0.0};
+        if (i <= j) {
+            int64_t b = threadIdx.x & 3;
+            for (; b + 12 < nparts; b += 16)
+#pragma unroll
+                for (int q = 0; q < 4; q++) h[q] += hparts[(b + 4 * q) * (j + 1) + i];
+            for (; b < nparts; b += 4) h[0] += hparts[b * (j + 1) + i];
+        }
+        double t = (h[0] + h[1]) + (h[2] + h[3]);
+        t += __shfl_xor_sync(0xffffffffu, t, 1);
+        t += __shfl_xor_sync(0xffffffffu, t, 2);
+        if ((threadIdx.x & 3) == 0 && i <= j) hs[i] = t;
+    }
+    __syncthreads();
     const int64_t r0 = (int64_t)blockIdx.x * kChunk;
     const int64_t r1 = r0 + kChunk < N ? r0 + kChunk : N;
     double s = 0.0;
     for (int64_t r = r0 + threadIdx.x; r < r1; r += blockDim.x) {
         double x = w[r];
-        for (int i = 0; i <= j; i++) x -= scal[S_H + i] * V[(int64_t)i * N + r];
+        int i = 0;
+        for (; i + 4 <= j + 1; i += 4) {       // four reads in flight
+            double v[4];
+#pragma unroll
+            for (int q = 0; q < 4; q++) v[q] = V[(int64_t)(i + q) * N + r];
+#pragma unroll
+            for (int q = 0; q < 4; q++) x -= hs[i + q] * v[q];
+        }
+        for (; i <= j; i++) x -= hs[i] * V[(int64_t)i * N + r];
         w[r] = x;
         s = fma(x, x, s);
     }
@@ -157,12 +236,26 @@ __global__ void __launch_bounds__(256) reorth_norm_kernel(int64_t N, double* w, 
     if (threadIdx.x == 0) part[blockIdx.x] = t;
 }
 
-// v_{j+1} = w / beta_j
-__global__ void scale_next_kernel(int64_t N, const double* w, double* V, int j, const double* scal) {
+// beta_j = |w| from the parts, breakdown test; v_{j+1} = w / beta_j
+__global__ void __launch_bounds__(256) scale_next_kernel(int64_t N, const double* w, double* V, int j,
+                                                         const double* part, int64_t nparts, double* scal) {
     if (scal[S_STOP] != 0.0) return;
-    int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= N) return;
-    V[(int64_t)(j + 1) * N + r] = w[r] / scal[S_BETA + j];
+    __shared__ double red[8];
+    const double beta = sqrt(sum_parts(part, nparts, red));
+    // every block comes to the same scale, whether block 0 has stored it yet or not
+    const double cand = fabs(scal[S_ALPHA + j]) + (j > 0 ? scal[S_BETA + j - 1] : 0.0);
+    const double scale = fmax(*(const volatile double*)&scal[S_SCALE], cand);
+    const bool stop = beta <= 1e-12 * scale;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        scal[S_SCALE] = scale;
+        scal[S_K] = (double)(j + 1);
+        scal[S_BETA + j] = stop ? 0.0 : beta;
+        if (stop) scal[S_STOP] = 1.0;
+    }
+    if (stop) return;
+    const int64_t r0 = (int64_t)blockIdx.x * kChunk;
+    const int64_t r1 = r0 + kChunk < N ? r0 + kChunk : N;
+    for (int64_t r = r0 + threadIdx.x; r < r1; r += blockDim.x) V[(int64_t)(j + 1) * N + r] = w[r] / beta;
 }
 
 // v_0 = v0 / |v0| (norm from part sums, fixed order)
@@ -176,6 +269,7 @@ __global__ void __launch_bounds__(256) sq_part_kernel(int64_t N, const double* v
     if (threadIdx.x == 0) part[blockIdx.x] = t;
 }
 
+// A chunk of rows per block; every block sums the parts in the same order.
 __global__ void __launch_bounds__(256) norm0_kernel(int64_t N, const double* v0, double* V, const double* part,
                                                     int64_t nparts, double* scal) {
     __shared__ double red[8];
@@ -185,12 +279,16 @@ __global__ void __launch_bounds__(256) norm0_kernel(int64_t N, const double* v0,
     double t = block_sum(s, red);
     if (threadIdx.x == 0) {
         nrm = sqrt(t);
-        for (int i = 0; i < S_TOTAL; i++) scal[i] = 0.0;
-        if (!(nrm > 0.0) || !isfinite(nrm)) scal[S_STOP] = 2.0;   // unusable start vector
+        if (blockIdx.x == 0) {
+            for (int i = 0; i < S_TOTAL; i++) scal[i] = 0.0;
+            if (!(nrm > 0.0) || !isfinite(nrm)) scal[S_STOP] = 2.0;   // unusable start vector
+        }
     }
     __syncthreads();
-    if (scal[S_STOP] != 0.0) return;
-    for (int64_t r = threadIdx.x; r < N; r += blockDim.x) V[r] = v0[r] / nrm;
+    if (!(nrm > 0.0) || !isfinite(nrm)) return;
+    const int64_t r0 = (int64_t)blockIdx.x * kChunk;
+    const int64_t r1 = r0 + kChunk < N ? r0 + kChunk : N;
+    for (int64_t r = r0 + threadIdx.x; r < r1; r += blockDim.x) V[r] = v0[r] / nrm;
 }
 
 // Number of eigenvalues of the symmetric tridiagonal (d, e) that are < x.
@@ -237,9 +335,9 @@ __device__ double sturm_edge(const double* d, const double* e, int k, double a, 
     return 0.5 * (a + b);
 }
 
-// Smallest and largest eigenvalue of T_k by multisection (one warp), then the bounds.
+// Smallest and largest eigenvalue of T_k by multisection (one warp each), then the bounds.
 __global__ void bounds_kernel(const double* scal, int64_t N, int64_t n_wanted, double* out) {
-    if (blockIdx.x != 0 || threadIdx.x >= 32) return;
+    __shared__ double theta[2];
     if (scal[S_STOP] == 2.0) {
         if (threadIdx.x == 0) out[0] = out[1] = out[2] = nan("");
         return;
@@ -256,9 +354,12 @@ __global__ void bounds_kernel(const double* scal, int64_t N, int64_t n_wanted, d
     double span = hi - lo;
     lo -= 1e-12 * (span + 1.0);
     hi += 1e-12 * (span + 1.0);
-    const double theta_min = sturm_edge(d, e, k, lo, hi, 1);
-    const double theta_max = sturm_edge(d, e, k, lo, hi, k);
+    const int end = threadIdx.x >> 5;
+    const double edge = sturm_edge(d, e, k, lo, hi, end == 0 ? 1 : k);
+    if ((threadIdx.x & 31) == 0) theta[end] = edge;
+    __syncthreads();
     if (threadIdx.x != 0) return;
+    const double theta_min = theta[0], theta_max = theta[1];
     const double resid = fabs(e[k - 1]);
     const double a0 = theta_min;
     const double bb = theta_max + resid;
@@ -270,11 +371,15 @@ __global__ void bounds_kernel(const double* scal, int64_t N, int64_t n_wanted, d
 
 }  // namespace
 
+// Two sets of parts: the SpMV's (or the norms'), and the dots'.
+static size_t lanczos_first_parts(int64_t N) {
+    const int64_t spmv_blocks = (N + kRowsPerBlock - 1) / kRowsPerBlock, chunks = (N + kChunk - 1) / kChunk;
+    return (size_t)((spmv_blocks > chunks ? spmv_blocks : chunks) + 1);
+}
+
 size_t lanczos_part_count(int64_t N, int steps) {
-    int64_t spmv_blocks = (N + kRowsPerBlock - 1) / kRowsPerBlock;
-    int64_t chunks = (N + kChunk - 1) / kChunk;
-    int64_t a = chunks * (steps + 1);
-    return (size_t)(spmv_blocks > a ? spmv_blocks : a) + S_TOTAL;
+    const int64_t chunks = (N + kChunk - 1) / kChunk;
+    return lanczos_first_parts(N) + (size_t)(chunks * (steps + 1)) + S_TOTAL;
 }
 
 int lanczos_run(const CsrDev& h, int steps, const double* v0, int64_t n_wanted, double* V, double* w,
@@ -286,29 +391,24 @@ int lanczos_run(const CsrDev& h, int steps, const double* v0, int64_t n_wanted, 
     const int64_t chunks = (N + kChunk - 1) / kChunk;
     const int64_t spmv_blocks = (N + kRowsPerBlock - 1) / kRowsPerBlock;
 
+    double* part2 = part + lanczos_first_parts(N);
     sq_part_kernel<<<(unsigned)chunks, 256, 0, s>>>(N, v0, part);
     CHFSI_LAUNCH_CHECK();
-    norm0_kernel<<<1, 256, 0, s>>>(N, v0, V, part, chunks, scal);
+    norm0_kernel<<<(unsigned)chunks, 256, 0, s>>>(N, v0, V, part, chunks, scal);
     CHFSI_LAUNCH_CHECK();
     for (int j = 0; j < k; j++) {
         const double* vj = V + (int64_t)j * N;
         spmv_dot_kernel<<<(unsigned)spmv_blocks, 256, 0, s>>>(N, h.row_ptr, h.col, val, h.nnz, vj, w, part,
                                                               scal, status);
         CHFSI_LAUNCH_CHECK();
-        finalize_kernel<<<1, 256, 0, s>>>(part, spmv_blocks, 1, scal + S_ALPHA + j, 0, j, scal);
+        three_term_dots_kernel<<<(unsigned)chunks, 256, 0, s>>>(N, w, V, j, part, spmv_blocks, part2, scal);
         CHFSI_LAUNCH_CHECK();
-        three_term_dots_kernel<<<(unsigned)chunks, 256, 0, s>>>(N, w, V, j, part, scal);
+        reorth_norm_kernel<<<(unsigned)chunks, 256, 0, s>>>(N, w, V, j, part2, chunks, part, scal);
         CHFSI_LAUNCH_CHECK();
-        finalize_kernel<<<j + 1, 256, 0, s>>>(part, chunks, j + 1, scal + S_H, 1, j, scal);
-        CHFSI_LAUNCH_CHECK();
-        reorth_norm_kernel<<<(unsigned)chunks, 256, 0, s>>>(N, w, V, j, part, scal);
-        CHFSI_LAUNCH_CHECK();
-        finalize_kernel<<<1, 256, 0, s>>>(part, chunks, 1, nullptr, 2, j, scal);
-        CHFSI_LAUNCH_CHECK();
-        scale_next_kernel<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(N, w, V, j, scal);
+        scale_next_kernel<<<(unsigned)chunks, 256, 0, s>>>(N, w, V, j, part, chunks, scal);
         CHFSI_LAUNCH_CHECK();
     }
-    bounds_kernel<<<1, 32, 0, s>>>(scal, N, n_wanted, dev_out);
+    bounds_kernel<<<1, 64, 0, s>>>(scal, N, n_wanted, dev_out);
     CHFSI_LAUNCH_CHECK();
     return CHFSI_OK;
 }
