@@ -440,7 +440,7 @@ int filter_columns(const FilterRun& R, const double* X, int64_t ldx, double* Y, 
             const int slices = R.prec && R.prec[k - 1] == CHFSI_F40_OZAKI ? 5 : 7;
             rc = ozaki_bsr_step(R.bsr64, n, static_cast<const double*>(io.cur), io.ldc,
                                 static_cast<const double*>(io.prev), io.ldp, static_cast<double*>(io.out), io.ldo,
-                                al[k], c, k >= 2 ? be[k] : 0.0, fl.oz, fl.oz_bytes, st, s, slices);
+                                al[k], c, k >= 2 ? be[k] : 0.0, fl.oz, fl.oz_bytes, st, s, slices, k - L - 1);
         } else if (H->kind == CHFSI_SPLIT) {
             // dense diagonal blocks on the tensor cores, then the sparse rest with that sum added
             rc = ozaki_blockdiag_apply(static_cast<const double*>(io.cur), io.ldc, N, H->split.block, n, fl.T, ldw,

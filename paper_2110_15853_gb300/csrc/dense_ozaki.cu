@@ -54,10 +54,10 @@
 //
 // What bounds it: the tensor pipe, at 908 cycles per K = 16 of the 28 slice products (their
 // work is 896) when nothing else runs on the SM; about 1150 in the filter step, since
-// the warps share the issue slots with the drains' conversions (6 of 61 ms) and a
+// the warps share the issue slots with the drains' conversions (6 of 60 ms) and a
 // drained group's MMAs come in narrower pieces.  20 FP64-accurate steps at 40^3, w = 3, 1024
-// states: 98.0 -> 61.4 ms (0.83 of the chunks, and 1.35 x the rate); 20 40-bit and 4
-// FP64-accurate steps at 48^3, w = 4, 1500 states: 266 -> 164 ms.
+// states: 98.0 -> 60.0 ms (0.83 of the chunks, and 1.35 x the rate); 20 40-bit and 4
+// FP64-accurate steps at 48^3, w = 4, 1500 states: 266 -> 161 ms.
 #include <algorithm>
 #include <type_traits>
 
@@ -239,6 +239,7 @@ struct OzArgs {
     const double* Yprev;      // nullptr: no beta term
     int64_t ldprev;
     double alpha, cshift, beta;
+    int* expNext;             // largest exponent field of each state of Y_out (zeroed before)
 };
 
 constexpr int kUnfolded = 1 << 30;
@@ -733,7 +734,8 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(const __grid_const
         // element take 8200 cycles an item at least and wait for Y_prev; done by the epilogue
         // warps (at once, or in pieces between the drains) they kept the drains and so
         // the MMAs waiting for a fifth of the time, and no registers or shared memory are left
-        // to hold an item's products for later, but L2 is.
+        // to hold an item's products for later, but L2 is.  They also leave the exponents that the
+        // next step's slices need (a pass over Y_out otherwise: 75 us of 3.1 ms at 40^3 x 1024).
         int n = 0;
         bool ok = true;
         for (int64_t item = blockIdx.x; ok && item < total; item += gridDim.x, n++) {
@@ -750,6 +752,7 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(const __grid_const
                 double* out = g.C + i0 * g.ldc + j;
                 const double* prev = g.Yprev ? g.Yprev + i0 * g.ldprev + j : nullptr;
                 double d[2][kStep], p[2][kStep];
+                int emax = 0;
                 auto load = [&](int b, int r) {
 #pragma unroll
                     for (int c = 0; c < kStep; c++) {
@@ -768,10 +771,13 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(const __grid_const
                         if (it.unfolded) D = fma(-g.cshift, g.Ycur[(i0 + r + c) * g.ldcur + j], D);
                         double y = g.alpha * D;
                         if (prev) y = fma(-g.beta, p[b][c], y);
-                        nonfinite |= (__double2hiint(y) & 0x7ff00000) == 0x7ff00000;
+                        const int ef = (__double2hiint(y) >> 20) & 0x7ff;
+                        emax = ef > emax ? ef : emax;
                         out[(r + c) * g.ldc] = y;
                     }
                 }
+                nonfinite |= emax == 0x7ff;
+                if (emax) atomicMax(g.expNext + j, emax);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&dempty[n & 1]);
@@ -1141,23 +1147,26 @@ int launch_slices(const double* src, int64_t ld, const OzOperand& o, int64_t Kto
     return CHFSI_OK;
 }
 
-// Exponents and digit planes of an operand; batch b reads src + b * src_bstride over
+// Exponents (unless have_exps) and digit planes of an operand; batch b reads src + b * src_bstride over
 // min(o.K, Ktot - b o.K) of the K dimension.  nplanes: digit planes written.
 int oz_prepare(const double* src, int64_t ld, bool trans, const OzOperand& o, int64_t Ktot, int64_t src_bstride,
-               unsigned* status, cudaStream_t s, int nplanes = kSlices) {
-    CHFSI_CUDA_TRY(cudaMemsetAsync(o.exps, 0, sizeof(int) * (size_t)o.padded_rows(), s));
+               unsigned* status, cudaStream_t s, int nplanes = kSlices, bool have_exps = false) {
     const int64_t brows = o.tiles * o.tile_rows;
-    if (trans) {
+    if (!have_exps) CHFSI_CUDA_TRY(cudaMemsetAsync(o.exps, 0, sizeof(int) * (size_t)o.padded_rows(), s));
+    if (have_exps) {
+        // the exponents are there (left by the step that made src)
+    } else if (trans) {
         const int span = exponent_span(o.K);
         dim3 grid((unsigned)((o.rows + 255) / 256), (unsigned)((o.K + span - 1) / span), (unsigned)o.nbatch);
         oz_exponents_kernel<true><<<grid, 256, 0, s>>>(src, ld, o.rows, o.K, Ktot, src_bstride, brows, span, o.exps,
                                                       status);
+        CHFSI_LAUNCH_CHECK();
     } else {
         dim3 grid((unsigned)((o.rows * 32 + 255) / 256), 1, (unsigned)o.nbatch);
         oz_exponents_kernel<false><<<grid, 256, 0, s>>>(src, ld, o.rows, o.K, Ktot, src_bstride, brows, 0, o.exps,
                                                        status);
+        CHFSI_LAUNCH_CHECK();
     }
-    CHFSI_LAUNCH_CHECK();
     if (o.tile_rows == kTileM)
         return trans ? launch_slices<true, kTileM>(src, ld, o, Ktot, src_bstride, nplanes, s)
                      : launch_slices<false, kTileM>(src, ld, o, Ktot, src_bstride, nplanes, s);
@@ -1335,6 +1344,7 @@ void oz_blockdiag_layout(Ar& ar, int64_t N, int B, int64_t n, OzBlockDiag* out) 
 // products of all its chunks share it.
 struct OzBsr {
     OzOperand Y;
+    int* exps[2] = {nullptr, nullptr};   // exponents of Y_cur and of the step's output, alternating
     unsigned char* H = nullptr;
     int32_t *chunk = nullptr, *count = nullptr;
     int* expH = nullptr;      // per grid row
@@ -1348,6 +1358,8 @@ void oz_bsr_layout(Ar& ar, int64_t nbr, int64_t nblocks, int64_t n, OzBsr* out) 
     b.chunk = ar.template take<int32_t>(stored);
     b.count = ar.template take<int32_t>((size_t)nbr);
     oz_operand_layout(ar, n, nbr * 64, 1, kTileM, &b.Y);
+    b.exps[0] = b.Y.exps;
+    b.exps[1] = ar.template take<int>((size_t)b.Y.padded_rows());
     b.expH = ar.template take<int>((size_t)(nbr * 64));
     if (out) *out = b;
 }
@@ -1493,7 +1505,7 @@ int ozaki_bsr_prepare(const BsrDev& h, int64_t n, double c, void* ws, size_t ws_
 
 int ozaki_bsr_step(const BsrDev& h, int64_t n, const double* Yc, int64_t ldc, const double* Yp, int64_t ldp,
                    double* Yo, int64_t ldo, double alpha, double c, double beta, void* ws, size_t ws_bytes,
-                   unsigned* status, cudaStream_t s, int slices) {
+                   unsigned* status, cudaStream_t s, int slices, int pass) {
     if (slices != 7 && slices != 5) return CHFSI_ERR_ARG;
     if (n <= 0 || h.nbr <= 0) return CHFSI_OK;
     if (ws_bytes < ozaki_bsr_bytes(h.nbr, h.nblocks, n)) return CHFSI_ERR_NOMEM;
@@ -1502,7 +1514,10 @@ int ozaki_bsr_step(const BsrDev& h, int64_t n, const double* Yc, int64_t ldc, co
     oz_bsr_layout(ar, h.nbr, h.nblocks, n, &b);
     const int64_t N = h.nbr * 64;
     int rc;
-    if ((rc = oz_prepare(Yc, ldc, true, b.Y, N, 0, status, s, slices))) return rc;
+    b.Y.exps = b.exps[pass & 1];
+    int* next = b.exps[(pass + 1) & 1];
+    if ((rc = oz_prepare(Yc, ldc, true, b.Y, N, 0, status, s, slices, pass > 0))) return rc;
+    CHFSI_CUDA_TRY(cudaMemsetAsync(next, 0, sizeof(int) * (size_t)b.Y.padded_rows(), s));
     OzArgs g{};
     g.A = b.Y.slices;
     g.B = b.H;
@@ -1537,6 +1552,7 @@ int ozaki_bsr_step(const BsrDev& h, int64_t n, const double* Yc, int64_t ldc, co
     g.alpha = alpha;
     g.cshift = c;
     g.beta = beta;
+    g.expNext = next;
     return launch_oz(g, CUtensorMap{}, g.pairs, s);
 }
 

@@ -167,12 +167,13 @@ int ozaki_gemm_nn(const double* A, int64_t lda, const double* B, int64_t ldb, in
 // iterates.  ozaki_bsr_prepare slices H once (rows of at most 128 blocks);
 // ozaki_bsr_step slices Y_cur and runs the step.  Both use one workspace (ozaki_bsr_bytes).
 // slices = 7: FP64-accurate; slices = 5: the 40-bit step (five digits per operand, the
-// 15 slice pairs of weight 2^-48 and above).
+// 15 slice pairs of weight 2^-48 and above).  pass: number of the step among consecutive
+// ones on one workspace, each reading the output of the one before (0: Y_cur is new).
 size_t ozaki_bsr_bytes(int64_t nbr, int64_t nblocks, int64_t n);
 int ozaki_bsr_prepare(const BsrDev& h, int64_t n, double c, void* ws, size_t ws_bytes, unsigned* status, cudaStream_t s);
 int ozaki_bsr_step(const BsrDev& h, int64_t n, const double* Yc, int64_t ldc, const double* Yp, int64_t ldp,
                    double* Yo, int64_t ldo, double alpha, double c, double beta, void* ws, size_t ws_bytes,
-                   unsigned* status, cudaStream_t s, int slices = 7);
+                   unsigned* status, cudaStream_t s, int slices = 7, int pass = 0);
 size_t ozaki_blockdiag_bytes(int64_t N, int B, int64_t n);
 int ozaki_blockdiag_prepare(const double* diag, int64_t N, int B, int64_t n, void* ws, size_t ws_bytes,
                             unsigned* status, cudaStream_t s);

@@ -1,7 +1,7 @@
 // Spectral bounds for Algorithm 1 (Sec. 3.4 takes eps_0, eps_ub^w, eps_ub^uw as
 // inputs without saying how they are found): k-step Lanczos with full
 // re-orthogonalisation on the GPU, then the extreme eigenvalues of the k x k
-// tridiagonal T_k by Sturm-sequence bisection in a one-thread kernel.
+// tridiagonal T_k by Sturm counts, a warp for each end and 32 points a round.
 //
 // Every scalar (alpha_j, beta_j, the re-orthogonalisation coefficients, the stop
 // flag) stays in device memory, so the k steps queue without host round trips.
