@@ -124,3 +124,41 @@ def test_closure_cholesky_blocks_and_inverse_levels(P, oracle_mod, n, precision)
     p = psi.cpu().numpy()
     assert np.max(np.abs(ritz.cpu().numpy() - theta)) <= 1e-10 * np.max(np.abs(theta))
     assert np.max(np.abs(p.T @ p - np.eye(n))) <= 1e-12
+
+
+@pytest.mark.parametrize("n", [1, 7, 8, 9, 16, 17, 24, 31, 33, 40, 47, 48, 49, 56, 64, 65, 104, 120, 193, 257, 301, 321])
+@pytest.mark.parametrize("schedule", [None, "f32x2"])
+def test_csr_steps_last_columns(P, oracle_mod, n, schedule):
+    """State counts whose last columns take each width of the FP64 step (64, 32, 16 and 8
+    columns, entries shared by groups of lanes) and each number of chunks per pass of the
+    two-float step, on rows of 0 to 40 entries (empty and single-entry rows among them)."""
+    rng = np.random.default_rng(n)
+    N, m = 75, 3
+    A = np.where(rng.random((N, N)) < rng.random((N, 1)) * 0.6, rng.standard_normal((N, N)), 0.0)
+    A[::13] = 0.0
+    A[5, :] = 0.0
+    A[5, 70] = 1.5
+    H = dense_to_csr(A / 10, keep_zeros=False)
+    X = rng.standard_normal((N, n))
+    a, b, a0 = 0.5, 2.0, -2.0
+    Hd = P.CsrMatrix.from_arrays(H["row_ptr"], H["col"], H["val"], device="cuda")
+    ws = P.Workspace("cuda")
+    Y = P.filter(Hd, _dev(X), m, a, b, a0, schedule=None if schedule is None else [schedule] * m, workspace=ws)
+    assert P.read_status(ws) == 0
+    assert rel_fro(Y.cpu().numpy(), oracle_mod.filter(H, X, m, a, b, a0)) <= 1e-12
+
+
+@pytest.mark.parametrize("N", [2, 3, 5, 31, 33, 63, 130, 511, 513, 1100])
+def test_lanczos_rows_per_warp_and_chunks(P, oracle_mod, N):
+    """Row counts around the four rows of a warp, the 32 of a block and the 512 of a vector
+    chunk, with rows of very different lengths."""
+    rng = np.random.default_rng(N)
+    A = np.where(rng.random((N, N)) < rng.random((N, 1)), rng.standard_normal((N, N)), 0.0)
+    A = (A + A.T) / 2 + np.diag(np.linspace(1.0, 5.0, N))
+    H = dense_to_csr(A, keep_zeros=False)
+    v0 = rng.standard_normal(N)
+    Hd = P.CsrMatrix.from_arrays(H["row_ptr"], H["col"], H["val"], device="cuda")
+    got = P.lanczos_bounds(Hd, _dev(v0), 12, 1)
+    want = oracle_mod.lanczos_bounds(H, v0, 12, 1)
+    scale = max(abs(x) for x in want)
+    assert max(abs(g - w) for g, w in zip(got, want)) <= 1e-10 * scale
