@@ -254,12 +254,12 @@ csr_step_body(int64_t N, const int64_t* __restrict__ row_ptr, const int32_t* __r
             // Entries are accumulated in their stored order when W = 32.  Two alternating
             // buffers: the gathers of the next entry are in flight while one is accumulated; a
             // bad column index (unstaged rows only) becomes a zero entry on row 0.
-            auto pass = [&](auto vv, auto ww, int64_t jbase) {
+            auto pass = [&](auto vv, auto ww, auto full, int64_t jbase) {
                 constexpr int VV = decltype(vv)::value, W = decltype(ww)::value, kGroups = 32 / W;
                 using G = Gathered<ACC, TG, VV>;
                 const int g = lane / W;
                 const int64_t j = jbase + (int64_t)(lane % W) * VV;
-                const bool on = j < n;
+                const bool on = decltype(full)::value || j < n;
                 ACC acc[VV];
 #pragma unroll
                 for (int v = 0; v < VV; v++) acc[v] = (ACC)0;
@@ -294,20 +294,25 @@ csr_step_body(int64_t N, const int64_t* __restrict__ row_ptr, const int32_t* __r
             };
             using std::integral_constant;
             // FP64 instructions an entry: 2 for 64 columns, 1 for 32, 1/2 for 16, 1/4 for 8
+            // (all 64 columns there: a pass of its own, without the lane test, which made the
+            // compiler spill; 52.55 -> 52.38 ms, 16 steps at 32^3 x 512)
             int64_t j = 0;
             while (j < n) {
                 const int64_t rest = n - j;
-                if (V == 2 && rest > 48) {
-                    pass(integral_constant<int, V>{}, integral_constant<int, 32>{}, j);
+                if (V == 2 && rest >= 64) {
+                    pass(integral_constant<int, V>{}, integral_constant<int, 32>{}, std::true_type{}, j);
+                    j += 32 * V;
+                } else if (V == 2 && rest > 48) {
+                    pass(integral_constant<int, V>{}, integral_constant<int, 32>{}, std::false_type{}, j);
                     j += 32 * V;
                 } else if (rest > 16) {
-                    pass(integral_constant<int, 1>{}, integral_constant<int, 32>{}, j);
+                    pass(integral_constant<int, 1>{}, integral_constant<int, 32>{}, std::false_type{}, j);
                     j += 32;
                 } else if (rest > 8) {
-                    pass(integral_constant<int, 1>{}, integral_constant<int, 16>{}, j);
+                    pass(integral_constant<int, 1>{}, integral_constant<int, 16>{}, std::false_type{}, j);
                     j += 16;
                 } else {
-                    pass(integral_constant<int, 1>{}, integral_constant<int, 8>{}, j);
+                    pass(integral_constant<int, 1>{}, integral_constant<int, 8>{}, std::false_type{}, j);
                     j += 8;
                 }
             }
