@@ -680,7 +680,7 @@ def ozaki_whole_step(P, torch, dev, stream, wl, H, Xd, Yref, theta_ref, bounds, 
         res = dict(schedule=f"{sched.count('ozaki40')} x ozaki40 + {sched.count('ozaki')} x ozaki",
                    filter_ms=t_f, filter_gflops=fl / (t_f * 1e-3) / 1e9,
                    filter_speedup_vs_f64=line["phases"]["filter_ms"] / t_f,
-                   slice_product_tflops=slice_products(sched) * 2.0 * nblocks * 4096 * n / (t_f * 1e-3) / 1e12,
+                   stored_block_slice_tflops=slice_products(sched) * 2.0 * nblocks * 4096 * n / (t_f * 1e-3) / 1e12,
                    y_rel_fro_err_vs_f64=y_err, status=status, closure_ms=t_c, ms=t_step,
                    speedup_vs_f64_step=line["phases"]["whole_step_ms"] / t_step,
                    host_layout_seconds_untimed=host_s, **_ritz_errors(th.cpu().numpy(), theta_ref, a))
@@ -896,7 +896,7 @@ def ozaki_bsr_variant(P, torch, dev, stream, Bd, Xp, Yb, m, a, b, a0, fl, nblock
                 lambda: P.filter(Bd, Xp, m, a, b, a0, schedule=sched, out=Yb, workspace=ws), reps=1)
     n = Xp.shape[1]
     return dict(ms=t, ms_per_step=t / m, gflops=fl / (t * 1e-3) / 1e9, speedup_vs_f64=t_f64 / t,
-                slice_product_tflops=slice_products(sched) * 2.0 * nblocks * 4096 * n / (t * 1e-3) / 1e12,
+                stored_block_slice_tflops=slice_products(sched) * 2.0 * nblocks * 4096 * n / (t * 1e-3) / 1e12,
                 status=P.read_status(ws), y_rel_fro_err_vs_f64=err_vs_ref(), **ritz_err())
 
 
