@@ -388,6 +388,15 @@ __global__ void dc_split_kernel(int64_t n, double* d, const double* e, double* e
     }
 }
 
+// Key of the order in which eigenvalues are ranked: that of the reals, -0 with 0, and every
+// NaN last, so that the ranks (ties by index) are a permutation whatever the values.
+// Integer instructions, off the FP64 pipe.
+__device__ __forceinline__ long long order_key(double x) {
+    const long long b = __double_as_longlong(x), mag = b & 0x7fffffffffffffffll;
+    if (mag > 0x7ff0000000000000ll) return 0x7fffffffffffffffll;
+    return b < 0 ? -mag : mag;
+}
+
 // Leaf eigenproblems by parallel (round-robin ordered) Jacobi; one block per leaf.
 // Writes ascending eigenvalues to w[l ..] and the eigenvectors into the diagonal block
 // Q[l.., l..] (the rest of Q is zero).
@@ -472,10 +481,10 @@ __global__ void __launch_bounds__(256) dc_leaf_kernel(int64_t n, const double* d
     // ascending order of the s real eigenvalues (the padding rows never mix with them)
     if (threadIdx.x < s) {
         const int i = threadIdx.x;
-        const double li = A[i][i];
+        const long long li = order_key(A[i][i]);
         int r = 0;
         for (int j = 0; j < s; j++) {
-            const double lj = A[j][j];
+            const long long lj = order_key(A[j][j]);
             r += (lj < li) || (lj == li && j < i);
         }
         rank[i] = r;
@@ -525,9 +534,14 @@ __device__ __forceinline__ Merge merge_at(int64_t half, int64_t n, MergeBufs& b)
 // place in the merged order by a binary search in the other half; the poles that stay are
 // numbered by a block-wide count.  Only when two neighbouring ones are close enough for a
 // rotation does one thread walk through them (the walk alone took 115 us a merge).
+// The places are a permutation, and perm a list of valid columns, only because both halves
+// are sorted numbers.  Where a pole, a weight or rho is not finite, or a half is not sorted
+// (after input that was not finite or a panel that gave up), the poles keep their
+// own order, all deflated, and the status word says so: nothing indexes with what
+// the workspace happened to hold.
 __global__ void __launch_bounds__(1024) dc_merge_prep_kernel(int64_t half, int64_t n, const double* w,
                                                              const double* Q, int64_t ldq, const double* ebak,
-                                                             MergeBufs b) {
+                                                             MergeBufs b, unsigned* status) {
     __shared__ int wcount[32], total;
     __shared__ double wmax[32];
     const Merge g = merge_at(half, n, b);
@@ -537,9 +551,11 @@ __global__ void __launch_bounds__(1024) dc_merge_prep_kernel(int64_t half, int64
     const double rho0 = ebak[m - 1];
     const double sg = rho0 >= 0.0 ? 1.0 : -1.0;
     double zz = 0.0, dmax = 0.0;
+    bool bad = !isfinite(rho0);
     for (int p = threadIdx.x; p < k; p += blockDim.x) {
         const double zp = p < n1 ? Q[(m - 1) * ldq + l + p] : Q[m * ldq + m + (p - n1)];
         const double d = sg * w[l + p];
+        bad |= !isfinite(zp) || !isfinite(d) || (p != 0 && p != n1 && !(w[l + p - 1] <= w[l + p]));
         b.z[p] = zp;
         b.D[p] = d;
         dmax = fmax(dmax, fabs(d));
@@ -554,6 +570,22 @@ __global__ void __launch_bounds__(1024) dc_merge_prep_kernel(int64_t half, int64
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
     const double rho_hat = fabs(rho0) * zz;
+    if (__syncthreads_or(bad)) {
+        for (int p = threadIdx.x; p < k; p += blockDim.x) {
+            b.perm[p] = p;
+            b.val[p] = b.D[p];
+            b.defl[p] = 1;
+            b.pos[p] = -1;
+        }
+        if (threadIdx.x == 0) {
+            b.par[0] = rho_hat;
+            b.par[1] = sg;
+            b.par[2] = 0.0;
+            b.par[3] = 0.0;
+            raise_status(status, DEV_NONFINITE);
+        }
+        return;
+    }
     const double zs = 1.0 / sqrt(zz > 0.0 ? zz : 1.0);
     // merged order of the two sorted halves (ascending when sg > 0, descending otherwise):
     // entry t of a half goes behind the entries of the other half that come before it (those
@@ -875,10 +907,10 @@ __global__ void __launch_bounds__(32 * kRootWarps) dc_rank2_kernel(int64_t half,
     const int lane = threadIdx.x & 31;
     const int64_t p = (int64_t)blockIdx.x * kRootWarps + (threadIdx.x >> 5);
     if (p >= k) return;
-    const double vp = b.D[p];
+    const long long vp = order_key(b.D[p]);
     int r = 0;
     for (int64_t q = lane; q < k; q += 32) {
-        const double vq = b.D[q];
+        const long long vq = order_key(b.D[q]);
         r += (vq < vp) || (vq == vp && q < p);
     }
 #pragma unroll
@@ -1165,7 +1197,7 @@ int eigh(double* A, int64_t lda, int64_t n, double* w, double* Q, int64_t ldq, v
         const unsigned nm = (unsigned)((n - half + 2 * half - 1) / (2 * half));
         const int64_t k = std::min(2 * half, n);      // the largest of them
         const unsigned kb = (unsigned)((k + 255) / 256);
-        dc_merge_prep_kernel<<<dim3(1, 1, nm), 1024, 0, s>>>(half, n, w, Q, ldq, ebak, mb);
+        dc_merge_prep_kernel<<<dim3(1, 1, nm), 1024, 0, s>>>(half, n, w, Q, ldq, ebak, mb, status);
         CHFSI_LAUNCH_CHECK();
         dc_rotate_kernel<<<dim3(kb, 1, nm), 256, 0, s>>>(half, n, Q, ldq, mb);
         CHFSI_LAUNCH_CHECK();
