@@ -55,6 +55,45 @@ __device__ double block_sum(double v) {
     return total;
 }
 
+// ------------------------------------------------------------------ 0. scale
+
+// The largest exponent field of A's entries (zeroed before) and, from it, the power of two
+// that takes the largest entry into [1/2, 1).  The solver works on that matrix, so that
+// products and squares of its rows neither overflow nor vanish for any finite A, and
+// kNegligible below is a fixed number.  An entry that is not finite is reported here.
+__global__ void __launch_bounds__(256) matrix_exponent_kernel(const double* __restrict__ A, int64_t lda, int64_t n,
+                                                              int* emax, unsigned* status) {
+    int m = 0;
+    for (int64_t r = blockIdx.x; r < n; r += gridDim.x)
+        for (int64_t c = threadIdx.x; c < n; c += blockDim.x) {
+            const int e = (__double2hiint(A[r * lda + c]) >> 20) & 0x7ff;
+            m = e > m ? e : m;
+        }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) {
+        if (m) atomicMax(emax, m);
+        if (m == 0x7ff) raise_status(status, DEV_NONFINITE);
+    }
+}
+
+// e of the scale 2^-e (0 where A is zero, subnormal throughout or not finite).
+__device__ __forceinline__ int scale_exponent(const int* emax) { return *emax == 0 || *emax == 0x7ff ? 0 : *emax - 1022; }
+
+// A *= 2^-e (exact unless the result is subnormal).
+__global__ void __launch_bounds__(256) scale_matrix_kernel(double* A, int64_t lda, int64_t n, const int* emax) {
+    const int e = scale_exponent(emax);
+    if (e == 0) return;
+    const double f = scalbn(1.0, -e);      // 2^-1024 (subnormal) .. 2^1021
+    for (int64_t r = blockIdx.x; r < n; r += gridDim.x)
+        for (int64_t c = threadIdx.x; c < n; c += blockDim.x) A[r * lda + c] *= f;
+}
+
+// w *= 2^e.
+__global__ void unscale_kernel(double* w, int64_t n, const int* emax) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) w[i] = scalbn(w[i], scale_exponent(emax));
+}
+
 // ------------------------------------------------------------------ 1. tridiagonalisation
 
 // A panel reduces kPanel32 columns j0 .. j0 + 31 against the trailing matrix as it stood at
@@ -85,10 +124,15 @@ constexpr int64_t kTriStaged = 20000;   // x in shared memory up to this n
 // a barrier that gave up, after which later panels do nothing.
 struct TriScalars {
     unsigned count, gave_up;
+    int emax;                    // largest exponent field of A
 };
 
+// A rest of x below 1e-140 of A's largest entry (in [1/2, 1)) is left out: with the squares of
+// scale = 1 / (x_0 - beta) below, a smaller one would overflow.
+constexpr double kNegligible = 1e-280;
+
 __device__ __forceinline__ void reflector(double x0, double sumsq, double& beta, double& t, double& scale) {
-    if (sumsq == 0.0) {
+    if (sumsq <= kNegligible) {
         beta = x0;
         t = 0.0;
         scale = 0.0;
@@ -1123,6 +1167,13 @@ int eigh(double* A, int64_t lda, int64_t n, double* w, double* Q, int64_t ldq, v
     MergeBufs& mb = u.mb;
     const bool oz = u.oz != nullptr;
 
+    CHFSI_CUDA_TRY(cudaMemsetAsync(u.tri, 0, sizeof(TriScalars), s));
+    const unsigned rows = (unsigned)std::min<int64_t>(n, 4 * 1024);
+    matrix_exponent_kernel<<<rows, 256, 0, s>>>(A, lda, n, &u.tri->emax, status);
+    CHFSI_LAUNCH_CHECK();
+    scale_matrix_kernel<<<rows, 256, 0, s>>>(A, lda, n, &u.tri->emax);
+    CHFSI_LAUNCH_CHECK();
+
     // 1. tridiagonalisation: a cooperative launch per panel, then the trailing product
     if (n >= 3) {
         const int dev = current_device();
@@ -1150,7 +1201,6 @@ int eigh(double* A, int64_t lda, int64_t n, double* w, double* Q, int64_t ldq, v
                                                 (int)(sizeof(double) * (kTriStaged + 2))));
             attr[dev] = true;
         }
-        CHFSI_CUDA_TRY(cudaMemsetAsync(u.tri, 0, sizeof(TriScalars), s));
         for (int64_t j0 = 0; j0 + 2 < n; j0 += kPanel32) {
             const int nc = (int)std::min<int64_t>(kPanel32, (n - 2) - j0);
             if (nc < kPanel32)   // rows nc .. 31 of V and W take part in the trailing product
@@ -1252,6 +1302,9 @@ int eigh(double* A, int64_t lda, int64_t n, double* w, double* Q, int64_t ldq, v
         copy_block_kernel<<<cells, 256, 0, s>>>(half, n, Q, ldq, mb);
         CHFSI_LAUNCH_CHECK();
     }
+
+    unscale_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(w, n, &u.tri->emax);
+    CHFSI_LAUNCH_CHECK();
 
     // 3. back-transformation Q = H_0 H_1 ... H_{n-3} Q, panels from the last
     const int64_t nref = n - 2;   // reflectors j = 0 .. n - 3

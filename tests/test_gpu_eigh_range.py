@@ -1,7 +1,10 @@
-"""The dense eigensolver and the closure on input outside the ordinary: entries that are not
-finite.  The call must end with the status that include/chfsi.h names, touch no memory but
-its own, and leave the context and the workspace usable: a finite matrix on the same
-workspace is solved as by LAPACK afterwards."""
+"""The dense eigensolver and the closure on input outside the ordinary.
+
+Entries that are not finite: the call must end with the status that include/chfsi.h names,
+touch no memory but its own, and leave the context and the workspace usable (a finite matrix
+on the same workspace is solved as by LAPACK afterwards).  Entries near the ends of the FP64
+range, and couplings whose squares vanish: the tolerances of the ordinary matrices
+(eigenvalues, residuals and orthogonality to 1e-12), a power of two taken out first."""
 import ctypes
 
 import numpy as np
@@ -68,6 +71,40 @@ def test_eigh_of_a_matrix_that_is_not_finite(P, n, value, where):
     status, w, Q = solve(A)
     assert status == 0
     _check(A, w, Q)
+
+
+@pytest.mark.parametrize("n", [3, 12, 32, 40, 97, 300])
+@pytest.mark.parametrize("exponent", [-1000, -500, -350, 350, 500, 1000])
+def test_eigh_of_any_magnitude(P, n, exponent):
+    A = _symmetric(n, n)
+    status, w, Q = _Solver(P, n)(np.ldexp(A, exponent))
+    assert status == 0
+    _check(A, np.ldexp(w, -exponent), Q)
+
+
+@pytest.mark.parametrize("n", [12, 40, 66, 300])
+@pytest.mark.parametrize("coupling", [1e-130, 1e-145, 1e-156, 1e-158, 1e-161, 1e-165, 1e-200, 1e-310])
+def test_eigh_of_blocks_that_hardly_couple(P, n, coupling):
+    A, h = _symmetric(n, n), n // 2
+    A[:h, h:] *= coupling
+    A[h:, :h] *= coupling
+    status, w, Q = _Solver(P, n)(A)
+    assert status == 0
+    _check(A, w, Q)
+
+
+@pytest.mark.parametrize("n", [40, 300])
+@pytest.mark.parametrize("exponent", [-400, 400])
+def test_closure_of_an_operator_of_any_magnitude(P, n, exponent):
+    N = 400
+    A, Y = _symmetric(N, 3), np.random.default_rng(n).standard_normal((N, n))
+    h = dense_to_csr(np.ldexp(A, exponent))
+    Hd = P.CsrMatrix.from_arrays(h["row_ptr"], h["col"], h["val"], device="cuda")
+    ritz, psi = P.rayleigh_ritz(Hd, torch.as_tensor(Y).cuda(), 2)
+    p, Qy = psi.cpu().numpy(), np.linalg.qr(Y)[0]
+    ref = np.linalg.eigvalsh(Qy.T @ A @ Qy)
+    assert np.max(np.abs(np.ldexp(ritz.cpu().numpy(), -exponent) - ref)) <= 1e-10 * np.max(np.abs(ref))
+    assert np.max(np.abs(p.T @ p - np.eye(n))) <= 1e-12
 
 
 @pytest.mark.parametrize("n", [40, 96, 300])
