@@ -82,6 +82,29 @@ def test_eigh_of_any_magnitude(P, n, exponent):
     _check(A, np.ldexp(w, -exponent), Q)
 
 
+@pytest.mark.parametrize("n", [300, 600, 1500, 2100])
+@pytest.mark.parametrize("kind", ["random", "spread", "dominant"])
+@pytest.mark.parametrize("scale", [1e-8, 1.0, 13.0])
+def test_eigh_panel_updates_of_any_norm(P, n, kind, scale):
+    """The trailing updates on the tensor cores (256 rows and more) to the accuracy of FP64 ones,
+    whatever A's norm is against its entries: a random matrix (norm sqrt(n) entries), a
+    spectrum in [1, 3], and a matrix of ones with a random part of 1e-3 (norm n entries).
+    Residual within 4 eps sqrt(n) of |A|_F, the growth of the rounding errors of n
+    reflections."""
+    if kind == "spread":
+        Qr = np.linalg.qr(np.random.default_rng(n).standard_normal((n, n)))[0]
+        A = (Qr * np.linspace(1.0, 3.0, n)) @ Qr.T
+        A = (A + A.T) / 2
+    else:
+        A = _symmetric(n, n) if kind == "random" else 1.0 + 1e-3 * _symmetric(n, n)
+    status, w, Q = _Solver(P, n)(A * scale)
+    assert status == 0
+    A, eps = A * scale, np.finfo(float).eps
+    assert np.linalg.norm(A @ Q - Q * w) <= 4 * eps * np.sqrt(n) * np.linalg.norm(A)
+    assert np.max(np.abs(w - np.linalg.eigvalsh(A))) <= 4 * eps * np.sqrt(n) * np.linalg.norm(A)
+    assert np.max(np.abs(Q.T @ Q - np.eye(n))) <= 1e-12
+
+
 @pytest.mark.parametrize("n", [12, 40, 66, 300])
 @pytest.mark.parametrize("coupling", [1e-130, 1e-145, 1e-156, 1e-158, 1e-161, 1e-165, 1e-200, 1e-310])
 def test_eigh_of_blocks_that_hardly_couple(P, n, coupling):
