@@ -368,7 +368,9 @@ int chfsi_eigh_workspace_size(int64_t n, size_t* bytes);
  * overwritten.  Q must not overlap A.  The call synchronises `stream` once per merge
  * of the divide and conquer.  Workspace (chfsi_eigh_workspace_size): the status word
  * and about 3 n^2 + 200 n doubles.  Errors: CHFSI_ERR_ARG, CHFSI_ERR_NOMEM,
- * CHFSI_ERR_UNSUPPORTED (n above 65535), CHFSI_ERR_CUDA.
+ * CHFSI_ERR_UNSUPPORTED (n above 65535), CHFSI_ERR_CUDA; in the status word
+ * CHFSI_ERR_NONFINITE (an entry that is not finite) and CHFSI_ERR_TIMEOUT (a bounded wait
+ * that gave up), after which w and Q are undefined.
  */
 int chfsi_eigh(double* A, int64_t lda, int64_t n, double* w, double* Q, int64_t ldq, void* ws,
                size_t ws_bytes, void* stream);
@@ -421,13 +423,14 @@ int chfsi_measure_pipe_peak(int32_t precision, double* flops_per_second, void* s
 unsigned long long chfsi_kernel_launches(void);
 
 /*
- * Limit, in nanoseconds, of the mbarrier waits in which one role of a tensor-core
- * kernel (chfsi_filter's BF16 steps on a BSR or hybrid operator, chfsi_ozaki_gemm and
- * the products that use it) waits on another: a copy producer on a free stage, the
- * MMA issuer on a loaded stage or a drained accumulator, the epilogue on a finished
- * accumulator.  A wait that runs out makes its CTA stop, wait for its own copies and
- * MMAs in flight (those waits keep a fixed 1 s bound), free its tensor memory and exit;
- * the call's status word then holds CHFSI_ERR_TIMEOUT and its outputs are undefined.
+ * Limit, in nanoseconds, of the waits of one part of a kernel on another: the mbarrier
+ * waits between the roles of a tensor-core kernel (chfsi_filter's BF16 steps on a BSR or
+ * hybrid operator, chfsi_ozaki_gemm and the products that use it: a copy producer on a
+ * free stage, the MMA issuer on a loaded stage or a drained accumulator, the epilogue on
+ * a finished accumulator) and the grid barriers of the eigensolver's panels.  A wait that
+ * runs out makes its CTA stop, wait for its own copies and MMAs in flight (those waits
+ * keep a fixed 1 s bound), free its tensor memory and exit; the call's status word then
+ * holds CHFSI_ERR_TIMEOUT and its outputs are undefined.
  * 0 restores the default of 1 s.  Process-wide, read at each launch; meant for tests
  * of that abort path (a limit of a few nanoseconds makes the first wait that does not
  * succeed at once run out).  Diagnostics only: the paper has no counterpart.

@@ -392,7 +392,9 @@ def ozaki_gemm(A: torch.Tensor, B: torch.Tensor, transpose_a: bool = False, symm
 
 def eigh(A: torch.Tensor, workspace: Optional[Workspace] = None):
     """(w ascending, Q) of a symmetric FP64 CUDA matrix by the library's dense
-    eigensolver (chfsi_eigh); A is not modified (a copy is factorised)."""
+    eigensolver (chfsi_eigh); A is not modified (a copy is factorised).  Waits for the result
+    and raises ChfsiError if the device found a non-finite value or gave up a wait (in a
+    stream capture it does neither)."""
     if A.dtype != torch.float64 or A.dim() != 2 or A.shape[0] != A.shape[1] or not A.is_cuda:
         raise ValueError("A must be a square float64 CUDA matrix")
     n = A.shape[0]
@@ -403,8 +405,10 @@ def eigh(A: torch.Tensor, workspace: Optional[Workspace] = None):
     sz = ctypes.c_size_t(0)
     check(lib.chfsi_eigh_workspace_size(n, ctypes.byref(sz)), "chfsi_eigh_workspace_size")
     ws = (workspace or Workspace(A.device)).get(sz.value)
-    check(lib.chfsi_eigh(_ptr(work), n, n, _ptr(w), _ptr(Q), n, _ptr(ws), ws.numel(), _stream_handle(A.device)),
-          "chfsi_eigh")
+    stream = _stream_handle(A.device)
+    check(lib.chfsi_eigh(_ptr(work), n, n, _ptr(w), _ptr(Q), n, _ptr(ws), ws.numel(), stream), "chfsi_eigh")
+    if n > 0 and not torch.cuda.is_current_stream_capturing():
+        check(lib.chfsi_read_status(_ptr(ws), stream), "chfsi_eigh")
     return w, Q
 
 

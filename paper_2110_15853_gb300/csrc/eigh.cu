@@ -153,11 +153,15 @@ struct TriPanel {
     TriScalars* tri;
     int* vwmax;                  // largest exponent fields of the panel's V and of its W (zeroed before)
     unsigned base;               // count at the start of this launch
+    uint64_t wait_ns;            // limit of a barrier's wait
     unsigned* status;
 };
 
 // Arrive at grid barrier number `b` of this launch; wait for it (bounded: the launch is
 // cooperative, so every block is resident, but a wait that gives up is flagged, not endless).
+// After it the panels to come do nothing, d, e and tau keep the zeros that they start with
+// where no panel got to, and the call ends with the status.  The clock is read every 1024
+// polls, or at each one for limits below a millisecond.
 __device__ __forceinline__ void grid_arrive(const TriPanel& a) {
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -170,14 +174,15 @@ __device__ __forceinline__ bool grid_wait(const TriPanel& a, unsigned b) {
     if (threadIdx.x == 0) {
         const unsigned target = a.base + (b + 1) * gridDim.x;
         const volatile unsigned* c = &a.tri->count;
+        const unsigned mask = a.wait_ns < 1000000ull ? 0u : 1023u;
         uint64_t t0 = 0;
         ok = 1;
         for (unsigned polls = 1; (int)(*c - target) < 0; polls++) {
-            if ((polls & 1023u) == 0) {
+            if ((polls & mask) == 0) {
                 uint64_t t;
                 asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
                 if (t0 == 0) t0 = t;
-                else if (t - t0 > 1000000000ull) {
+                else if (t - t0 > a.wait_ns) {
                     a.tri->gave_up = 1;
                     raise_status(a.status, DEV_TIMEOUT);
                     ok = 0;
@@ -1122,14 +1127,14 @@ size_t eigh_ozaki_bytes(int64_t n) {
 template <typename Ar>
 void eigh_layout(Ar& ar, int64_t n, EighBufs* out) {
     EighBufs u{};
+    u.tri = ar.template take<TriScalars>(1);
+    u.vwmax = ar.template take<int>(2 * (size_t)(n / kPanel32 + 1));
     u.d = ar.template take<double>(n);
     u.e = ar.template take<double>(n);
     u.tau = ar.template take<double>(n);
     u.ebak = ar.template take<double>(n);
     u.part = ar.template take<double>(kMaxTriBlocks);
     u.dots = ar.template take<double>(2 * kPanel32);
-    u.tri = ar.template take<TriScalars>(1);
-    u.vwmax = ar.template take<int>(2 * (size_t)(n / kPanel32 + 1));
     u.PV = ar.template take<double>((size_t)(3 * kPanel32) * n);
     u.ybuf = ar.template take<double>(n);
     MergeBufs& b = u.mb;
@@ -1195,8 +1200,8 @@ int eigh(double* A, int64_t lda, int64_t n, double* w, double* Q, int64_t ldq, v
     MergeBufs& mb = u.mb;
     const bool oz = u.oz != nullptr;
 
-    // the scalars and, behind them, the panels' exponents
-    CHFSI_CUDA_TRY(cudaMemsetAsync(u.tri, 0, (size_t)((char*)(u.vwmax + 2 * (n / kPanel32 + 1)) - (char*)u.tri), s));
+    // the scalars and, behind them, the panels' exponents, d, e and tau
+    CHFSI_CUDA_TRY(cudaMemsetAsync(u.tri, 0, (size_t)((char*)(tau + n) - (char*)u.tri), s));
     const unsigned rows = (unsigned)std::min<int64_t>(n, 4 * 1024);
     matrix_exponent_kernel<<<rows, 256, 0, s>>>(A, lda, n, &u.tri->emax, status);
     CHFSI_LAUNCH_CHECK();
@@ -1223,6 +1228,7 @@ int eigh(double* A, int64_t lda, int64_t n, double* w, double* Q, int64_t ldq, v
         tp.e = e;
         tp.tau = tau;
         tp.tri = u.tri;
+        tp.wait_ns = pipeline_wait_ns();
         tp.status = status;
         static bool attr[kMaxDevices] = {};
         if (!attr[dev]) {

@@ -154,3 +154,39 @@ def test_closure_of_an_operator_or_a_block_that_is_not_finite(P, n, passes, valu
     Qy = np.linalg.qr(Y)[0]
     assert np.max(np.abs(th - np.linalg.eigvalsh(Qy.T @ A @ Qy))) <= 1e-10 * np.max(np.abs(th))
     assert np.max(np.abs(p.T @ p - np.eye(n))) <= (1e-12 if passes == 2 else 1e-9)
+
+
+@pytest.mark.parametrize("n", [100, 300, 700])
+def test_a_grid_barrier_that_gives_up(P, n):
+    """With a limit of a few nanoseconds the first barrier of a panel that is not complete at
+    once gives up: the status says so, in chfsi_eigh, in the binding and in the closure,
+    and the next call on the same workspace is right."""
+    from paper_2110_15853_gb300 import _abi
+    A, solve = _symmetric(n, n), _Solver(P, n)
+    h = dense_to_csr(_symmetric(800, 1))
+    Hd = P.CsrMatrix.from_arrays(h["row_ptr"], h["col"], h["val"], device="cuda")
+    Y = torch.as_tensor(np.random.default_rng(n).standard_normal((800, n))).cuda()
+    lib = P.load()
+    assert lib.chfsi_set_pipeline_wait_limit(4) == 0
+    try:
+        assert solve(A)[0] == _abi.CHFSI_ERR_TIMEOUT
+        for call in (lambda: P.eigh(torch.as_tensor(A).cuda()), lambda: P.rayleigh_ritz(Hd, Y, 2)):
+            with pytest.raises(P.ChfsiError) as e:
+                call()
+            assert e.value.code == _abi.CHFSI_ERR_TIMEOUT
+    finally:
+        assert lib.chfsi_set_pipeline_wait_limit(0) == 0
+    status, w, Q = solve(A)
+    assert status == 0
+    _check(A, w, Q)
+    w, Q = P.eigh(torch.as_tensor(A).cuda())
+    _check(A, w.cpu().numpy(), Q.cpu().numpy())
+
+
+def test_eigh_binding_raises_on_a_matrix_that_is_not_finite(P):
+    from paper_2110_15853_gb300 import _abi
+    A = _symmetric(20, 0)
+    A[3, 4] = A[4, 3] = np.nan
+    with pytest.raises(P.ChfsiError) as e:
+        P.eigh(torch.as_tensor(A).cuda())
+    assert e.value.code == _abi.CHFSI_ERR_NONFINITE
