@@ -1243,13 +1243,22 @@ int eigh(double* A, int64_t lda, int64_t n, double* w, double* Q, int64_t ldq, v
             // a warp per row of the product and its dots, at most one block per SM: fewer blocks
             // meet sooner at the barriers
             const int64_t rows = n - j0 - 1 + 2 * kPanel32;
-            const unsigned grid = (unsigned)std::min<int64_t>(sms, (rows + kTriWarps - 1) / kTriWarps);
+            unsigned grid = (unsigned)std::min<int64_t>(sms, (rows + kTriWarps - 1) / kTriWarps);
             tp.j0 = j0;
             tp.nc = nc;
             tp.vwmax = u.vwmax + 2 * (j0 / kPanel32);
             void* args[] = {&tp};
-            CHFSI_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)tri_panel_kernel, dim3(grid), dim3(kTriThreads),
-                                                       args, tp.staged ? sizeof(double) * (size_t)(n - j0 + 2) : 0, s));
+            // a stream whose context has fewer SMs than the device refuses a grid that cannot be
+            // resident; the kernel runs on any grid, so a smaller one is taken from there on
+            const size_t smem = tp.staged ? sizeof(double) * (size_t)(n - j0 + 2) : 0;
+            cudaError_t err;
+            while ((err = cudaLaunchCooperativeKernel((const void*)tri_panel_kernel, dim3(grid), dim3(kTriThreads), args,
+                                                      smem, s)) == cudaErrorCooperativeLaunchTooLarge &&
+                   grid > 1) {
+                (void)cudaGetLastError();
+                sms = (int)(grid = (grid + 1) / 2);
+            }
+            CHFSI_CUDA_TRY(err);
             CHFSI_LAUNCH_CHECK();
             tp.base += grid * (unsigned)(2 * nc - 1);
             const int64_t jn = j0 + nc, mp = n - jn;

@@ -190,3 +190,38 @@ def test_eigh_binding_raises_on_a_matrix_that_is_not_finite(P):
     with pytest.raises(P.ChfsiError) as e:
         P.eigh(torch.as_tensor(A).cuda())
     assert e.value.code == _abi.CHFSI_ERR_NONFINITE
+
+
+@pytest.fixture(scope="module")
+def stream_of_few_sms():
+    """A stream of a green context with the smallest share of the SMs that the driver gives."""
+    torch.cuda.init()
+    torch.zeros(1, device="cuda")
+    cu = ctypes.CDLL("libcuda.so.1")
+    if not hasattr(cu, "cuGreenCtxStreamCreate"):
+        pytest.skip("the driver has no green contexts")
+    ok = lambda rc: rc == 0 or pytest.fail(f"driver error {rc}")
+    resource = ctypes.c_char * 144                       # CUdevResource
+    dev, every, some, rest = ctypes.c_int(), resource(), resource(), resource()
+    groups, desc, ctx, stream = ctypes.c_uint(1), ctypes.c_void_p(), ctypes.c_void_p(), ctypes.c_void_p()
+    ok(cu.cuDeviceGet(ctypes.byref(dev), torch.cuda.current_device()))
+    ok(cu.cuDeviceGetDevResource(dev, every, 1))         # CU_DEV_RESOURCE_TYPE_SM
+    ok(cu.cuDevSmResourceSplitByCount(some, ctypes.byref(groups), every, rest, 0, 1))
+    ok(cu.cuDevResourceGenerateDesc(ctypes.byref(desc), some, 1))
+    ok(cu.cuGreenCtxCreate(ctypes.byref(ctx), desc, dev, 1))
+    ok(cu.cuGreenCtxStreamCreate(ctypes.byref(stream), ctx, 1, 0))
+    yield torch.cuda.ExternalStream(stream.value)
+    torch.cuda.synchronize()
+    ok(cu.cuStreamDestroy_v2(stream))
+    ok(cu.cuGreenCtxDestroy(ctx))
+
+
+@pytest.mark.parametrize("n", [40, 300, 1500])
+def test_eigh_on_a_stream_of_few_sms(P, stream_of_few_sms, n):
+    """The grid of the tridiagonalisation's panels shrinks to what can be resident."""
+    A = _symmetric(n, n)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream_of_few_sms):
+        w, Q = P.eigh(torch.as_tensor(A).cuda())
+        w, Q = w.cpu().numpy(), Q.cpu().numpy()
+    _check(A, w, Q)
