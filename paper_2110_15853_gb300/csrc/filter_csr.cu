@@ -11,12 +11,13 @@
 // beta = 0 is the plain product H X of the subspace projection (step 3), and with
 // (alpha_k, beta_{k+1}) on the adjoint iterates it is the reverse recurrence.
 //
-// Layout: one CTA owns kWarps consecutive rows (one warp per row).  The CTA's
+// Layout: one CTA owns kWarps (or half as many) consecutive rows, one warp per row.  The CTA's
 // slice of the CSR arrays (values and column indices, contiguous because the rows
 // are consecutive) is staged once into shared memory with cp.async and reused for
 // every column chunk of the row.  Lanes own V consecutive columns (vector loads:
 // double2 for FP64, float4 for FP32, 4 x bf16 for the BF16 operand); a chunk is
-// 32 * V * U columns.  Accumulation order over a row's entries is the stored order.
+// 32 * V * U columns.  Accumulation order over a row's entries is the stored order, for every
+// column alike: a column's result has the same bits wherever it stands in the block.
 // Every column index is range-checked while staging; a bad one is replaced by a
 // zero entry and reported in the status word, so no access leaves the buffers.
 #include <type_traits>
@@ -220,16 +221,22 @@ csr_step_body(int64_t N, const int64_t* __restrict__ row_ptr, const int32_t* __r
 
     const int64_t r = r0 + warp;
     if (r < r_end) {
-        int64_t rb = clampp(row_ptr[r]), re = clampp(row_ptr[r + 1]);
-        if (re < rb) { re = rb; bad = true; }
-        if (rb < p_lo || re > p_hi) { rb = re = p_lo; bad = true; }
-        const TH* hv = staged ? s_val + (rb - p_lo) : val + rb;
-        const int32_t* hc = staged ? s_col + (rb - p_lo) : col + rb;
-        const int len = (int)(re - rb);
+        // The entries of row rr (< r_end).
+        auto entries = [&](int64_t rr, const TH*& hv, const int32_t*& hc) -> int {
+            int64_t rb = clampp(row_ptr[rr]), re = clampp(row_ptr[rr + 1]);
+            if (re < rb) { re = rb; bad = true; }
+            if (rb < p_lo || re > p_hi) { rb = re = p_lo; bad = true; }
+            hv = staged ? s_val + (rb - p_lo) : val + rb;
+            hc = staged ? s_col + (rb - p_lo) : col + rb;
+            return (int)(re - rb);
+        };
+        const TH* hv;
+        const int32_t* hc;
+        const int len = entries(r, hv, hc);
         bool nonfinite = false;
 
-        // The output of VV columns from j on, from their sums.
-        auto finish = [&](int64_t j, auto& acc) {
+        // The output of VV columns from j on of row r, from their sums.
+        auto finish = [&](int64_t r, int64_t j, auto& acc) {
             constexpr int VV = sizeof(acc) / sizeof(acc[0]);
             ACC yc[VV], out[VV];
             ldv<ACC, TC, VV>(Yc + r * ldc + j, yc);
@@ -249,70 +256,98 @@ csr_step_body(int64_t N, const int64_t* __restrict__ row_ptr, const int32_t* __r
         };
         if constexpr (std::is_same<ACC, double>::value) {
             // FP64: bound by the pipe, on which an instruction takes the same time whatever its
-            // active lanes, so that the last columns are matched to the warp: W lanes a row
-            // entry, 32 / W entries at once (their sums added at the end), VV columns a lane.
-            // Entries are accumulated in their stored order when W = 32.  Two alternating
-            // buffers: the gathers of the next entry are in flight while one is accumulated; a
-            // bad column index (unstaged rows only) becomes a zero entry on row 0.
-            auto pass = [&](auto vv, auto ww, auto full, int64_t jbase) {
-                constexpr int VV = decltype(vv)::value, W = decltype(ww)::value, kGroups = 32 / W;
+            // active lanes.  Two alternating buffers: the gathers of the next entry are in flight
+            // while one is accumulated; a bad column index (unstaged rows only) becomes a
+            // zero entry on row 0.
+            auto pass = [&](auto vv, auto full, int64_t jbase) {      // 32 VV columns of row r
+                constexpr int VV = decltype(vv)::value;
                 using G = Gathered<ACC, TG, VV>;
-                const int g = lane / W;
-                const int64_t j = jbase + (int64_t)(lane % W) * VV;
+                const int64_t j = jbase + (int64_t)lane * VV;
                 const bool on = decltype(full)::value || j < n;
                 ACC acc[VV];
 #pragma unroll
                 for (int v = 0; v < VV; v++) acc[v] = (ACC)0;
-                if (Ya && on && g == 0) ldv<double, double, VV>(Ya + r * lda + j, acc);
-                auto fetch = [&](int t, G& y, ACC& h) {
-                    const int q = t * kGroups + g;
-                    h = (ACC)0;
-                    y.zero();
-                    if (kGroups > 1 && q >= len) return;
+                if (Ya && on) ldv<double, double, VV>(Ya + r * lda + j, acc);
+                auto fetch = [&](int q, G& y, ACC& h) {
                     int32_t cj = hc[q];
                     h = cvt<ACC>(hv[q]);
+                    y.zero();
                     if (!staged && (cj < 0 || (int64_t)cj >= N)) { bad = true; cj = 0; h = (ACC)0; }
                     if (on) y.load(Yg + (int64_t)cj * ldg + j);
                 };
-                const int steps = (len + kGroups - 1) / kGroups;
                 G ya, yb;
                 ACC ha = (ACC)0, hb = (ACC)0;
-                if (steps > 0) fetch(0, ya, ha);
+                if (len > 0) fetch(0, ya, ha);
                 int t = 0;
-                for (; t + 1 < steps; t += 2) {
+                for (; t + 1 < len; t += 2) {
                     fetch(t + 1, yb, hb);
                     ya.madd(ha, acc);
-                    if (t + 2 < steps) fetch(t + 2, ya, ha);
+                    if (t + 2 < len) fetch(t + 2, ya, ha);
                     yb.madd(hb, acc);
                 }
-                if (t < steps) ya.madd(ha, acc);
+                if (t < len) ya.madd(ha, acc);
+                if (on) finish(r, j, acc);
+            };
+            // The last 16 or 8 columns: W lanes a row, so that a warp takes 32 / W of the CTA's rows at
+            // once (the other warps are done) and an instruction serves them all; every row
+            // still adds its entries in stored order.
+            auto last_columns = [&](auto ww, int64_t jbase) {
+                constexpr int W = decltype(ww)::value, kRows = 32 / W, kAhead = 4;
+                if (r0 + warp * kRows >= r_end) return;
+                const int64_t rr = r0 + warp * kRows + lane / W, j = jbase + lane % W;
+                const TH* lv = hv;
+                const int32_t* lc = hc;
+                const int mine = rr < r_end && j < n ? entries(rr, lv, lc) : 0;
+                const int longest = __reduce_max_sync(0xffffffffu, mine);
+                ACC acc[1] = {(ACC)0};
+                if (Ya && rr < r_end && j < n) ldv<double, double, 1>(Ya + rr * lda + j, acc);
+                Gathered<ACC, TG, 1> y[kAhead];
+                ACC h[kAhead];
+                auto fetch = [&](int q, int b) {
+                    h[b] = (ACC)0;
+                    y[b].zero();
+                    if (q >= mine) return;
+                    int32_t cj = lc[q];
+                    h[b] = cvt<ACC>(lv[q]);
+                    if (!staged && (cj < 0 || (int64_t)cj >= N)) { bad = true; cj = 0; h[b] = (ACC)0; }
+                    y[b].load(Yg + (int64_t)cj * ldg + j);
+                };
 #pragma unroll
-                for (int o = W; o < 32; o <<= 1)
+                for (int b = 0; b < kAhead; b++) fetch(b, b);
+                for (int t = 0; t < longest; t += kAhead) {
 #pragma unroll
-                    for (int v = 0; v < VV; v++) acc[v] += __shfl_xor_sync(0xffffffffu, acc[v], o);
-                if (on && g == 0) finish(j, acc);
+                    for (int b = 0; b < kAhead; b++) {
+                        if (t + b < mine) y[b].madd(h[b], acc);
+                        fetch(t + b + kAhead, b);
+                    }
+                }
+                if (rr < r_end && j < n) finish(rr, j, acc);
             };
             using std::integral_constant;
             // FP64 instructions an entry: 2 for 64 columns, 1 for 32, 1/2 for 16, 1/4 for 8
             // (all 64 columns there: a pass of its own, without the lane test, which made the
-            // compiler spill; 52.55 -> 52.38 ms, 16 steps at 32^3 x 512)
+            // compiler spill; 52.55 -> 52.38 ms, 16 steps at 32^3 x 512).  33 to 48 columns
+            // take 32 and 16 where the rows fill the FP64 pipes, and one pass below 32
+            // rows an SM, where a pass is a chain of gathers: 40 columns and 10 steps on 8000
+            // rows of 300 entries 2.62 -> 2.52 ms, on 1728 rows of 100 0.31 against 0.48 ms.
+            constexpr int64_t kFilled = 5000;
             int64_t j = 0;
             while (j < n) {
                 const int64_t rest = n - j;
                 if (V == 2 && rest >= 64) {
-                    pass(integral_constant<int, V>{}, integral_constant<int, 32>{}, std::true_type{}, j);
+                    pass(integral_constant<int, V>{}, std::true_type{}, j);
                     j += 32 * V;
-                } else if (V == 2 && rest > 48) {
-                    pass(integral_constant<int, V>{}, integral_constant<int, 32>{}, std::false_type{}, j);
+                } else if (V == 2 && rest > (N < kFilled ? 32 : 48)) {
+                    pass(integral_constant<int, V>{}, std::false_type{}, j);
                     j += 32 * V;
                 } else if (rest > 16) {
-                    pass(integral_constant<int, 1>{}, integral_constant<int, 32>{}, std::false_type{}, j);
+                    pass(integral_constant<int, 1>{}, std::false_type{}, j);
                     j += 32;
                 } else if (rest > 8) {
-                    pass(integral_constant<int, 1>{}, integral_constant<int, 16>{}, std::false_type{}, j);
+                    last_columns(integral_constant<int, 16>{}, j);
                     j += 16;
                 } else {
-                    pass(integral_constant<int, 1>{}, integral_constant<int, 8>{}, std::false_type{}, j);
+                    last_columns(integral_constant<int, 8>{}, j);
                     j += 8;
                 }
             }
@@ -368,7 +403,7 @@ csr_step_body(int64_t N, const int64_t* __restrict__ row_ptr, const int32_t* __r
 #pragma unroll
             for (int u = 0; u < U; u++) {
                 if (!on[u]) continue;
-                finish(j0 + u * 32 * V, acc[u]);
+                finish(r, j0 + u * 32 * V, acc[u]);
             }
         }
         }
