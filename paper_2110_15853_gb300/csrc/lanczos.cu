@@ -20,6 +20,9 @@ constexpr int kChunk = 512;          // vector kernels: rows per block, two a th
                                      // of 152 idle at N = 64000)
 constexpr int kUnroll = 4;           // SpMV: entries in flight per lane
 constexpr int kMaxSteps = 64;
+constexpr int kGroups = 256;                        // groups of parts
+constexpr int64_t kMaxPartReads = (int64_t)1 << 22; // by all blocks of a kernel: 32 MB from L2, about the
+                                                    // 5 us of a launch that groups them
 
 // scal layout
 enum {
@@ -121,7 +124,9 @@ __global__ void __launch_bounds__(256) spmv_dot_kernel(int64_t N, const int64_t*
 
 // The sum of nparts partial sums, on every thread: each block of the kernels below adds up
 // the parts that it needs itself, in the same order as every other (a launch of one block
-// for each of the three sums of a step took 6.5 us).
+// for each of the three sums of a step took 6.5 us).  The reads of all blocks grow with N^2,
+// so where there are more than kMaxPartReads of them group_parts_kernel adds up kGroups
+// groups of parts first: 20 steps at 4.2 M rows of 27 entries took 125 ms without it.
 __device__ __forceinline__ double sum_parts(const double* part, int64_t nparts, double* red) {
     __shared__ double total;
     double s = 0.0;
@@ -130,6 +135,27 @@ __device__ __forceinline__ double sum_parts(const double* part, int64_t nparts, 
     if (threadIdx.x == 0) total = t;
     __syncthreads();
     return total;
+}
+
+// out[g][i] = sum over the parts b of group g of part[b][i], i < ncol (cols: ncol rounded up to
+// a power of two), a block per group of consecutive parts, in a fixed order.
+__global__ void __launch_bounds__(256) group_parts_kernel(const double* __restrict__ part, int64_t nparts, int ncol,
+                                                          int cols, double* __restrict__ out, const double* scal) {
+    if (scal && scal[S_STOP] != 0.0) return;
+    __shared__ double red[256];
+    const int i = threadIdx.x & (cols - 1), sub = threadIdx.x / cols, subs = 256 / cols;
+    const int64_t per = (nparts + gridDim.x - 1) / gridDim.x, lo = per * blockIdx.x;
+    const int64_t hi = lo + per < nparts ? lo + per : nparts;
+    double s = 0.0;
+    if (i < ncol)
+#pragma unroll 4
+        for (int64_t b = lo + sub; b < hi; b += subs) s += part[b * ncol + i];
+    red[threadIdx.x] = s;
+    for (int o = 128; o >= cols; o >>= 1) {
+        __syncthreads();
+        if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+    }
+    if ((int)threadIdx.x < ncol) out[(int64_t)blockIdx.x * ncol + threadIdx.x] = red[threadIdx.x];
 }
 
 // alpha_j from the SpMV's parts; w -= alpha_j v_j + beta_{j-1} v_{j-1}; part[b*(j+1) + i] =
@@ -371,7 +397,7 @@ __global__ void bounds_kernel(const double* scal, int64_t N, int64_t n_wanted, d
 
 }  // namespace
 
-// Two sets of parts: the SpMV's (or the norms'), and the dots'.
+// Two sets of parts, the SpMV's (or the norms') and the dots', and one of groups.
 static size_t lanczos_first_parts(int64_t N) {
     const int64_t spmv_blocks = (N + kRowsPerBlock - 1) / kRowsPerBlock, chunks = (N + kChunk - 1) / kChunk;
     return (size_t)((spmv_blocks > chunks ? spmv_blocks : chunks) + 1);
@@ -379,7 +405,23 @@ static size_t lanczos_first_parts(int64_t N) {
 
 size_t lanczos_part_count(int64_t N, int steps) {
     const int64_t chunks = (N + kChunk - 1) / kChunk;
-    return lanczos_first_parts(N) + (size_t)(chunks * (steps + 1)) + S_TOTAL;
+    return lanczos_first_parts(N) + (size_t)(chunks * (steps + 1)) + (size_t)kGroups * kMaxSteps;
+}
+
+// Partial sums for a kernel of `blocks` blocks that each read all of them: `count` x ncol
+// at p, added up in groups first where those reads are too many.
+struct Parts {
+    const double* p;
+    int64_t count;
+};
+static int group_parts(Parts& q, int ncol, int64_t blocks, double* groups, const double* scal, cudaStream_t s) {
+    if (blocks * q.count * ncol <= kMaxPartReads) return CHFSI_OK;
+    int cols = 1;
+    while (cols < ncol) cols *= 2;
+    group_parts_kernel<<<kGroups, 256, 0, s>>>(q.p, q.count, ncol, cols, groups, scal);
+    CHFSI_LAUNCH_CHECK();
+    q = Parts{groups, kGroups};
+    return CHFSI_OK;
 }
 
 int lanczos_run(const CsrDev& h, int steps, const double* v0, int64_t n_wanted, double* V, double* w,
@@ -392,20 +434,31 @@ int lanczos_run(const CsrDev& h, int steps, const double* v0, int64_t n_wanted, 
     const int64_t spmv_blocks = (N + kRowsPerBlock - 1) / kRowsPerBlock;
 
     double* part2 = part + lanczos_first_parts(N);
+    double* groups = part2 + chunks * (steps + 1);
+
     sq_part_kernel<<<(unsigned)chunks, 256, 0, s>>>(N, v0, part);
     CHFSI_LAUNCH_CHECK();
-    norm0_kernel<<<(unsigned)chunks, 256, 0, s>>>(N, v0, V, part, chunks, scal);
+    int rc;
+    Parts q{part, chunks};
+    if ((rc = group_parts(q, 1, chunks, groups, nullptr, s))) return rc;
+    norm0_kernel<<<(unsigned)chunks, 256, 0, s>>>(N, v0, V, q.p, q.count, scal);
     CHFSI_LAUNCH_CHECK();
     for (int j = 0; j < k; j++) {
         const double* vj = V + (int64_t)j * N;
         spmv_dot_kernel<<<(unsigned)spmv_blocks, 256, 0, s>>>(N, h.row_ptr, h.col, val, h.nnz, vj, w, part,
                                                               scal, status);
         CHFSI_LAUNCH_CHECK();
-        three_term_dots_kernel<<<(unsigned)chunks, 256, 0, s>>>(N, w, V, j, part, spmv_blocks, part2, scal);
+        q = Parts{part, spmv_blocks};
+        if ((rc = group_parts(q, 1, chunks, groups, scal, s))) return rc;
+        three_term_dots_kernel<<<(unsigned)chunks, 256, 0, s>>>(N, w, V, j, q.p, q.count, part2, scal);
         CHFSI_LAUNCH_CHECK();
-        reorth_norm_kernel<<<(unsigned)chunks, 256, 0, s>>>(N, w, V, j, part2, chunks, part, scal);
+        q = Parts{part2, chunks};
+        if ((rc = group_parts(q, j + 1, chunks, groups, scal, s))) return rc;
+        reorth_norm_kernel<<<(unsigned)chunks, 256, 0, s>>>(N, w, V, j, q.p, q.count, part, scal);
         CHFSI_LAUNCH_CHECK();
-        scale_next_kernel<<<(unsigned)chunks, 256, 0, s>>>(N, w, V, j, part, chunks, scal);
+        q = Parts{part, chunks};
+        if ((rc = group_parts(q, 1, chunks, groups, scal, s))) return rc;
+        scale_next_kernel<<<(unsigned)chunks, 256, 0, s>>>(N, w, V, j, q.p, q.count, scal);
         CHFSI_LAUNCH_CHECK();
     }
     bounds_kernel<<<1, 64, 0, s>>>(scal, N, n_wanted, dev_out);

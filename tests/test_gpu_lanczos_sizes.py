@@ -1,0 +1,58 @@
+"""The Lanczos bounds over the range of sizes: operators of millions of rows, whose partial
+sums are added up in groups, against the oracle, and the time a row, which must not grow with
+the number of rows."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    from paper_2110_15853_gb300 import build
+    build.build()
+    import paper_2110_15853_gb300 as P
+    return P
+
+
+def _tridiagonal(N):
+    """Rows of two or three entries, columns ascending, on the device."""
+    i = torch.arange(N, device="cuda", dtype=torch.int64)
+    cols = torch.stack((i - 1, i, i + 1), 1)
+    vals = torch.stack((torch.cos(0.5 * (i - 1)), 3.0 + torch.sin(0.1 * i), torch.cos(0.5 * i)), 1).double()
+    keep = (cols >= 0) & (cols < N)
+    rp = torch.zeros(N + 1, dtype=torch.int64, device="cuda")
+    rp[1:] = torch.cumsum(keep.sum(1), 0)
+    return rp, cols[keep].to(torch.int32), vals[keep].contiguous()
+
+
+# the dots are grouped from about 0.1 M rows on (20 steps), the SpMV's parts from 0.26 M
+@pytest.mark.parametrize("N,steps", [(120011, 20), (300000, 20), (1100003, 17), (600001, 33)])
+def test_bounds_of_a_large_operator(P, oracle_mod, N, steps):
+    rp, col, val = _tridiagonal(N)
+    H = dict(N=N, nnz=col.numel(), row_ptr=rp.cpu().numpy(), col=col.cpu().numpy(), val=val.cpu().numpy())
+    v0 = np.random.default_rng(N).standard_normal(N)
+    got = P.lanczos_bounds(P.CsrMatrix(rp, col, val, N), torch.as_tensor(v0).cuda(), steps, N // 100)
+    want = oracle_mod.lanczos_bounds(H, v0, steps, N // 100)
+    assert max(abs(g - w) for g, w in zip(got, want)) <= 1e-10 * max(abs(x) for x in want)
+
+
+def test_time_grows_with_the_rows_and_no_faster(P):
+    """Four times the rows: the traffic of a step is linear in them, so the time grows about four
+    times; half as much again is allowed (sums over all parts in every block made it seven)."""
+    times = []
+    for N in (1 << 20, 1 << 22):
+        rp, col, val = _tridiagonal(N)
+        H, ws = P.CsrMatrix(rp, col, val, N), P.Workspace("cuda")
+        v0 = torch.randn(N, dtype=torch.float64, device="cuda")
+        best = np.inf
+        for _ in range(5):
+            t0, t1 = torch.cuda.Event(True), torch.cuda.Event(True)
+            t0.record()
+            P.lanczos_bounds(H, v0, 20, N // 100, workspace=ws)
+            t1.record()
+            torch.cuda.synchronize()
+            best = min(best, t0.elapsed_time(t1))
+        times.append(best)
+    assert times[1] <= 6.0 * times[0], times
