@@ -14,8 +14,14 @@ namespace chfsi {
 
 namespace {
 
-constexpr int kRowsPerWarp = 4;      // SpMV: rows whose sums a warp adds up together
-constexpr int kRowsPerBlock = 8 * kRowsPerWarp;
+// SpMV: rows whose sums a warp adds up together, 4, or 1 where rows have kLongRow entries and
+// more on average (a sum's six additions a lane are then few beside its entries, and few
+// long rows need all the warps: 20 steps on 5000 rows of 5000 entries 4.73 -> 2.17 ms, on
+// 20000 of 1500 2.48 -> 2.36, while on 64000 of 300 four rows take 2.32 and one row 2.60).
+constexpr int kRowsPerWarp = 4;
+constexpr int64_t kLongRow = 512;
+inline int rows_per_warp(int64_t N, int64_t nnz) { return nnz >= kLongRow * N ? 1 : kRowsPerWarp; }
+inline int64_t spmv_block_count(int64_t N, int rows) { return (N + 8 * rows - 1) / (8 * rows); }
 constexpr int kChunk = 512;          // vector kernels: rows per block, two a thread (2048 left 120 SMs
                                      // of 152 idle at N = 64000)
 constexpr int kUnroll = 4;           // SpMV: entries in flight per lane
@@ -49,25 +55,27 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
     return t;   // valid on thread 0
 }
 
-// w = H v ; part[b] = sum over the block's rows of v[r] w[r].  A warp takes four rows, their
+// w = H v ; part[b] = sum over the block's rows of v[r] w[r].  A warp takes kRows rows, their
 // entries strided over the lanes with kUnroll in flight a lane (the column index, then the
-// gather, are dependent reads), and adds up the four rows' lane sums together: six
+// gather, are dependent reads), and adds up four rows' lane sums together: six
 // FP64 additions a lane where row by row took twenty, half of the FP64 pipe's time on rows of
 // 300 entries (83 -> 64 us at 19.2 M entries; reading them takes 34).
+template <int kRows>
 __global__ void __launch_bounds__(256) spmv_dot_kernel(int64_t N, const int64_t* __restrict__ row_ptr,
                                                        const int32_t* __restrict__ col,
                                                        const double* __restrict__ val, int64_t nnz,
                                                        const double* __restrict__ v, double* w, double* part,
                                                        const double* scal, unsigned* status) {
     if (scal[S_STOP] != 0.0) return;
-    __shared__ double rowdot[kRowsPerBlock];
+    static_assert(kRows == 4 || kRows == 1, "lane sums of four rows, or of one");
+    __shared__ double rowdot[8 * kRows];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t r0 = (int64_t)blockIdx.x * kRowsPerBlock + warp * kRowsPerWarp;
-    int64_t ptr = lane <= kRowsPerWarp && r0 + lane <= N ? row_ptr[r0 + lane] : 0;
-    double s[kRowsPerWarp];
+    const int64_t r0 = (int64_t)blockIdx.x * (8 * kRows) + warp * kRows;
+    int64_t ptr = lane <= kRows && r0 + lane <= N ? row_ptr[r0 + lane] : 0;
+    double s[kRows];
     bool bad = false;
 #pragma unroll
-    for (int q = 0; q < kRowsPerWarp; q++) {
+    for (int q = 0; q < kRows; q++) {
         s[q] = 0.0;
         if (r0 + q >= N) continue;
         int64_t b = __shfl_sync(0xffffffffu, ptr, q), e = __shfl_sync(0xffffffffu, ptr, q + 1);
@@ -94,28 +102,34 @@ __global__ void __launch_bounds__(256) spmv_dot_kernel(int64_t N, const int64_t*
                 if (p + 32 * u < e) s[q] = fma(h[u], x[u], s[q]);
         }
     }
-    // lanes 8 q .. 8 q + 7 end with the sum of row q
-    const bool up16 = lane & 16, up8 = lane & 8;
-    double t0 = up16 ? s[2] : s[0], t1 = up16 ? s[3] : s[1];
-    t0 += __shfl_xor_sync(0xffffffffu, up16 ? s[0] : s[2], 16);
-    t1 += __shfl_xor_sync(0xffffffffu, up16 ? s[1] : s[3], 16);
-    double t = up8 ? t1 : t0;
-    t += __shfl_xor_sync(0xffffffffu, up8 ? t0 : t1, 8);
+    // lanes 8 q .. 8 q + 7 end with the sum of row q (kRows = 1: all lanes with the row's)
+    constexpr int kLanes = 32 / kRows;
+    double t;
+    if constexpr (kRows == 4) {
+        const bool up16 = lane & 16, up8 = lane & 8;
+        double t0 = up16 ? s[2] : s[0], t1 = up16 ? s[3] : s[1];
+        t0 += __shfl_xor_sync(0xffffffffu, up16 ? s[0] : s[2], 16);
+        t1 += __shfl_xor_sync(0xffffffffu, up16 ? s[1] : s[3], 16);
+        t = up8 ? t1 : t0;
+        t += __shfl_xor_sync(0xffffffffu, up8 ? t0 : t1, 8);
+    } else {
+        t = s[0];
+    }
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    for (int o = kRows == 4 ? 4 : 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
     if (__any_sync(0xffffffffu, bad) && lane == 0) raise_status(status, DEV_PATTERN);
-    const int64_t r = r0 + lane / 8;
-    if ((lane & 7) == 0) {
+    const int64_t r = r0 + lane / kLanes;
+    if (lane % kLanes == 0) {
         double d = 0.0;
         if (r < N) {
             w[r] = t;
             d = v[r] * t;
         }
-        rowdot[warp * kRowsPerWarp + lane / 8] = d;
+        rowdot[warp * kRows + lane / kLanes] = d;
     }
     __syncthreads();
     if (warp == 0) {
-        double d = rowdot[lane];
+        double d = lane < 8 * kRows ? rowdot[lane] : 0.0;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
         if (lane == 0) part[blockIdx.x] = d;
@@ -399,7 +413,7 @@ __global__ void bounds_kernel(const double* scal, int64_t N, int64_t n_wanted, d
 
 // Two sets of parts, the SpMV's (or the norms') and the dots', and one of groups.
 static size_t lanczos_first_parts(int64_t N) {
-    const int64_t spmv_blocks = (N + kRowsPerBlock - 1) / kRowsPerBlock, chunks = (N + kChunk - 1) / kChunk;
+    const int64_t spmv_blocks = spmv_block_count(N, 1), chunks = (N + kChunk - 1) / kChunk;
     return (size_t)((spmv_blocks > chunks ? spmv_blocks : chunks) + 1);
 }
 
@@ -431,7 +445,9 @@ int lanczos_run(const CsrDev& h, int steps, const double* v0, int64_t n_wanted, 
     if (k < 1 || k > kMaxSteps) return CHFSI_ERR_ARG;
     const double* val = static_cast<const double*>(h.val);
     const int64_t chunks = (N + kChunk - 1) / kChunk;
-    const int64_t spmv_blocks = (N + kRowsPerBlock - 1) / kRowsPerBlock;
+    const int rows = rows_per_warp(N, h.nnz);
+    const int64_t spmv_blocks = spmv_block_count(N, rows);
+    auto spmv = rows == 1 ? spmv_dot_kernel<1> : spmv_dot_kernel<kRowsPerWarp>;
 
     double* part2 = part + lanczos_first_parts(N);
     double* groups = part2 + chunks * (steps + 1);
@@ -445,8 +461,7 @@ int lanczos_run(const CsrDev& h, int steps, const double* v0, int64_t n_wanted, 
     CHFSI_LAUNCH_CHECK();
     for (int j = 0; j < k; j++) {
         const double* vj = V + (int64_t)j * N;
-        spmv_dot_kernel<<<(unsigned)spmv_blocks, 256, 0, s>>>(N, h.row_ptr, h.col, val, h.nnz, vj, w, part,
-                                                              scal, status);
+        spmv<<<(unsigned)spmv_blocks, 256, 0, s>>>(N, h.row_ptr, h.col, val, h.nnz, vj, w, part, scal, status);
         CHFSI_LAUNCH_CHECK();
         q = Parts{part, spmv_blocks};
         if ((rc = group_parts(q, 1, chunks, groups, scal, s))) return rc;
