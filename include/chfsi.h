@@ -144,14 +144,17 @@ typedef struct {
                                  (chfsi_rayleigh_ritz_ex) its dense products; in a filter
                                  schedule the FP64 steps of a BSR or hybrid operator, its
                                  64 x 64 blocks as Ozaki products (rows of at most 128
-                                 blocks), FP64 iterates and recurrence                   */
+                                 blocks), FP64 iterates and recurrence (the shift c in
+                                 the digits of H's diagonal in block rows where
+                                 |H_ii - c| <= |H_ii| throughout, an FP64 multiply-add
+                                 in the others)                                          */
 #define CHFSI_F40_OZAKI 5     /* filter schedules only, wherever CHFSI_F64_OZAKI steps may
                                  run: the same step with the first five of the seven
                                  slices of each operand (40-bit operands, truncated) and
                                  the 15 slice pairs of weight 2^-48 and above, each term
                                  within about 2^-40 of its row scales (2^16 finer than
                                  FP32) for about half the tensor-core work; FP64 iterates
-                                 and recurrence.  Not in the paper: a precision knob of
+                                 and recurrence, the shift as there.  Not in the paper: a precision knob of
                                  this library, for the early steps of a schedule whose
                                  last steps are CHFSI_F64_OZAKI                          */
 

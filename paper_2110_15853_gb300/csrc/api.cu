@@ -436,7 +436,8 @@ int filter_columns(const FilterRun& R, const double* X, int64_t ldx, double* Y, 
         }
         io.out = f64_buf(k); io.out_t = Buf::F64; io.ldo = f64_ld(k);
         if (oz_tail) {
-            // H's blocks as Ozaki products on the tensor cores, FP64 recurrence
+            // H's blocks (and c, where their digits take it) as Ozaki products on the tensor
+            // cores, FP64 recurrence
             const int slices = R.prec && R.prec[k - 1] == CHFSI_F40_OZAKI ? 5 : 7;
             rc = ozaki_bsr_step(R.bsr64, n, static_cast<const double*>(io.cur), io.ldc,
                                 static_cast<const double*>(io.prev), io.ldp, static_cast<double*>(io.out), io.ldo,

@@ -1372,9 +1372,11 @@ void oz_bsr_layout(Ar& ar, int64_t nbr, int64_t nblocks, int64_t n, OzBsr* out) 
 // not reach) adds nothing to the product and is left out of it.
 // The shift c goes into the digits of the diagonal (of H_ii - c as a two-float sum), so that
 // the step's output need not read Y_cur again nor spend a third FP64 operation an element
-// (8192 outputs an item at two operations a cycle) on it -- where that leaves no grid row
-// of the block row with a larger scale, so that no digit loses weight; other block rows,
-// and those without a stored diagonal block, are marked kUnfolded.
+// (8192 outputs an item at two operations a cycle) on it -- where |H_ii - c| <= |H_ii| for every
+// grid row of the block row, so that no scale grows and the rounding of Y_cur to 56 (40)
+// bits is multiplied by no larger a diagonal than without the shift; other block rows,
+// and those without a stored diagonal block, are marked kUnfolded, and their shift is an
+// FP64 multiply-add on Y_cur itself.
 __global__ void __launch_bounds__(256) oz_bsr_prepare_kernel(const double* __restrict__ val,
                                                              const int32_t* __restrict__ brow_ptr,
                                                              const int32_t* __restrict__ bcol, int64_t nblocks,
@@ -1384,14 +1386,14 @@ __global__ void __launch_bounds__(256) oz_bsr_prepare_kernel(const double* __res
     __shared__ int rowmax[64];
     __shared__ unsigned char flag[kMaxChunks];
     __shared__ int16_t list[kMaxChunks + kStageChunks];
-    __shared__ int kept, padded, grown;
+    __shared__ int kept, padded, larger;
     const int64_t R = blockIdx.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int qb, nq;
     bool bad_ptr = false, bad = false;
     bsr_row_range(brow_ptr, nblocks, R, qb, nq, bad_ptr);
     for (int p = threadIdx.x; p < nq * kBlockChunks; p += 256) flag[p] = 0;
-    if (threadIdx.x == 0) grown = 0;
+    if (threadIdx.x == 0) larger = 0;
     __syncthreads();
     int qd = -1;        // the first diagonal block of the row
     int m[8] = {};      // largest exponent fields, without that block's diagonal
@@ -1426,11 +1428,11 @@ __global__ void __launch_bounds__(256) oz_bsr_prepare_kernel(const double* __res
     const double hii = qd >= 0 ? val[(int64_t)(qb + qd) * 4096 + r * 65] : 0.0;
     const double sd = hii - c, back = sd + c, err = (hii - back) + ((back - sd) - c);   // hii - c = sd + err
     const int ed = (__double2hiint(hii) >> 20) & 0x7ff, es = (__double2hiint(sd) >> 20) & 0x7ff;
-    const int em = rowmax[r], plain = em > ed ? em : ed, shifted = em > es ? em : es;
-    if (threadIdx.x < 64 && shifted > plain) grown = 1;
+    const int em = rowmax[r];
+    if (threadIdx.x < 64 && !(fabs(sd) <= fabs(hii))) larger = 1;
     __syncthreads();
-    const bool fold = qd >= 0 && c != 0.0 && !grown;
-    const int efm = fold ? shifted : plain;
+    const bool fold = qd >= 0 && c != 0.0 && !larger;
+    const int efd = fold ? es : ed, efm = em > efd ? em : efd;
     if (fold && threadIdx.x < kBlockChunks) flag[qd * kBlockChunks + threadIdx.x] = 1;
     __syncthreads();
     if (warp == 0) {
