@@ -57,10 +57,11 @@ __device__ double block_sum(double v) {
 
 // ------------------------------------------------------------------ 0. scale
 
-// The largest exponent field of A's entries (zeroed before) and, from it, the power of two
-// that takes the largest entry into [1/2, 1).  The solver works on that matrix, so that
-// products and squares of its rows neither overflow nor vanish for any finite A, and
-// kNegligible below is a fixed number.  An entry that is not finite is reported here.
+// The largest exponent field of A's entries (zeroed before) and, where the largest entry is not
+// within 2^-64 .. 2^64, the power of two that takes it into [1/2, 1).  Products and squares
+// of the rows of the matrix that the solver works on then neither overflow nor vanish for
+// any finite A, and kNegligible below is a fixed number.  An entry that is not finite is
+// reported here.
 __global__ void __launch_bounds__(256) matrix_exponent_kernel(const double* __restrict__ A, int64_t lda, int64_t n,
                                                               int* emax, unsigned* status) {
     int m = 0;
@@ -76,8 +77,11 @@ __global__ void __launch_bounds__(256) matrix_exponent_kernel(const double* __re
     }
 }
 
-// e of the scale 2^-e (0 where A is zero, subnormal throughout or not finite).
-__device__ __forceinline__ int scale_exponent(const int* emax) { return *emax == 0 || *emax == 0x7ff ? 0 : *emax - 1022; }
+// e of the scale 2^-e (0 also where A is zero, subnormal throughout or not finite).
+__device__ __forceinline__ int scale_exponent(const int* emax) {
+    const int m = *emax, e = m - 1022;
+    return m == 0 || m == 0x7ff || (e >= -64 && e <= 64) ? 0 : e;
+}
 
 // A *= 2^-e (exact unless the result is subnormal).
 __global__ void __launch_bounds__(256) scale_matrix_kernel(double* A, int64_t lda, int64_t n, const int* emax) {
@@ -91,7 +95,8 @@ __global__ void __launch_bounds__(256) scale_matrix_kernel(double* A, int64_t ld
 // w *= 2^e.
 __global__ void unscale_kernel(double* w, int64_t n, const int* emax) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) w[i] = scalbn(w[i], scale_exponent(emax));
+    const int e = scale_exponent(emax);
+    if (i < n && e != 0) w[i] = scalbn(w[i], e);
 }
 
 // ------------------------------------------------------------------ 1. tridiagonalisation
@@ -127,7 +132,7 @@ struct TriScalars {
     int emax;                    // largest exponent field of A
 };
 
-// A rest of x below 1e-140 of A's largest entry (in [1/2, 1)) is left out: with the squares of
+// A rest of x below 1e-140 (A's largest entry is 2^-64 and more) is left out: with the squares of
 // scale = 1 / (x_0 - beta) below, a smaller one would overflow.
 constexpr double kNegligible = 1e-280;
 
@@ -423,18 +428,21 @@ __global__ void __launch_bounds__(kTriThreads) tri_panel_kernel(const __grid_con
     }
 }
 
-// V *= 2^h, W *= 2^-h in the columns of the trailing matrix, before an Ozaki product: V W
-// stays as it is, and both come to the same largest magnitude.  A row of the product's
-// operands holds entries of V and of W under one power-of-two scale, so that the
-// smaller kind loses as many digits as W (of A's norm) and V (of 1's) differ: residuals of
-// 9e-14 |A| for 1500 x 1500 ones with a random part of 1e-3, 1e-14 with FP64 updates, 7e-15
-// with this pass (an eigensolve of 640 rows takes 12.57 ms with it, 12.50 without).
+// V *= 2^h, W *= 2^-h in the columns of the trailing matrix, before an Ozaki product, where their
+// largest magnitudes are 2^4 and more apart: V W stays as it is, and both come to the same
+// size.  A row of the product's operands holds entries of V and of W under one
+// power-of-two scale, so that the smaller kind loses as many of the 56 bits as W (of
+// A's spread) and V (of 1's) differ by.  Three of them leave it at the accuracy of FP64 updates;
+// 1500 x 1500 ones with a random part of 1e-3 left residuals of 9e-14 |A| (FP64 1e-14, with
+// this pass 7e-15).  2 - 3 us a panel.
 __global__ void __launch_bounds__(256) panel_balance_kernel(double* PV, int64_t n, int64_t jn, const int* vwmax) {
+    const int apart = vwmax[0] && vwmax[1] ? vwmax[1] - vwmax[0] : 0, h = apart / 2;
     const int64_t c = jn + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int h = vwmax[0] && vwmax[1] ? (vwmax[1] - vwmax[0]) / 2 : 0;
-    if (h == 0 || c >= n) return;
-    const bool w = blockIdx.y >= kPanel32 && blockIdx.y < 2 * kPanel32;       // rows V, W, V
-    PV[(int64_t)blockIdx.y * n + c] = scalbn(PV[(int64_t)blockIdx.y * n + c], w ? -h : h);
+    if (abs(apart) < 4 || c >= n) return;
+    for (int t = 0; t < 3 * kPanel32; t++) {          // rows V, W, V
+        double* p = PV + (int64_t)t * n + c;
+        *p = scalbn(*p, t / kPanel32 == 1 ? -h : h);
+    }
 }
 
 // The last 2 x 2 (or 1 x 1) block of T.
@@ -1127,14 +1135,14 @@ size_t eigh_ozaki_bytes(int64_t n) {
 template <typename Ar>
 void eigh_layout(Ar& ar, int64_t n, EighBufs* out) {
     EighBufs u{};
-    u.tri = ar.template take<TriScalars>(1);
-    u.vwmax = ar.template take<int>(2 * (size_t)(n / kPanel32 + 1));
     u.d = ar.template take<double>(n);
     u.e = ar.template take<double>(n);
     u.tau = ar.template take<double>(n);
     u.ebak = ar.template take<double>(n);
     u.part = ar.template take<double>(kMaxTriBlocks);
     u.dots = ar.template take<double>(2 * kPanel32);
+    u.tri = ar.template take<TriScalars>(1);
+    u.vwmax = ar.template take<int>(2 * (size_t)(n / kPanel32 + 1));
     u.PV = ar.template take<double>((size_t)(3 * kPanel32) * n);
     u.ybuf = ar.template take<double>(n);
     MergeBufs& b = u.mb;
@@ -1200,8 +1208,8 @@ int eigh(double* A, int64_t lda, int64_t n, double* w, double* Q, int64_t ldq, v
     MergeBufs& mb = u.mb;
     const bool oz = u.oz != nullptr;
 
-    // the scalars and, behind them, the panels' exponents, d, e and tau
-    CHFSI_CUDA_TRY(cudaMemsetAsync(u.tri, 0, (size_t)((char*)(tau + n) - (char*)u.tri), s));
+    // d, e and tau, and with what lies behind them the scalars and the panels' exponents
+    CHFSI_CUDA_TRY(cudaMemsetAsync(u.d, 0, (size_t)((char*)(u.vwmax + 2 * (n / kPanel32 + 1)) - (char*)u.d), s));
     const unsigned rows = (unsigned)std::min<int64_t>(n, 4 * 1024);
     matrix_exponent_kernel<<<rows, 256, 0, s>>>(A, lda, n, &u.tri->emax, status);
     CHFSI_LAUNCH_CHECK();
@@ -1268,8 +1276,7 @@ int eigh(double* A, int64_t lda, int64_t n, double* w, double* Q, int64_t ldq, v
             double* C22 = A + jn * lda + jn;
             int rc;
             if (oz && mp >= kOzakiMinN) {
-                panel_balance_kernel<<<dim3((unsigned)((mp + 255) / 256), 3 * kPanel32), 256, 0, s>>>(u.PV, n, jn,
-                                                                                                     tp.vwmax);
+                panel_balance_kernel<<<(unsigned)((mp + 255) / 256), 256, 0, s>>>(u.PV, n, jn, tp.vwmax);
                 CHFSI_LAUNCH_CHECK();
                 if ((rc = ozaki_gemm_tn(Vop, n, Wop, n, 2 * kPanel32, mp, mp, C22, lda, true, u.oz, u.oz_bytes, status,
                                         s, true)))
