@@ -146,8 +146,8 @@ typedef struct {
                                  64 x 64 blocks as Ozaki products (rows of at most 128
                                  blocks), FP64 iterates and recurrence (the shift c in
                                  the digits of H's diagonal in block rows where
-                                 |H_ii - c| <= |H_ii| throughout, an FP64 multiply-add
-                                 in the others)                                          */
+                                 |H_ii - c| <= 2 |H_ii| throughout, an FP64
+                                 multiply-add in the others)                             */
 #define CHFSI_F40_OZAKI 5     /* filter schedules only, wherever CHFSI_F64_OZAKI steps may
                                  run: the same step with the first five of the seven
                                  slices of each operand (40-bit operands, truncated) and

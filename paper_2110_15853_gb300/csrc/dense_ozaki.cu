@@ -1372,11 +1372,12 @@ void oz_bsr_layout(Ar& ar, int64_t nbr, int64_t nblocks, int64_t n, OzBsr* out) 
 // not reach) adds nothing to the product and is left out of it.
 // The shift c goes into the digits of the diagonal (of H_ii - c as a two-float sum), so that
 // the step's output need not read Y_cur again nor spend a third FP64 operation an element
-// (8192 outputs an item at two operations a cycle) on it -- where |H_ii - c| <= |H_ii| for every
-// grid row of the block row, so that no scale grows and the rounding of Y_cur to 56 (40)
-// bits is multiplied by no larger a diagonal than without the shift; other block rows,
-// and those without a stored diagonal block, are marked kUnfolded, and their shift is an
-// FP64 multiply-add on Y_cur itself.
+// (8192 outputs an item at two operations a cycle) on it -- where, for every grid row of the
+// block row, no scale grows and |H_ii - c| <= 2 |H_ii|, so that the rounding of Y_cur to 56
+// (40) bits is multiplied by at most twice the diagonal that it meets without the shift
+// (c within -1 .. 3 times the diagonal: all rows of the grid operators, whose errors against
+// 64 bits fell with the fold); other block rows, and those without a stored diagonal
+// block, are marked kUnfolded, and their shift is an FP64 multiply-add on Y_cur itself.
 __global__ void __launch_bounds__(256) oz_bsr_prepare_kernel(const double* __restrict__ val,
                                                              const int32_t* __restrict__ brow_ptr,
                                                              const int32_t* __restrict__ bcol, int64_t nblocks,
@@ -1429,7 +1430,7 @@ __global__ void __launch_bounds__(256) oz_bsr_prepare_kernel(const double* __res
     const double sd = hii - c, back = sd + c, err = (hii - back) + ((back - sd) - c);   // hii - c = sd + err
     const int ed = (__double2hiint(hii) >> 20) & 0x7ff, es = (__double2hiint(sd) >> 20) & 0x7ff;
     const int em = rowmax[r];
-    if (threadIdx.x < 64 && !(fabs(sd) <= fabs(hii))) larger = 1;
+    if (threadIdx.x < 64 && (!(fabs(sd) <= 2.0 * fabs(hii)) || es > (em > ed ? em : ed))) larger = 1;
     __syncthreads();
     const bool fold = qd >= 0 && c != 0.0 && !larger;
     const int efd = fold ? es : ed, efm = em > efd ? em : efd;
