@@ -56,6 +56,25 @@ inline int current_device() {
     return d;
 }
 
+// SMs of the current device (kept per device), 0 without one.
+inline int sm_count() {
+    static int cache[kMaxDevices] = {};
+    const int dev = current_device();
+    if (dev < 0) return 0;
+    if (!cache[dev]) {
+        int v = 0;
+        if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+        cache[dev] = v;
+    }
+    return cache[dev];
+}
+// The same for rules that also run where there is no device (workspace sizes): a GB300's
+// 152 there.
+inline int64_t sm_count_or_default() {
+    const int n = sm_count();
+    return n > 0 ? n : 152;
+}
+
 __device__ __forceinline__ void raise_status(unsigned* st, unsigned bits) {
     if (st) atomicOr(st, bits);
 }

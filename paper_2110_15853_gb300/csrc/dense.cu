@@ -161,7 +161,7 @@ __global__ void reduce_parts_kernel(const double* __restrict__ part, int splits,
 int gemm_tile(int64_t M, int64_t Nc, int64_t batches, bool upper) {
     int64_t tm = (M + 63) / 64, tn = (Nc + 63) / 64, tiles = tm * tn;
     if (upper) tiles = tm * (tm + 1) / 2;
-    return tiles * batches < 4 * 152 ? 16 : 64;
+    return tiles * batches < 4 * sm_count_or_default() ? 16 : 64;
 }
 
 int run_gemm(const GemmArgs& g, cudaStream_t s) {
@@ -386,18 +386,19 @@ __global__ void convert_values_kernel(const double* __restrict__ src, float* dst
 }  // namespace
 
 int gemm_tn_splits(int64_t K, int64_t n) {
+    const int64_t sms = sm_count_or_default();
     int64_t tiles = ((n + 63) / 64);
     tiles = tiles * (tiles + 1) / 2;
-    int64_t want = (4 * 152 + tiles - 1) / tiles;        // about four 64 x 64 tiles per SM
+    int64_t want = (4 * sms + tiles - 1) / tiles;        // about four 64 x 64 tiles per SM
     int64_t maxs = (K + 2047) / 2048;                    // keep >= 2048 rows per split
     int64_t s = want < maxs ? want : maxs;
     // fewer tiles than that: 16 x 16 tiles (run_gemm), enough splits for a dozen of them per
     // SM while each keeps 256 rows
-    if (tiles * s < 4 * 152) {
-        const int64_t t = (n + 15) / 16, more = (12 * 152 + t * (t + 1) / 2 - 1) / (t * (t + 1) / 2);
+    if (tiles * s < 4 * sms) {
+        const int64_t t = (n + 15) / 16, more = (12 * sms + t * (t + 1) / 2 - 1) / (t * (t + 1) / 2);
         const int64_t most = (K + 255) / 256, want16 = more < most ? more : most;
         if (want16 > s) s = want16;
-        if (tiles * s >= 4 * 152) s = (4 * 152 - 1) / tiles;
+        if (tiles * s >= 4 * sms) s = (4 * sms - 1) / tiles;
     }
     if (s < 1) s = 1;
     if (s > 64) s = 64;

@@ -1196,7 +1196,7 @@ struct OzPlan {
 
 // M x Nc output, K reduction; tn_form: C = A^T B (split over K), else C = A B.
 template <typename Ar>
-void oz_layout(Ar& ar, bool tn_form, int64_t M, int64_t Nc, int64_t K, bool same, int sms, OzPlan* plan) {
+void oz_layout(Ar& ar, bool tn_form, int64_t M, int64_t Nc, int64_t K, bool same, OzPlan* plan) {
     OzPlan p;
     p.same = same;
     oz_operand_layout(ar, M, K, 1, kTileM, &p.A);
@@ -1204,7 +1204,7 @@ void oz_layout(Ar& ar, bool tn_form, int64_t M, int64_t Nc, int64_t K, bool same
     else oz_operand_layout(ar, Nc, K, 1, kTileN, &p.B);
     if (tn_form) {
         const int64_t tm = (M + kTileM - 1) / kTileM, tn = (Nc + kTileN - 1) / kTileN;
-        p.splits = oz_splits(tm * tn, (int)(p.A.chunks / kStageChunks), sms > 0 ? sms : 148);
+        p.splits = oz_splits(tm * tn, (int)(p.A.chunks / kStageChunks), (int)sm_count_or_default());
         p.part = ar.template take<double>((size_t)p.splits * (tm * kTileM) * (tn * kTileN));
     }
     if (plan) *plan = p;
@@ -1561,7 +1561,7 @@ int ozaki_bsr_step(const BsrDev& h, int64_t n, const double* Yc, int64_t ldc, co
 
 size_t ozaki_workspace_bytes(bool tn_form, int64_t M, int64_t Nc, int64_t K, bool same) {
     CountAr ar;
-    oz_layout(ar, tn_form, M, Nc, K, same, tc::sm_count(), nullptr);
+    oz_layout(ar, tn_form, M, Nc, K, same, nullptr);
     return ar.s.used;
 }
 
@@ -1577,7 +1577,7 @@ int ozaki_gemm_tn(const double* A, int64_t lda, const double* B, int64_t ldb, in
     if (ws_bytes < ozaki_workspace_bytes(true, M, Nc, K, same)) return CHFSI_ERR_NOMEM;
     Arena ar(ws, ws_bytes);
     OzPlan p;
-    oz_layout(ar, true, M, Nc, K, same, tc::sm_count(), &p);
+    oz_layout(ar, true, M, Nc, K, same, &p);
     int rc;
     if ((rc = oz_prepare(A, lda, true, p.A, K, 0, status, s))) return rc;
     if (!same && (rc = oz_prepare(B, ldb, true, p.B, K, 0, status, s))) return rc;
@@ -1591,7 +1591,7 @@ int ozaki_gemm_nn(const double* A, int64_t lda, const double* B, int64_t ldb, in
     if (ws_bytes < ozaki_workspace_bytes(false, M, Nc, K, false)) return CHFSI_ERR_NOMEM;
     Arena ar(ws, ws_bytes);
     OzPlan p;
-    oz_layout(ar, false, M, Nc, K, false, tc::sm_count(), &p);
+    oz_layout(ar, false, M, Nc, K, false, &p);
     int rc;
     if ((rc = oz_prepare(A, lda, false, p.A, K, 0, status, s))) return rc;
     if ((rc = oz_prepare(B, ldb, true, p.B, K, 0, status, s))) return rc;   // B_hat = B^T: rows are B's columns

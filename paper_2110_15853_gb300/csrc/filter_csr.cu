@@ -455,7 +455,7 @@ int launch(const CsrDev& h, const void* hval, int64_t n, const StepIO& io, doubl
     // FP64 on few rows: 4 rows a CTA, for an even share of them on every SM (1728 rows: 432
     // CTAs, at most 3 an SM, where 216 of 8 rows gave some SMs twice the rows of others)
     int warps = kWarps;
-    if (std::is_same<ACC, double>::value && h.N < 152 * 8 * kWarps) {
+    if (std::is_same<ACC, double>::value && h.N < sm_count_or_default() * 8 * kWarps) {
         warps = kWarps / 2;
         cap = kCapMax / 2;
     }

@@ -120,17 +120,5 @@ inline int make_map_bf16(CUtensorMap* map, const void* base, int64_t cols, int64
     return r == CUDA_SUCCESS ? CHFSI_OK : CHFSI_ERR_CUDA;
 }
 
-inline int sm_count() {
-    static int cache[kMaxDevices] = {};
-    const int dev = current_device();
-    if (dev < 0) return 0;
-    if (!cache[dev]) {
-        int v = 0;
-        if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-        cache[dev] = v;
-    }
-    return cache[dev];
-}
-
 }  // namespace tc
 }  // namespace chfsi
