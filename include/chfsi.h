@@ -287,8 +287,8 @@ int chfsi_rayleigh_ritz_workspace_size(const chfsi_matrix* H, int64_t n_cols,
  *      (cholqr_passes = 2 repeats it on X_F: CholQR2);
  *   3. H_F = X_F^T (H X_F);
  *   4. H_F Q = Q Lambda (ascending eigenvalues), by the library's dense eigensolver
- *      (the algorithm of chfsi_eigh, which synchronises `stream` once per merge of
- *      its divide and conquer);
+ *      (the algorithm of chfsi_eigh, which synchronises `stream` once per level of
+ *      merges above 256 rows of its divide and conquer);
  *   5. Psi = X_F Q.
  * With cholqr_passes = 2 the second pass's X_F = X1 R2^-1 is not formed: steps 3 and 5
  * use H_F = R2^-T (X1^T H X1) R2^-1 and Psi = X1 (R2^-1 Q), the same quantities in exact
@@ -312,10 +312,11 @@ int chfsi_rayleigh_ritz_ex_workspace_size(const chfsi_matrix* H, int64_t n_cols,
  * precision = CHFSI_F64 (the same as chfsi_rayleigh_ritz), CHFSI_F32X2
  * (two-float products on the FP32 pipe, about 48 significant bits; needs the CSR
  * layout) or CHFSI_F64_OZAKI (the dense products as chfsi_ozaki_gemm on the BF16
- * tensor cores, about 48 significant bits of the row scales; H X_F in two-float
- * arithmetic on a CSR operator, in FP64 on a BSR one).  The Cholesky
- * factorisation, the triangular inverse and the eigensolve stay FP64 in all
- * three.  Same arguments, errors and synchronisation as chfsi_rayleigh_ritz.
+ * tensor cores, about 48 significant bits of the row scales; H X_F as an Ozaki step on
+ * a BSR or hybrid operator with block rows of at most 128 blocks, in two-float
+ * arithmetic on a CSR one, else in FP64).  The Cholesky factorisation and the triangular
+ * inverse are FP64 in the first two; with CHFSI_F64_OZAKI their products of 256 rows
+ * and more are Ozaki products too.  The eigensolve is chfsi_eigh's in all three.  Same arguments, errors and synchronisation as chfsi_rayleigh_ritz.
  */
 int chfsi_rayleigh_ritz_ex(const chfsi_matrix* H, const double* Y, int64_t ldy, int64_t n_cols,
                            double* Psi, int64_t ldpsi, double* ritz, int32_t cholqr_passes,
@@ -326,7 +327,7 @@ int chfsi_rayleigh_ritz_ex(const chfsi_matrix* H, const double* Y, int64_t ldy, 
 #define CHFSI_OP_TN 0              /* C = A^T B: A is K x M (lda), B is K x Nc (ldb)          */
 #define CHFSI_OP_NN 1              /* C = A B:   A is M x K (lda), B is K x Nc (ldb)          */
 #define CHFSI_GEMM_SYMMETRIC 1     /* TN, M == Nc, C known to be symmetric (Y^T Y, X^T H X):
-                                      the 128 x 128 tiles on and above the diagonal are
+                                      the 128 x 64 tiles that reach the upper triangle are
                                       computed, the others mirrored                          */
 #define CHFSI_GEMM_B_UPPER 2       /* NN, B upper triangular (B[k][j] = 0 for k > j)          */
 
@@ -341,8 +342,8 @@ int chfsi_ozaki_gemm_workspace_size(int32_t op, int64_t M, int64_t Nc, int64_t K
  * balanced 8-bit digits, each digit slice exact in BF16; the 28 slice products
  * with digit weights down to 2^-64 run as tcgen05 MMAs, one FP32 accumulator per digit
  * level, each drained before its sums pass 2^24 units, so that the accumulation is
- * exact (integer multiples, whatever the tensor cores' rounding) and ends in two
- * 64-bit integers per element.  The only errors are the 56-bit rounding of the inputs
+ * exact (integer multiples, whatever the tensor cores' rounding) and ends in one
+ * 96-bit integer per element.  The only errors are the 56-bit rounding of the inputs
  * and the dropped slice pairs: |C_ij - (A_hat B_hat^T)_ij| is below K 2^-50 times the
  * product of the two rows' largest magnitudes (errors of random sign make it about
  * sqrt(K) times that in practice).  Row-major blocks with leading dimensions; C
@@ -368,9 +369,11 @@ int chfsi_eigh_workspace_size(int64_t n, size_t* bytes);
  * (deflation, secular equation by bracketed rational-model steps, eigenvector weights recomputed from the
  * roots), back-transformation in panels of 64 reflectors.  w: n doubles, ascending.
  * Q: n x n (ldq), Q[k * ldq + i] = component k of the eigenvector of w[i].  A is
- * overwritten.  Q must not overlap A.  The call synchronises `stream` once per merge
- * of the divide and conquer.  Workspace (chfsi_eigh_workspace_size): the status word
- * and about 3 n^2 + 200 n doubles.  Errors: CHFSI_ERR_ARG, CHFSI_ERR_NOMEM,
+ * overwritten.  Q must not overlap A.  For 256 <= n <= 8192 the products of 256 rows
+ * and more are FP64-accurate Ozaki products on the tensor cores, and the call
+ * synchronises `stream` once per level of merges above 256 rows of the divide and
+ * conquer.  Workspace (chfsi_eigh_workspace_size): the status word, about 3 n^2 + 435 n
+ * doubles and, for those n, 3.6 n^2 more for the slices.  Errors: CHFSI_ERR_ARG, CHFSI_ERR_NOMEM,
  * CHFSI_ERR_UNSUPPORTED (n above 65535), CHFSI_ERR_CUDA; in the status word
  * CHFSI_ERR_NONFINITE (an entry that is not finite) and CHFSI_ERR_TIMEOUT (a bounded wait
  * that gave up), after which w and Q are undefined.

@@ -931,9 +931,10 @@ int rr_run_f32x2(const chfsi_matrix* H, const double* Y, int64_t ldy, int64_t N,
     return rr_finish(rl, st, s);
 }
 
-// Steps 2, 3 and 5 with the dense products on the tensor cores (Ozaki slices) and
-// H X_F in two-float arithmetic (FP64 on a BSR-only operator); the Cholesky
-// factorisation, the triangular inverse and the eigensolve stay FP64.
+// Steps 2, 3 and 5 with the dense products on the tensor cores (Ozaki slices), those of the
+// Cholesky factorisation, the triangular inverse and the eigensolve from 256 rows on among
+// them, and H X_F as an Ozaki BSR step on 64 x 64 blocks, in two-float arithmetic on a CSR
+// operator, in FP64 on blocks in rows too long for that step.
 int rr_run_ozaki(const chfsi_matrix* H, const double* Y, int64_t ldy, int64_t N, int64_t n, double* Psi,
                  int64_t ldpsi, double* ritz, int passes, bool bsr_hx, const RRLayout& rl, unsigned* st,
                  cudaStream_t s) {

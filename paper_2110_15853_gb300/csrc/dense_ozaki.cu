@@ -91,7 +91,6 @@ constexpr int kThreads = 32 * (4 + kEpiWarps);        // a warpgroup for the pro
 constexpr int kRegsIssue = 88, kRegsEpilogue = 208;
 constexpr uint32_t kTmemCols = 512;
 constexpr int kMaxSlots = 7;
-constexpr int kMaxGroups = 3;                         // accumulator groups, and drains on the way at once
 constexpr int kEvents = 4;                            // barrier pairs of the drains
 static_assert(kColsPerThread == 32, "TMEM loads of 8 columns, batches of 8 and 16");
 
@@ -224,15 +223,15 @@ struct OzArgs {
     // BSR filter-step mode (bsr != 0): A_hat = Y_cur^T (states x grid points), B_hat = the
     // non-zero 8-column chunks of H's 64-row block rows; a work item is one block row
     // (the 64 output columns, grid rows R * 64 ..) against one tile of 128 states, its K
-    // the row's chunks, and the epilogue applies the recurrence
-    // Y_out = alpha (H Y_cur - c Y_cur) - beta Y_prev in FP64 (output in C, ldc).
+    // the row's chunks; the epilogue leaves the products in C (ldc), where the output warps
+    // apply the recurrence Y_out = alpha (H Y_cur - c Y_cur) - beta Y_prev in FP64.
     int bsr;
     int slices;               // digit slices per operand in the products: 7, or 5 (BSR mode)
     const int32_t* brow_ptr;
     const int32_t* hchunk;    // Y_cur chunk of each stored chunk of H (row R from brow_ptr[R] * 8 on)
     const int32_t* hcount;    // stored chunks of each block row (a multiple of kStageChunks),
                               // kUnfolded set where c is not in H's digits
-    int64_t nbr, nblocks;
+    int64_t nblocks;
     const int* expH;          // exponent field of each grid row of H (over its block row)
     const double* Ycur;
     int64_t ldcur;
@@ -246,7 +245,7 @@ constexpr int kUnfolded = 1 << 30;
 
 struct Item {
     int batch, tm, tn, kb0, KB;
-    bool unfolded;            // BSR mode: the epilogue subtracts c Y_cur
+    bool unfolded;            // BSR mode: the output warps subtract c Y_cur
     int64_t qc;               // BSR mode: first stored chunk of the row
 };
 
@@ -561,7 +560,7 @@ __global__ void __launch_bounds__(kThreads, 1) oz_gemm_kernel(const __grid_const
         // elected lane issues.
         // Drain number e uses barrier pair e % kEvents; pend_g is the last drain of group g
         // (five slices: pend1 and pend2 of the two sets of E4-E6), -1 once waited for, so that
-        // at most kMaxGroups drains are on the way.
+        // at most three drains are on the way.
         const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
         const uint32_t ring = __shfl_sync(0xffffffffu, sa(smem), 0);
         const uint32_t leader = elect_one() ? 1u : 0u;
@@ -1175,7 +1174,7 @@ int oz_prepare(const double* src, int64_t ld, bool trans, const OzOperand& o, in
 }
 
 // Split-K count for a product whose output has `tiles` tiles: at most kMaxItemKB
-// K-blocks per work item (the range of the 64-bit accumulators), and enough items
+// K-blocks per work item (the range of the 96-bit sums), and enough items
 // for about one per SM while each split keeps at least 2048 K.
 int oz_splits(int64_t tiles, int kb_total, int sms) {
     const int64_t need = (kb_total + kMaxItemKB - 1) / kMaxItemKB;
@@ -1545,7 +1544,6 @@ int ozaki_bsr_step(const BsrDev& h, int64_t n, const double* Yc, int64_t ldc, co
     g.brow_ptr = h.brow_ptr;
     g.hchunk = b.chunk;
     g.hcount = b.count;
-    g.nbr = h.nbr;
     g.nblocks = h.nblocks;
     g.expH = b.expH;
     g.Ycur = Yc;

@@ -13,8 +13,9 @@
 //      multiplies the subproblem vectors by the eigenvectors of D + rho z z^T;
 //   3. back-transformation Q = Q_H Q_T in panels of 64 reflectors (compact WY form
 //      I - V T V^T, three matrix products per panel).
-// Everything runs in this library's kernels (FP64 on the DFMA pipe); the host only
-// orders the launches.
+// Everything runs in this library's kernels, FP64 on the DFMA pipe or, for the products from
+// 256 rows on, FP64-accurate Ozaki products on the tensor cores; the host orders the
+// launches and reads the merges' sizes.
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -1330,8 +1331,8 @@ int eigh(double* A, int64_t lda, int64_t n, double* w, double* Q, int64_t ldq, v
         dc_gather_kernel<<<cells, 256, 0, s>>>(half, n, Q, ldq, mb);
         CHFSI_LAUNCH_CHECK();
         // Gn (k x kn) = G (k x kn) U (kn x kn), kn <= k the merge's count of non-deflated poles:
-        // FP64 products of all merges in one launch that reads kn on the device, or from
-        // 512 rows on Ozaki products one by one (kn copied to the host, once a level)
+        // FP64 products of all merges in one launch that reads kn on the device, or with more
+        // than kMergeFp64 rows Ozaki products one by one (kn copied to the host, once a level)
         int rc;
         if (oz && k > kMergeFp64) {
             kns.resize(nm);

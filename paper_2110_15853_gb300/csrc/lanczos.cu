@@ -34,8 +34,7 @@ constexpr int64_t kMaxPartReads = (int64_t)1 << 22; // by all blocks of a kernel
 enum {
     S_ALPHA = 0,                 // [kMaxSteps]
     S_BETA = kMaxSteps,          // [kMaxSteps]
-    S_H = 2 * kMaxSteps,         // [kMaxSteps + 1] re-orthogonalisation coefficients
-    S_K = 3 * kMaxSteps + 1,     // number of completed steps (as double)
+    S_K = 2 * kMaxSteps,         // number of completed steps (as double)
     S_STOP = S_K + 1,            // 1.0 after breakdown
     S_SCALE = S_STOP + 1,        // running max |alpha_i| + beta_{i-1}
     S_TOTAL = S_SCALE + 1,
