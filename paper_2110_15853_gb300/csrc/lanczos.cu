@@ -16,10 +16,11 @@ namespace {
 
 // SpMV: rows whose sums a warp adds up together, 4, or 1 where rows have kLongRow entries and
 // more on average (a sum's six additions a lane are then few beside its entries, and few
-// long rows need all the warps: 20 steps on 5000 rows of 5000 entries 4.73 -> 2.17 ms, on
-// 20000 of 1500 2.48 -> 2.36, while on 64000 of 300 four rows take 2.32 and one row 2.60).
+// long rows need all the warps).  20 steps with four rows and with one: 5000 rows of 5000
+// entries 4.73 and 2.17 ms, 8000 of 1500 2.09 and 1.69, 64000 of 1500 5.52 and 5.28; but 64000 of
+// 600 3.05 and 3.21, 262144 of 655 10.4 and 11.3, 64000 of 300 2.32 and 2.60.
 constexpr int kRowsPerWarp = 4;
-constexpr int64_t kLongRow = 512;
+constexpr int64_t kLongRow = 1024;
 inline int rows_per_warp(int64_t N, int64_t nnz) { return nnz >= kLongRow * N ? 1 : kRowsPerWarp; }
 inline int64_t spmv_block_count(int64_t N, int rows) { return (N + 8 * rows - 1) / (8 * rows); }
 constexpr int kChunk = 512;          // vector kernels: rows per block, two a thread (2048 left 120 SMs

@@ -58,9 +58,9 @@ def test_time_grows_with_the_rows_and_no_faster(P):
     assert times[1] <= 6.0 * times[0], times
 
 
-@pytest.mark.parametrize("N", [9, 513, 520, 700])
+@pytest.mark.parametrize("N", [9, 513, 520, 700, 1021, 1024, 1033])
 def test_bounds_of_an_operator_with_long_rows(P, oracle_mod, N):
-    """Dense operators around the row length from which a warp takes one row (512 entries)."""
+    """Dense operators around the row length from which a warp takes one row (1024 entries)."""
     A = np.random.default_rng(N).standard_normal((N, N))
     A = (A + A.T) / 2
     rp = np.arange(N + 1, dtype=np.int64) * N
