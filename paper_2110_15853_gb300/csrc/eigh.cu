@@ -436,14 +436,18 @@ __global__ void __launch_bounds__(kTriThreads) tri_panel_kernel(const __grid_con
 // A's spread) and V (of 1's) differ by.  Three of them leave it at the accuracy of FP64 updates;
 // 1500 x 1500 ones with a random part of 1e-3 left residuals of 9e-14 |A| (FP64 1e-14, with
 // this pass 7e-15).  2 - 3 us a panel.
+constexpr int kBalanceRows = 8;
 __global__ void __launch_bounds__(256) panel_balance_kernel(double* PV, int64_t n, int64_t jn, const int* vwmax) {
     const int apart = vwmax[0] && vwmax[1] ? vwmax[1] - vwmax[0] : 0, h = apart / 2;
     const int64_t c = jn + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (abs(apart) < 4 || c >= n) return;
-    for (int t = 0; t < 3 * kPanel32; t++) {          // rows V, W, V
-        double* p = PV + (int64_t)t * n + c;
-        *p = scalbn(*p, t / kPanel32 == 1 ? -h : h);
-    }
+    const int t0 = blockIdx.y * kBalanceRows;           // rows V, W, V
+    const double f = scalbn(1.0, t0 / kPanel32 == 1 ? -h : h);
+    double x[kBalanceRows];
+#pragma unroll
+    for (int t = 0; t < kBalanceRows; t++) x[t] = PV[(t0 + t) * n + c];
+#pragma unroll
+    for (int t = 0; t < kBalanceRows; t++) PV[(t0 + t) * n + c] = x[t] * f;
 }
 
 // The last 2 x 2 (or 1 x 1) block of T.
@@ -1277,7 +1281,8 @@ int eigh(double* A, int64_t lda, int64_t n, double* w, double* Q, int64_t ldq, v
             double* C22 = A + jn * lda + jn;
             int rc;
             if (oz && mp >= kOzakiMinN) {
-                panel_balance_kernel<<<(unsigned)((mp + 255) / 256), 256, 0, s>>>(u.PV, n, jn, tp.vwmax);
+                panel_balance_kernel<<<dim3((unsigned)((mp + 255) / 256), 3 * kPanel32 / kBalanceRows), 256, 0, s>>>(
+                    u.PV, n, jn, tp.vwmax);
                 CHFSI_LAUNCH_CHECK();
                 if ((rc = ozaki_gemm_tn(Vop, n, Wop, n, 2 * kPanel32, mp, mp, C22, lda, true, u.oz, u.oz_bytes, status,
                                         s, true)))
