@@ -53,9 +53,10 @@
 // (bounded) for its copies and MMAs in flight, frees TMEM and exits.
 //
 // What bounds it: the tensor pipe, at 908 cycles per K = 16 of the 28 slice products (their
-// work is 896) when nothing else runs on the SM; about 1150 in the filter step, since
-// the warps share the issue slots with the drains' conversions (6 of 60 ms) and a
-// drained group's MMAs come in narrower pieces.  20 FP64-accurate steps at 40^3, w = 3, 1024
+// work is 896) when nothing else runs on the SM; over a launch 1240 in a Gram product and
+// 1350 in the filter step (pipe 74% and 66% active), since the warps share the issue slots
+// with the drains' conversions (6 of 60 ms), a drained group's MMAs come in narrower
+// pieces, and an item ends with three drains in turn.  The 40-bit step takes 915 for 480.  20 FP64-accurate steps at 40^3, w = 3, 1024
 // states: 98.0 -> 60.0 ms (0.83 of the chunks, and 1.35 x the rate); 20 40-bit and 4
 // FP64-accurate steps at 48^3, w = 4, 1500 states: 266 -> 161 ms.
 #include <algorithm>
