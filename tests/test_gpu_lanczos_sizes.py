@@ -73,18 +73,21 @@ def test_bounds_of_an_operator_with_long_rows(P, oracle_mod, N):
 
 
 def test_few_long_rows_take_all_the_warps(P):
-    """5000 rows of 5000 entries: twenty steps read 6 GB, 0.9 ms of the memory's rate; a warp
-    for each row takes 2.2 ms, a warp for four rows took 4.7."""
-    N = 5000
-    rp = torch.arange(N + 1, device="cuda", dtype=torch.int64) * N
-    H = P.CsrMatrix(rp, torch.arange(N, device="cuda", dtype=torch.int32).repeat(N),
-                    torch.rand(N * N, dtype=torch.float64, device="cuda"), N)
-    v0, ws, best = torch.randn(N, dtype=torch.float64, device="cuda"), P.Workspace("cuda"), np.inf
-    for _ in range(5):
-        t0, t1 = torch.cuda.Event(True), torch.cuda.Event(True)
-        t0.record()
-        P.lanczos_bounds(H, v0, 20, 50, workspace=ws)
-        t1.record()
-        torch.cuda.synchronize()
-        best = min(best, t0.elapsed_time(t1))
-    assert best <= 3.5, best
+    """25 million entries as 5000 rows of 5000 and as 83333 of 300: the same reads of H, and less of
+    everything else in the first (0.75 of the time; 1.6 with a warp for four of the 5000 rows)."""
+    times = []
+    for N, K in ((83333, 300), (5000, 5000)):
+        rp = torch.arange(N + 1, device="cuda", dtype=torch.int64) * K
+        col = (torch.arange(N, device="cuda")[:, None] + torch.arange(K, device="cuda")) % N
+        H = P.CsrMatrix(rp, col.sort(1)[0].to(torch.int32).reshape(-1), torch.rand(N * K, dtype=torch.float64, device="cuda"),
+                        N)
+        v0, ws, best = torch.randn(N, dtype=torch.float64, device="cuda"), P.Workspace("cuda"), np.inf
+        for _ in range(5):
+            t0, t1 = torch.cuda.Event(True), torch.cuda.Event(True)
+            t0.record()
+            P.lanczos_bounds(H, v0, 20, 50, workspace=ws)
+            t1.record()
+            torch.cuda.synchronize()
+            best = min(best, t0.elapsed_time(t1))
+        times.append(best)
+    assert times[1] <= 1.2 * times[0], times
